@@ -2,8 +2,9 @@
 
 Argument marshalling only: every step of the hot path -- K/V refresh, active-row
 attention, the entropy gate -- runs in the library's kernels.  torch is used for
-device memory and streams.  There is no CPU fallback: importing this package
-without the built library raises.
+device memory and streams.  The entry points called once per layer or per step are
+marshalled by a compiled module (csrc/ec_python.cpp), the rest through ctypes.
+There is no CPU fallback: importing this package without the built library raises.
 
 Functions carry the names of the C entry points declared in
 ``include/entropycache.h``:
@@ -84,6 +85,10 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+try:
+    from . import _ec_python as _native
+except ImportError as e:
+    raise ImportError(f"{e}: build it with `python paper_2603_18489_b200/build.py` (there is no fallback path)") from e
 
 
 def status_string(status: int) -> str:
@@ -160,26 +165,22 @@ def ec_workspace_init(workspace: torch.Tensor, stream=None) -> None:
 
 def ec_kv_refresh(desc: ec_attn_desc, k_cache, v_cache, k_new, v_new, active_idx, stream=None) -> None:
     """k_cache[b, h, active_idx[b, i], :] = k_new[b, i, h, :] (and V), in place, asynchronously."""
-    n_active = int(k_new.shape[1])
-    _check(lib.ec_kv_refresh(ctypes.byref(desc), _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache"),
-                             _dev(k_new, "k_new"), _dev(v_new, "v_new"), _dev(active_idx, "active_idx"),
-                             n_active, _stream(stream)), "ec_kv_refresh")
+    status = _native.kv_refresh(desc, k_cache, v_cache, k_new, v_new, active_idx, stream)
+    if status:
+        raise EcError(status, "ec_kv_refresh")
 
 
 def ec_attend(desc: ec_attn_desc, q, k_new, v_new, k_cache, v_cache, active_idx, out=None,
               workspace=None, dev_status=None, stream=None) -> torch.Tensor:
     """Refresh the active rows (if k_new/v_new are given), then attend from the
     active rows over the whole cache.  Returns `out` [B, n_active, H_q, D]."""
-    n_active = int(q.shape[1])
     if out is None:
         out = torch.empty_like(q)
     if workspace is None:
-        workspace = new_workspace(ec_attend_workspace_bytes(desc, n_active), q.device)
-    _check(lib.ec_attend(ctypes.byref(desc), _dev(q, "q"), _dev(k_new, "k_new"), _dev(v_new, "v_new"),
-                         _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache"), _dev(active_idx, "active_idx"),
-                         n_active, _dev(out, "out"), _dev(workspace, "workspace"),
-                         workspace.numel() * workspace.element_size(), _dev(dev_status, "dev_status"),
-                         _stream(stream)), "ec_attend")
+        workspace = new_workspace(ec_attend_workspace_bytes(desc, int(q.shape[1])), q.device)
+    status = _native.attend(desc, q, k_new, v_new, k_cache, v_cache, active_idx, out, workspace, dev_status, stream)
+    if status:
+        raise EcError(status, "ec_attend")
     return out
 
 
@@ -189,29 +190,13 @@ def ec_entropy_gate(logits, vocab: int, rows_per_seq: int, decoded_flags, tau: f
     """One pass over logits [R, row_stride]: per-row argmax / confidence / entropy,
     per-sequence maximum entropy over the flagged rows and the skip (0) / recompute (1)
     decision.  Outputs are device tensors; nothing is synchronised."""
-    if logits.dim() != 2 or not logits.is_cuda:
-        raise ValueError("logits must be a 2-D CUDA tensor [n_rows, row_stride]")
-    R, stride = int(logits.shape[0]), int(logits.stride(0))
-    dev = logits.device
-    n_seq = R // rows_per_seq if rows_per_seq > 0 else 0
-    if want_rows:
-        argmax_out = torch.empty(R, dtype=torch.int32, device=dev) if argmax_out is None else argmax_out
-        conf_out = torch.empty(R, dtype=torch.float32, device=dev) if conf_out is None else conf_out
-        entropy_out = torch.empty(R, dtype=torch.float32, device=dev) if entropy_out is None else entropy_out
-    if max_entropy_out is None:
-        max_entropy_out = torch.empty(n_seq, dtype=torch.float32, device=dev)
-    if decision_out is None:
-        decision_out = torch.empty(n_seq, dtype=torch.int32, device=dev)
     if workspace is None:
-        workspace = new_workspace(ec_entropy_gate_workspace_bytes(R, vocab), dev)
-    if logits.stride(1) != 1:
-        raise ValueError("logits rows must be contiguous")
-    _check(lib.ec_entropy_gate(ctypes.c_void_p(logits.data_ptr()), _dtype_code(logits), R, int(vocab), stride,
-                               int(rows_per_seq), _dev(decoded_flags, "decoded_flags"), float(tau),
-                               _dev(argmax_out, "argmax_out"), _dev(conf_out, "conf_out"),
-                               _dev(entropy_out, "entropy_out"), _dev(max_entropy_out, "max_entropy_out"),
-                               _dev(decision_out, "decision_out"), _dev(workspace, "workspace"),
-                               workspace.numel() * workspace.element_size(), _stream(stream)), "ec_entropy_gate")
+        workspace = new_workspace(ec_entropy_gate_workspace_bytes(logits.shape[0], vocab), logits.device)
+    status, argmax_out, conf_out, entropy_out, max_entropy_out, decision_out = _native.gate(
+        logits, vocab, rows_per_seq, decoded_flags, tau, argmax_out, conf_out, entropy_out, max_entropy_out,
+        decision_out, workspace, want_rows, stream)
+    if status:
+        raise EcError(status, "ec_entropy_gate")
     return dict(argmax=argmax_out, conf=conf_out, entropy=entropy_out, max_entropy=max_entropy_out,
                 decision=decision_out)
 
@@ -259,19 +244,9 @@ def ec_select_recent(history, state, decoded_flags, window_start, block: int, de
     """Eq. 2-3 and the bookkeeping of Appendix A after the decode of a step (argument marshalling only).
     history int32 [B, L]; state int32 [B, 4]; decoded_flags uint8 [B * block]; window_start, decision int32 [B];
     active_idx int32 [B, n_cap] (out)."""
-    batch, ctx_len = history.shape
-    if history.dtype != torch.int32 or state.dtype != torch.int32 or active_idx.dtype != torch.int32:
-        raise TypeError("history, state and active_idx must be int32")
-    if decoded_flags.dtype != torch.uint8 or window_start.dtype != torch.int32 or decision.dtype != torch.int32:
-        raise TypeError("decoded_flags must be uint8, window_start and decision int32")
-    if tuple(state.shape) != (batch, 4) or active_idx.shape[0] != batch or decoded_flags.numel() != batch * block:
-        raise ValueError("state must be [B, 4], active_idx [B, n_cap], decoded_flags [B * block]")
-    if window_start.numel() != batch or decision.numel() != batch:
-        raise ValueError("window_start and decision must hold one entry per sequence")
-    _check(lib.ec_select_recent(_dev(history, "history"), int(ctx_len), int(batch), _dev(state, "state"),
-                                _dev(decoded_flags, "decoded_flags"), _dev(window_start, "window_start"), int(block),
-                                _dev(decision, "decision"), int(k), _dev(active_idx, "active_idx"),
-                                int(active_idx.shape[1]), _stream(stream)), "ec_select_recent")
+    status = _native.select_recent(history, state, decoded_flags, window_start, block, decision, k, active_idx, stream)
+    if status:
+        raise EcError(status, "ec_select_recent")
 
 
 def ec_entropy_gate_decode(logits, vocab: int, rows_per_seq: int, masked, conf_threshold: float, tau: float, tokens, *,
@@ -279,33 +254,13 @@ def ec_entropy_gate_decode(logits, vocab: int, rows_per_seq: int, masked, conf_t
                            decision_out=None, workspace=None, want_rows: bool = True, stream=None) -> dict:
     """The gate with confidence-based parallel decoding in front of it (argument marshalling only).  `masked`
     (uint8 [R]) and `tokens` (int32 [R]) are updated in place.  Outputs are device tensors; nothing is synchronised."""
-    if logits.dim() != 2:
-        raise ValueError("logits must be [n_rows, row_stride]")
-    n_rows, stride = logits.shape
-    dev = logits.device
-    n_seq = n_rows // rows_per_seq if rows_per_seq > 0 else 0
-    if masked.dtype != torch.uint8 or tokens.dtype != torch.int32 or masked.numel() != n_rows or tokens.numel() != n_rows:
-        raise ValueError("masked must be uint8 [n_rows], tokens int32 [n_rows]")
-    if decoded_out is None:
-        decoded_out = torch.empty(n_rows, dtype=torch.uint8, device=dev)
-    if want_rows:
-        argmax_out = torch.empty(n_rows, dtype=torch.int32, device=dev) if argmax_out is None else argmax_out
-        conf_out = torch.empty(n_rows, dtype=torch.float32, device=dev) if conf_out is None else conf_out
-        entropy_out = torch.empty(n_rows, dtype=torch.float32, device=dev) if entropy_out is None else entropy_out
-    if max_entropy_out is None:
-        max_entropy_out = torch.empty(n_seq, dtype=torch.float32, device=dev)
-    if decision_out is None:
-        decision_out = torch.empty(n_seq, dtype=torch.int32, device=dev)
     if workspace is None:
-        workspace = new_workspace(ec_entropy_gate_workspace_bytes(n_rows, vocab), dev)
-    _check(lib.ec_entropy_gate_decode(_dev(logits, "logits"), _dtype_code(logits), int(n_rows), int(vocab), int(stride),
-                                      int(rows_per_seq), _dev(masked, "masked"), float(conf_threshold), float(tau),
-                                      _dev(decoded_out, "decoded_out"), _dev(tokens, "tokens"),
-                                      _dev(argmax_out, "argmax_out"), _dev(conf_out, "conf_out"),
-                                      _dev(entropy_out, "entropy_out"), _dev(max_entropy_out, "max_entropy_out"),
-                                      _dev(decision_out, "decision_out"), _dev(workspace, "workspace"),
-                                      workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ec_entropy_gate_decode")
+        workspace = new_workspace(ec_entropy_gate_workspace_bytes(logits.shape[0], vocab), logits.device)
+    status, decoded_out, argmax_out, conf_out, entropy_out, max_entropy_out, decision_out = _native.gate_decode(
+        logits, vocab, rows_per_seq, masked, conf_threshold, tau, tokens, decoded_out, argmax_out, conf_out, entropy_out,
+        max_entropy_out, decision_out, workspace, want_rows, stream)
+    if status:
+        raise EcError(status, "ec_entropy_gate_decode")
     return dict(argmax=argmax_out, conf=conf_out, entropy=entropy_out, decoded=decoded_out, max_entropy=max_entropy_out,
                 decision=decision_out)
 
@@ -314,26 +269,14 @@ def ec_entropy_gate_metrics(logits, vocab: int, rows_per_seq: int, decoded_flags
                             stream=None) -> dict:
     """ec_entropy_gate plus the entropy sum and the maximum confidence over the decoded rows (Section 5.3 of the
     paper); argument marshalling only.  Outputs are device tensors; nothing is synchronised."""
-    if logits.dim() != 2:
-        raise ValueError("logits must be [n_rows, row_stride]")
-    n_rows, stride = logits.shape
-    dev = logits.device
-    n_seq = n_rows // rows_per_seq if rows_per_seq > 0 else 0
-    f32 = lambda n: torch.empty(n, dtype=torch.float32, device=dev)
-    out = dict(argmax=torch.empty(n_rows, dtype=torch.int32, device=dev), conf=f32(n_rows), entropy=f32(n_rows),
-               max_entropy=f32(n_seq), decision=torch.empty(n_seq, dtype=torch.int32, device=dev),
-               entropy_sum=f32(n_seq), max_conf=f32(n_seq))
     if workspace is None:
-        workspace = new_workspace(ec_entropy_gate_workspace_bytes(n_rows, vocab), dev)
-    _check(lib.ec_entropy_gate_metrics(_dev(logits, "logits"), _dtype_code(logits), int(n_rows), int(vocab), int(stride),
-                                       int(rows_per_seq), _dev(decoded_flags, "decoded_flags"), float(tau),
-                                       _dev(out["argmax"], "argmax"), _dev(out["conf"], "conf"),
-                                       _dev(out["entropy"], "entropy"), _dev(out["max_entropy"], "max_entropy"),
-                                       _dev(out["decision"], "decision"), _dev(out["entropy_sum"], "entropy_sum"),
-                                       _dev(out["max_conf"], "max_conf"), _dev(workspace, "workspace"),
-                                       workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ec_entropy_gate_metrics")
-    return out
+        workspace = new_workspace(ec_entropy_gate_workspace_bytes(logits.shape[0], vocab), logits.device)
+    status, argmax, conf, entropy, max_entropy, decision, entropy_sum, max_conf = _native.gate_metrics(
+        logits, vocab, rows_per_seq, decoded_flags, tau, workspace, stream)
+    if status:
+        raise EcError(status, "ec_entropy_gate_metrics")
+    return dict(argmax=argmax, conf=conf, entropy=entropy, max_entropy=max_entropy, decision=decision,
+                entropy_sum=entropy_sum, max_conf=max_conf)
 
 
 def ec_select_recent_sliding(history, state, masked, decoded_flags, window: int, decision, k: int, active_idx,
@@ -341,16 +284,6 @@ def ec_select_recent_sliding(history, state, masked, decoded_flags, window: int,
     """ec_select_recent for sliding-window decoding (argument marshalling only).  masked uint8 [B, L] (in/out);
     active_idx int32 [B, n_cap] holds the current window in its first `window` entries on entry and the next row
     list on return."""
-    batch, ctx_len = history.shape
-    if history.dtype != torch.int32 or state.dtype != torch.int32 or active_idx.dtype != torch.int32:
-        raise TypeError("history, state and active_idx must be int32")
-    if masked.dtype != torch.uint8 or decoded_flags.dtype != torch.uint8 or decision.dtype != torch.int32:
-        raise TypeError("masked and decoded_flags must be uint8, decision int32")
-    if tuple(masked.shape) != (batch, ctx_len) or tuple(state.shape) != (batch, 4) or active_idx.shape[0] != batch:
-        raise ValueError("masked must be [B, L], state [B, 4], active_idx [B, n_cap]")
-    if decoded_flags.numel() != batch * window or decision.numel() != batch:
-        raise ValueError("decoded_flags must be [B * window], decision [B]")
-    _check(lib.ec_select_recent_sliding(_dev(history, "history"), int(ctx_len), int(batch), _dev(state, "state"),
-                                        _dev(masked, "masked"), _dev(decoded_flags, "decoded_flags"), int(window),
-                                        _dev(decision, "decision"), int(k), _dev(active_idx, "active_idx"),
-                                        int(active_idx.shape[1]), _stream(stream)), "ec_select_recent_sliding")
+    status = _native.select_recent_sliding(history, state, masked, decoded_flags, window, decision, k, active_idx, stream)
+    if status:
+        raise EcError(status, "ec_select_recent_sliding")

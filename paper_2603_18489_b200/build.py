@@ -1,4 +1,4 @@
-"""Builds libentropycache.so (sm_100a only) in-tree, beside this file.
+"""Builds libentropycache.so (sm_100a only) and its Python marshalling module in-tree, beside this file.
 
     python paper_2603_18489_b200/build.py [--force] [--verbose]
 
@@ -8,6 +8,7 @@ Each .cu under csrc/ is compiled to an object under _build/ (git-ignored) and
 the objects are linked into one shared library with a static CUDA runtime, so
 the library needs nothing but the driver at load time (driver entry points
 are resolved through the runtime, so it also loads on a machine without one).
+csrc/ec_python.cpp becomes _ec_python.so, linked against that library and PyTorch's.
 """
 from __future__ import annotations
 
@@ -16,6 +17,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -23,6 +25,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libentropycache.so")
+PY_SRC = os.path.join(CSRC, "ec_python.cpp")
+PY_LIB = os.path.join(HERE, "_ec_python.so")
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -54,6 +58,29 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_python_module(force: bool, verbose: bool) -> None:
+    if not force and _newer(PY_LIB, [PY_SRC] + glob.glob(os.path.join(INCLUDE, "*.h"))):
+        return
+    import torch                      # for its headers and libraries only
+    t = os.path.dirname(torch.__file__)
+    tmp = PY_LIB + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], "-I", os.path.join(t, "include"),
+           "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), PY_SRC, "-o", tmp,
+           "-L", HERE, "-l:libentropycache.so", "-L", os.path.join(t, "lib"),
+           "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
+    if verbose:
+        print(" ".join(cmd), flush=True)
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode:
+        raise RuntimeError(f"{cmd[0]} failed on {PY_SRC}")
+    os.replace(tmp, PY_LIB)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJDIR, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
@@ -73,6 +100,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
         os.replace(tmp, LIB)
+    _build_python_module(force, verbose)
     return LIB
 
 
