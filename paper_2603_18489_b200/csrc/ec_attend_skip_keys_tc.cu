@@ -13,10 +13,11 @@
 // taken by two auxiliary warps that read P^T back from shared memory (where the softmax threads put it for the
 // second product), so the softmax threads carry no running sums.  With N = 96 (the paper's default budget k = 64
 // gives 96 active rows) two softmax warpgroups share the columns of a key.
-//   softmax  the reference maxima m[q] (log2 units) are shared by all keys of the CTA and live in shared memory.
-//            The common path computes p = 2^(s*scale*log2e - m[q]) with no reduction at all; a barrier-wide OR
-//            tells whether any score exceeds its reference by more than 2^8 (always true on the first tile):
-//            only then the column maxima are reduced, m is raised, and O^T and the row sums are rescaled;
+//   softmax  the references m[q] (log2 units) are shared by all keys of the CTA and live in shared memory.  The first
+//            is the score of one valid key; p = 2^(s*scale*log2e - m[q]) needs no reduction as long as no score exceeds
+//            its reference by more than 2^60 (bf16 and fp32 have room for that, and a reference is never above the true
+//            maximum).  A barrier-wide OR tells: only then the column maxima are reduced, m is raised, and O^T and the
+//            row sums are rescaled;
 //   grid     (C, B*H_kv*n_sub) as clusters of C <= 8 CTAs (any count, not only powers of two) that split one
 //            head's 128-key tiles, chosen so that the most-loaded SM streams the fewest tiles; CTAs that hold a
 //            single tile are small enough for two per SM.  With grouped-query attention the query heads of a kv
@@ -38,21 +39,25 @@
 //            for later steps, ordered against nothing.  (Keys
 //            in a different order, the same sum.)  When a CTA holds a single cache tile the extra tiles get a CTA of
 //            their own, so that nobody streams two tiles through one stage;
-//   merge    CTA c of the cluster owns the output columns d in [c*DL, (c+1)*DL): once every CTA of the cluster is
-//            past its last product (first cluster barrier, arrive early / wait late) each softmax thread puts its
-//            O^T row (one output column, all queries) into a local staging chunk per owner, next to m and l; one
-//            bulk copy per owner moves the chunk into the owner's shared memory and completes on the owner's
-//            mbarrier; the owner combines the C partials, normalises and writes out[b, i, h, d]; a second cluster
-//            barrier keeps every CTA's shared memory alive until its peers have read it.
-// warp 0: TMA producer; warp 1: stale-key masks, then tcgen05.mma issue; next 4 (or 8) warps: softmax; last two
-// warps: cache update and row sums.  Launched with programmatic stream serialisation; global memory is touched only after
-// griddepcontrol.wait.  Every mbarrier wait is bounded (EC_ERR_TIMEOUT in dev_status, CTA-wide abort flag: an
+//   merge    CTA c of the cluster owns the output columns d in [c*DL, (c+1)*DL).  Every CTA leaves its O (un-normalised),
+//            m and l in its own shared memory; after a cluster barrier the owners read their columns of all C partials out
+//            of the peers (128-byte pieces: a warp whose lanes read different rows takes 2.1 us for what this does in 0.6),
+//            combine, normalise and store; a second cluster barrier keeps every CTA's shared memory alive until its
+//            peers have read it.
+// What bounds it: HBM at long contexts (L = 4096, one sequence, 34 rows: 68.8 MB in 17.1 us), the serial path below that:
+// a launch of one tile per CTA takes 7.6 us, of which the dependency wait is 0.8, Q 0.5, the scores 1.2, the softmax
+// 1.2, P V and the row sums 0.7, the merge 1.9 with its barriers and the exit 0.7.  Code that runs once is fetched
+// about as slowly as it runs, so this path is kept short: index arithmetic before the wait, rolled loops in the merge.
+// warp 0: TMA producer; warp 1: tcgen05.mma issue; next 4 (or 8) warps: Q, softmax; the auxiliary warps: stale-key bits,
+// cache update, row sums.  Launched with programmatic stream serialisation; what the previous kernel wrote is read only
+// after griddepcontrol.wait.  Every mbarrier wait is bounded (EC_ERR_TIMEOUT in dev_status, CTA-wide abort flag: an
 // aborted CTA stores no output); the CTA always frees its TMEM and exits.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 namespace ec {
@@ -70,20 +75,27 @@ constexpr uint32_t STAGE = 2 * TILE;       // K tile + V tile: 64 KB
 constexpr int kMaxStages = 6;              // ring slots of one tile (32 KB) each
 constexpr int kMaxSlots = 96;              // query slots (packed rows) of one CTA column
 constexpr int kMaxActive = 256;            // active rows of a sequence (refresh list, row chunks)
-constexpr int kMaxTiles = 1024;            // key tiles of one CTA (bits of the patch mask)
+constexpr int kMaxTiles = 1024;            // key tiles of one CTA
 
 enum { B_FULL = 0, B_EMPTY = kMaxStages, B_SFULL = 2 * kMaxStages, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 1,
-       B_PSUM = B_PVDONE + 1, B_QFULL = B_PSUM + 1, B_LIST = B_QFULL + 1, B_RECV = B_LIST + 1,
-       B_COUNT = B_RECV + 1 };
+       B_PSUM = B_PVDONE + 1, B_QFULL = B_PSUM + 1, B_LIST = B_QFULL + 1, B_COUNT = B_LIST + 1 };
 
 constexpr uint32_t kBarBytes = (B_COUNT * 8u + 15u) & ~15u;   // the barrier block, padded so that what follows is 16-byte aligned
 
-// order-preserving map float -> int (for integer warp reductions of a maximum) and back
-__device__ __forceinline__ int f2ord(float f) {
-    const int i = __float_as_int(f);
-    return i >= 0 ? i : (i ^ 0x7fffffff);
+// A probability may exceed its reference by this power of two before the references are raised: sums and products stay
+// far from the fp32 range, and bf16 carries fp32's exponents, so nothing is lost.
+constexpr float kRaise = 60.f;
+
+// a CTA's partial for the merge: O, m and l
+__host__ __device__ constexpr uint32_t partial_bytes(int n) { return (uint32_t)n * (HD * 4u + 8u); }
+
+// the value is needed here: the compiler reads it now
+template <typename V>
+__device__ __forceinline__ void touch(V v) {
+    if constexpr (sizeof(V) == 8) asm volatile("" ::"l"((unsigned long long)v) : "memory");
+    else if constexpr (std::is_same_v<V, float>) asm volatile("" ::"f"(v) : "memory");
+    else asm volatile("" ::"r"((uint32_t)v) : "memory");
 }
-__device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i : (i ^ 0x7fffffff)); }
 
 // COLS consecutive 32-bit columns of this thread's TMEM lane -> registers (and back).  ALIGNED32: the first column is
 // a multiple of 32 (one 32-column access, then the rest); otherwise 16-column accesses at multiples of 16.
@@ -122,6 +134,8 @@ struct KeysParams {
     int32_t* dev_status;
     int n_active, ctx_len, n_q_heads, n_kv_heads;
     int group;        // query heads of one kv head handled by one CTA column (a divisor of H_q / H_kv)
+    int group_inv;    // ceil(2^16 / group): r / group = (r * group_inv) >> 16 for packed rows r < 256
+    int quads_inv;    // ceil(2^16 / (dl / 4)), for the items of the merge
     int rows_chunk;   // active rows handled by one CTA column (the last chunk may hold fewer)
     int n_sub_r;      // row chunks = ceil(n_active / rows_chunk)
     int n_sub;        // CTA columns per kv head = ((H_q / H_kv) / group) * n_sub_r
@@ -129,10 +143,9 @@ struct KeysParams {
     int shift;        // 1: the first CTA of the cluster takes one cache tile more and the last, which also visits the
                       // fresh tiles, one less (ranges of the CTAs in between move up by one tile)
     int n_extra;      // key tiles of fresh rows attended by the last CTA of every cluster (0: nothing to refresh)
-    int dl;           // output columns merged by one CTA of the cluster (even; the last CTA may own fewer)
-    int q_tma;        // 1: the producer fetches Q with one TMA box (one query head per column); 0: softmax warps stage it
+    int dl;           // output columns merged by one CTA of the cluster (a multiple of 8; the last CTAs may own fewer)
     uint32_t off_p, off_stage, off_list, off_bar;   // shared-memory carve (bytes from the 1024-aligned base); Q is at 0;
-                                                    // off_list: the stale-key bits, 16 bytes per refreshed cache tile
+                                                    // off_list: the stale-key bits, 16 bytes per cache tile
     float scale_log2;
     // Nanoseconds the memory system needs for one stage of every CTA that streams its own K/V: the producer spaces
     // the first fill of its ring by this much per stage, so that the stages of the launch arrive one wave after the
@@ -148,20 +161,18 @@ struct alignas(16) KeysShared {
     uint32_t tmem;
     int abort_flag;
     int pad[2];
-    int slow_flag[2][2];                       // [tile parity][warpgroup]: the softmax of that tile raised its references
-    uint32_t patch_mask[kMaxTiles / 32];       // bit t: cache tile t of this CTA holds a refreshed (stale) position
-    uint16_t slot_base[kMaxTiles / 32];        // refreshed tiles before word w of the mask: tile -> row of the stale-key bits
+    volatile int raised[2];                    // [warpgroup]: the last tile whose softmax raised its references
     alignas(16) float m[kMaxSlots];            // reference maxima of the query rows, log2 units (read as float2)
     alignas(16) float factor[2][kMaxSlots];    // [tile parity]: rescale factors of that tile's slow path
     alignas(16) float lpart[2][kMaxSlots];     // row sums of the CTA's keys, one partial per group of row-sum threads
-    int colmax[4][kMaxSlots];                  // per-warp column maxima (ordered ints) of the current slow path
+    float colmax[4][kMaxSlots];                // per-warp column maxima of the current slow path
 };
 
 template <int N>
 __global__ void __launch_bounds__(64 + (N > 64 ? 256 : 128) + aux_threads(N), N <= 64 ? 2 : 1)
 attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                        const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kn,
-                        const __grid_constant__ CUtensorMap map_vn, const KeysParams p) {
+                        const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
+                        const KeysParams p) {
     static_assert(N == 48 || N == 64 || N == 96, "query-row slots per CTA");
     constexpr int WG = N > 64 ? 2 : 1;          // softmax warpgroups: each takes NH of a key's N scores
     constexpr int NH = N / WG;
@@ -180,7 +191,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     const uint32_t bars = base + p.off_bar;
     KeysShared* sh = reinterpret_cast<KeysShared*>(gbase + p.off_bar + kBarBytes);
     volatile int* abort_flag = &sh->abort_flag;
-    uint32_t* stale = reinterpret_cast<uint32_t*>(gbase + p.off_list);   // [refreshed cache tile][4]: a bit per stale key
+    uint32_t* stale = reinterpret_cast<uint32_t*>(gbase + p.off_list);   // [cache tile][4]: a bit per stale key
     auto bar = [&](int idx) { return bars + idx * 8; };
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -202,12 +213,11 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     const int XT = (refresh && split == p.n_splits - 1) ? p.n_extra : 0;
     const int T = XT + TC;           // tiles this CTA visits: >= 1 by construction of the plan
     const int key_lo = t_begin * BK, key_hi = min(p.ctx_len, t_end * BK);
-    // exchange areas of the merge, from the start of the (then dead) Q / P^T / stage memory: C staging chunks (one per
-    // owner), C receive chunks (one per source).  A chunk holds
-    // [N queries][DL columns] floats of O^T, then m[N], then l[N].
-    const uint32_t chunk_floats = (uint32_t)(N * DL + 2 * N);
-    const uint32_t chunk_bytes = chunk_floats * 4u;
-    const uint32_t stg_off = 0, recv_off = (uint32_t)C * chunk_bytes;
+    // partial of this CTA for the merge, over the (then dead) Q / P^T / stage memory: [query][PITCH] floats of O, then
+    // (m, l)[N]; the peers read it from here
+    constexpr uint32_t PITCH = HD;
+    constexpr uint32_t ML_OFF = N * PITCH * 4;
+    const int own_dl = max(0, min(DL, HD - split * DL));   // output columns this CTA owns (a multiple of 8)
 
     // ---- set-up ------------------------------------------------------------------------------
     // Under programmatic dependent launch this CTA starts while the tail of the previous kernel still runs.  Whatever
@@ -219,8 +229,8 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     if (tid == 0) {
         for (int i = 0; i < B_COUNT; ++i) {
             uint32_t count = 1;
-            if (i == B_PFULL || (i == B_QFULL && !p.q_tma)) count = kSoft;
-            if (i == B_PSUM) count = kAuxThreads;
+            if (i == B_PFULL || i == B_QFULL) count = kSoft;
+            if (i == B_PSUM || i == B_LIST) count = kAuxThreads;
             mbar_init(bar(i), count);
         }
         sh->abort_flag = 0;
@@ -236,15 +246,15 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             prefetch_map(&map_k);
             prefetch_map(&map_v);
         }
-        if (p.q_tma) prefetch_map(&map_q);
         if (p.k_new) {
             prefetch_map(&map_kn);
             prefetch_map(&map_vn);
         }
-        if (C > 1) mbar_expect_tx(bar(B_RECV), (uint32_t)C * chunk_bytes);   // the peers' partials, one chunk each
     }
-    if (tid < kMaxTiles / 32) sh->patch_mask[tid] = 0u;
+    if (refresh)
+        for (int w = tid; w < TC * 4; w += kThreads) stale[w] = 0u;
     if (tid < N) sh->m[tid] = -INFINITY;
+    if (tid < 2) sh->raised[tid] = -1;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s2u(&sh->tmem)), "r"(TM_COLS)
                      : "memory");
@@ -254,30 +264,41 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     __syncthreads();
     fence_after();
     const uint32_t tmem = sh->tmem;
-    pdl_wait();                    // the previous kernel of the stream has completed; global memory may be touched
-    pdl_launch_dependents();
+    // Q: where this thread's 16-byte pieces of the packed rows come from (element offsets; -1: no such row).  Worked out
+    // here, before the wait below, because what follows it is the serial path of a short launch.
+    constexpr int kPieces = N * (HD / 8) / kSoft;
+    int q_off[kPieces];
+    if (warp >= 2 && warp < 2 + 4 * WG) {
+        const int stid = tid - 64;
+#pragma unroll
+        for (int u = 0; u < kPieces; ++u) {
+            const int row = (stid >> 4) + u * (kSoft / 16);
+            const int i = (row * p.group_inv) >> 16, jh = row - i * p.group;
+            q_off[u] = row < rows_total ? ((i0 + i) * p.n_q_heads + hq0 + jh) * HD + (stid & 15) * 8 : -1;
+            touch(q_off[u]);
+        }
+    }
+    const __nv_bfloat16* q_seq = p.q + (long long)b * p.n_active * p.n_q_heads * HD;
+    touch(q_seq);
+    if (warp != 0) pdl_wait();     // the previous kernel of the stream has completed; its results may be read
+    if (tid == 32) pdl_launch_dependents();
+    __syncwarp();
+
+    // First fill of the ring: cache tile j of every CTA is asked for j * stagger_ns after the first, so the first tiles of
+    // all CTAs land before anybody's second, and requests stay queued while they are consumed.  (Asked for all at once,
+    // the tiles of the whole launch arrive together after the time of all of them, and the memory system then idles
+    // until the first slot is free again.)
+    auto pace = [&](int j) {
+        if (j == 0 || j >= TC || !p.stagger_ns) return;
+        const unsigned long long due = t_fill + (unsigned long long)j * p.stagger_ns;
+        while (global_timer_ns() < due) __nanosleep(64);
+    };
 
     if (warp == 0) {
         // ================================ TMA producer ======================================
         if (lane == 0) {
-            if (p.q_tma) {   // Q first: [half][row][64 columns] of this head's rows, rows past n_active read as zero
-                mbar_expect_tx(bar(B_QFULL), (uint32_t)N * 256u);
-                tma_load_5d(base, &map_q, 0, i0, hq0, 0, b, bar(B_QFULL));   // rows past the chunk land in unused slots
-            }
-            const bool first_asked = t_fill != 0;   // ring entry 0 (the first cache tile) is already on its way
-            if (!first_asked) t_fill = global_timer_ns();
-            for (int n = 0; n < 2 * T; ++n) {   // ring entry n: K of tile n / 2 (even n) or its V (odd n)
-                const int j = n >> 1, s = n % NS, u = n / NS;
-                if (first_asked && j == 0) continue;
-                if (u == 0 && !(n & 1) && j > 0 && j < TC && p.stagger_ns) {
-                    // First fill of the ring: cache tile j of every CTA is asked for j * stagger_ns after the first, so
-                    // the first tiles of all CTAs land before anybody's second, and requests stay queued while they
-                    // are consumed.  (Asked for all at once, the tiles of the whole launch arrive together after
-                    // the time of all of them, and the memory system then idles until the first slot is free again.)
-                    const unsigned long long due = t_fill + (unsigned long long)j * p.stagger_ns;
-                    while (global_timer_ns() < due) __nanosleep(64);
-                }
-                if (u > 0) mbar_wait(bar(B_EMPTY + s), (u - 1) & 1, abort_flag, p.dev_status);
+            auto load = [&](int n) {   // ring entry n: K of tile n / 2 (even n) or its V (odd n)
+                const int j = n >> 1, s = n % NS;
                 const uint32_t dst = base + p.off_stage + s * TILE;
                 mbar_expect_tx(bar(B_FULL + s), TILE);
                 if (j >= TC) {   // active rows [128 x, 128 x + 128) of this kv head, fresh; rows past n_active read as zero
@@ -285,74 +306,54 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 } else {
                     tma_load_4d(dst, (n & 1) ? &map_v : &map_k, 0, (t_begin + j) * BK, 0, bh, bar(B_FULL + s));
                 }
+            };
+            int n = 0;
+            if (p.early_cache) {
+                const int fill = min(NS, 2 * TC);
+                for (n = TC > 0 ? 2 : 0; n < fill; ++n) {   // entries 0 and 1 are already on their way
+                    if (!(n & 1)) pace(n >> 1);
+                    load(n);
+                }
+                n = fill;
             }
+            pdl_wait();
+            if (n == 0) t_fill = global_timer_ns();
+            for (; n < 2 * T; ++n) {
+                if (n < NS) { if (!(n & 1)) pace(n >> 1); }
+                else mbar_wait(bar(B_EMPTY + n % NS), (n / NS - 1) & 1, abort_flag, p.dev_status);
+                load(n);
+            }
+        } else {
+            pdl_wait();
         }
+        __syncwarp();
     } else if (warp == 1) {
-        // ================= stale-key masks, then MMA issue (lane 0) =================================
-        if (refresh) {
-            // which cached keys of this CTA's range are about to be refreshed: they are attended from k_new / v_new (as
-            // extra tiles, by the last CTA of the cluster), so their cached copies must not count
-            int posv[kMaxActive / 32];
-#pragma unroll
-            for (int k = 0; k < kMaxActive / 32; ++k) {
-                const int i = k * 32 + lane;
-                posv[k] = -1;
-                if (k * 32 >= p.n_active) continue;   // uniform: nothing of the list left
-                if (i < p.n_active) posv[k] = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
-            }
-#pragma unroll
-            for (int k = 0; k < kMaxActive / 32; ++k) {
-                if (k * 32 >= p.n_active) break;
-                if (posv[k] >= key_lo && posv[k] < key_hi) {
-                    const int tile = (posv[k] - key_lo) / BK;
-                    atomicOr(&sh->patch_mask[tile >> 5], 1u << (tile & 31));
-                }
-            }
-            __syncwarp();
-            {   // rows of the bit table: refreshed tiles in tile order (exclusive prefix count over the mask words)
-                const int cnt = __popc(sh->patch_mask[lane]);
-                int incl = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += v;
-                }
-                sh->slot_base[lane] = (uint16_t)(incl - cnt);
-                const int total = __shfl_sync(0xffffffffu, incl, 31);
-                for (int w = lane; w < total * 4; w += 32) stale[w] = 0u;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < kMaxActive / 32; ++k) {
-                if (k * 32 >= p.n_active) break;
-                if (posv[k] >= key_lo && posv[k] < key_hi) {
-                    const int r = posv[k] - key_lo, tile = r / BK, kk = r % BK;
-                    const int slot = sh->slot_base[tile >> 5] + __popc(sh->patch_mask[tile >> 5] & ((1u << (tile & 31)) - 1u));
-                    atomicOr(&stale[slot * 4 + (kk >> 5)], 1u << (kk & 31));
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_LIST));   // release: the masks above are visible to whoever waits
-            __syncwarp();
-        }
+        // ================================ MMA issue (lane 0) ========================================
         if (lane == 0) {
             constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
             constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
             constexpr uint32_t QHALF = N * 128;                   // bytes of one 64-column half of the Q tile
-            auto issue_s = [&](int j) {
-                const int s = (2 * j) % NS;
+            const uint64_t desc_q = smem_desc(base, 16, 1024), desc_p = smem_desc(base + p.off_p, SUB, 1024);
+            auto products_s = [&](int slot, int buf) {
+                const uint64_t desc_k = smem_desc(base + p.off_stage + slot * TILE, 16, 1024);
                 fence_after();
-                const uint32_t kst = base + p.off_stage + s * TILE;
 #pragma unroll
-                for (int k = 0; k < HD / 16; ++k) {
-                    const uint32_t koff = (k & 3) * 32;
-                    mma_ss(tmem + TM_S + (j & 1) * NP, smem_desc(kst + (k >> 2) * SUB + koff, 16, 1024),
-                           smem_desc(base + (k >> 2) * QHALF + koff, 16, 1024), IDESC_S, k > 0);
-                }
-                commit(bar(B_SFULL + (j & 1)));
-                commit(bar(B_EMPTY + s));   // the K slot is free once these products have run
+                for (int k = 0; k < HD / 16; ++k)
+                    mma_ss(tmem + TM_S + buf * NP, desc_k + ((k >> 2) * SUB + (k & 3) * 32) / 16,
+                           desc_q + ((k >> 2) * QHALF + (k & 3) * 32) / 16, IDESC_S, k > 0);
             };
-            // S of tile j needs the tile (and its patch); P V of tile j needs P^T from the softmax.  Whichever is ready
+            auto products_pv = [&](int slot, bool accumulate) {
+                const uint64_t desc_v = smem_desc(base + p.off_stage + slot * TILE, SUB, 1024);
+                fence_after();
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k)
+                    mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (accumulate || k > 0));
+            };
+            // Both products once on whatever shared memory holds, before there is anything to do: the results are
+            // overwritten (S of tile 1, the first P V), but the code has been fetched when the first tile needs it.
+            products_s(0, 1);
+            products_pv(0, false);
+            // S of tile j needs the tile; P V of tile j needs P^T from the softmax.  Whichever is ready
             // is issued: P V of a tile does not wait for the next tile to land (its commit frees the stage for the
             // producer), S may run one tile ahead of P V (two S^T buffers).
             mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
@@ -360,22 +361,20 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             SpinGuard guard;
             while (next_pv < T) {
                 bool progressed = false;
-                if (next_s < T && next_s <= next_pv + 1 && mbar_try(bar(B_FULL + (2 * next_s) % NS), ((2 * next_s) / NS) & 1)) {
-                    issue_s(next_s);   // (the tile has landed)
+                if (next_s < T && next_s <= next_pv + 1 && mbar_test(bar(B_FULL + (2 * next_s) % NS), ((2 * next_s) / NS) & 1)) {
+                    const int s = (2 * next_s) % NS;
+                    products_s(s, next_s & 1);   // (the tile has landed)
+                    commit(bar(B_SFULL + (next_s & 1)));
+                    commit(bar(B_EMPTY + s));    // the K slot is free once these products have run
                     ++next_s;
                     progressed = true;
                 }
-                if (mbar_try(bar(B_PFULL), next_pv & 1) &&
-                    mbar_try(bar(B_FULL + (2 * next_pv + 1) % NS), ((2 * next_pv + 1) / NS) & 1)) {   // P^T is there, V has landed
-                    const int j = next_pv;
-                    const uint32_t vst = base + p.off_stage + ((2 * j + 1) % NS) * TILE;
-                    fence_after();
-#pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        mma_ss(tmem + TM_O, smem_desc(vst + k * 2048, SUB, 1024), smem_desc(base + p.off_p + k * 2048, SUB, 1024),
-                               IDESC_PV, (j > 0 || k > 0));
+                if (mbar_test(bar(B_PFULL), next_pv & 1) &&
+                    mbar_test(bar(B_FULL + (2 * next_pv + 1) % NS), ((2 * next_pv + 1) / NS) & 1)) {   // P^T is there, V has landed
+                    const int s = (2 * next_pv + 1) % NS;
+                    products_pv(s, next_pv > 0);
                     commit(bar(B_PVDONE));
-                    commit(bar(B_EMPTY + (2 * j + 1) % NS));
+                    commit(bar(B_EMPTY + s));
                     ++next_pv;
                     progressed = true;
                 }
@@ -384,8 +383,17 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             }
         }
     } else if (warp >= 2 + 4 * WG) {
-        // ===== auxiliary warps: the fresh rows into the cache (for later steps); row sums of P^T =====
+        // ===== auxiliary warps: stale-key bits; the fresh rows into the cache (for later steps); row sums of P^T =====
         const int atid = tid - (64 + kSoft);
+        if (refresh) {
+            // which cached keys of this CTA's range are about to be refreshed: they are attended from k_new / v_new (as
+            // extra tiles, by the last CTA of the cluster), so their cached copies must not count
+            for (int i = atid; i < p.n_active; i += kAuxThreads) {
+                const int r = (p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i) - key_lo;
+                if (r >= 0 && r < key_hi - key_lo) atomicOr(&stale[r >> 5], 1u << (r & 31));
+            }
+            mbar_arrive(bar(B_LIST));   // release: the bits above are visible to whoever waits
+        }
         // row sums: this thread adds up column pair cp of the keys [k_lo, k_lo + BK / kParts) of every tile
         const bool summer = atid < kPairs * kParts;
         const int cp = atid % kPairs, col = 2 * cp, gch = col >> 3;
@@ -399,7 +407,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 // rows' K/V into the cache, for later steps: the fresh tile is in shared memory once its stage is full,
                 // so the rows leave from there as plain 16-byte stores (thread = one 16-byte piece of a row, four rows
                 // per pass; the tile is 128-byte swizzled).  Nothing in this launch depends on these stores.  The stage
-                // is overwritten (by the merge's exchange areas) only after the row sums of the last visit, which this
+                // is overwritten (by the partial of the merge) only after the row sums of the last visit, which this
                 // thread reports after it has read its pieces.  (One TMA store per row and half took 3.5 us for 34
                 // rows: 136 requests of 128 bytes, served one after the other.)
                 const int x = j - TC;
@@ -422,7 +430,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             // P^T of tile j is in shared memory
             mbar_wait(bar(B_PFULL), j & 1, abort_flag, p.dev_status);
             if (summer) {
-                if (sh->slow_flag[j & 1][col / NH]) {   // the references of these columns were raised at this tile
+                if (sh->raised[col / NH] == j) {   // the references of these columns were raised at this tile
                     acc0 *= sh->factor[j & 1][col];
                     acc1 *= sh->factor[j & 1][col + 1];
                 }
@@ -444,25 +452,28 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             mbar_arrive(bar(B_PSUM));   // P^T of tile j has been read (release: the row sums above are visible)
         }
     } else {
-        // ================== Q staging (grouped heads), softmax (warps 2 ..) ========================
+        // ================================ Q, softmax (warps 2 ..) ===================================
         const int stid = tid - 64;
         const int wg = stid >> 7;                    // warpgroup: columns [wg * NH, (wg + 1) * NH) of every key
         const int c0 = wg * NH;
         const int st_w = stid & 127;
         constexpr uint32_t QHALF = N * 128;
-        // Q rows of this kv head -> swizzled K-major tile of N rows (rows past rows_total are zero)
-        for (int c = stid; c < (p.q_tma ? 0 : N * (HD / 8)); c += kSoft) {
-            const int row = c >> 4, ch = c & 15;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (row < rows_total) {
-                const int i = i0 + row / p.group, jh = row % p.group;
-                v = __ldg(reinterpret_cast<const uint4*>(
-                    p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hq0 + jh) * HD + ch * 8));
+        // Q rows of this kv head -> swizzled K-major tile of N rows (rows past rows_total are zero): all of a thread's
+        // loads are issued before the first is stored
+        {
+            const int ch = stid & 15;
+            uint4 v[kPieces];
+#pragma unroll
+            for (int u = 0; u < kPieces; ++u) {
+                v[u] = make_uint4(0u, 0u, 0u, 0u);
+                ldg_nc_v4_pred(v[u], q_seq + q_off[u], q_off[u] >= 0);
             }
-            const uint32_t off = (ch >> 3) * QHALF + (row >> 3) * 1024 + (row & 7) * 128 + (((ch & 7) ^ (row & 7)) << 4);
-            *reinterpret_cast<uint4*>(gbase + off) = v;
-        }
-        if (!p.q_tma) {
+#pragma unroll
+            for (int u = 0; u < kPieces; ++u) {
+                const int row = (stid >> 4) + u * (kSoft / 16);
+                const uint32_t off = (ch >> 3) * QHALF + (row >> 3) * 1024 + (row & 7) * 128 + (((ch & 7) ^ (row & 7)) << 4);
+                *reinterpret_cast<uint4*>(gbase + off) = v[u];
+            }
             fence_async_smem();     // Q (generic proxy) -> visible to the tensor core (async proxy)
             mbar_arrive(bar(B_QFULL));
         }
@@ -496,59 +507,63 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             if (j >= TC) {
                 past_end = !((fresh_ok >> (j - TC)) & 1u);
             } else {
-                const int t = j;
-                past_end = (t_begin + t) * BK + kk >= p.ctx_len;
+                past_end = (t_begin + j) * BK + kk >= p.ctx_len;
                 if (!masks_ready) {
                     mbar_wait(bar(B_LIST), 0, abort_flag, p.dev_status);
                     masks_ready = true;
                 }
-                if (refresh && ((sh->patch_mask[t >> 5] >> (t & 31)) & 1u)) {
-                    const int slot = sh->slot_base[t >> 5] + __popc(sh->patch_mask[t >> 5] & ((1u << (t & 31)) - 1u));
-                    past_end = past_end || ((stale[slot * 4 + (kk >> 5)] >> (kk & 31)) & 1u);
-                }
+                if (refresh) past_end = past_end || ((stale[j * 4 + (kk >> 5)] >> (kk & 31)) & 1u);
             }
-            // d = s * scale * log2(e) - m[q]; does any score exceed its reference by more than 2^8?
+            if (j == 0) {
+                // First reference: the scores of the first valid key among the first warp's 32 (any key that counts
+                // will do: a reference is never above the true maximum, and probabilities may exceed it by 2^kRaise).
+                if (quarter == 0) {
+                    uint32_t sr[NH];
+                    ld_row<NH, WG == 1>(s_addr, sr);
+                    const uint32_t valid = __ballot_sync(0xffffffffu, !past_end);
+                    if (lane == __ffs(valid) - 1) {
+#pragma unroll
+                        for (int c = 0; c < NH; c += 4)
+                            *reinterpret_cast<float4*>(&sh->m[c0 + c]) =
+                                make_float4(__uint_as_float(sr[c]) * sl2, __uint_as_float(sr[c + 1]) * sl2,
+                                            __uint_as_float(sr[c + 2]) * sl2, __uint_as_float(sr[c + 3]) * sl2);
+                    }
+                }
+                named_barrier(bar_sync, 128);
+            }
+            // d = s * scale * log2(e) - m[q]; does any score exceed its reference by more than 2^kRaise?
             f32x2 d2[NH / 2];
-            auto load_d = [&]() {
+            while (true) {
                 uint32_t sr[NH];
                 ld_row<NH, WG == 1>(s_addr, sr);
+                float dmx0 = -INFINITY, dmx1 = -INFINITY;
 #pragma unroll
                 for (int i = 0; i < NH / 2; ++i) {
                     const float2 mm = *reinterpret_cast<const float2*>(&sh->m[c0 + 2 * i]);
                     d2[i] = fma2(pk(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), sl2_2, pk(-mm.x, -mm.y));
                     if (past_end) d2[i] = pk(-INFINITY, -INFINITY);   // probability 0 for every query
+                    float d0, d1;
+                    upk(d2[i], d0, d1);
+                    if (i & 1) dmx1 = max3(dmx1, d0, d1); else dmx0 = max3(dmx0, d0, d1);
                 }
-            };
-            load_d();
-            float dmx0 = -INFINITY, dmx1 = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < NH / 2; ++i) {
-                float d0, d1;
-                upk(d2[i], d0, d1);
-                if (i & 1) dmx1 = max3(dmx1, d0, d1); else dmx0 = max3(dmx0, d0, d1);
-            }
-            const bool slow = named_barrier_or(bar_or, 128, fmaxf(dmx0, dmx1) > 8.f);
-            if (st_w == 0) sh->slow_flag[j & 1][wg] = slow ? 1 : 0;   // for the row-sum threads (read after "P full")
-            if (slow) {
+                if (!named_barrier_or(bar_or, 128, fmaxf(dmx0, dmx1) > kRaise)) break;
                 // ---- rare path: raise the references to the column maxima of this tile, rescale O^T (the row-sum
-                //      threads rescale their sums by the same factors) ----
-                {
-                    uint32_t sr[NH];   // the raw scores once more (they stay in tensor memory until S of tile j + 2)
-                    ld_row<NH, WG == 1>(s_addr, sr);
+                //      threads rescale their sums by the same factors), and once more ----
+                ld_row<NH, WG == 1>(s_addr, sr);
 #pragma unroll
-                    for (int c = 0; c < NH; ++c) {
-                        const int o = __reduce_max_sync(0xffffffffu, f2ord(past_end ? -INFINITY : __uint_as_float(sr[c])));
-                        if (lane == (c & 31)) sh->colmax[quarter][c0 + c] = o;
-                    }
+                for (int c = 0; c < NH; ++c) {
+                    const float o = redux_max(past_end ? -INFINITY : __uint_as_float(sr[c]));
+                    if (lane == (c & 31)) sh->colmax[quarter][c0 + c] = o;
                 }
                 named_barrier(bar_sync, 128);
                 if (st_w < NH) {
                     const int c = c0 + st_w;
-                    const int o = max(max(sh->colmax[0][c], sh->colmax[1][c]), max(sh->colmax[2][c], sh->colmax[3][c]));
+                    const float o = fmaxf(fmaxf(sh->colmax[0][c], sh->colmax[1][c]), fmaxf(sh->colmax[2][c], sh->colmax[3][c]));
                     const float m_old = sh->m[c];
-                    const float m_new = fmaxf(m_old, ord2f(o) * sl2);
+                    const float m_new = fmaxf(m_old, o * sl2);
                     sh->factor[j & 1][c] = (m_old == -INFINITY) ? 0.f : fast_exp2(m_old - m_new);
                     sh->m[c] = m_new;
+                    if (st_w == 0) sh->raised[wg] = j;   // for the row-sum threads (read after "P full")
                 }
                 named_barrier(bar_sync, 128);
                 if (j > 0) {   // O^T holds the tiles before j: P V of tile j - 1 must have completed
@@ -561,7 +576,6 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                     for (int c = 0; c < NH; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * sh->factor[j & 1][c0 + c]);
                     st_row<NH, WG == 1>(o_addr, o);
                 }
-                load_d();   // against the raised references
             }
             uint32_t pw[NH / 2];
 #pragma unroll
@@ -587,16 +601,11 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         }
         mbar_wait(bar(B_PVDONE), (T - 1) & 1, abort_flag, p.dev_status);   // Q, P^T and the K/V stages are dead from here on
         fence_after();
-        if (C > 1) {
-            // first cluster barrier, arrive half: the peers may write their partials into this CTA's receive chunks
-            // (nothing is published by it, so no memory ordering is attached)
-            __syncwarp();
-            cluster_arrive_relaxed();
-        }
-        mbar_wait(bar(B_PSUM), (T - 1) & 1, abort_flag, p.dev_status);     // the row sums are complete
-
         uint32_t o[NH];
         ld_row<NH, WG == 1>(tmem + lane_addr + TM_O + c0, o);
+        fence_before();
+        named_arrive(7, kSoft + 32);   // tensor memory has been read: the MMA warp may free it
+        mbar_wait(bar(B_PSUM), (T - 1) & 1, abort_flag, p.dev_status);     // the row sums are complete
         if (C == 1) {
             // ---- single CTA per (sequence, kv head): normalise and store column kk of every query row ----
             if (!*abort_flag) {
@@ -604,130 +613,86 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 for (int c = 0; c < NH; ++c) {
                     if (c0 + c < rows_total) {
                         const float l = sh->lpart[0][c0 + c] + (kParts == 2 ? sh->lpart[1][c0 + c] : 0.f);
-                        const int i = i0 + (c0 + c) / p.group, jh = (c0 + c) % p.group;
-                        __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hq0 + jh) * HD;
+                        const int i = ((c0 + c) * p.group_inv) >> 16, jh = c0 + c - i * p.group;
+                        __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i0 + i) * p.n_q_heads + hq0 + jh) * HD;
                         dst[kk] = __float2bfloat16_rn(__uint_as_float(o[c]) / l);
                     }
                 }
             }
         } else {
-            // ---- this thread's O^T row (output column kk, its warpgroup's queries) -> the staging chunk of the
-            //      CTA that owns column kk; consecutive lanes write consecutive words ----
-            float* stg = reinterpret_cast<float*>(gbase + stg_off) + (kk / DL) * chunk_floats + (kk % DL);
+            // ---- this thread's O^T row (output column kk, its warpgroup's queries), m and l into this CTA's partial:
+            //      consecutive lanes write consecutive words ----
+            float* part = reinterpret_cast<float*>(gbase) + kk;
 #pragma unroll
             for (int c = 0; c < NH; ++c)
-                if (c0 + c < rows_total) stg[(c0 + c) * DL] = __uint_as_float(o[c]);
-            if (st_w < NH) {   // every owner also gets this CTA's m[q] and l[q]
+                if (c0 + c < rows_total) part[(c0 + c) * PITCH] = __uint_as_float(o[c]);
+            if (st_w < NH) {
                 const int c = c0 + st_w;
                 const float l = sh->lpart[0][c] + (kParts == 2 ? sh->lpart[1][c] : 0.f);
-                for (int ow = 0; ow < C; ++ow) {
-                    float* ml = reinterpret_cast<float*>(gbase + stg_off) + ow * chunk_floats + N * DL;
-                    ml[c] = sh->m[c];
-                    ml[N + c] = l;
-                }
-            }
-            fence_async_smem();   // staging (generic proxy) -> bulk copies (async proxy)
-            named_barrier(6, kSoft);
-            __syncwarp();
-            cluster_wait();       // every CTA of the cluster is past its main loop
-            if (stid < C) {       // one bulk copy per owner into the owner's receive chunk of this source
-                const uint32_t src = base + stg_off + (uint32_t)stid * chunk_bytes;
-                const uint32_t dst = map_to_cta(base + recv_off + (uint32_t)split * chunk_bytes, stid);
-                bulk_copy_to_peer(dst, src, chunk_bytes, map_to_cta(bar(B_RECV), stid));
+                *reinterpret_cast<float2*>(gbase + ML_OFF + c * 8) = make_float2(sh->m[c], l);
             }
         }
     }
-
-    if (C > 1) {
-        if (!(warp >= 2 && warp < 2 + 4 * WG)) {   // the other warps' halves of the first cluster barrier
-            __syncwarp();
-            cluster_arrive_relaxed();
-            cluster_wait();
-        }
-        // ---- merge the C partials of the output columns this CTA owns -------------------------
-        mbar_wait(bar(B_RECV), 0, abort_flag, p.dev_status);
-        // second cluster barrier, arrive half: this CTA holds every peer's partial, so the peers' copies out of their
-        // staging chunks have completed; the wait half, before leaving, overlaps the merge
-        __syncwarp();
-        cluster_arrive_relaxed();
-        const float* recv = reinterpret_cast<const float*>(gbase + recv_off);
-        // a thread owns two adjacent output columns of a query row (one 4-byte store) and works out the row's weights
-        // 2^(m_s - m) / l itself: the sixteen or so threads of a row repeat that, but nobody waits for a table
-        const int own_dl = min(DL, HD - split * DL);   // output columns this CTA owns (even)
-        if (!*abort_flag && (DL & 3) == 0 && (own_dl & 3) == 0) {
-            // four adjacent output columns of a query row per item (one 8-byte store)
-            const int quads = own_dl / 4;
-            for (int idx = tid; idx < rows_total * quads; idx += kThreads) {
-                const int qq = idx / quads, dq = idx % quads;
-                float m = -INFINITY;
-#pragma unroll
-                for (int s = 0; s < 8; ++s)
-                    if (s < C) m = fmaxf(m, recv[s * chunk_floats + N * DL + qq]);
-                float l = 0.f;
-                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    if (s < C) {
-                        const float* ch = recv + s * chunk_floats;
-                        const float e = fast_exp2(ch[N * DL + qq] - m);
-                        const float4 v = *reinterpret_cast<const float4*>(ch + qq * DL + 4 * dq);
-                        l = fmaf(e, ch[N * DL + N + qq], l);
-                        a.x = fmaf(e, v.x, a.x);
-                        a.y = fmaf(e, v.y, a.y);
-                        a.z = fmaf(e, v.z, a.z);
-                        a.w = fmaf(e, v.w, a.w);
-                    }
-                }
-                const float inv = 1.f / l;
-                const int i = i0 + qq / p.group, jh = qq % p.group;
-                __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hq0 + jh) * HD + split * DL + 4 * dq;
-                *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(a.z * inv, a.w * inv));
-            }
-        } else if (!*abort_flag) {
-            const int half_dl = own_dl / 2;
-            for (int idx = tid; idx < rows_total * half_dl; idx += kThreads) {
-                const int qq = idx / half_dl, dp = idx % half_dl;
-                float ms[8], ls[8];
-                float2 v[8];
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    if (s < C) {
-                        const float* ch = recv + s * chunk_floats;
-                        ms[s] = ch[N * DL + qq];
-                        ls[s] = ch[N * DL + N + qq];
-                        v[s] = *reinterpret_cast<const float2*>(ch + qq * DL + 2 * dp);
-                    } else {
-                        ms[s] = -INFINITY;
-                        ls[s] = 0.f;
-                        v[s] = make_float2(0.f, 0.f);
-                    }
-                }
-                const float m = fmaxf(fmaxf(fmaxf(ms[0], ms[1]), fmaxf(ms[2], ms[3])), fmaxf(fmaxf(ms[4], ms[5]), fmaxf(ms[6], ms[7])));
-                float l = 0.f, a0 = 0.f, a1 = 0.f;
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const float e = fast_exp2(ms[s] - m);   // 0 for the sources that do not exist
-                    l = fmaf(e, ls[s], l);
-                    a0 = fmaf(e, v[s].x, a0);
-                    a1 = fmaf(e, v[s].y, a1);
-                }
-                const float inv = 1.f / l;
-                const int i = i0 + qq / p.group, jh = qq % p.group;
-                __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hq0 + jh) * HD + split * DL + 2 * dp;
-                *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(a0 * inv, a1 * inv);
-            }
-        }
-        // no CTA leaves while a peer may still copy out of its staging chunks
-        __syncwarp();
-        cluster_wait();
-    }
-
-    fence_before();
-    __syncthreads();
     if (warp == 1) {
+        __syncwarp();
+        named_barrier(7, kSoft + 32);
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TM_COLS) : "memory");
     }
+    if (C == 1) return;
+
+    // ---- merge the C partials of the output columns this CTA owns: a thread takes a query row and four adjacent columns
+    //      (consecutive threads read consecutive words), reads them out of the peers' shared memory and works out its row's
+    //      weights 2^(m_s - m) / l itself: the few threads of a row repeat that, but nobody waits for a table.
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();           // the partials of all CTAs are complete
+    const int quads = DL / 4;
+    if (!*abort_flag) {
+#pragma unroll 1
+        for (int idx = tid; idx < rows_total * quads; idx += kThreads) {
+            const int qq = (idx * p.quads_inv) >> 16, d0 = (idx - qq * quads) * 4;
+            if (d0 >= own_dl) continue;
+            const uint32_t at = base + ((uint32_t)qq * PITCH + (uint32_t)(split * DL + d0)) * 4u;
+            float m = -INFINITY, l = 0.f, a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+            for (int s0 = 0; s0 < C; s0 += 4) {   // four sources at a time: their loads are in flight together
+                float ms[4], ls[4], x[4][4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int s = min(s0 + k, C - 1);
+                    ld_peer_v2(map_to_cta(base + ML_OFF + (uint32_t)qq * 8u, s), ms[k], ls[k]);
+                    ld_peer_v4(map_to_cta(at, s), x[k]);
+                }
+                float mn = m;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (s0 + k >= C) ms[k] = -INFINITY;
+                    mn = fmaxf(mn, ms[k]);
+                }
+                const float f = m == -INFINITY ? 0.f : fast_exp2(m - mn);
+                m = mn;
+                l *= f;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) a[v] *= f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float e = fast_exp2(ms[k] - mn);
+                    l = fmaf(e, ls[k], l);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) a[v] = fmaf(e, x[k][v], a[v]);
+                }
+            }
+            const float inv = 1.f / l;
+            const int i = (qq * p.group_inv) >> 16, jh = qq - i * p.group;
+            __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i0 + i) * p.n_q_heads + hq0 + jh) * HD + split * DL + d0;
+            *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(a[0] * inv, a[1] * inv), pack_bf16x2(a[2] * inv, a[3] * inv));
+        }
+    }
+    // no CTA leaves while a peer may still read its partial
+    __syncwarp();
+    cluster_arrive_relaxed();
+    cluster_wait();
 }
 
 // ---- host side ---------------------------------------------------------------------------
@@ -745,21 +710,6 @@ bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len) {
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// q [B, n, H_q, 128] bf16 (one query head per CTA column) seen as 5-D {64 columns, row, head, half, sequence}:
-// the box {64, N, 1, 2, 1} lands as [half][row][64 columns], the K-major Q tile; rows past n read as zero
-bool make_q_map(CUtensorMap* map, const void* q, int batch, int n_active, int n_q_heads, int n_slots) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[5] = {64, (cuuint64_t)n_active, (cuuint64_t)n_q_heads, 2, (cuuint64_t)batch};
-    const cuuint64_t strides[4] = {(cuuint64_t)n_q_heads * HD * 2, (cuuint64_t)HD * 2, 128,
-                                   (cuuint64_t)n_active * n_q_heads * HD * 2};
-    const cuuint32_t box[5] = {64, (cuuint32_t)n_slots, 1, 2, 1};
-    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(q), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 struct KeysPlan {
     bool ok;
     int group, rows_chunk, n_sub_r, n_sub;   // heads and active rows per CTA column, row chunks, CTA columns per kv head
@@ -774,8 +724,8 @@ constexpr uint32_t kSmemTwoPerSm = 115712;   // (228 KB per SM - 2 x 1 KB reserv
 constexpr int tm_columns(int n_slots) { return 3 * (n_slots <= 64 ? 64 : 128) <= 256 ? 256 : 512; }
 
 // shared-memory carve for n_slots query slots and ns stages; `fresh`: room for the stale-key bits (16 bytes per
-// refreshed cache tile, of which there are at most n_active)
-void carve(KeysPlan& pl, int n_active, int ns, bool fresh) {
+// cache tile of a CTA, of which it may hold one more than tiles_per_split)
+void carve(KeysPlan& pl, int ns, bool fresh) {
     uint32_t off = (uint32_t)pl.n_slots * 256u;   // Q
     off = (off + 1023u) & ~1023u;
     pl.off_p = off;
@@ -783,7 +733,7 @@ void carve(KeysPlan& pl, int n_active, int ns, bool fresh) {
     pl.off_stage = off;
     off += (uint32_t)ns * TILE;
     pl.off_list = off;
-    off += fresh ? (uint32_t)n_active * 16u : 0u;
+    off += fresh ? (uint32_t)(pl.tiles_per_split + 1) * 16u : 0u;
     pl.off_bar = off;
     off += kBarBytes + (uint32_t)sizeof(KeysShared) + 16u;
     pl.smem_bytes = off + 1024u;
@@ -872,19 +822,18 @@ KeysPlan make_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
         for (int own = 0; own <= (fresh ? 1 : 0); ++own) {                     // own: the fresh tiles get their own CTA
             const int c = cs + own;
             if (c > 8) continue;
-            int dl = (HD + c - 1) / c;
-            dl += dl & 1;
-            if ((c - 1) * dl >= HD) continue;                                  // an owner without columns
+            const int dl = ((HD + c - 1) / c + 7) & ~7;                        // (the last CTAs may own fewer columns, or none)
             const int last_tiles = key_tiles - (cs - 1) * tps;
             const int visits = own ? (tps > pl.n_extra ? tps : pl.n_extra)
                                    : (tps > last_tiles + pl.n_extra ? tps : last_tiles + pl.n_extra);
             KeysPlan t = pl;
             int ns = 2 * visits < kMaxStages ? 2 * visits : kMaxStages;   // ring slots: a K and a V slot per tile in flight
-            carve(t, n_active, ns, fresh);
-            while (ns > 2 && t.smem_bytes > kSmemMax) carve(t, n_active, --ns, fresh);
+            t.tiles_per_split = tps;
+            carve(t, ns, fresh);
+            while (ns > 2 && t.smem_bytes > kSmemMax) carve(t, --ns, fresh);
             if (t.smem_bytes > kSmemMax || (ns < 4 && visits > 1)) continue;
-            // the exchange areas of the merge (2 c chunks) reuse the Q / P^T / stage memory
-            if (c > 1 && 2 * (size_t)c * (pl.n_slots * dl + 2 * pl.n_slots) * 4 > t.off_list) continue;
+            // the partial of the merge reuses the Q / P^T / stage memory
+            if (c > 1 && partial_bytes(pl.n_slots) > t.off_list) continue;
             const int per_sm = (t.smem_bytes <= kSmemTwoPerSm && tm_cols <= 256) ? 2 : 1;
             const long long ctas = columns * c;
             if (ctas > (long long)per_sm * sms) continue;
@@ -909,7 +858,7 @@ KeysPlan make_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
         }
     }
     pl.ok = best_cost >= 0;
-    if (pl.ok) carve(pl, n_active, pl.n_stages, fresh);
+    if (pl.ok) carve(pl, pl.n_stages, fresh);
     return pl;
 }
 
@@ -954,8 +903,7 @@ double stream_bytes_per_ns() {
 
 template <int N>
 cudaError_t launch_n(const KeysPlan& pl, const KeysParams& p, const CUtensorMap& mk, const CUtensorMap& mv,
-                     const CUtensorMap& mq, const CUtensorMap& mkn, const CUtensorMap& mvn,
-                     int bh, cudaStream_t stream) {
+                     const CUtensorMap& mkn, const CUtensorMap& mvn, int bh, cudaStream_t stream) {
     static PerDeviceOnce attr_once;
     if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_skip_keys_kernel<N>, (int)kSmemMax); ea != cudaSuccess)
         return ea;
@@ -973,7 +921,7 @@ cudaError_t launch_n(const KeysPlan& pl, const KeysParams& p, const CUtensorMap&
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_skip_keys_kernel<N>, mk, mv, mq, mkn, mvn, p);
+    return cudaLaunchKernelEx(&cfg, attend_skip_keys_kernel<N>, mk, mv, mkn, mvn, p);
 }
 
 }  // namespace
@@ -1006,9 +954,7 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
     if (!make_cache_map(&map_k, a.k_cache, bh, a.d.ctx_len) || !make_cache_map(&map_v, a.v_cache, bh, a.d.ctx_len))
         return cudaErrorInvalidValue;
     KeysParams p{};
-    CUtensorMap map_q = map_k, map_kn = map_k, map_vn = map_v;   // placeholders unless q_tma / fresh
-    p.q_tma = (pl.group == 1) ? 1 : 0;   // one query head per CTA column: its rows are one TMA box
-    if (p.q_tma && !make_q_map(&map_q, a.q, a.d.batch, a.n_active, a.d.n_q_heads, pl.n_slots)) return cudaErrorInvalidValue;
+    CUtensorMap map_kn = map_k, map_vn = map_v;   // placeholders unless fresh
     if (fresh && (!make_fresh_map(&map_kn, k_new, a.d.batch, a.n_active, a.d.n_kv_heads) ||
                   !make_fresh_map(&map_vn, v_new, a.d.batch, a.n_active, a.d.n_kv_heads)))
         return cudaErrorInvalidValue;
@@ -1025,6 +971,7 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
     p.n_q_heads = a.d.n_q_heads;
     p.n_kv_heads = a.d.n_kv_heads;
     p.group = pl.group;
+    p.group_inv = (65536 + pl.group - 1) / pl.group;
     p.rows_chunk = pl.rows_chunk;
     p.n_sub_r = pl.n_sub_r;
     p.n_sub = pl.n_sub;
@@ -1034,6 +981,7 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
     p.n_stages = pl.n_stages;
     p.n_extra = pl.n_extra;
     p.dl = pl.dl;
+    p.quads_inv = (65536 + pl.dl / 4 - 1) / (pl.dl / 4);
     p.off_p = pl.off_p;
     p.off_stage = pl.off_stage;
     p.off_list = pl.off_list;
@@ -1047,9 +995,9 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
         p.stagger_ns = (uint32_t)(ns < 3000.0 ? ns : 3000.0);
     }
     const int cols = bh * pl.n_sub;
-    return pl.n_slots == 48   ? launch_n<48>(pl, p, map_k, map_v, map_q, map_kn, map_vn, cols, stream)
-           : pl.n_slots == 64 ? launch_n<64>(pl, p, map_k, map_v, map_q, map_kn, map_vn, cols, stream)
-                              : launch_n<96>(pl, p, map_k, map_v, map_q, map_kn, map_vn, cols, stream);
+    return pl.n_slots == 48   ? launch_n<48>(pl, p, map_k, map_v, map_kn, map_vn, cols, stream)
+           : pl.n_slots == 64 ? launch_n<64>(pl, p, map_k, map_v, map_kn, map_vn, cols, stream)
+                              : launch_n<96>(pl, p, map_k, map_v, map_kn, map_vn, cols, stream);
 }
 
 }  // namespace ec

@@ -41,6 +41,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// the same without the hardware's suspended wait: for a thread that polls several barriers
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // bounded wait (a poll count and one second of wall time); on failure raises the CTA's abort flag (every later wait
 // then returns at once) and reports EC_ERR_TIMEOUT through the caller's status word
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* dev_status) {
@@ -57,7 +67,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatil
     *abort_flag = 1;
     if (dev_status) atomicExch(dev_status, (int)EC_ERR_TIMEOUT);
 }
-// bookkeeping of a bounded polling loop over several barriers (same limits as mbar_wait): call tick() after a round
+// bookkeeping of a bounded polling loop over several barriers (one second of wall time): call tick() after a round
 // without progress; it returns false when the loop should give up (limit reached: abort raised; or abort already set)
 struct SpinGuard {
     uint32_t n = 0;
@@ -67,7 +77,7 @@ struct SpinGuard {
         if (*abort_flag) return false;
         const unsigned long long now = global_timer_ns();
         if (t0 == 0) t0 = now;
-        if (n < kSpinLimit && now - t0 <= kWaitLimitNs) return true;
+        if (now - t0 <= kWaitLimitNs) return true;
         *abort_flag = 1;
         if (dev_status) atomicExch(dev_status, (int)EC_ERR_TIMEOUT);
         return false;
@@ -202,6 +212,13 @@ __device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t
 __device__ __forceinline__ void st_peer_f32(uint32_t addr_cluster, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr_cluster), "f"(v) : "memory");
 }
+// loads from a peer CTA's shared memory (address from map_to_cta)
+__device__ __forceinline__ void ld_peer_v4(uint32_t addr_cluster, float* r) {
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(addr_cluster) : "memory");
+}
+__device__ __forceinline__ void ld_peer_v2(uint32_t addr_cluster, float& a, float& b) {
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(addr_cluster) : "memory");
+}
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 // named barrier over n_threads threads that also ORs a predicate across them
 __device__ __forceinline__ bool named_barrier_or(int id, int n_threads, bool pred) {
@@ -212,6 +229,9 @@ __device__ __forceinline__ bool named_barrier_or(int id, int n_threads, bool pre
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r) : "r"(id), "r"(n_threads), "r"((uint32_t)pred) : "memory");
     return r != 0;
+}
+__device__ __forceinline__ void named_arrive(int id, int n_threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }
 __device__ __forceinline__ void named_barrier(int id, int n_threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
@@ -243,6 +263,12 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
     f32x2 r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// maximum over the lanes of a warp
+__device__ __forceinline__ float redux_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {

@@ -1,0 +1,29 @@
+"""GPU parity at the sizes where single paths of the kernels can go wrong: cluster sizes whose CTAs merge unequal
+shares of the output, references of the softmax taken from the rare path, edges of tiles and of dispatch rules.
+Each against the fp64 oracle, with the tolerances of test_gpu_attend.py."""
+import numpy as np
+import pytest
+
+import ec_synth as syn
+from test_gpu_attend import _check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L,n", [(64, 1), (257, 34), (500, 33), (640, 48), (769, 34), (900, 60), (896, 96)])
+def test_cluster_sizes_with_unequal_output_shares(L, n):
+    """Two heads, so the keys split over as many CTAs as there are tiles (one to eight with the fresh rows' own CTA):
+    the CTAs own 128, 64, 48, 32, 24 or 16 output columns, the last ones fewer or none."""
+    w = syn.Workload(97, "clusters", syn.BF16, 1, 2, 2, 128, 0, L, 1, 0, 64)
+    t = syn.attn_inputs(w, n, active_idx=syn.arbitrary_active_idx(1, L, n, seed=17 * L + n), std_qk=0.9, std_v=0.5)
+    _check(w, t)
+    _check(w, t, refresh=False)
+
+
+@pytest.mark.parametrize("std,L", [(0.3, 1024), (2.5, 1024), (14.0, 600)])
+def test_first_keys_of_a_tile_all_refreshed(std, L):
+    """The first 32 keys of every second tile are refreshed, so no cached key of the warp that supplies a CTA's first
+    reference counts and the reference comes from the rare path; with std 14 scores exceed references by far."""
+    idx = np.concatenate([np.arange(i, i + 32) for i in range(0, min(L, 700), 256)])[None].astype(np.int32)
+    w = syn.Workload(98, "stale", syn.BF16, 1, 8, 8, 128, 0, L, 1, 0, 64)
+    _check(w, syn.attn_inputs(w, idx.shape[1], active_idx=idx, std_qk=std, std_v=0.5))
