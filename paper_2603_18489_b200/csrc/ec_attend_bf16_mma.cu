@@ -1,21 +1,26 @@
 // ec_attend, bf16 storage, warp-level tensor-core path (mma.sync m16n8k16, fp32
-// accumulation): active-row bidirectional attention over the full cache
-// (Appendix A of the paper, partial branch; the full branch when n_active == L).
+// accumulation): refresh and active-row bidirectional attention over the full cache
+// (Appendix A of the paper, partial branch; the full branch when n_active == L) in ONE launch.
 //
 // Work decomposition
 //   - The query rows that share one kv head -- n_active rows x g = H_q/H_kv query
 //     heads -- are flattened into one row axis r = i*g + j (GQA packing), cut into
 //     64-row tiles; one CTA (4 warps x 16 rows) owns one tile.
 //   - Keys are cut into 64-key tiles.  When there are few row tiles (skip step:
-//     34 active rows) the key axis is also split across CTAs ("split-KV"): each
-//     split writes an un-normalised partial (m, l, O) to the workspace and a small
-//     combine kernel merges them.  Every K/V byte is read by exactly one CTA per
-//     row tile, so the skip step streams the cache once.
-//   - K/V tiles are staged in shared memory with 16-byte cp.async copies (two
-//     stages), XOR-swizzled so ldmatrix is bank-conflict free.
+//     34 active rows) up to eight CTAs, a cluster, split the keys of a row tile; each leaves
+//     (m, l, O) un-normalised in its shared memory and, after a cluster barrier, merges a share
+//     of the rows out of its peers' (partials in global memory and a second launch took 5.4 us more).
+//   - K/V tiles are staged in shared memory with 16-byte cp.async copies, XOR-swizzled so ldmatrix
+//     is bank-conflict free.  A key that is being refreshed is read from k_new / v_new (a table of
+//     the CTA's keys, filled from the index list), so nothing waits for the cache update; the row
+//     tiles of a kv head share the writing of the cache.
 //   - Softmax is online (running max / sum per row, exp2 with the scale folded
 //     in); P is re-packed from the S accumulators into A fragments in registers.
+// What bounds it: latency on partial steps of 64-wide heads (four sequences of 1000 keys, 48 rows, 12 query heads on 4:
+// 9.5 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
+// per clock and SM, measured) on full ones.
 #include "ec_common.cuh"
+#include "ec_tc_ptx.cuh"
 
 namespace ec {
 namespace {
@@ -23,6 +28,11 @@ namespace {
 constexpr int BM = 64;   // query rows per CTA
 constexpr int BN = 64;   // keys per tile
 constexpr int kThreads = 128;
+// K/V stages in shared memory.  A tile computes in about half the time its data takes to arrive, so two tiles have to be
+// on their way (9.5 us against 13.4 with one); with 128-wide heads two stages are what fits two CTAs per SM.
+template <int D>
+__host__ __device__ constexpr int stages() { return D == 64 ? 3 : 2; }
+constexpr int kMaxMapKeys = 8192;   // keys of one CTA beyond which the refresh is a launch of its own
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -63,28 +73,35 @@ __device__ __forceinline__ uint32_t swz(int row, int chunk) {
 
 struct MmaParams {
     const __nv_bfloat16* q;
-    const __nv_bfloat16* k_cache;
-    const __nv_bfloat16* v_cache;
+    const __nv_bfloat16* k_new;   // nullptr: attend without refreshing
+    const __nv_bfloat16* v_new;
+    __nv_bfloat16* k_cache;
+    __nv_bfloat16* v_cache;
+    const int32_t* active_idx;    // nullptr: identity
     __nv_bfloat16* out;
-    float* part_o;   // [B*Hkv, n_splits, rows_total, D]
-    float2* part_ml; // [B*Hkv, n_splits, rows_total]  (m in log2 units, l)
     int n_active, ctx_len, n_q_heads, n_kv_heads, group;  // group = H_q / H_kv
     int rows_total;   // n_active * group
-    int n_splits, tiles_per_split;
+    int row_tiles, n_splits, tiles_per_split;
     float scale_log2;  // scale * log2(e)
 };
 
 template <int D>
-__global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p) {
+__global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(const MmaParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int TILE_BYTES = BN * D * 2;
     constexpr int CHUNKS = D / 8;  // 16-byte chunks per row
+    constexpr int ST = stages<D>();
     unsigned char* sQ = smem;                       // BM x D
-    unsigned char* sK = smem + BM * D * 2;          // 2 stages
-    unsigned char* sV = sK + 2 * TILE_BYTES;        // 2 stages
+    unsigned char* sK = smem + BM * D * 2;          // ST stages
+    unsigned char* sV = sK + ST * TILE_BYTES;       // ST stages
+    float2* s_ml = reinterpret_cast<float2*>(sV + ST * TILE_BYTES);   // (m, l) per row, for the merge
+    int* map = reinterpret_cast<int*>(s_ml + BM);   // [key of this CTA]: active row that refreshes it, or -1
+    float* part = reinterpret_cast<float*>(sK);     // the partial of the merge, over the stages: [BM][PP]
+    constexpr int PP = D + 8;                       // row pitch: fragment stores of eight rows cover all banks
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int row_tile = blockIdx.x, split = blockIdx.y, bh = blockIdx.z;
+    const int split = blockIdx.x % p.n_splits, unit = blockIdx.x / p.n_splits;
+    const int row_tile = unit % p.row_tiles, bh = unit / p.row_tiles;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
     const int r0 = row_tile * BM;
 
@@ -94,6 +111,14 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
 
     const __nv_bfloat16* kbase = p.k_cache + ((long long)bh * p.ctx_len) * D;
     const __nv_bfloat16* vbase = p.v_cache + ((long long)bh * p.ctx_len) * D;
+
+    const int key_lo = t_begin * BN, n_keys = min(p.ctx_len, t_end * BN) - key_lo;
+    const bool fresh = p.k_new != nullptr, mapped = fresh && p.active_idx != nullptr;
+    if (mapped)
+        for (int k = tid; k < n_keys; k += kThreads) map[k] = -1;
+    __syncthreads();
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
 
     // ---- stage Q (rows beyond rows_total are zero-filled) --------------------------
     for (int c = tid; c < BM * CHUNKS; c += kThreads) {
@@ -105,18 +130,40 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
             p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + ch * 8;
         cp_async16(smem_u32(sQ) + swz<D>(row, ch), src, ok);
     }
+    if (mapped) {
+        for (int i = tid; i < p.n_active; i += kThreads) {
+            const int k = __ldg(p.active_idx + (long long)b * p.n_active + i) - key_lo;
+            if (k >= 0 && k < n_keys) map[k] = i;
+        }
+        __syncthreads();
+    }
+    // keys that no table sends elsewhere: the cache's panel of this head, or (identity list) the fresh tensor's rows
+    const bool identity = fresh && !mapped;
+    const long long new0 = ((long long)b * p.n_active * p.n_kv_heads + hk) * D;
+    const int new_stride = p.n_kv_heads * D, key_stride = identity ? new_stride : D;
+    const __nv_bfloat16 *ksrc0 = identity ? p.k_new + new0 : kbase, *vsrc0 = identity ? p.v_new + new0 : vbase;
     auto load_kv = [&](int tile, int stage) {
         const int key0 = tile * BN;
         for (int c = tid; c < BN * CHUNKS; c += kThreads) {
             const int row = c / CHUNKS, ch = c % CHUNKS;
             const bool ok = key0 + row < p.ctx_len;
-            const long long off = (long long)(ok ? key0 + row : 0) * D + ch * 8;
-            cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz<D>(row, ch), kbase + off, ok);
-            cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz<D>(row, ch), vbase + off, ok);
+            const long long off = ok ? (long long)(key0 + row) * key_stride : 0;
+            const __nv_bfloat16 *ks = ksrc0 + off, *vs = vsrc0 + off;
+            if (mapped && ok) {
+                const int i = map[key0 + row - key_lo];
+                if (i >= 0) {
+                    ks = p.k_new + new0 + (long long)i * new_stride;
+                    vs = p.v_new + new0 + (long long)i * new_stride;
+                }
+            }
+            cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz<D>(row, ch), ks + ch * 8, ok);
+            cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz<D>(row, ch), vs + ch * 8, ok);
         }
     };
-    if (t_begin < t_end) load_kv(t_begin, 0);
-    cp_async_commit();
+    for (int s = 0; s < ST - 1; ++s) {
+        if (t_begin + s < t_end) load_kv(t_begin + s, s);
+        cp_async_commit();
+    }
 
     // ---- per-thread state ----------------------------------------------------------
     uint32_t qf[D / 16][4];
@@ -127,11 +174,11 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
 
     bool q_loaded = false;
     for (int t = t_begin; t < t_end; ++t) {
-        const int stage = (t - t_begin) & 1;
-        if (t + 1 < t_end) load_kv(t + 1, stage ^ 1);
+        const int stage = (t - t_begin) % ST;
+        cp_async_wait<ST - 2>();
+        __syncthreads();   // the tile has landed, and everyone is done with the one before it, whose stage is refilled now
+        if (t + ST - 1 < t_end) load_kv(t + ST - 1, (t - t_begin + ST - 1) % ST);
         cp_async_commit();
-        cp_async_wait<1>();
-        __syncthreads();
 
         if (!q_loaded) {
             q_loaded = true;
@@ -217,9 +264,19 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
                 mma_bf16(o[2 * db + 1], pf, vf[2], vf[3]);
             }
         }
-        __syncthreads();  // everyone is done with this stage before it is refilled
+        // refreshed keys into the cache, from the landed tile: the row tiles that walk over these keys take turns
+        if (fresh && t % p.row_tiles == row_tile) {
+            for (int c = tid; c < BN * CHUNKS; c += kThreads) {
+                const int row = c / CHUNKS, ch = c % CHUNKS, key = key0 + row;
+                if (key >= p.ctx_len || (mapped && map[key - key_lo] < 0)) continue;
+                const long long at = ((long long)bh * p.ctx_len + key) * D + ch * 8;
+                *reinterpret_cast<uint4*>(p.k_cache + at) = *reinterpret_cast<const uint4*>(sK + stage * TILE_BYTES + swz<D>(row, ch));
+                *reinterpret_cast<uint4*>(p.v_cache + at) = *reinterpret_cast<const uint4*>(sV + stage * TILE_BYTES + swz<D>(row, ch));
+            }
+        }
     }
     cp_async_wait<0>();
+    __syncthreads();   // everyone is done with the stages before they become the partial
 
     // ---- epilogue ------------------------------------------------------------------
 #pragma unroll
@@ -227,13 +284,16 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
         l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
         l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
     }
+    auto out_row = [&](int r) {   // where packed row r goes
+        const int i = r / p.group, j = r - i * p.group;
+        return p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D;
+    };
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r = r0 + warp * 16 + (lane >> 2) + 8 * h;
-        if (r >= p.rows_total) continue;
+        const int row = warp * 16 + (lane >> 2) + 8 * h, r = r0 + row;
         if (p.n_splits == 1) {
-            const int i = r / p.group, j = r % p.group;
-            __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D;
+            if (r >= p.rows_total) continue;
+            __nv_bfloat16* dst = out_row(r);
             const float inv = 1.f / l_run[h];
 #pragma unroll
             for (int n = 0; n < D / 8; ++n) {
@@ -241,53 +301,54 @@ __global__ void __launch_bounds__(kThreads) attend_mma_kernel(const MmaParams p)
                 *reinterpret_cast<uint32_t*>(dst + n * 8 + 2 * (lane & 3)) = v;
             }
         } else {
-            const long long slot = ((long long)bh * p.n_splits + split) * p.rows_total + r;
-            float* dst = p.part_o + slot * D;
 #pragma unroll
             for (int n = 0; n < D / 8; ++n)
-                *reinterpret_cast<float2*>(dst + n * 8 + 2 * (lane & 3)) = make_float2(o[n][2 * h], o[n][2 * h + 1]);
-            if ((lane & 3) == 0) p.part_ml[slot] = make_float2(m_run[h], l_run[h]);
+                *reinterpret_cast<float2*>(part + row * PP + n * 8 + 2 * (lane & 3)) = make_float2(o[n][2 * h], o[n][2 * h + 1]);
+            if ((lane & 3) == 0) s_ml[row] = make_float2(m_run[h], l_run[h]);
         }
     }
-}
+    if (p.n_splits == 1) return;
 
-// merge the split-KV partials of one (sequence, kv head, row): out = sum_s w_s O_s / sum_s w_s l_s,
-// w_s = 2^(m_s - max m)
-template <int D>
-__global__ void __launch_bounds__(128) attend_combine_kernel(const MmaParams p) {
-    const int lane = threadIdx.x & 31;
-    const int bh = blockIdx.z;
-    const int r = blockIdx.x * 4 + (threadIdx.x >> 5);  // one warp per flattened row
-    if (r >= p.rows_total) return;
-    const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
-    float m = -INFINITY;
-    for (int s = 0; s < p.n_splits; ++s)
-        m = fmaxf(m, __ldcg(&p.part_ml[((long long)bh * p.n_splits + s) * p.rows_total + r]).x);
-    constexpr int DPL = D / 32;
-    float acc[DPL];
+    // ---- each CTA of the cluster merges a share of the rows: out = sum_s w_s O_s / sum_s w_s l_s, w_s = 2^(m_s - max m) ----
+    tc::cluster_arrive();
+    tc::cluster_wait();
+    const int valid = min(BM, p.rows_total - r0), per = (valid + p.n_splits - 1) / p.n_splits;
+    const int rows_here = min(per, valid - split * per);
+    for (int idx = tid; idx < rows_here * (D / 4); idx += kThreads) {
+        const int row = split * per + idx / (D / 4), ch = idx % (D / 4);
+        float mm[8], ll[8], x[8][4], M = -INFINITY, L = 0.f;
 #pragma unroll
-    for (int t = 0; t < DPL; ++t) acc[t] = 0.f;
-    float l = 0.f;
-    for (int s = 0; s < p.n_splits; ++s) {
-        const long long slot = ((long long)bh * p.n_splits + s) * p.rows_total + r;
-        const float2 ml = __ldcg(&p.part_ml[slot]);
-        if (ml.y <= 0.f) continue;  // an empty split
-        const float w = fast_exp2(ml.x - m);
-        l = fmaf(w, ml.y, l);
-        const float* src = p.part_o + slot * D;
+        for (int q = 0; q < 8; ++q) {
+            const int src = min(q, p.n_splits - 1);
+            tc::ld_peer_v2(tc::map_to_cta(smem_u32(s_ml + row), src), mm[q], ll[q]);
+            tc::ld_peer_v4(tc::map_to_cta(smem_u32(part + row * PP + ch * 4), src), x[q]);
+        }
 #pragma unroll
-        for (int t = 0; t < DPL; ++t) acc[t] = fmaf(w, __ldcg(src + lane + 32 * t), acc[t]);
+        for (int q = 0; q < 8; ++q) {
+            if (q >= p.n_splits) mm[q] = -INFINITY;
+            M = fmaxf(M, mm[q]);
+        }
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float w = fast_exp2(mm[q] - M);
+            L = fmaf(w, ll[q], L);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] = fmaf(w, x[q][e], acc[e]);
+        }
+        const float inv = 1.f / L;
+        *reinterpret_cast<uint2*>(out_row(r0 + row) + ch * 4) =
+            make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
     }
-    const int i = r / p.group, j = r % p.group;
-    __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D;
-    const float inv = 1.f / l;
-#pragma unroll
-    for (int t = 0; t < DPL; ++t) dst[lane + 32 * t] = __float2bfloat16_rn(acc[t] * inv);
+    tc::cluster_arrive_relaxed();   // no CTA leaves while a peer may still read its partial
+    tc::cluster_wait();
 }
 
 struct Plan {
     int row_tiles, n_splits, tiles_per_split, rows_total;
 };
+// Keys of a row tile split over up to eight CTAs (a cluster; at least one tile each) while the launch stays within the
+// three CTAs an SM holds: a CTA is a serial chain of tiles (about 1 us each when nothing hides their latency).
 Plan make_plan(const ec_attn_desc& d, int n_active) {
     Plan pl;
     const int g = d.n_q_heads / d.n_kv_heads;
@@ -295,9 +356,9 @@ Plan make_plan(const ec_attn_desc& d, int n_active) {
     pl.row_tiles = (pl.rows_total + BM - 1) / BM;
     const int key_tiles = (d.ctx_len + BN - 1) / BN;
     const long long base = (long long)pl.row_tiles * d.batch * d.n_kv_heads;
-    const long long want = 2LL * sm_count();
-    int splits = (int)((want + base - 1) / base);
+    int splits = (int)(3LL * sm_count() / base);
     if (splits < 1) splits = 1;
+    if (splits > 8) splits = 8;
     if (splits > key_tiles) splits = key_tiles;
     pl.tiles_per_split = (key_tiles + splits - 1) / splits;
     pl.n_splits = (key_tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
@@ -305,11 +366,15 @@ Plan make_plan(const ec_attn_desc& d, int n_active) {
 }
 
 template <int D>
-cudaError_t launch_d(const AttendArgs& a, const Plan& pl, cudaStream_t stream) {
+cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, const void* v_new, const int32_t* active_idx,
+                     cudaStream_t stream) {
     MmaParams p;
     p.q = static_cast<const __nv_bfloat16*>(a.q);
-    p.k_cache = static_cast<const __nv_bfloat16*>(a.k_cache);
-    p.v_cache = static_cast<const __nv_bfloat16*>(a.v_cache);
+    p.k_cache = static_cast<__nv_bfloat16*>(const_cast<void*>(a.k_cache));
+    p.v_cache = static_cast<__nv_bfloat16*>(const_cast<void*>(a.v_cache));
+    p.k_new = static_cast<const __nv_bfloat16*>(k_new);
+    p.v_new = static_cast<const __nv_bfloat16*>(v_new);
+    p.active_idx = active_idx;
     p.out = static_cast<__nv_bfloat16*>(a.out);
     p.n_active = a.n_active;
     p.ctx_len = a.d.ctx_len;
@@ -317,41 +382,49 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, cudaStream_t stream) {
     p.n_kv_heads = a.d.n_kv_heads;
     p.group = a.d.n_q_heads / a.d.n_kv_heads;
     p.rows_total = pl.rows_total;
+    p.row_tiles = pl.row_tiles;
     p.n_splits = pl.n_splits;
     p.tiles_per_split = pl.tiles_per_split;
     p.scale_log2 = a.scale * kLog2e;
-    const long long slots = (long long)a.d.batch * a.d.n_kv_heads * pl.n_splits * pl.rows_total;
-    p.part_o = static_cast<float*>(a.workspace);
-    p.part_ml = reinterpret_cast<float2*>(static_cast<char*>(a.workspace) + (size_t)slots * D * sizeof(float));
-    constexpr int smem = (BM + 4 * BN) * D * 2;
-    static PerDeviceOnce attr_once;
-    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D>, smem); ea != cudaSuccess) return ea;
-    const dim3 grid(pl.row_tiles, pl.n_splits, a.d.batch * a.d.n_kv_heads);
-    attend_mma_kernel<D><<<grid, kThreads, smem, stream>>>(p);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (pl.n_splits > 1) {
-        const dim3 cgrid((pl.rows_total + 3) / 4, 1, a.d.batch * a.d.n_kv_heads);
-        attend_combine_kernel<D><<<cgrid, 128, 0, stream>>>(p);
-        e = cudaGetLastError();
+    const long long ctas = (long long)a.d.batch * a.d.n_kv_heads * pl.row_tiles * pl.n_splits;
+    if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    int map_keys = k_new && active_idx ? pl.tiles_per_split * BN : 0;
+    if (map_keys > kMaxMapKeys) {   // no room for the table of keys
+        if (const cudaError_t e = launch_refresh(a.d, p.k_cache, p.v_cache, k_new, v_new, active_idx, a.n_active, stream);
+            e != cudaSuccess)
+            return e;
+        p.k_new = p.v_new = nullptr;
+        map_keys = 0;
     }
-    return e;
+    constexpr int smem = (BM + 2 * stages<D>() * BN) * D * 2 + BM * (int)sizeof(float2);
+    static_assert(BM * (D + 8) * 4 <= 4 * BN * D * 2, "the partial of the merge fits over the stages");
+    static PerDeviceOnce attr_once;
+    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem + (size_t)map_keys * 4;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = pl.n_splits;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D>, p);
 }
 
 }  // namespace
 
-size_t attend_workspace_bytes(const ec_attn_desc& d, int n_active) {
-    if (d.dtype != EC_BF16 || n_active <= 0) return 16;
-    const Plan pl = make_plan(d, n_active);
-    if (pl.n_splits <= 1) return 16;
-    const size_t slots = (size_t)d.batch * d.n_kv_heads * pl.n_splits * pl.rows_total;
-    return slots * ((size_t)d.head_dim * sizeof(float) + sizeof(float2)) + 16;
-}
-
-cudaError_t launch_attend_bf16(const AttendArgs& a, cudaStream_t stream) {
+cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
+                               cudaStream_t stream) {
     if (a.n_active == 0) return cudaSuccess;
     const Plan pl = make_plan(a.d, a.n_active);
-    return a.d.head_dim == 64 ? launch_d<64>(a, pl, stream) : launch_d<128>(a, pl, stream);
+    return a.d.head_dim == 64 ? launch_d<64>(a, pl, k_new, v_new, active_idx, stream)
+                              : launch_d<128>(a, pl, k_new, v_new, active_idx, stream);
 }
 
 }  // namespace ec

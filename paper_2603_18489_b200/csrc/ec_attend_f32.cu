@@ -1,112 +1,327 @@
-// ec_attend, fp32 storage: active-row bidirectional attention over the full
-// cache (Appendix A of the paper, partial branch; the full branch when every row
-// is active) computed entirely in fp32 on the FMA pipes.
+// ec_attend, fp32 storage: refresh and active-row bidirectional attention over the full cache (Appendix A of the paper,
+// partial branch; the full branch when every row is active) in ONE launch, entirely in fp32 on the FMA pipes (the
+// tolerance that goes with fp32 tensors, 1e-5 relative, rules out tf32 tensor cores).
 //
-// fp32 tensors are the small validation geometry; the tight tolerance that goes
-// with them (1e-5 relative) rules out tf32 tensor cores, so this is a plain SIMT
-// kernel: one warp per (sequence, active row, query head).
-//   scores : lane l takes key c*32+l of a 32-key chunk and dots its K row with
-//            the query (staged in shared memory, read as broadcast float4);
-//   softmax: online over chunks (running max m, running sum l), accurate expf;
-//   PV     : every lane owns head_dim/32 output columns; the chunk's 32
-//            probabilities are broadcast by shuffle and V rows are read coalesced.
+//   grid    a CTA of 128 threads takes 32 packed query rows (active row x query heads of one kv head) and a range of
+//           32-key tiles; up to eight CTAs, a cluster, split the keys of a row tile when there are few row tiles, so
+//           that a partial step of a small model still spreads over the chip.
+//   tile    K and V tiles come by 16-byte asynchronous copies into one of two stages.  Thread (tr, tk) = (tid / 16,
+//           tid % 16) holds rows 4 tr .. 4 tr + 3: it forms their scores against keys tk and tk + 16 (packed fp32x2 over even
+//           and odd columns: two partial sums), the 16 threads of a row exchange maxima and sums by shuffles, and
+//           probabilities go through shared memory to the same warp, which accumulates D / 16 output columns a thread.
+//   refresh a key that is being refreshed is read from k_new / v_new (a table of the CTA's keys, filled from the index
+//           list), so nothing waits for the cache update; the row tiles of a kv head share the writing of the cache,
+//           whose refreshed rows nobody reads.
+//   merge   every CTA leaves O (un-normalised), m and l of its keys in shared memory; after a cluster barrier each
+//           combines a share of the rows out of its peers' memory.
+// What bounds it: latency at the sizes it is for.  34 rows x 4 heads of 64 over 256 keys: 6.0 us a call (a warp per query
+// row that walks over all keys, behind a refresh launch, took 30.7).  At large sizes the FMA pipe: 438 rows x 8 heads of
+// four sequences 82 us (511).
 #include "ec_common.cuh"
+#include "ec_tc_ptx.cuh"
 
 namespace ec {
 namespace {
 
-constexpr int kWarpsPerCta = 4;
+using namespace tc;
+
+constexpr int kThreads = 128, BM = 32, BN = 32;
+constexpr int kMaxMapKeys = 8192;   // keys of one CTA beyond which the refresh is a launch of its own
+
+struct F32Params {
+    const float *q, *k_new, *v_new;
+    float *k_cache, *v_cache, *out;
+    const int32_t* active_idx;
+    int n_active, ctx_len, n_q_heads, n_kv_heads, group, rows_total, row_tiles, n_splits, tiles_per_split;
+    float scale;
+};
+
+// shared memory, in floats (D-float rows padded by four: eight rows read as float4 then cover all banks)
+template <int D>
+struct Carve {
+    static constexpr int P = D + 4;
+    static constexpr int q = 0, kv = q + BM * P, stage = 2 * BN * P, p = kv + 2 * stage, pp = BN + 4;
+    static constexpr int ml = p + BM * pp, map = ml + 2 * BM;
+    static constexpr int part = kv;   // the partial of the merge, over the stages: [BM][D]
+    static size_t bytes(int map_keys) { return (size_t)(map + map_keys) * 4; }
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+    const int sz = valid ? 16 : 0;   // 0: the 16 bytes are zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sz) : "memory");
+}
 
 template <int D>
-__global__ void __launch_bounds__(kWarpsPerCta * 32) attend_f32_kernel(
-    const float* __restrict__ q, const float* __restrict__ k_cache, const float* __restrict__ v_cache,
-    float* __restrict__ out, int batch, int n_active, int ctx_len, int n_q_heads, int n_kv_heads, float scale) {
-    __shared__ __align__(16) float s_q[kWarpsPerCta][D];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long job = (long long)blockIdx.x * kWarpsPerCta + warp;
-    const long long n_jobs = (long long)batch * n_active * n_q_heads;
-    if (job >= n_jobs) return;  // whole warp leaves together; no block-wide barrier below
-    const int hq = (int)(job % n_q_heads);
-    const long long bi = job / n_q_heads;
-    const long long b = bi / n_active;
-    const int hk = hq / (n_q_heads / n_kv_heads);
-    constexpr int DPL = D / 32;  // output columns per lane
+__global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p) {
+    using C = Carve<D>;
+    constexpr int D4 = D / 4, OC = D / 16;   // float4 pieces of a row; output columns of a thread
+    extern __shared__ __align__(16) float sm[];
+    const int tid = threadIdx.x, tr = tid >> 4, tk = tid & 15;
+    const int split = blockIdx.x % p.n_splits, unit = blockIdx.x / p.n_splits;
+    const int row_tile = unit % p.row_tiles, bh = unit / p.row_tiles;
+    const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
+    const int r0 = row_tile * BM;
+    const int n_tiles = (p.ctx_len + BN - 1) / BN;
+    const int t0 = split * p.tiles_per_split, t1 = min(n_tiles, t0 + p.tiles_per_split);
+    const int key_lo = t0 * BN, key_hi = min(p.ctx_len, t1 * BN);
+    const bool fresh = p.k_new != nullptr;
+    const bool mapped = fresh && p.active_idx != nullptr;
+    int* map = reinterpret_cast<int*>(sm + C::map);   // [key of this CTA]: active row that refreshes it, or -1
+    if (mapped)
+        for (int k = tid; k < key_hi - key_lo; k += kThreads) map[k] = -1;
+    __syncthreads();
+    pdl_wait();
+    pdl_launch_dependents();
 
-    const float* qrow = q + job * D;
-#pragma unroll
-    for (int t = 0; t < DPL; ++t) s_q[warp][lane + 32 * t] = qrow[lane + 32 * t];
-    __syncwarp();
-
-    const float* kb = k_cache + ((b * n_kv_heads + hk) * (long long)ctx_len) * D;
-    const float* vb = v_cache + ((b * n_kv_heads + hk) * (long long)ctx_len) * D;
-
-    float m = -INFINITY, l = 0.f;
-    float acc[DPL];
-#pragma unroll
-    for (int t = 0; t < DPL; ++t) acc[t] = 0.f;
-
-    for (int c0 = 0; c0 < ctx_len; c0 += 32) {
-        const int j = c0 + lane;
-        float s = -INFINITY;
-        if (j < ctx_len) {
-            const float4* kr = reinterpret_cast<const float4*>(kb + (long long)j * D);
-            const float4* qs = reinterpret_cast<const float4*>(s_q[warp]);
-            float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;  // four partial sums: shorter chains, smaller error
-#pragma unroll
-            for (int d4 = 0; d4 < D / 4; ++d4) {
-                const float4 kv = __ldg(kr + d4);
-                const float4 qv = qs[d4];
-                d0 = fmaf(qv.x, kv.x, d0);
-                d1 = fmaf(qv.y, kv.y, d1);
-                d2 = fmaf(qv.z, kv.z, d2);
-                d3 = fmaf(qv.w, kv.w, d3);
-            }
-            s = ((d0 + d1) + (d2 + d3)) * scale;
-        }
-        float cmax = s;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-        const float m_new = fmaxf(m, cmax);
-        const float corr = (m == -INFINITY) ? 0.f : expf(m - m_new);
-        const float p = (j < ctx_len) ? expf(s - m_new) : 0.f;
-        float psum = p;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-        l = fmaf(l, corr, psum);
-        m = m_new;
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) acc[t] *= corr;
-        const int cnt = min(32, ctx_len - c0);
-        for (int jj = 0; jj < cnt; ++jj) {
-            const float pj = __shfl_sync(0xffffffffu, p, jj);
-            const float* vr = vb + (long long)(c0 + jj) * D;
-#pragma unroll
-            for (int t = 0; t < DPL; ++t) acc[t] = fmaf(pj, __ldg(vr + lane + 32 * t), acc[t]);
-        }
+    for (int c = tid; c < BM * D4; c += kThreads) {
+        const int row = c / D4, ch = c % D4, r = r0 + row;
+        const bool ok = r < p.rows_total;
+        const int i = ok ? r / p.group : 0, j = ok ? r - i * p.group : 0;
+        const float* src = p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + ch * 4;
+        cp_async16(s2u(sm + C::q + row * C::P + ch * 4), src, ok);
     }
-    float* orow = out + job * D;
-    const float inv = 1.f / l;
+    if (mapped) {
+        for (int i = tid; i < p.n_active; i += kThreads) {
+            const int k = __ldg(p.active_idx + (long long)b * p.n_active + i) - key_lo;
+            if (k >= 0 && k < key_hi - key_lo) map[k] = i;
+        }
+        __syncthreads();
+    }
+    const float *kc = p.k_cache + (long long)bh * p.ctx_len * D, *vc = p.v_cache + (long long)bh * p.ctx_len * D;
+    // the fresh row behind a key of this CTA, or -1
+    auto fresh_row = [&](int key) { return !fresh ? -1 : mapped ? map[key - key_lo] : key; };
+    auto load_kv = [&](int t, int stage) {
+        float* ks = sm + C::kv + stage * C::stage;
+        for (int c = tid; c < BN * D4; c += kThreads) {
+            const int row = c / D4, ch = c % D4, key = t * BN + row;
+            const bool ok = key < p.ctx_len;
+            const float *ksrc = kc, *vsrc = vc;
+            if (ok) {
+                const int i = fresh_row(key);
+                const long long at = i < 0 ? (long long)key * D : (((long long)b * p.n_active + i) * p.n_kv_heads + hk) * D;
+                ksrc = (i < 0 ? kc : p.k_new) + at + ch * 4;
+                vsrc = (i < 0 ? vc : p.v_new) + at + ch * 4;
+            }
+            cp_async16(s2u(ks + row * C::P + ch * 4), ksrc, ok);
+            cp_async16(s2u(ks + (BN + row) * C::P + ch * 4), vsrc, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (t0 < t1) load_kv(t0, 0);
+
+    float m[4], l[4], o[4][OC];
 #pragma unroll
-    for (int t = 0; t < DPL; ++t) orow[lane + 32 * t] = acc[t] * inv;
+    for (int r = 0; r < 4; ++r) {
+        m[r] = -INFINITY;
+        l[r] = 0.f;
+#pragma unroll
+        for (int c = 0; c < OC; ++c) o[r][c] = 0.f;
+    }
+    for (int t = t0; t < t1; ++t) {
+        const int stage = (t - t0) & 1;
+        if (t + 1 < t1) {
+            load_kv(t + 1, stage ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const float *ks = sm + C::kv + stage * C::stage, *vs = ks + BN * C::P;
+        // ---- scores of four rows against two keys ----
+        f32x2 acc[4][2];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = pk(0.f, 0.f);
+#pragma unroll 4
+        for (int ch = 0; ch < D4; ++ch) {
+            const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(ks + tk * C::P + ch * 4);
+            const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(ks + (tk + 16) * C::P + ch * 4);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(sm + C::q + (4 * tr + r) * C::P + ch * 4);
+                acc[r][0] = fma2(qv.y, k0.y, fma2(qv.x, k0.x, acc[r][0]));
+                acc[r][1] = fma2(qv.y, k1.y, fma2(qv.x, k1.x, acc[r][1]));
+            }
+        }
+        const bool in0 = t * BN + tk < p.ctx_len, in1 = t * BN + tk + 16 < p.ctx_len;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float a0, a1, b0, b1;
+            upk(acc[r][0], a0, a1);
+            upk(acc[r][1], b0, b1);
+            const float s0 = in0 ? (a0 + a1) * p.scale : -INFINITY, s1 = in1 ? (b0 + b1) * p.scale : -INFINITY;
+            float mx = fmaxf(s0, s1);
+#pragma unroll
+            for (int d = 8; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+            const float m_new = fmaxf(m[r], mx);   // finite: every tile holds a key of the context
+            const float corr = m[r] == -INFINITY ? 0.f : expf(m[r] - m_new);
+            const float p0 = in0 ? expf(s0 - m_new) : 0.f, p1 = in1 ? expf(s1 - m_new) : 0.f;
+            float sum = p0 + p1;
+#pragma unroll
+            for (int d = 8; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            l[r] = fmaf(l[r], corr, sum);
+            m[r] = m_new;
+#pragma unroll
+            for (int c = 0; c < OC; ++c) o[r][c] *= corr;
+            sm[C::p + (4 * tr + r) * C::pp + tk] = p0;
+            sm[C::p + (4 * tr + r) * C::pp + tk + 16] = p1;
+        }
+        __syncwarp();   // the probabilities of a row are written and read by the same warp
+        // ---- O += P V: output columns 4 tk .. 4 tk + 3 (and 64 + 4 tk .. for D = 128) ----
+#pragma unroll 2
+        for (int k4 = 0; k4 < BN; k4 += 4) {
+            float4 pr[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) pr[r] = *reinterpret_cast<const float4*>(sm + C::p + (4 * tr + r) * C::pp + k4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int c = 0; c < OC; c += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(vs + (k4 + k) * C::P + c * 16 + 4 * tk);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const float pv = k == 0 ? pr[r].x : k == 1 ? pr[r].y : k == 2 ? pr[r].z : pr[r].w;
+                        o[r][c] = fmaf(pv, v.x, o[r][c]);
+                        o[r][c + 1] = fmaf(pv, v.y, o[r][c + 1]);
+                        o[r][c + 2] = fmaf(pv, v.z, o[r][c + 2]);
+                        o[r][c + 3] = fmaf(pv, v.w, o[r][c + 3]);
+                    }
+                }
+            }
+        }
+        // refreshed keys into the cache, from the landed tile: the row tiles that walk over these keys take turns
+        if (fresh && t % p.row_tiles == row_tile) {
+            for (int c = tid; c < BN * D4; c += kThreads) {
+                const int row = c / D4, ch = c % D4, key = t * BN + row;
+                if (key >= p.ctx_len || fresh_row(key) < 0) continue;
+                const long long at = ((long long)bh * p.ctx_len + key) * D + ch * 4;
+                *reinterpret_cast<float4*>(p.k_cache + at) = *reinterpret_cast<const float4*>(ks + row * C::P + ch * 4);
+                *reinterpret_cast<float4*>(p.v_cache + at) = *reinterpret_cast<const float4*>(vs + row * C::P + ch * 4);
+            }
+        }
+        __syncthreads();   // everyone is done with this stage before it is refilled (or becomes the partial)
+    }
+
+    auto out_row = [&](int r) {   // where packed row r goes
+        const int i = r / p.group, j = r - i * p.group;
+        return p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D;
+    };
+    if (p.n_splits == 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r0 + 4 * tr + r >= p.rows_total) continue;
+            float* dst = out_row(r0 + 4 * tr + r);
+            const float inv = 1.f / l[r];
+#pragma unroll
+            for (int c = 0; c < OC; c += 4)
+                *reinterpret_cast<float4*>(dst + c * 16 + 4 * tk) =
+                    make_float4(o[r][c] * inv, o[r][c + 1] * inv, o[r][c + 2] * inv, o[r][c + 3] * inv);
+        }
+        return;
+    }
+    // ---- partial of this CTA, then each CTA of the cluster merges its share of the rows ----
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int c = 0; c < OC; c += 4)
+            *reinterpret_cast<float4*>(sm + C::part + (4 * tr + r) * D + c * 16 + 4 * tk) =
+                make_float4(o[r][c], o[r][c + 1], o[r][c + 2], o[r][c + 3]);
+        if (tk == 0) *reinterpret_cast<float2*>(sm + C::ml + 2 * (4 * tr + r)) = make_float2(m[r], l[r]);
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int per = (BM + p.n_splits - 1) / p.n_splits;   // rows merged by one CTA
+    const int rows_here = min(per, min(BM, p.rows_total - r0) - split * per);
+    for (int idx = tid; idx < rows_here * D4; idx += kThreads) {
+        const int row = split * per + idx / D4, ch = idx % D4;
+        float mm[8], ll[8], x[8][4], M = -INFINITY, L = 0.f;
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const int src = min(s, p.n_splits - 1);
+            ld_peer_v2(map_to_cta(s2u(sm + C::ml + 2 * row), src), mm[s], ll[s]);
+            ld_peer_v4(map_to_cta(s2u(sm + C::part + row * D + ch * 4), src), x[s]);
+        }
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            if (s >= p.n_splits) mm[s] = -INFINITY;
+            M = fmaxf(M, mm[s]);
+        }
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const float e = mm[s] == -INFINITY ? 0.f : expf(mm[s] - M);
+            L = fmaf(e, ll[s], L);
+            a.x = fmaf(e, x[s][0], a.x);
+            a.y = fmaf(e, x[s][1], a.y);
+            a.z = fmaf(e, x[s][2], a.z);
+            a.w = fmaf(e, x[s][3], a.w);
+        }
+        const float inv = 1.f / L;
+        *reinterpret_cast<float4*>(out_row(r0 + row) + ch * 4) = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+    }
+    cluster_arrive_relaxed();   // no CTA leaves while a peer may still read its partial
+    cluster_wait();
+}
+
+template <int D>
+cudaError_t launch_d(const F32Params& p, int batch, cudaStream_t stream) {
+    static PerDeviceOnce once;
+    const size_t smem = Carve<D>::bytes(p.k_new && p.active_idx ? p.tiles_per_split * BN : 0);
+    if (const cudaError_t e = ensure_dynamic_smem(once, attend_f32_kernel<D>, (int)Carve<D>::bytes(kMaxMapKeys)); e != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((long long)batch * p.n_kv_heads * p.row_tiles * p.n_splits), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = p.n_splits;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, attend_f32_kernel<D>, p);
 }
 
 }  // namespace
 
-cudaError_t launch_attend_f32(const AttendArgs& a, cudaStream_t stream) {
-    const long long n_jobs = (long long)a.d.batch * a.n_active * a.d.n_q_heads;
-    if (n_jobs == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((n_jobs + kWarpsPerCta - 1) / kWarpsPerCta);
-    const float* q = static_cast<const float*>(a.q);
-    const float* k = static_cast<const float*>(a.k_cache);
-    const float* v = static_cast<const float*>(a.v_cache);
-    float* o = static_cast<float*>(a.out);
-    if (a.d.head_dim == 64)
-        attend_f32_kernel<64><<<grid, kWarpsPerCta * 32, 0, stream>>>(
-            q, k, v, o, a.d.batch, a.n_active, a.d.ctx_len, a.d.n_q_heads, a.d.n_kv_heads, a.scale);
-    else
-        attend_f32_kernel<128><<<grid, kWarpsPerCta * 32, 0, stream>>>(
-            q, k, v, o, a.d.batch, a.n_active, a.d.ctx_len, a.d.n_q_heads, a.d.n_kv_heads, a.scale);
-    return cudaGetLastError();
+cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
+                              cudaStream_t stream) {
+    if (a.n_active == 0) return cudaSuccess;
+    F32Params p{};
+    p.q = static_cast<const float*>(a.q);
+    p.k_new = static_cast<const float*>(k_new);
+    p.v_new = static_cast<const float*>(v_new);
+    p.k_cache = static_cast<float*>(const_cast<void*>(a.k_cache));
+    p.v_cache = static_cast<float*>(const_cast<void*>(a.v_cache));
+    p.out = static_cast<float*>(a.out);
+    p.active_idx = active_idx;
+    p.n_active = a.n_active;
+    p.ctx_len = a.d.ctx_len;
+    p.n_q_heads = a.d.n_q_heads;
+    p.n_kv_heads = a.d.n_kv_heads;
+    p.group = a.d.n_q_heads / a.d.n_kv_heads;
+    p.rows_total = a.n_active * p.group;
+    p.row_tiles = (p.rows_total + BM - 1) / BM;
+    p.scale = a.scale;
+    // The keys of a row tile are split over as many CTAs (at most eight, at least a tile each) as keep the launch within
+    // four CTAs per SM, which is what shared memory leaves room for.
+    const int n_tiles = (a.d.ctx_len + BN - 1) / BN;
+    const long long units = (long long)a.d.batch * a.d.n_kv_heads * p.row_tiles;
+    int splits = 1;
+    while (splits < 8 && 2 * splits <= n_tiles && 2 * splits * units <= 4LL * sm_count()) splits *= 2;
+    p.tiles_per_split = (n_tiles + splits - 1) / splits;
+    p.n_splits = (n_tiles + p.tiles_per_split - 1) / p.tiles_per_split;
+    if (units * p.n_splits > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    if (k_new && active_idx && p.tiles_per_split * BN > kMaxMapKeys) {   // no room for the table of keys
+        if (const cudaError_t e = launch_refresh(a.d, p.k_cache, p.v_cache, k_new, v_new, active_idx, a.n_active, stream);
+            e != cudaSuccess)
+            return e;
+        p.k_new = p.v_new = nullptr;
+    }
+    return a.d.head_dim == 64 ? launch_d<64>(p, a.d.batch, stream) : launch_d<128>(p, a.d.batch, stream);
 }
 
 }  // namespace ec

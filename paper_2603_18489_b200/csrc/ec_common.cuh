@@ -117,9 +117,12 @@ struct AttendArgs {
     void* refresh_k_dst = nullptr;
     void* refresh_v_dst = nullptr;
 };
-size_t attend_workspace_bytes(const ec_attn_desc& d, int n_active);
-cudaError_t launch_attend_f32(const AttendArgs& a, cudaStream_t stream);
-cudaError_t launch_attend_bf16(const AttendArgs& a, cudaStream_t stream);      // mma.sync path (any head_dim)
+// fp32: refresh and attention in one launch (k_new == nullptr: attention alone)
+cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
+                              cudaStream_t stream);
+// mma.sync path (any head_dim): refresh and attention in one launch (k_new == nullptr: attention alone)
+cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
+                               cudaStream_t stream);
 // fused skip-step path (bf16, head_dim 128, n_active * H_q/H_kv <= 256): refresh + attention + merge in one launch
 bool attend_skip_supported(const ec_attn_desc& d, int n_active);
 // host-only descriptions of the launch the plan functions choose ("kernel<instantiation> grid=... cluster=..."),

@@ -9,7 +9,11 @@
 // source, so reads are fully coalesced and writes are coalesced per head row.
 // With idx == nullptr the list is the identity (recompute step) and the kernel
 // is a [n, H, D] -> [H, n, D] layout-changing copy.
+//
+// A partial step moves some tens of KB and is a launch latency long, so the kernel is launched with programmatic stream
+// serialisation: its start overlaps the end of the kernel before it.
 #include "ec_common.cuh"
+#include "ec_tc_ptx.cuh"
 
 namespace ec {
 namespace {
@@ -29,6 +33,8 @@ __global__ void __launch_bounds__(256) refresh_kernel(uint4* __restrict__ k_cach
     const long long bi = bih / n_kv_heads;
     const int i = (int)(bi % n_active);
     const long long b = bi / n_active;
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
     const int pos = idx ? __ldg(idx + bi) : i;
     if (pos < 0 || pos >= ctx_len) return;  // never write outside the cache
     const long long dst = ((b * n_kv_heads + h) * ctx_len + pos) * row_vecs + piece;
@@ -48,10 +54,18 @@ cudaError_t launch_refresh(const ec_attn_desc& d, void* k_cache, void* v_cache, 
     const long long total = (long long)d.batch * n_active * d.n_kv_heads * row_vecs;
     if (total == 0) return cudaSuccess;
     const dim3 grid((unsigned)((total + 255) / 256), 2);
-    refresh_kernel<<<grid, 256, 0, stream>>>(static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache),
-                                             static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
-                                             active_idx, n_active, d.ctx_len, d.n_kv_heads, row_vecs, total);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, refresh_kernel, static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache),
+                              static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), active_idx, n_active,
+                              d.ctx_len, d.n_kv_heads, row_vecs, total);
 }
 
 }  // namespace ec
