@@ -25,7 +25,7 @@
 //               the tensor pipe for the same row tile.
 //   warp 18     recompute steps only: every cache row is overwritten by the fresh row of the same position, so the
 //               launch reads K/V straight from the token-major k_new / v_new (only the tensor map's strides
-//               differ) and this warp copies them into the cache meanwhile: no separate refresh pass.
+//               differ) and this warp stores landed tiles into the cache meanwhile: no separate refresh pass.
 // TMEM (512 columns): S_0 [0,128), S_1 [128,256), O_0 [256,384), O_1 [384,512).
 // Shared memory: Q_0, Q_1 (32 KB each, staged once), five 32 KB K/V slots, barriers: 225 KB, one CTA per SM.
 // Every mbarrier wait is bounded; a wait that runs out sets EC_ERR_TIMEOUT in the caller's dev_status word and
@@ -56,17 +56,17 @@ constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
 enum { B_FULL = 0, B_EMPTY = kSlots, B_SFULL = 2 * kSlots, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 2,
-       B_QFULL = B_PVDONE + 2, B_COUNT = B_QFULL + 1 };
+       B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 1, B_COUNT = B_VERDICT + 1 };
+
+// first pass: a row's sum may grow to this before the unit is done again with running maxima
+constexpr float kMaxSum = 1.152921504606846976e18f;   // 2^60
 
 struct DenseParams {
     const __nv_bfloat16* q;
     __nv_bfloat16* out;
     // recompute step: the K/V this launch reads are the token-major fresh tensors [B, L, Hkv, 128]; its copy warp
-    // writes them into the caches [B, Hkv, L, 128] (nullptr: nothing to copy)
-    const uint4* k_src;
-    const uint4* v_src;
-    uint4* k_dst;
-    uint4* v_dst;
+    // stores their tiles into the caches [B, Hkv, L, 128]
+    int copy;
     int32_t* dev_status;
     int n_active, ctx_len, n_q_heads, n_kv_heads, group, rows_total;
     // Grouped-query shapes run with one unit per QUERY head (the kernel then sees n_kv_heads = n_q_heads = H_q and
@@ -84,13 +84,15 @@ constexpr int kPartFloats = BM * (HD + 2);   // one row tile of one part
 
 __global__ void __launch_bounds__(kThreads, 1)
 attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                    const __grid_constant__ CUtensorMap map_q, const DenseParams p) {
+                    const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kd,
+                    const __grid_constant__ CUtensorMap map_vd, const DenseParams p) {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
     const uint32_t bars = base + OFF_BAR;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + OFF_BAR + B_COUNT * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + OFF_BAR + B_COUNT * 8 + 4);
+    volatile int* again = reinterpret_cast<volatile int*>(gbase + OFF_BAR + B_COUNT * 8 + 8);   // verdict of the first pass
     float* xch = reinterpret_cast<float*>(gbase + OFF_XCH);
     auto bar = [&](int idx) { return bars + idx * 8; };
     if (base - s2u(smem_raw) + SMEM_NEEDED > SMEM_BYTES) {   // never with the 1024-byte alignment the runtime gives
@@ -116,7 +118,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         prefetch_map(&map_k);
         prefetch_map(&map_v);
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 2) ? 256u : 1u);
+            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 2) ? 256u : (p.copy && i >= B_EMPTY && i < B_EMPTY + kSlots) ? 2u : 1u);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -141,49 +143,72 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             mbar_expect_tx(bar(B_QFULL), (uint32_t)n_tiles_q * TILE);
             for (int t = 0; t < n_tiles_q; ++t)
                 tma_load_5d(base + OFF_Q + t * TILE, &map_q, 0, r_pair + t * BM, hk, 0, b, bar(B_QFULL));
-            for (int n = 0; n < 2 * T; ++n) {   // ring index: K_j = 2j, V_j = 2j + 1
-                const int slot = n % kSlots, u = n / kSlots;
+            for (int n = 0; n < 4 * T; ++n) {   // ring index: K_j = 2j, V_j = 2j + 1; from 2T on the second pass
+                if (n == 2 * T) {
+                    mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                    if (!*again) break;
+                }
+                const int slot = n % kSlots, u = n / kSlots, j = (n >> 1) % T;
                 if (u > 0) mbar_wait(bar(B_EMPTY + slot), (u - 1) & 1, abort_flag, p.dev_status);
                 mbar_expect_tx(bar(B_FULL + slot), TILE);
-                tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, (j0 + (n >> 1)) * BN, 0, hk_kv, b, bar(B_FULL + slot));
+                tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, (j0 + j) * BN, 0, hk_kv, b, bar(B_FULL + slot));
             }
         }
     } else if (warp == 1) {
         // ================================ MMA issuer ========================================
         if (lane == 0) {
             constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
-            auto wait_full = [&](int n) { mbar_wait(bar(B_FULL + n % kSlots), (n / kSlots) & 1, abort_flag, p.dev_status); };
-            auto issue_s = [&](int t, int j) {
-                const uint32_t kst = base + OFF_RING + ((2 * j) % kSlots) * TILE;
+            const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024);
+            auto issue_s = [&](int t, int slot_k) {
+                const uint64_t desc_k = smem_desc(base + OFF_RING + slot_k * TILE, 16, 1024);
 #pragma unroll
                 for (int k = 0; k < HD / 16; ++k) {
-                    const uint32_t koff = (k >> 2) * SUB + (k & 3) * 32;
-                    mma_ss(tmem + TM_S + t * 128, smem_desc(base + OFF_Q + t * TILE + koff, 16, 1024),
-                           smem_desc(kst + koff, 16, 1024), IDESC_S, k > 0);
+                    const uint32_t koff = ((k >> 2) * SUB + (k & 3) * 32) / 16;
+                    mma_ss(tmem + TM_S + t * 128, desc_q + t * (TILE / 16) + koff, desc_k + koff, IDESC_S, k > 0);
                 }
                 commit(bar(B_SFULL + t));
             };
             mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
-            wait_full(0);
-            fence_after();
-            for (int t = 0; t < n_tiles_q; ++t) issue_s(t, 0);
-            commit(bar(B_EMPTY + 0));   // K_0 is free once both S(0) have run
-            for (int j = 0; j < T; ++j) {
-                wait_full(2 * j + 1);   // V_j
-                if (j + 1 < T) wait_full(2 * j + 2);   // K_{j+1}
-                const uint32_t vst = base + OFF_RING + ((2 * j + 1) % kSlots) * TILE;
-                for (int t = 0; t < n_tiles_q; ++t) {
-                    mbar_wait(bar(B_PFULL + t), j & 1, abort_flag, p.dev_status);
-                    fence_after();
-#pragma unroll
-                    for (int k = 0; k < BN / 16; ++k)
-                        mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + k * 8, smem_desc(vst + k * 2048, SUB, 1024),
-                               IDESC_PV, (j > 0 || k > 0));
-                    commit(bar(B_PVDONE + t));
-                    if (j + 1 < T) issue_s(t, j + 1);
+            int slot = 0;          // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...
+            uint32_t phase = 0, p_phase = 0;
+            auto advance = [&]() {
+                const int s = slot;
+                if (++slot == kSlots) slot = 0, phase ^= 1;
+                return s;
+            };
+            for (int pass = 0; pass < 2; ++pass) {
+                if (pass == 1) {
+                    mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                    if (!*again) break;
                 }
-                commit(bar(B_EMPTY + (2 * j + 1) % kSlots));              // V_j
-                if (j + 1 < T) commit(bar(B_EMPTY + (2 * j + 2) % kSlots));   // K_{j+1}
+                mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+                fence_after();
+                for (int t = 0; t < n_tiles_q; ++t) issue_s(t, slot);
+                commit(bar(B_EMPTY + advance()));   // K_0 is free once both S(0) have run
+                for (int j = 0; j < T; ++j, p_phase ^= 1) {
+                    mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+                    const int vs = advance();            // V_j
+                    int ks = 0;
+                    const bool more = j + 1 < T;
+                    if (more) {
+                        mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+                        ks = advance();                  // K_{j+1}
+                    }
+                    const uint64_t desc_v = smem_desc(base + OFF_RING + vs * TILE, SUB, 1024);
+                    for (int t = 0; t < n_tiles_q; ++t) {
+                        mbar_wait(bar(B_PFULL + t), p_phase, abort_flag, p.dev_status);
+                        fence_after();
+                        // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95
+#pragma unroll
+                        for (int k = 0; k < BN / 16; ++k)
+                            mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
+                                   IDESC_PV, (j > 0 || k > 0));
+                        if (more) issue_s(t, ks);
+                        commit(bar(B_PVDONE + t));
+                    }
+                    commit(bar(B_EMPTY + vs));
+                    if (more) commit(bar(B_EMPTY + ks));
+                }
             }
         }
     } else if (warp < 2 + kSoftThreads / 32) {
@@ -205,8 +230,77 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             float m_used = -INFINITY, l_run = 0.f;
             const float sl2 = p.scale_log2;
             const f32x2 sl2_2 = pk(sl2, sl2);
-            for (int j = 0; j < T; ++j) {
-                mbar_wait(bar(B_SFULL + t), j & 1, abort_flag, p.dev_status);
+            // ---- first pass: no running maximum.  The reference of a row is its largest score among the first eight keys
+            //      (both threads of the row read those), so a thread needs nothing from its partner and nothing is
+            //      reduced: probabilities may exceed 1 by what fp32 and bf16 exponents have room for, and the row sum
+            //      tells at the end whether they stayed within it. ----
+            {
+                f32x2 mneg2 = pk(0.f, 0.f), sum2[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};
+                for (int j = 0; j < T; ++j) {
+                    mbar_wait(bar(B_SFULL + t), j & 1, abort_flag, p.dev_status);
+                    fence_after();
+                    if (j == 0) {
+                        uint32_t r8[8];
+                        ld8(tm_s, r8);
+                        wait_ld();
+                        float mx = __uint_as_float(r8[0]);
+#pragma unroll
+                        for (int c = 1; c < 8; ++c)
+                            if (j0 * BN + c < p.ctx_len) mx = fmaxf(mx, __uint_as_float(r8[c]));
+                        m_used = mx * sl2;
+                        mneg2 = pk(-m_used, -m_used);
+                        named_barrier(pair_bar, 64);   // both threads of the row have read what P is about to overwrite
+                    }
+                    uint32_t sr[2][32];
+                    ld32(tm_s + h * 64, sr[0]);
+                    wait_ld();
+                    ld32(tm_s + h * 64 + 32, sr[1]);   // on its way while the first 32 scores are worked on
+                    const int key0 = (j0 + j) * BN + h * 64;
+                    const bool ragged = key0 + 64 > p.ctx_len;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (q == 1) wait_ld();
+                        if (ragged) {
+#pragma unroll
+                            for (int c = 0; c < 32; ++c)
+                                if (key0 + q * 32 + c >= p.ctx_len) sr[q][c] = 0xff800000u;   // -inf
+                        }
+                        uint32_t pw[16];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            const f32x2 d2 = fma2(pk(__uint_as_float(sr[q][2 * c]), __uint_as_float(sr[q][2 * c + 1])), sl2_2, mneg2);
+                            float d0, d1;
+                            upk(d2, d0, d1);
+                            const float e0 = fast_exp2(d0), e1 = fast_exp2(d1);
+                            sum2[c & 1] = add2(sum2[c & 1], pk(e0, e1));
+                            pw[c] = pack_bf16x2(e0, e1);
+                        }
+                        // P (bf16 pairs) over the first half of this thread's own scores
+                        st16(tm_s + h * 64 + q * 16, pw);
+                    }
+                    wait_st();
+                    fence_before();
+                    mbar_arrive(bar(B_PFULL + t));
+                }
+                float a0, a1, b0, b1;
+                upk(sum2[0], a0, a1);
+                upk(sum2[1], b0, b1);
+                l_run = (a0 + a1) + (b0 + b1);   // this half's share of the row sum
+            }
+            int done = T;   // tiles of both passes behind us
+            const bool redo = named_barrier_or(9, n_tiles_q * 256, !(l_run <= kMaxSum));
+            if (ws == 0 && lane == 0) {
+                *again = redo ? 1 : 0;
+                mbar_arrive(bar(B_VERDICT));
+            }
+            // ---- second pass, only if a score left the first one's range: running maxima ----
+            if (redo) {
+                m_used = -INFINITY;
+                l_run = 0.f;
+                done = 2 * T;
+            }
+            for (int j = 0; redo && j < T; ++j) {
+                mbar_wait(bar(B_SFULL + t), (T + j) & 1, abort_flag, p.dev_status);
                 fence_after();
                 uint32_t sr[BN / 2];
                 ld32(tm_s + h * 64, sr);
@@ -254,7 +348,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (need_rescale) {
                     // O holds tiles < j: P V of tile j - 1 must have completed before the accumulator is scaled;
                     // each of the two threads of a row scales its 64 columns
-                    mbar_wait(bar(B_PVDONE + t), (j - 1) & 1, abort_flag, p.dev_status);
+                    mbar_wait(bar(B_PVDONE + t), (T + j - 1) & 1, abort_flag, p.dev_status);
                     fence_after();
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
@@ -266,15 +360,15 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         st32(tm_o + h * 64 + c * 32, o);
                     }
                 }
-                // P (bf16 pairs) over the first 64 columns of S_t: this thread's 64 keys are columns [32 h, 32 h + 32)
-                st32(tm_s + h * 32, pw);
+                // P (bf16 pairs) over the first half of this thread's own scores
+                st32(tm_s + h * 64, pw);
                 wait_st();
                 fence_before();
                 mbar_arrive(bar(B_PFULL + t));
             }
 
             // ---- epilogue ------------------------------------------------------------------------
-            mbar_wait(bar(B_PVDONE + t), (T - 1) & 1, abort_flag, p.dev_status);
+            mbar_wait(bar(B_PVDONE + t), (done - 1) & 1, abort_flag, p.dev_status);
             fence_after();
             *xch_mine = l_run;
             named_barrier(pair_bar, 64);
@@ -327,38 +421,33 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         }
         fence_before();
-    } else if (p.k_dst != nullptr && part == 0) {
+    } else if (p.copy && lane == 0) {
         // ====================== copy warp: this CTA's share of the refresh ============================
-        // The (row-tile pair, kv head) CTAs of a head split its positions evenly; a position's K and V rows
-        // (256 bytes each) go from [b, pos, hk, :] to [b, hk, pos, :].  Two rows per warp instruction, eight
-        // instructions in flight.  Nobody reads the cache in this launch.
-        // (with one unit per query head, the kv_div units of a real kv head share its positions as well)
+        // The key tiles that stream through the ring ARE the fresh rows: those of this CTA's share go from shared memory to
+        // the cache by TMA (the same box through the cache's map; rows past L are not written), so the cache update reads
+        // nothing.  The units of a kv head (its query heads' row-tile pairs) take turns by tile.  Nobody reads the cache
+        // in this launch.  (A warp that copied its share of the rows through registers took longer than the six key
+        // tiles of a unit at L = 768.)
         const int hk_kv = hk / p.kv_div;
-        const int n_share = p.n_pairs * p.kv_div;
-        const int per = (p.ctx_len + n_share - 1) / n_share;
-        const int pos0 = ((hk % p.kv_div) * p.n_pairs + pair) * per, pos1 = min(p.ctx_len, pos0 + per);
-        const int sub = lane >> 4, piece = lane & 15;
-        for (int pos = pos0; pos < pos1; pos += 16) {
-            uint4 kv[8], vv[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int pp = pos + 2 * u + sub;
-                if (pp < pos1) {
-                    const long long src = (((long long)b * p.ctx_len + pp) * p.n_kv_real + hk_kv) * 16 + piece;
-                    kv[u] = __ldg(p.k_src + src);
-                    vv[u] = __ldg(p.v_src + src);
-                }
+        const int n_share = p.n_pairs * p.kv_div, mine = (hk % p.kv_div) * p.n_pairs + pair;
+        int slot = 0;
+        uint32_t phase = 0;
+        for (int n = 0; n < 4 * T; ++n) {   // (on a second pass the tiles only pass by)
+            if (n == 2 * T) {
+                mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                if (!*again) break;
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int pp = pos + 2 * u + sub;
-                if (pp < pos1) {
-                    const long long dst = (((long long)b * p.n_kv_real + hk_kv) * p.ctx_len + pp) * 16 + piece;
-                    p.k_dst[dst] = kv[u];
-                    p.v_dst[dst] = vv[u];
-                }
+            mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+            const int j = j0 + (n >> 1);
+            if (n < 2 * T && j % n_share == mine && !*abort_flag) {
+                tma_store_5d((n & 1) ? &map_vd : &map_kd, base + OFF_RING + slot * TILE, 0, j * BN, 0, hk_kv, b);
+                bulk_commit();
+                bulk_wait_read();   // the slot has been read
             }
+            mbar_arrive(bar(B_EMPTY + slot));
+            if (++slot == kSlots) slot = 0, phase ^= 1;
         }
+        bulk_wait();
     }
 
     __syncthreads();
@@ -497,7 +586,7 @@ bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
     const long long pairs = ((long long)n_active + 2 * BM - 1) / (2 * BM);
     const long long bh = (long long)d.batch * d.n_q_heads;
     if (pairs * bh > 0x3fffffffLL) return false;
-    return pairs * bh >= sm_count() / 2;
+    return pairs * bh >= sm_count() / 4;
 }
 
 size_t attend_dense_workspace_bytes(const ec_attn_desc& d, int n_active) {
@@ -521,11 +610,11 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     DenseParams p;
     p.q = static_cast<const __nv_bfloat16*>(a.q);
     p.out = static_cast<__nv_bfloat16*>(a.out);
-    const bool copy = a.kv_token_major && a.refresh_k_dst && a.refresh_v_dst;
-    p.k_src = copy ? static_cast<const uint4*>(a.k_cache) : nullptr;
-    p.v_src = copy ? static_cast<const uint4*>(a.v_cache) : nullptr;
-    p.k_dst = copy ? static_cast<uint4*>(a.refresh_k_dst) : nullptr;
-    p.v_dst = copy ? static_cast<uint4*>(a.refresh_v_dst) : nullptr;
+    p.copy = a.kv_token_major && a.refresh_k_dst && a.refresh_v_dst;
+    CUtensorMap map_kd = map_k, map_vd = map_v;   // placeholders unless copying
+    if (p.copy && (!make_kv_map(&map_kd, a.refresh_k_dst, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false) ||
+                   !make_kv_map(&map_vd, a.refresh_v_dst, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false)))
+        return cudaErrorInvalidValue;
     p.dev_status = a.dev_status;
     p.n_active = a.n_active;
     p.ctx_len = a.d.ctx_len;
@@ -571,7 +660,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (const cudaError_t el = cudaLaunchKernelEx(&cfg, attend_dense_kernel, map_k, map_v, map_q, p); el != cudaSuccess) return el;
+    if (const cudaError_t el = cudaLaunchKernelEx(&cfg, attend_dense_kernel, map_k, map_v, map_q, map_kd, map_vd, p); el != cudaSuccess) return el;
     if (pl.split == 1) return cudaSuccess;
     CombineParams c{p.part, p.out, pl.n_pairs, pl.n_full, pl.split, a.n_active, a.d.n_q_heads, a.n_active};
     cfg.gridDim = dim3((pl.units - pl.n_full) * 8, 1, 1);   // (cut unit, row tile, 32-row group)
