@@ -9,20 +9,20 @@
 //     S^T[128 keys x N]  = K_tile[128 keys x 128] . Q[N x 128]^T          (A = K tile, B = Q, both K-major)
 //     O^T[128 d    x N] += V_tile^T[128 d x 128 keys] . P^T[128 keys x N]  (A = V tile MN-major, B = P^T MN-major)
 // so a softmax thread owns one KEY (TMEM lane) and its scores against the query slots: all 128 lanes work, one
-// exponential per (key, query), no padding rows, a pipeline step covers 128 keys.  The row sums sum_keys P are
-// taken by two auxiliary warps that read P^T back from shared memory (where the softmax threads put it for the
-// second product), so the softmax threads carry no running sums.  With N = 96 (the paper's default budget k = 64
-// gives 96 active rows) two softmax warpgroups share the columns of a key.
+// exponential per (key, query), no padding rows, a pipeline step covers 128 keys.  A thread keeps its key lane's share of
+// every row sum in registers; they are added up over the lanes once, at the end.  (Two auxiliary warps that read P^T back
+// from shared memory took 1.2 us a tile and set the pace: 15.9 us a launch at L = 1983 with 96 rows, now 13.7.)  With
+// N = 96 (the paper's default budget k = 64 gives 96 active rows) two softmax warpgroups share the columns of a key.
 //   softmax  the references m[q] (log2 units) are shared by all keys of the CTA and live in shared memory.  The first
 //            is the score of one valid key; p = 2^(s*scale*log2e - m[q]) needs no reduction as long as no score exceeds
 //            its reference by more than 2^60 (bf16 and fp32 have room for that, and a reference is never above the true
 //            maximum).  A barrier-wide OR tells: only then the column maxima are reduced, m is raised, and O^T and the
 //            row sums are rescaled;
 //   grid     (C, B*H_kv*n_sub) as clusters of C <= 8 CTAs (any count, not only powers of two) that split one
-//            head's 128-key tiles, chosen so that the most-loaded SM streams the fewest tiles; CTAs that hold a
-//            single tile are small enough for two per SM.  With grouped-query attention the query heads of a kv
-//            head are packed into the N axis; when they exceed the slots the heads (and, beyond 96 active rows,
-//            the rows) are spread over n_sub CTA columns that stream the same K/V (L2 serves the repeats);
+//            head's 128-key tiles, chosen so that the most-loaded SM streams the fewest tiles.  With grouped-query
+//            attention the query heads of a kv head are packed into the N axis; when they exceed the slots the heads
+//            (and, beyond 96 active rows, the rows) are spread over n_sub CTA columns that stream the same K/V (L2
+//            serves the repeats);
 //   K/V      the producer warp issues its TMA loads in key order through a ring of NS slots of 32 KB (K_0 V_0 K_1 V_1
 //            ...: a K slot is free again as soon as the scores of its tile are computed, a V slot after the second
 //            product, and an odd slot count is possible, which is what lets the 96-slot instantiation keep two and
@@ -34,22 +34,21 @@
 //            fresh tensors (a [128 rows x 128] box of k_new is laid out exactly like a cache tile) after its cache
 //            tiles (visited first they held a ring stage through the start of the stream and set that CTA two tile
 //            times behind its peers), while every CTA masks the stale cached keys of the refreshed positions (a bit per key, built from
-//            the index list).  The attention therefore never waits for the cache update: the auxiliary warps of that
-//            CTA copy the fresh rows from the landed tile to the cache in global memory with plain 16-byte stores,
-//            for later steps, ordered against nothing.  (Keys
-//            in a different order, the same sum.)  When a CTA holds a single cache tile the extra tiles get a CTA of
-//            their own, so that nobody streams two tiles through one stage;
+//            the index list).  The attention therefore never waits for the cache update: the auxiliary warps copy the
+//            fresh rows to the cache in global memory, for later steps, ordered against nothing.  (Keys in a different
+//            order, the same sum.)  When a CTA holds a single cache tile the extra tiles get a CTA of their own;
 //   merge    CTA c of the cluster owns the output columns d in [c*DL, (c+1)*DL).  Every CTA leaves its O (un-normalised),
 //            m and l in its own shared memory; after a cluster barrier the owners read their columns of all C partials out
 //            of the peers (128-byte pieces: a warp whose lanes read different rows takes 2.1 us for what this does in 0.6),
 //            combine, normalise and store; a second cluster barrier keeps every CTA's shared memory alive until its
 //            peers have read it.
-// What bounds it: HBM at long contexts (L = 4096, one sequence, 34 rows: 68.8 MB in 17.1 us), the serial path below that:
-// a launch of one tile per CTA takes 7.6 us, of which the dependency wait is 0.8, Q 0.5, the scores 1.2, the softmax
-// 1.2, P V and the row sums 0.7, the merge 1.9 with its barriers and the exit 0.7.  Code that runs once is fetched
-// about as slowly as it runs, so this path is kept short: index arithmetic before the wait, rolled loops in the merge.
+// What bounds it: HBM at long contexts (L = 4096, one sequence, 34 rows: 68.8 MB in 16.2 us), the serial path below that:
+// a launch of one tile per CTA takes 7.1 us: dependency wait 0.8, Q 0.5, scores 1.2, softmax 1.2, P V 0.6, the merge 1.9
+// with its barriers, the exit 0.7.  Code that runs once is fetched about as slowly as it runs, so this path is kept
+// short: index arithmetic before the wait, rolled loops in the merge.  One CTA per SM: with 128 registers a thread, which
+// two would need, the softmax spills and the launches of L = 768 to 4096 take 0.7 to 2 us more.
 // warp 0: TMA producer; warp 1: tcgen05.mma issue; next 4 (or 8) warps: Q, softmax; the auxiliary warps: stale-key bits,
-// cache update, row sums.  Launched with programmatic stream serialisation; what the previous kernel wrote is read only
+// cache update.  Launched with programmatic stream serialisation; what the previous kernel wrote is read only
 // after griddepcontrol.wait.  Every mbarrier wait is bounded (EC_ERR_TIMEOUT in dev_status, CTA-wide abort flag: an
 // aborted CTA stores no output); the CTA always frees its TMEM and exits.
 #include "ec_common.cuh"
@@ -66,9 +65,8 @@ namespace {
 using namespace tc;
 
 constexpr int BK = 128, HD = 128;
-// auxiliary warps (cache update and row sums): two, or four for the 96-slot instantiation, whose row sums over twice
-// the columns otherwise trail the softmax and hold up the merge
-__host__ __device__ constexpr int aux_threads(int n) { return n > 64 ? 128 : 64; }
+constexpr int kAuxThreads = 64;            // auxiliary warps: stale-key bits and cache update
+__host__ __device__ constexpr int block_threads(int n) { return 64 + (n > 64 ? 256 : 128) + kAuxThreads; }
 constexpr uint32_t SUB = 128 * 128;        // [128 rows x 64 bf16], 128-byte swizzle: 16 KB
 constexpr uint32_t TILE = 2 * SUB;         // [128 x 128] bf16
 constexpr uint32_t STAGE = 2 * TILE;       // K tile + V tile: 64 KB
@@ -78,7 +76,7 @@ constexpr int kMaxActive = 256;            // active rows of a sequence (refresh
 constexpr int kMaxTiles = 1024;            // key tiles of one CTA
 
 enum { B_FULL = 0, B_EMPTY = kMaxStages, B_SFULL = 2 * kMaxStages, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 1,
-       B_PSUM = B_PVDONE + 1, B_QFULL = B_PSUM + 1, B_LIST = B_QFULL + 1, B_COUNT = B_LIST + 1 };
+       B_QFULL = B_PVDONE + 1, B_LIST = B_QFULL + 1, B_COUNT = B_LIST + 1 };
 
 constexpr uint32_t kBarBytes = (B_COUNT * 8u + 15u) & ~15u;   // the barrier block, padded so that what follows is 16-byte aligned
 
@@ -97,7 +95,7 @@ __device__ __forceinline__ void touch(V v) {
     else asm volatile("" ::"r"((uint32_t)v) : "memory");
 }
 
-// COLS consecutive 32-bit columns of this thread's TMEM lane -> registers (and back).  ALIGNED32: the first column is
+// COLS consecutive 32-bit columns of this thread's TMEM lane -> registers.  ALIGNED32: the first column is
 // a multiple of 32 (one 32-column access, then the rest); otherwise 16-column accesses at multiples of 16.
 template <int COLS, bool ALIGNED32>
 __device__ __forceinline__ void ld_row(uint32_t taddr, uint32_t* r) {
@@ -111,18 +109,6 @@ __device__ __forceinline__ void ld_row(uint32_t taddr, uint32_t* r) {
     }
     wait_ld();
 }
-template <int COLS, bool ALIGNED32>
-__device__ __forceinline__ void st_row(uint32_t taddr, const uint32_t* r) {
-    if (ALIGNED32) {
-        st32(taddr, r);
-        if (COLS == 48) st16(taddr + 32, r + 32); else st32(taddr + 32, r + 32);
-    } else {
-#pragma unroll
-        for (int c = 0; c < COLS; c += 16) st16(taddr + c, r + c);
-    }
-    wait_st();
-}
-
 struct KeysParams {
     const __nv_bfloat16* q;
     const __nv_bfloat16* k_new;   // nullptr: attend without refreshing
@@ -133,12 +119,14 @@ struct KeysParams {
     __nv_bfloat16* out;
     int32_t* dev_status;
     int n_active, ctx_len, n_q_heads, n_kv_heads;
-    int group;        // query heads of one kv head handled by one CTA column (a divisor of H_q / H_kv)
+    int q_per_kv;     // H_q / H_kv
+    int group;        // query heads of one kv head handled by one CTA column (the last one may have fewer: its packed
+                      // rows keep the stride, the rows of the heads it lacks are empty)
     int group_inv;    // ceil(2^16 / group): r / group = (r * group_inv) >> 16 for packed rows r < 256
     int quads_inv;    // ceil(2^16 / (dl / 4)), for the items of the merge
     int rows_chunk;   // active rows handled by one CTA column (the last chunk may hold fewer)
     int n_sub_r;      // row chunks = ceil(n_active / rows_chunk)
-    int n_sub;        // CTA columns per kv head = ((H_q / H_kv) / group) * n_sub_r
+    int n_sub;        // CTA columns per kv head = ceil(q_per_kv / group) * n_sub_r
     int n_splits, tiles_per_split, n_stages;
     int shift;        // 1: the first CTA of the cluster takes one cache tile more and the last, which also visits the
                       // fresh tiles, one less (ranges of the CTAs in between move up by one tile)
@@ -161,15 +149,13 @@ struct alignas(16) KeysShared {
     uint32_t tmem;
     int abort_flag;
     int pad[2];
-    volatile int raised[2];                    // [warpgroup]: the last tile whose softmax raised its references
     alignas(16) float m[kMaxSlots];            // reference maxima of the query rows, log2 units (read as float2)
     alignas(16) float factor[2][kMaxSlots];    // [tile parity]: rescale factors of that tile's slow path
-    alignas(16) float lpart[2][kMaxSlots];     // row sums of the CTA's keys, one partial per group of row-sum threads
-    float colmax[4][kMaxSlots];                // per-warp column maxima of the current slow path
+    float col[4][kMaxSlots];                   // per warp and column: maxima of the current slow path, at the end row sums
 };
 
 template <int N>
-__global__ void __launch_bounds__(64 + (N > 64 ? 256 : 128) + aux_threads(N), N <= 64 ? 2 : 1)
+__global__ void __launch_bounds__(block_threads(N), 1)
 attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                         const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
                         const KeysParams p) {
@@ -177,14 +163,11 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     constexpr int WG = N > 64 ? 2 : 1;          // softmax warpgroups: each takes NH of a key's N scores
     constexpr int NH = N / WG;
     constexpr int kSoft = 128 * WG;
-    constexpr int kAuxThreads = aux_threads(N);
-    constexpr int kThreads = 64 + kSoft + kAuxThreads;
+    constexpr int kThreads = block_threads(N);
     // tensor-memory columns: S^T x 2 and O^T at multiples of NP (the slots rounded up to 64 or 128)
     constexpr uint32_t NP = N <= 64 ? 64 : 128;
     constexpr uint32_t TM_S = 0, TM_O = 2 * NP;
     constexpr uint32_t TM_COLS = (3 * NP <= 256) ? 256 : 512;
-    // row-sum threads: a column pair and a share of the tile's keys each
-    constexpr int kPairs = N / 2, kParts = (kAuxThreads / kPairs) >= 2 ? 2 : 1;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
@@ -197,7 +180,9 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = blockIdx.x, bh = blockIdx.y / p.n_sub, sub = blockIdx.y % p.n_sub;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
-    const int hq0 = (hk * (p.n_sub / p.n_sub_r) + sub / p.n_sub_r) * p.group;   // first query head of this CTA
+    const int hg = sub / p.n_sub_r * p.group;                                  // first query head of this CTA in its kv head
+    const int hq0 = hk * p.q_per_kv + hg;                                      // ... and of all
+    const int heads = min(p.group, p.q_per_kv - hg);                           // (the last column may have fewer)
     const int i0 = (sub % p.n_sub_r) * p.rows_chunk;                           // first active row of this CTA
     const int rows_total = min(p.rows_chunk, p.n_active - i0) * p.group;       // packed query rows of this CTA
     const int C = p.n_splits;
@@ -230,7 +215,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         for (int i = 0; i < B_COUNT; ++i) {
             uint32_t count = 1;
             if (i == B_PFULL || i == B_QFULL) count = kSoft;
-            if (i == B_PSUM || i == B_LIST) count = kAuxThreads;
+            if (i == B_LIST) count = kAuxThreads;
             mbar_init(bar(i), count);
         }
         sh->abort_flag = 0;
@@ -254,7 +239,6 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     if (refresh)
         for (int w = tid; w < TC * 4; w += kThreads) stale[w] = 0u;
     if (tid < N) sh->m[tid] = -INFINITY;
-    if (tid < 2) sh->raised[tid] = -1;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s2u(&sh->tmem)), "r"(TM_COLS)
                      : "memory");
@@ -274,7 +258,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         for (int u = 0; u < kPieces; ++u) {
             const int row = (stid >> 4) + u * (kSoft / 16);
             const int i = (row * p.group_inv) >> 16, jh = row - i * p.group;
-            q_off[u] = row < rows_total ? ((i0 + i) * p.n_q_heads + hq0 + jh) * HD + (stid & 15) * 8 : -1;
+            q_off[u] = (row < rows_total && jh < heads) ? ((i0 + i) * p.n_q_heads + hq0 + jh) * HD + (stid & 15) * 8 : -1;
             touch(q_off[u]);
         }
     }
@@ -383,7 +367,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             }
         }
     } else if (warp >= 2 + 4 * WG) {
-        // ===== auxiliary warps: stale-key bits; the fresh rows into the cache (for later steps); row sums of P^T =====
+        // ===== auxiliary warps: stale-key bits; the fresh rows into the cache (for later steps) =====
         const int atid = tid - (64 + kSoft);
         if (refresh) {
             // which cached keys of this CTA's range are about to be refreshed: they are attended from k_new / v_new (as
@@ -394,62 +378,33 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             }
             mbar_arrive(bar(B_LIST));   // release: the bits above are visible to whoever waits
         }
-        // row sums: this thread adds up column pair cp of the keys [k_lo, k_lo + BK / kParts) of every tile
-        const bool summer = atid < kPairs * kParts;
-        const int cp = atid % kPairs, col = 2 * cp, gch = col >> 3;
-        const int k_lo = (atid / kPairs) * (BK / kParts);
-        const unsigned char* pcol = gbase + p.off_p + (gch >> 3) * SUB + (col & 7) * 2;
-        float acc0 = 0.f, acc1 = 0.f;
-
-        for (int j = 0; j < T; ++j) {
-            if (j >= TC && sub == 0) {
-                // One CTA per (sequence, kv head) -- the one that attends to the fresh tiles -- also puts the active
-                // rows' K/V into the cache, for later steps: the fresh tile is in shared memory once its stage is full,
-                // so the rows leave from there as plain 16-byte stores (thread = one 16-byte piece of a row, four rows
-                // per pass; the tile is 128-byte swizzled).  Nothing in this launch depends on these stores.  The stage
-                // is overwritten (by the partial of the merge) only after the row sums of the last visit, which this
-                // thread reports after it has read its pieces.  (One TMA store per row and half took 3.5 us for 34
-                // rows: 136 requests of 128 bytes, served one after the other.)
-                const int x = j - TC;
-                mbar_wait(bar(B_FULL + (2 * j) % NS), ((2 * j) / NS) & 1, abort_flag, p.dev_status);           // the fresh K tile
-                mbar_wait(bar(B_FULL + (2 * j + 1) % NS), ((2 * j + 1) / NS) & 1, abort_flag, p.dev_status);   // and V tile
-                const unsigned char* ktile = gbase + p.off_stage + ((2 * j) % NS) * TILE;
-                const unsigned char* vtile = gbase + p.off_stage + ((2 * j + 1) % NS) * TILE;
-                const int ch = atid & 15;   // piece of the row: columns [8 ch, 8 ch + 8)
-                const int n_rows = min(BK, p.n_active - x * BK);
-                for (int r = atid >> 4; r < n_rows; r += kAuxThreads / 16) {
-                    const int i = x * BK + r;
-                    const int pos = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
-                    if (pos < 0 || pos >= p.ctx_len) continue;
-                    const uint32_t off = (ch >> 3) * SUB + (r >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4);
-                    const long long dst = (((long long)bh * p.ctx_len + pos) * HD + ch * 8);
-                    *reinterpret_cast<uint4*>(p.k_cache + dst) = *reinterpret_cast<const uint4*>(ktile + off);
-                    *reinterpret_cast<uint4*>(p.v_cache + dst) = *reinterpret_cast<const uint4*>(vtile + off);
-                }
-            }
-            // P^T of tile j is in shared memory
-            mbar_wait(bar(B_PFULL), j & 1, abort_flag, p.dev_status);
-            if (summer) {
-                if (sh->raised[col / NH] == j) {   // the references of these columns were raised at this tile
-                    acc0 *= sh->factor[j & 1][col];
-                    acc1 *= sh->factor[j & 1][col + 1];
-                }
-#pragma unroll 4
-                for (int k8 = 0; k8 < BK / kParts; k8 += 8) {
+        if (refresh && sub == 0) {
+            // The CTAs of one column also put the active rows' K/V into the cache, for later steps, each a share of the
+            // rows: straight from the fresh tensors, eight 16-byte pieces in flight per thread.  Nothing in this launch
+            // depends on these stores.
+            const int pieces = p.n_active * 32;   // [row][K, V][16 pieces]
+            for (int c0 = split * kAuxThreads + atid; c0 < pieces; c0 += 8 * C * kAuxThreads) {
+                uint4 v[8];
+                int pos[8];
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) {
-                        const int k = k_lo + k8 + r;
-                        const uint32_t w = *reinterpret_cast<const uint32_t*>(pcol + (k >> 3) * 1024 + r * 128 + (((gch & 7) ^ r) << 4));
-                        acc0 += __uint_as_float(w << 16);
-                        acc1 += __uint_as_float(w & 0xffff0000u);
+                for (int u = 0; u < 8; ++u) {
+                    const int c = c0 + u * C * kAuxThreads, i = c >> 5;
+                    pos[u] = -1;
+                    if (c < pieces) {
+                        pos[u] = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
+                        const __nv_bfloat16* src = (c & 16) ? p.v_new : p.k_new;
+                        v[u] = __ldg(reinterpret_cast<const uint4*>(
+                            src + (((long long)b * p.n_active + i) * p.n_kv_heads + hk) * HD + (c & 15) * 8));
                     }
                 }
-                if (j == T - 1) {
-                    sh->lpart[atid / kPairs][col] = acc0;
-                    sh->lpart[atid / kPairs][col + 1] = acc1;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int c = c0 + u * C * kAuxThreads;
+                    if (pos[u] < 0 || pos[u] >= p.ctx_len) continue;
+                    __nv_bfloat16* dst = (c & 16) ? p.v_cache : p.k_cache;
+                    *reinterpret_cast<uint4*>(dst + ((long long)bh * p.ctx_len + pos[u]) * HD + (c & 15) * 8) = v[u];
                 }
             }
-            mbar_arrive(bar(B_PSUM));   // P^T of tile j has been read (release: the row sums above are visible)
         }
     } else {
         // ================================ Q, softmax (warps 2 ..) ===================================
@@ -495,6 +450,9 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 if (pos >= 0 && pos < p.ctx_len) fresh_ok |= 1u << x;
             }
         }
+        f32x2 lsum[NH / 2];   // this key lane's share of the row sums: probabilities as rounded for the second product
+#pragma unroll
+        for (int i = 0; i < NH / 2; ++i) lsum[i] = pk(0.f, 0.f);
         bool masks_ready = !refresh;   // the stale-key bits are awaited once, before the first cache tile
 
         for (int j = 0; j < T; ++j) {
@@ -531,64 +489,74 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 }
                 named_barrier(bar_sync, 128);
             }
-            // d = s * scale * log2(e) - m[q]; does any score exceed its reference by more than 2^kRaise?
-            f32x2 d2[NH / 2];
+            // d = s * scale * log2(e) - m[q], p = 2^d; does any score exceed its reference by more than 2^kRaise?
+            uint32_t pw[NH / 2];
             while (true) {
-                uint32_t sr[NH];
-                ld_row<NH, WG == 1>(s_addr, sr);
                 float dmx0 = -INFINITY, dmx1 = -INFINITY;
+                uint32_t sr[2][16];
+                ld16(s_addr, sr[0]);
 #pragma unroll
-                for (int i = 0; i < NH / 2; ++i) {
-                    const float2 mm = *reinterpret_cast<const float2*>(&sh->m[c0 + 2 * i]);
-                    d2[i] = fma2(pk(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), sl2_2, pk(-mm.x, -mm.y));
-                    if (past_end) d2[i] = pk(-INFINITY, -INFINITY);   // probability 0 for every query
-                    float d0, d1;
-                    upk(d2[i], d0, d1);
-                    if (i & 1) dmx1 = max3(dmx1, d0, d1); else dmx0 = max3(dmx0, d0, d1);
+                for (int q = 0; q < NH / 16; ++q) {   // sixteen columns at a time, the next ones on their way
+                    wait_ld16(sr[q & 1]);
+                    if (q + 1 < NH / 16) ld16(s_addr + 16 * (q + 1), sr[(q + 1) & 1]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 mm = *reinterpret_cast<const float2*>(&sh->m[c0 + 16 * q + 2 * i]);
+                        f32x2 d2 = fma2(pk(__uint_as_float(sr[q & 1][2 * i]), __uint_as_float(sr[q & 1][2 * i + 1])), sl2_2,
+                                        pk(-mm.x, -mm.y));
+                        if (past_end) d2 = pk(-INFINITY, -INFINITY);   // probability 0 for every query
+                        float d0, d1;
+                        upk(d2, d0, d1);
+                        if (i & 1) dmx1 = max3(dmx1, d0, d1); else dmx0 = max3(dmx0, d0, d1);
+                        pw[8 * q + i] = pack_bf16x2(fast_exp2(d0), fast_exp2(d1));
+                    }
                 }
                 if (!named_barrier_or(bar_or, 128, fmaxf(dmx0, dmx1) > kRaise)) break;
-                // ---- rare path: raise the references to the column maxima of this tile, rescale O^T (the row-sum
-                //      threads rescale their sums by the same factors), and once more ----
-                ld_row<NH, WG == 1>(s_addr, sr);
+                // ---- rare path: raise the references to the column maxima of this tile, rescale O^T and the row sums by
+                //      the same factors, and once more ----
 #pragma unroll
-                for (int c = 0; c < NH; ++c) {
-                    const float o = redux_max(past_end ? -INFINITY : __uint_as_float(sr[c]));
-                    if (lane == (c & 31)) sh->colmax[quarter][c0 + c] = o;
+                for (int q = 0; q < NH / 16; ++q) {
+                    ld16(s_addr + 16 * q, sr[0]);
+                    wait_ld16(sr[0]);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const float o = redux_max(past_end ? -INFINITY : __uint_as_float(sr[0][c]));
+                        if (lane == (16 * q + c) % 32) sh->col[quarter][c0 + 16 * q + c] = o;
+                    }
                 }
                 named_barrier(bar_sync, 128);
                 if (st_w < NH) {
                     const int c = c0 + st_w;
-                    const float o = fmaxf(fmaxf(sh->colmax[0][c], sh->colmax[1][c]), fmaxf(sh->colmax[2][c], sh->colmax[3][c]));
+                    const float o = fmaxf(fmaxf(sh->col[0][c], sh->col[1][c]), fmaxf(sh->col[2][c], sh->col[3][c]));
                     const float m_old = sh->m[c];
                     const float m_new = fmaxf(m_old, o * sl2);
                     sh->factor[j & 1][c] = (m_old == -INFINITY) ? 0.f : fast_exp2(m_old - m_new);
                     sh->m[c] = m_new;
-                    if (st_w == 0) sh->raised[wg] = j;   // for the row-sum threads (read after "P full")
                 }
                 named_barrier(bar_sync, 128);
                 if (j > 0) {   // O^T holds the tiles before j: P V of tile j - 1 must have completed
                     mbar_wait(bar(B_PVDONE), (j - 1) & 1, abort_flag, p.dev_status);
                     fence_after();
-                    uint32_t o[NH];
                     const uint32_t o_addr = tmem + lane_addr + TM_O + c0;
-                    ld_row<NH, WG == 1>(o_addr, o);
 #pragma unroll
-                    for (int c = 0; c < NH; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * sh->factor[j & 1][c0 + c]);
-                    st_row<NH, WG == 1>(o_addr, o);
+                    for (int q = 0; q < NH / 16; ++q) {
+                        ld16(o_addr + 16 * q, sr[0]);
+                        wait_ld16(sr[0]);
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            sr[0][c] = __float_as_uint(__uint_as_float(sr[0][c]) * sh->factor[j & 1][c0 + 16 * q + c]);
+                        st16(o_addr + 16 * q, sr[0]);
+                    }
+                    wait_st();
+#pragma unroll
+                    for (int i = 0; i < NH / 2; ++i) {
+                        const float2 f = *reinterpret_cast<const float2*>(&sh->factor[j & 1][c0 + 2 * i]);
+                        lsum[i] = mul2(lsum[i], pk(f.x, f.y));
+                    }
                 }
             }
-            uint32_t pw[NH / 2];
-#pragma unroll
-            for (int i = 0; i < NH / 2; ++i) {
-                float d0, d1;
-                upk(d2[i], d0, d1);
-                pw[i] = pack_bf16x2(fast_exp2(d0), fast_exp2(d1));
-            }
-            // the P^T buffer is free once P V of the previous tile has completed and its row sums have been taken
-            if (j > 0) {
-                mbar_wait(bar(B_PVDONE), (j - 1) & 1, abort_flag, p.dev_status);
-                mbar_wait(bar(B_PSUM), (j - 1) & 1, abort_flag, p.dev_status);
-            }
+            // the P^T buffer is free once P V of the previous tile has completed
+            if (j > 0) mbar_wait(bar(B_PVDONE), (j - 1) & 1, abort_flag, p.dev_status);
 #pragma unroll
             for (int ch = 0; ch < NH / 8; ++ch) {
                 const int gch = (c0 >> 3) + ch;      // 16-byte chunk (8 slots) of the whole P^T row
@@ -598,6 +566,37 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             fence_async_smem();
             fence_before();
             mbar_arrive(bar(B_PFULL));
+#pragma unroll
+            for (int i = 0; i < NH / 2; ++i)   // (while the second product runs)
+                lsum[i] = add2(lsum[i], pk(__uint_as_float(pw[i] << 16), __uint_as_float(pw[i] & 0xffff0000u)));
+        }
+        {   // row sums over the warp's 32 keys: each step halves the columns a lane holds, the last adds neighbours
+            float v[NH];
+#pragma unroll
+            for (int i = 0; i < NH / 2; ++i) upk(lsum[i], v[2 * i], v[2 * i + 1]);
+            int first = c0;
+#pragma unroll
+            for (int step = 1; step <= 4; ++step) {
+                const int n = NH >> step, o = 32 >> step;
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int i = 0; i < n; ++i) {
+                    const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+                first += up ? n : 0;
+            }
+#pragma unroll
+            for (int i = 0; i < NH / 16; ++i) {
+                v[i] += __shfl_xor_sync(0xffffffffu, v[i], 1);
+                if (!(lane & 1)) sh->col[quarter][first + i] = v[i];
+            }
+        }
+        named_barrier(bar_sync, 128);
+        auto row_sum = [&](int c) { return (sh->col[0][c] + sh->col[1][c]) + (sh->col[2][c] + sh->col[3][c]); };
+        if (C == 1) {
+            if (st_w < NH) sh->factor[0][c0 + st_w] = 1.f / row_sum(c0 + st_w);
+            named_barrier(bar_sync, 128);
         }
         mbar_wait(bar(B_PVDONE), (T - 1) & 1, abort_flag, p.dev_status);   // Q, P^T and the K/V stages are dead from here on
         fence_after();
@@ -605,17 +604,16 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         ld_row<NH, WG == 1>(tmem + lane_addr + TM_O + c0, o);
         fence_before();
         named_arrive(7, kSoft + 32);   // tensor memory has been read: the MMA warp may free it
-        mbar_wait(bar(B_PSUM), (T - 1) & 1, abort_flag, p.dev_status);     // the row sums are complete
         if (C == 1) {
             // ---- single CTA per (sequence, kv head): normalise and store column kk of every query row ----
             if (!*abort_flag) {
 #pragma unroll
                 for (int c = 0; c < NH; ++c) {
                     if (c0 + c < rows_total) {
-                        const float l = sh->lpart[0][c0 + c] + (kParts == 2 ? sh->lpart[1][c0 + c] : 0.f);
                         const int i = ((c0 + c) * p.group_inv) >> 16, jh = c0 + c - i * p.group;
+                        if (jh >= heads) continue;
                         __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i0 + i) * p.n_q_heads + hq0 + jh) * HD;
-                        dst[kk] = __float2bfloat16_rn(__uint_as_float(o[c]) / l);
+                        dst[kk] = __float2bfloat16_rn(__uint_as_float(o[c]) * sh->factor[0][c0 + c]);
                     }
                 }
             }
@@ -628,8 +626,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 if (c0 + c < rows_total) part[(c0 + c) * PITCH] = __uint_as_float(o[c]);
             if (st_w < NH) {
                 const int c = c0 + st_w;
-                const float l = sh->lpart[0][c] + (kParts == 2 ? sh->lpart[1][c] : 0.f);
-                *reinterpret_cast<float2*>(gbase + ML_OFF + c * 8) = make_float2(sh->m[c], l);
+                *reinterpret_cast<float2*>(gbase + ML_OFF + c * 8) = make_float2(sh->m[c], row_sum(c));
             }
         }
     }
@@ -652,7 +649,8 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
 #pragma unroll 1
         for (int idx = tid; idx < rows_total * quads; idx += kThreads) {
             const int qq = (idx * p.quads_inv) >> 16, d0 = (idx - qq * quads) * 4;
-            if (d0 >= own_dl) continue;
+            const int i = (qq * p.group_inv) >> 16, jh = qq - i * p.group;
+            if (d0 >= own_dl || jh >= heads) continue;
             const uint32_t at = base + ((uint32_t)qq * PITCH + (uint32_t)(split * DL + d0)) * 4u;
             float m = -INFINITY, l = 0.f, a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -684,7 +682,6 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 }
             }
             const float inv = 1.f / l;
-            const int i = (qq * p.group_inv) >> 16, jh = qq - i * p.group;
             __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i0 + i) * p.n_q_heads + hq0 + jh) * HD + split * DL + d0;
             *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(a[0] * inv, a[1] * inv), pack_bf16x2(a[2] * inv, a[3] * inv));
         }
@@ -713,7 +710,7 @@ bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len) {
 struct KeysPlan {
     bool ok;
     int group, rows_chunk, n_sub_r, n_sub;   // heads and active rows per CTA column, row chunks, CTA columns per kv head
-    int n_slots, n_splits, tiles_per_split, n_stages, n_extra, dl, ctas_per_sm, shift;
+    int n_slots, n_splits, tiles_per_split, n_stages, n_extra, dl, shift;
     uint32_t off_p, off_stage, off_list, off_bar, smem_bytes;
 };
 
@@ -756,7 +753,7 @@ int resident_clusters_of(int c, uint32_t smem) {
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c, 1, 1);
-    cfg.blockDim = dim3(64 + (N > 64 ? 256 : 128) + aux_threads(N), 1, 1);
+    cfg.blockDim = dim3(block_threads(N), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -792,74 +789,98 @@ int resident_clusters(int n_slots, int c, uint32_t smem) {
 }
 
 // fresh: the call refreshes (k_new / v_new given), so the last CTA of every cluster also visits the fresh tiles
-KeysPlan make_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
+KeysPlan compute_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
     KeysPlan pl{};
-    // a CTA column takes the largest divisor of the H_q / H_kv heads of a kv head whose packed rows fit the query
-    // slots; the other columns of that kv head stream the same K/V (from L2) for their own heads
     const int g = d.n_q_heads / d.n_kv_heads;
-    pl.group = g;
-    while (pl.group > 1 && (g % pl.group != 0 || (long long)n_active * pl.group > kMaxSlots)) --pl.group;
-    // more active rows than slots: the rows are cut into equal chunks, one CTA column each
-    pl.n_sub_r = (n_active * pl.group + kMaxSlots - 1) / kMaxSlots;
-    pl.rows_chunk = (n_active + pl.n_sub_r - 1) / pl.n_sub_r;
-    pl.n_sub_r = (n_active + pl.rows_chunk - 1) / pl.rows_chunk;
-    pl.n_sub = (g / pl.group) * pl.n_sub_r;
-    const int rows = pl.rows_chunk * pl.group;
-    pl.n_slots = rows <= 48 ? 48 : rows <= 64 ? 64 : 96;
-    pl.n_extra = fresh ? (n_active + BK - 1) / BK : 0;
-    const int tm_cols = tm_columns(pl.n_slots);
     const int key_tiles = (d.ctx_len + BK - 1) / BK;
-    const long long columns = (long long)d.batch * d.n_kv_heads * pl.n_sub;   // grid.y
     const int sms = sm_count();
-    // Cluster shape: cs CTAs split the cache tiles (every one at least one tile); the fresh tiles go to the last of
-    // them, or to one more CTA of their own (worth it when a CTA holds so few tiles that one more would be felt, and
-    // needed when it has a single stage).  All CTAs resident at once (two per SM when they are small); the most-loaded SM
-    // streams as few tiles as possible; among equals, more CTAs (more SMs pulling).
     long long best_cost = -1, best_ctas = 0;
-    for (int cs = 1; cs <= 8 && cs <= key_tiles; ++cs) {
-        const int tps = (key_tiles + cs - 1) / cs;
-        if ((key_tiles + tps - 1) / tps != cs || tps > kMaxTiles) continue;   // this cs leaves a CTA empty
-        for (int own = 0; own <= (fresh ? 1 : 0); ++own) {                     // own: the fresh tiles get their own CTA
-            const int c = cs + own;
-            if (c > 8) continue;
-            const int dl = ((HD + c - 1) / c + 7) & ~7;                        // (the last CTAs may own fewer columns, or none)
-            const int last_tiles = key_tiles - (cs - 1) * tps;
-            const int visits = own ? (tps > pl.n_extra ? tps : pl.n_extra)
-                                   : (tps > last_tiles + pl.n_extra ? tps : last_tiles + pl.n_extra);
-            KeysPlan t = pl;
-            int ns = 2 * visits < kMaxStages ? 2 * visits : kMaxStages;   // ring slots: a K and a V slot per tile in flight
-            t.tiles_per_split = tps;
-            carve(t, ns, fresh);
-            while (ns > 2 && t.smem_bytes > kSmemMax) carve(t, --ns, fresh);
-            if (t.smem_bytes > kSmemMax || (ns < 4 && visits > 1)) continue;
-            // the partial of the merge reuses the Q / P^T / stage memory
-            if (c > 1 && partial_bytes(pl.n_slots) > t.off_list) continue;
-            const int per_sm = (t.smem_bytes <= kSmemTwoPerSm && tm_cols <= 256) ? 2 : 1;
-            const long long ctas = columns * c;
-            if (ctas > (long long)per_sm * sms) continue;
-            const int fit = resident_clusters(pl.n_slots, c, t.smem_bytes);   // (-1: no device to ask, keep the estimate)
-            if (fit >= 0 && columns > fit) continue;
-            // cost in quarter tiles: the fresh tiles arrive early (they are small and mostly in L2), so on a shared CTA
-            // they count a quarter of a cache tile
-            const long long cost = 4LL * tps * ((ctas + sms - 1) / sms) + ((fresh && !own) ? pl.n_extra : 0);
-            if (best_cost < 0 || cost < best_cost || (cost == best_cost && ctas > best_ctas)) {
+    // A CTA column takes `group` query heads of a kv head; the columns of a kv head stream the same K/V (from L2).  Fewer
+    // columns leave more CTAs for splitting the keys, but more packed rows make a tile dearer.
+    for (int cols = 1; cols <= g; ++cols) {
+        KeysPlan base = KeysPlan{};
+        base.group = (g + cols - 1) / cols;
+        if ((g + base.group - 1) / base.group != cols) continue;
+        if (base.group > 1 && (long long)n_active * base.group > kMaxSlots) continue;
+        // more active rows than slots: the rows are cut into equal chunks, one CTA column each
+        base.n_sub_r = (n_active * base.group + kMaxSlots - 1) / kMaxSlots;
+        base.rows_chunk = (n_active + base.n_sub_r - 1) / base.n_sub_r;
+        base.n_sub_r = (n_active + base.rows_chunk - 1) / base.rows_chunk;
+        base.n_sub = cols * base.n_sub_r;
+        const int rows = base.rows_chunk * base.group;
+        base.n_slots = rows <= 48 ? 48 : rows <= 64 ? 64 : 96;
+        base.n_extra = fresh ? (n_active + BK - 1) / BK : 0;
+        const long long columns = (long long)d.batch * d.n_kv_heads * base.n_sub;   // grid.y
+        // Cluster shape: cs CTAs split the cache tiles (every one at least one tile); the fresh tiles go to the last of
+        // them, or to one more CTA of their own (worth it when a CTA holds so few tiles that one more would be felt).
+        // All CTAs resident at once; the most-loaded SM streams as few tiles as possible; among equals, more CTAs (more
+        // SMs pulling).
+        for (int cs = 1; cs <= 8 && cs <= key_tiles; ++cs) {
+            const int tps = (key_tiles + cs - 1) / cs;
+            if ((key_tiles + tps - 1) / tps != cs || tps > kMaxTiles) continue;   // this cs leaves a CTA empty
+            for (int own = 0; own <= (fresh ? 1 : 0); ++own) {                     // own: the fresh tiles get their own CTA
+                const int c = cs + own;
+                if (c > 8) continue;
+                const int dl = ((HD + c - 1) / c + 7) & ~7;                        // (the last CTAs may own fewer columns, or none)
+                const int last_tiles = key_tiles - (cs - 1) * tps;
+                const int visits = own ? (tps > base.n_extra ? tps : base.n_extra)
+                                       : (tps > last_tiles + base.n_extra ? tps : last_tiles + base.n_extra);
+                KeysPlan t = base;
+                int ns = 2 * visits < kMaxStages ? 2 * visits : kMaxStages;   // ring slots: a K and a V slot per tile in flight
+                t.tiles_per_split = tps;
+                carve(t, ns, fresh);
+                while (ns > 2 && t.smem_bytes > kSmemMax) carve(t, --ns, fresh);
+                if (t.smem_bytes > kSmemMax || (ns < 4 && visits > 1)) continue;
+                // the partial of the merge reuses the Q / P^T / stage memory
+                if (c > 1 && partial_bytes(t.n_slots) > t.off_list) continue;
+                const long long ctas = columns * c;
+                if (ctas > sms) continue;   // one CTA per SM: registers
+                // Cost in quarter tiles (about 0.25 us): the fresh tiles arrive early (they are small and mostly in L2), so
+                // on a shared CTA they count a quarter of a cache tile.  96 slots: a tile takes 1.3 us where the memory
+                // system does not set the pace (48: 1.0), and the launch around the tiles up to 3 us more.
+                const long long cost = (t.n_slots == 96 ? 5LL * tps + 13 : 4LL * tps) + ((fresh && !own) ? t.n_extra : 0);
+                if (best_cost >= 0 && (cost > best_cost || (cost == best_cost && ctas <= best_ctas))) continue;
+                const int fit = resident_clusters(t.n_slots, c, t.smem_bytes);   // (-1: no device to ask, keep the estimate)
+                if (fit >= 0 && columns > fit) continue;
                 best_cost = cost;
                 best_ctas = ctas;
+                pl = t;
                 pl.n_splits = c;
-                pl.tiles_per_split = tps;
                 // The CTA that also visits the fresh tiles has one visit more than its peers, and the cluster waits for
                 // it at the merge.  The memory system serves whoever asks, so giving that CTA one cache tile less (and
                 // the first CTA one more) lets it finish its stream early and spend the difference on the extra visit.
                 pl.shift = (fresh && !own && cs >= 2 && tps >= 2 && last_tiles == tps) ? 1 : 0;
                 pl.dl = dl;
-                pl.ctas_per_sm = per_sm;
-                pl.n_stages = ns;
+                pl.ok = true;
             }
         }
     }
-    pl.ok = best_cost >= 0;
-    if (pl.ok) carve(pl, pl.n_stages, fresh);
     return pl;
+}
+
+// The plan of the last geometry a thread asked for is kept: a layer loop asks for the same one at every call, twice (a
+// plan takes 1 to 2 us of host time, a launch 3).
+KeysPlan make_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
+    struct Key {
+        int dev, batch, ctx_len, n_q_heads, n_kv_heads, n_active, fresh;
+        bool operator==(const Key& o) const {
+            return dev == o.dev && batch == o.batch && ctx_len == o.ctx_len && n_q_heads == o.n_q_heads &&
+                   n_kv_heads == o.n_kv_heads && n_active == o.n_active && fresh == o.fresh;
+        }
+    };
+    static thread_local Key last{-2, 0, 0, 0, 0, 0, 0};
+    static thread_local KeysPlan plan;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        dev = -1;
+    }
+    const Key key{dev, d.batch, d.ctx_len, d.n_q_heads, d.n_kv_heads, n_active, fresh ? 1 : 0};
+    if (!(key == last)) {
+        plan = compute_keys_plan(d, n_active, fresh);
+        last = key;
+    }
+    return plan;
 }
 
 // k_new / v_new [B, n, H_kv, 128] bf16 seen as 5-D {64 columns, active row, half, kv head, sequence}: one box
@@ -909,7 +930,7 @@ cudaError_t launch_n(const KeysPlan& pl, const KeysParams& p, const CUtensorMap&
         return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(pl.n_splits, bh, 1);
-    cfg.blockDim = dim3(64 + (N > 64 ? 256 : 128) + aux_threads(N), 1, 1);
+    cfg.blockDim = dim3(block_threads(N), 1, 1);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute at[2];
@@ -940,7 +961,7 @@ bool attend_skip_keys_supported(const ec_attn_desc& d, int n_active, bool fresh)
 void attend_skip_keys_describe(const ec_attn_desc& d, int n_active, bool fresh, char* buf, size_t len) {
     const KeysPlan pl = make_keys_plan(d, n_active, fresh);
     snprintf(buf, len, "attend_skip_keys_kernel<%d> grid=(%d,%d) cluster=%d ring_slots=%d smem=%u ctas_per_sm=%d fresh_tiles=%d",
-             pl.n_slots, pl.n_splits, d.batch * d.n_kv_heads * pl.n_sub, pl.n_splits, pl.n_stages, pl.smem_bytes, pl.ctas_per_sm,
+             pl.n_slots, pl.n_splits, d.batch * d.n_kv_heads * pl.n_sub, pl.n_splits, pl.n_stages, pl.smem_bytes, 1,
              pl.n_extra);
 }
 
@@ -971,6 +992,7 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
     p.n_q_heads = a.d.n_q_heads;
     p.n_kv_heads = a.d.n_kv_heads;
     p.group = pl.group;
+    p.q_per_kv = a.d.n_q_heads / a.d.n_kv_heads;
     p.group_inv = (65536 + pl.group - 1) / pl.group;
     p.rows_chunk = pl.rows_chunk;
     p.n_sub_r = pl.n_sub_r;
