@@ -5,24 +5,19 @@
 //
 // R*V*sizeof(elem) bytes are read exactly once; the arithmetic is about seven instructions per element.
 //   grid  = (splits, R): CTA (s, r) owns the columns [s*chunk, (s+1)*chunk) of row r; the split count is
-//           chosen so that the whole grid is about one resident wave (4 CTAs per SM);
-//   CTA   : (inputs below 24 MB; larger ones: every thread loads its own vectors through four rolling registers,
-//           no producer warp)  8 consumer warps and one producer warp.  The producer's lane 0 moves the chunk through a ring of
-//           three 16 KB stages in shared memory with bulk copies (cp.async.bulk, completion on an mbarrier, L2
-//           evict-first), as far ahead as the ring allows, so the bytes in flight per SM are the rings of its
-//           resident CTAs and do not depend on the consumers' registers;
-//   loop  : a consumer thread takes the 16-byte vectors (bf16x8 / f32x4) t, t + 256, ... of the chunk in ascending
-//           order, four per stage, and keeps a running
+//           chosen so that the whole grid is about one resident wave (4 CTAs of 256 threads per SM);
+//   loop  : a thread takes the 16-byte vectors (bf16x8 / f32x4) t, t + 256, ... of the chunk in ascending
+//           order through four rolling registers and keeps a running
 //           (max, S, T) with S = sum 2^d, T = sum 2^d * d, d = x*log2(e) - base: one ex2.approx per element
 //           and one packed fp32x2 FMA, add and FMA per pair of elements.  The base follows the maximum lazily: it moves, and S and T
 //           are rescaled (S' = 2^dl S, T' = 2^dl (T + dl S), dl = old base - new base), only when a value
 //           exceeds it by more than 2^64, so the common path has no data-dependent branch.  Logits are
 //           clamped from below at -1e38 (packed bf16 max on the raw words), which keeps d finite:
 //           -inf and finfo.min-style masks get probability 0 without a per-element special case;
-//   argmax: the thread remembers the iteration that raised its maximum; after the CTA-wide maximum is
-//           known, only the threads that attained it look at that iteration's vectors again for the
+//   argmax: the thread remembers the vector that raised its maximum; after the warp's maximum is
+//           known, only the threads that attained it look at that vector again for the
 //           first column (ties -> smallest index, through every reduction stage);
-//   reduce: sums rescaled to the CTA's base and added (shuffles + shared memory);
+//   reduce: sums rescaled to the warp's base and added (shuffles), the warps' results merged behind one barrier;
 //   merge : CTA partial (M, S, T, idx) -> workspace, one atomic ticket; the last CTA of a sequence
 //           (no spinning: tickets only count arrivals) merges the partials of every row of the
 //           sequence, writes H = ln S - ln2 * T / S, conf = 2^(M*log2e - base) / S and argmax, takes
@@ -30,10 +25,13 @@
 //           than 32 splits, use two ticket levels instead (last CTA of a row, then last row of the sequence).
 // The entropy identity used: with p_j = 2^{d_j} / S,  -sum p_j ln p_j = ln S - ln2 * T / S
 // for any common base, so no partial ever needs the true row maximum.
-// The kernel is launched with programmatic stream serialisation and touches global memory only after
-// griddepcontrol.wait.  Every mbarrier wait is bounded (one second); a CTA whose wait gave up waits, bounded
-// again, for its copies in flight, still arrives at its ticket with a poison bit, and the sequence then reports
-// decision -1 instead of a value computed from missing data.
+// What bounds it: at [256, 126464] bf16 (17.9 us, 10 of them at the copy rate) about 5 us of launch, ramp, reduction,
+// tickets and the finishing CTA, and 2.5 us of arithmetic that the stream does not hide (15.4 us without any); at
+// [32, 126464] (7.0 us) the fixed part alone.  Also timed at [256, 126464]: twelve vectors ahead through asynchronous
+// copies 17.9 (fp32 26.6 against 24.2), two batches of four in registers 18.6, 3 to 21 CTAs a row 19.5 to 38; a ring of
+// bulk copies with a producer warp took 19.7, and 7.4 at [32, 126464].
+// The kernel is launched with programmatic stream serialisation, touches global memory only after
+// griddepcontrol.wait and waits for nothing else.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
@@ -42,16 +40,12 @@
 namespace ec {
 namespace {
 
-constexpr int kGateThreads = 256;      // consumer threads of a CTA (a producer warp comes on top)
+constexpr int kGateThreads = 256;
 constexpr int kCtasPerSm = 4;
 constexpr int kVec = 8;  // columns per thread in one slab of kGateThreads * kVec columns (chunk granularity)
 constexpr int kMaxSplits = 96;
 constexpr float kDClamp = -150.0f;  // 2^-150 flushes to 0 (ftz)
-constexpr int kStages = 3;                          // ring of staged buffers per CTA
-constexpr int kInFlight = 4;                        // rolling variant: 16-byte vectors a thread keeps in flight
-constexpr int kStageVecs = 4 * kGateThreads;        // 16-byte vectors per stage: four per consumer thread
-constexpr uint32_t kStageBytes = kStageVecs * 16u;
-constexpr int kPoison = 1 << 20;                    // added to a ticket by a CTA whose wait gave up
+constexpr int kInFlight = 4;         // 16-byte vectors a thread keeps in flight
 constexpr int kSingleLevelMaxRows = 64;
 constexpr float kRebase = 64.f;     // the base moves when a value exceeds it by more than 2^kRebase
 constexpr unsigned int kXMinBf16x2 = 0xFE96FE96u;   // two bf16 of about -1e38: lower clamp of the logits
@@ -104,25 +98,6 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// global -> shared bulk copy that completes on an mbarrier; the source is read once, so it leaves L2 first
-__device__ __forceinline__ uint64_t evict_first_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t policy) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
-}
-__device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-// barrier of the 256 consumer threads (the producer warp leaves early)
-__device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kGateThreads) : "memory"); }
 __device__ __forceinline__ unsigned int max_bf16x2(unsigned int a, unsigned int b) {
     unsigned int d;
     asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -146,7 +121,6 @@ struct Loader<__nv_bfloat16> {
     static __device__ __forceinline__ unsigned int max_word(const uint4& u) {
         return max_bf16x2(max_bf16x2(u.x, u.y), max_bf16x2(u.z, u.w));
     }
-    static __device__ __forceinline__ unsigned int max_words(unsigned int a, unsigned int b) { return max_bf16x2(a, b); }
     static __device__ __forceinline__ float word_max(unsigned int w) {
         return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
     }
@@ -180,9 +154,6 @@ struct Loader<float> {
     static __device__ __forceinline__ unsigned int max_word(const uint4& u) {
         return __float_as_uint(fmaxf(fmaxf(__uint_as_float(u.x), __uint_as_float(u.y)),
                                      fmaxf(__uint_as_float(u.z), __uint_as_float(u.w))));
-    }
-    static __device__ __forceinline__ unsigned int max_words(unsigned int a, unsigned int b) {
-        return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
     }
     static __device__ __forceinline__ float word_max(unsigned int w) { return __uint_as_float(w); }
     static __device__ __forceinline__ void widen(const uint4& u, float (&x)[4]) {
@@ -251,36 +222,43 @@ __device__ __forceinline__ float finish_row(const GateParams& p, int row, int la
     return H;
 }
 
-// kStaged: the logits come through the bulk-copy ring (a producer warp on top of the consumers); otherwise every
-// thread loads its own vectors into a rolling set of kInFlight registers.  The ring wins on small inputs (three
-// stages are on their way before any consumer has started: 7.5 against 8.3 us at [32, 126464]), the rolling loads on
-// large ones (17.8 against 19.7 us at [256, 126464]): the host picks by size.
-template <typename T, bool kStaged>
-__global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm) gate_kernel(const GateParams p) {
-    __shared__ float s_m[kGateThreads / 32];
-    __shared__ int s_i[kGateThreads / 32];
-    __shared__ float s_S[kGateThreads / 32], s_T[kGateThreads / 32];
+template <typename T>
+__global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const GateParams p) {
+    constexpr int kWarps = kGateThreads / 32;
+    __shared__ float4 s_part[kWarps];
     __shared__ float s_H[kSingleLevelMaxRows];
     __shared__ float s_conf[kSingleLevelMaxRows];
     __shared__ int s_arg[kSingleLevelMaxRows];
     __shared__ int s_last;
-    __shared__ __align__(8) unsigned long long s_bar[2 * kStages];
-    __shared__ volatile int s_abort;
-    __shared__ volatile int s_issued;
-    extern __shared__ __align__(128) unsigned char s_ring[];
-    const uint32_t ring0 = tc::s2u(s_ring), full0 = tc::s2u(&s_bar[0]), empty0 = tc::s2u(&s_bar[kStages]);
 
-    constexpr int EPV = Loader<T>::EPV;
+    using L = Loader<T>;
+    constexpr int EPV = L::EPV;
     const int row = blockIdx.y, split = blockIdx.x, tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const T* rowp = reinterpret_cast<const T*>(p.logits) + (long long)row * p.row_stride;
     const int c0 = split * p.chunk;
     const int c_end = min(p.vocab, c0 + p.chunk);
 
+    // Thread t owns the whole vectors t, t + 256, ... of the chunk.  They pass through a rolling set of kInFlight registers:
+    // as soon as a vector has been consumed its register is given to the load kInFlight vectors ahead.  The ragged end
+    // of a row (a vocabulary that is no multiple of the vector length) is handled by element below.
+    constexpr int kVStride = kGateThreads * EPV;
+    const int n_vec = (c_end - c0) / EPV;
+    const int n_mine = n_vec > tid ? (n_vec - tid + kGateThreads - 1) / kGateThreads : 0;
+    const T* mine = rowp + c0 + tid * EPV;
+    uint4 raw[kInFlight];
+    auto fetch = [&](int i, uint4& v) {
+        if (i < n_mine) v = __ldcs(reinterpret_cast<const uint4*>(mine + (long long)i * kVStride));   // streamed once
+    };
+    tc::pdl_wait();                 // the previous kernel of the stream has completed: the logits are final
+    tc::pdl_launch_dependents();
+#pragma unroll
+    for (int r = 0; r < kInFlight; ++r) fetch(r, raw[r]);
+
     // running state: maximum, exponent base, and S, T as two packed lanes each
     float m = -INFINITY, base = base_of(-INFINITY);
     f32x2 S2 = pack2(0.f, 0.f), T2 = pack2(0.f, 0.f);
-    int mcol = -1, mspan = 0;   // where the maximum was raised: first column, and how many elements (a vector or one)
+    int mat = -1;               // the vector that raised the maximum last
     const f32x2 kL2 = pack2(kLog2e, kLog2e);
     auto rebase_if_needed = [&](float vmax) {
         if (fmaf(vmax, kLog2e, -base) > kRebase) {   // rare
@@ -297,58 +275,18 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
             base = nb;
         }
     };
-
-    // ---- the chunk's whole vectors, staged through shared memory --------------------------------------------------
-    // Warp 8 lane 0 issues one bulk copy per stage (16 KB = four vectors per consumer thread) into a ring of kStages
-    // buffers, as far ahead as the ring allows; the bytes in flight per SM (the ring of every resident CTA) are what
-    // the pass lives on, not the consumers' registers.  Consumer thread t takes the vectors t, t + 256, t + 512, ...
-    // of the chunk in ascending order.  The ragged end of a row (a vocabulary that is no multiple of the vector
-    // length) is handled element by element below.
-    const int n_vec = (c_end - c0) / EPV;                                  // whole vectors of the chunk
-    const int n_stage = (n_vec + kStageVecs - 1) / kStageVecs;
-    if (tid == 0) {
-        if (kStaged) {
-#pragma unroll
-            for (int i = 0; i < kStages; ++i) { tc::mbar_init(full0 + 8u * i, 1); tc::mbar_init(empty0 + 8u * i, kGateThreads / 32); }
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        s_abort = 0;
-        s_issued = -1;
-    }
-    __syncthreads();
-    pdl_wait();                 // the previous kernel of the stream has completed: the logits are final
-    pdl_launch_dependents();
-    if (kStaged && warp == kGateThreads / 32) {            // the producer warp
-        if (lane == 0) {
-            const unsigned char* src = reinterpret_cast<const unsigned char*>(rowp + c0);
-            const uint64_t policy = evict_first_policy();
-            int s = 0;
-            for (; s < n_stage; ++s) {
-                const int slot = s % kStages;
-                if (s >= kStages) tc::mbar_wait(empty0 + 8u * slot, ((s / kStages) - 1) & 1, &s_abort, nullptr);
-                if (s_abort) break;
-                const uint32_t bytes = (uint32_t)min(kStageVecs, n_vec - s * kStageVecs) * 16u;
-                tc::mbar_expect_tx(full0 + 8u * slot, bytes);
-                bulk_load(ring0 + (uint32_t)slot * kStageBytes, src + (size_t)s * kStageBytes, bytes, full0 + 8u * slot, policy);
-            }
-            s_issued = s;
-        }
-        return;
-    }
-    auto consume = [&](uint4 raw, int col) {
-        Loader<T>::clamp(raw);
-        const float vmax = Loader<T>::word_max(Loader<T>::max_word(raw));
+    auto consume = [&](uint4 v, int i) {
+        L::clamp(v);
+        const float vmax = L::word_max(L::max_word(v));
         rebase_if_needed(vmax);
-        const bool up = vmax > m;   // strictly greater: the first vector of a tie survives
-        m = up ? vmax : m;
-        mcol = up ? col : mcol;
-        mspan = up ? EPV : mspan;
+        mat = vmax > m ? i : mat;   // strictly greater: the first vector of a tie survives
+        m = fmaxf(m, vmax);
         const f32x2 nb2 = pack2(-base, -base);
         f32x2 x2[EPV / 2];
-        Loader<T>::widen2(raw, x2);
+        L::widen2(v, x2);
 #pragma unroll
-        for (int i = 0; i < EPV / 2; ++i) {
-            const f32x2 d2 = fma2(x2[i], kL2, nb2);
+        for (int e = 0; e < EPV / 2; ++e) {
+            const f32x2 d2 = fma2(x2[e], kL2, nb2);
             float d0, d1;
             unpack2(d2, d0, d1);
             const f32x2 e2 = pack2(fast_exp2(d0), fast_exp2(d1));
@@ -356,69 +294,25 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
             T2 = fma2(e2, d2, T2);
         }
     };
-    if (!kStaged) {
-        // Thread t owns the vectors t, t + 256, ... of the chunk.  They pass through a rolling set of kInFlight
-        // registers: as soon as a vector has been consumed its register is given to the load kInFlight vectors ahead.
-        constexpr int kVStride = kGateThreads * EPV;
-        const int n_mine = n_vec > tid ? (n_vec - tid + kGateThreads - 1) / kGateThreads : 0;
-        const T* mine = rowp + c0 + tid * EPV;
-        uint4 raw[kInFlight];
+    int i0 = 0;
+    for (; i0 + kInFlight <= n_mine; i0 += kInFlight) {
 #pragma unroll
-        for (int v = 0; v < kInFlight; ++v)
-            if (v < n_mine) raw[v] = __ldcs(reinterpret_cast<const uint4*>(mine + (long long)v * kVStride));   // streamed once
-        int i0 = 0;
-        for (; i0 + kInFlight <= n_mine; i0 += kInFlight) {
-#pragma unroll
-            for (int v = 0; v < kInFlight; ++v) {
-                consume(raw[v], c0 + (i0 + v) * kVStride + tid * EPV);
-                if (i0 + v + kInFlight < n_mine)
-                    raw[v] = __ldcs(reinterpret_cast<const uint4*>(mine + (long long)(i0 + v + kInFlight) * kVStride));
-            }
+        for (int r = 0; r < kInFlight; ++r) {
+            consume(raw[r], i0 + r);
+            fetch(i0 + r + kInFlight, raw[r]);
         }
-#pragma unroll
-        for (int v = 0; v < kInFlight; ++v)
-            if (i0 + v < n_mine) consume(raw[v], c0 + (i0 + v) * kVStride + tid * EPV);
     }
-    for (int s = 0; kStaged && s < n_stage; ++s) {
-        const int slot = s % kStages;
-        tc::mbar_wait(full0 + 8u * slot, (s / kStages) & 1, &s_abort, nullptr);
-        if (s_abort) break;
-        const uint32_t at = ring0 + (uint32_t)slot * kStageBytes + (uint32_t)tid * 16u;
-        uint4 raw[kStageVecs / kGateThreads];
 #pragma unroll
-        for (int k = 0; k < kStageVecs / kGateThreads; ++k) raw[k] = lds_v4(at + (uint32_t)k * kGateThreads * 16u);
-#pragma unroll
-        for (int k = 0; k < kStageVecs / kGateThreads; ++k) {
-            const int v = s * kStageVecs + k * kGateThreads + tid;
-            if (v < n_vec) consume(raw[k], c0 + v * EPV);
-        }
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(empty0 + 8u * slot);   // the stage's bytes are in registers or consumed
-    }
-    consumer_sync();
-    if (s_abort) {      // uniform: nothing raises the flag after the barrier above
-        // a wait gave up (one second): the copies already issued still target this CTA's shared memory, so the CTA
-        // stays until they have landed (bounded again) and reports through the poisoned ticket below
-        if (tid == 0) {
-            unsigned long long t0 = tc::global_timer_ns();
-            while (s_issued < 0 && tc::global_timer_ns() - t0 < tc::kWaitLimitNs) {}
-            const int issued = max(0, s_issued);
-            for (int s = max(0, issued - kStages); s < issued; ++s) {
-                t0 = tc::global_timer_ns();
-                while (!tc::mbar_try(full0 + 8u * (s % kStages), (s / kStages) & 1) && tc::global_timer_ns() - t0 < tc::kWaitLimitNs) {}
-            }
-        }
-        consumer_sync();
-    }
+    for (int r = 0; r < kInFlight; ++r)
+        if (i0 + r < n_mine) consume(raw[r], i0 + r);
+    int tail_col = -1;
     {   // the ragged end of the chunk: fewer than EPV columns, one element per thread
         const int col = c0 + n_vec * EPV + tid;
         if (col < c_end) {
-            const float x = Loader<T>::one(rowp + col);
+            const float x = L::one(rowp + col);
             rebase_if_needed(x);
-            const bool up = x > m;
-            m = up ? x : m;
-            mcol = up ? col : mcol;
-            mspan = up ? 1 : mspan;
+            tail_col = x > m ? col : -1;
+            m = fmaxf(m, x);
             float s0, s1, t0, t1;
             unpack2(S2, s0, s1);
             unpack2(T2, t0, t1);
@@ -429,33 +323,25 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
         }
     }
 
-    // ---- CTA-wide maximum; the threads that attained it find its first column ---------------------------
-    // every thread asks again for the vector that raised its maximum (an L2 hit, in flight during the reduction); only
-    // the threads that attained the CTA's maximum will look at it
+    // ---- warp maximum; the threads that attained it find its first column in the vector that raised it --------
+    // (every thread asks again for that vector: an L2 hit, in flight during the reduction)
     uint4 again = make_uint4(0u, 0u, 0u, 0u);
-    if (mspan == EPV) again = __ldg(reinterpret_cast<const uint4*>(rowp + mcol));
-    float wm = m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-    if (lane == 0) s_m[warp] = wm;
-    consumer_sync();
-    float M = s_m[0];
-#pragma unroll
-    for (int w = 1; w < kGateThreads / 32; ++w) M = fmaxf(M, s_m[w]);
+    if (mat >= 0) again = __ldg(reinterpret_cast<const uint4*>(mine + (long long)mat * kVStride));
+    const float M = tc::redux_max(m);
     int idx = 0x7fffffff;
-    if (m == M && mcol >= 0) {
-        if (mspan == EPV) {
+    if (m == M) {
+        if (tail_col >= 0) {
+            idx = tail_col;
+        } else if (mat >= 0) {
             float x[EPV];
-            Loader<T>::clamp(again);
-            Loader<T>::widen(again, x);
+            L::clamp(again);
+            L::widen(again, x);
 #pragma unroll
-            for (int i = EPV - 1; i >= 0; --i)   // descending: the smallest column survives
-                if (x[i] == M) idx = mcol + i;
-        } else {
-            idx = mcol;   // a single element of the ragged end
+            for (int e = EPV - 1; e >= 0; --e)   // descending: the smallest column survives
+                if (x[e] == M) idx = c0 + mat * kVStride + tid * EPV + e;
         }
     }
-    // ---- sums against the CTA's base, first column of the maximum --------------------------------------
+    // ---- sums against the warp's base, first column of the maximum --------------------------------------
     float S, Tt;
     {
         float s0, s1, t0, t1;
@@ -474,29 +360,35 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
     for (int o = 16; o > 0; o >>= 1) {
         S += __shfl_xor_sync(0xffffffffu, S, o);
         Tt += __shfl_xor_sync(0xffffffffu, Tt, o);
-        idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, o));
     }
-    if (lane == 0) { s_S[warp] = S; s_T[warp] = Tt; s_i[warp] = idx; }
-    consumer_sync();
+    idx = __reduce_min_sync(0xffffffffu, idx);
+    if (lane == 0) s_part[warp] = make_float4(M, S, Tt, __int_as_float(idx));
+    __syncthreads();
 
-    // ---- publish the partial; count arrivals (tickets only count, nothing spins) --------------------
+    // ---- publish the CTA's partial; count arrivals (tickets only count, nothing spins) --------------------
     const int seq = row / p.rows_per_seq;
-    if (tid == 0) {
-        float Ss = 0.f, Ts = 0.f;
-        int Midx = 0x7fffffff;
+    if (warp == 0) {
+        const float4 f = s_part[lane % kWarps];
+        Partial acc;
+        acc.M = f.x; acc.S = f.y; acc.T = f.z; acc.idx = __float_as_int(f.w);
 #pragma unroll
-        for (int w = 0; w < kGateThreads / 32; ++w) { Ss += s_S[w]; Ts += s_T[w]; Midx = min(Midx, s_i[w]); }
-        *reinterpret_cast<float4*>(&p.partials[(long long)row * p.splits + split]) =
-            make_float4(M, Ss, Ts, __int_as_float(Midx));
-        // a CTA whose wait gave up still arrives, with the poison bit: the sequence then reports decision -1
-        const int mine = 1 + (s_abort ? kPoison : 0);
-        const int old = p.single_level ? ticket_add(&p.seq_ticket[seq], mine) : ticket_add(&p.row_ticket[row], mine);
-        const int expected = p.single_level ? p.rows_per_seq * p.splits : p.splits;
-        s_last = ((old & (kPoison - 1)) == expected - 1 ? 1 : 0) | (old + mine >= kPoison ? 2 : 0);
+        for (int o = kWarps / 2; o > 0; o >>= 1) {
+            Partial q;
+            q.M = __shfl_xor_sync(0xffffffffu, acc.M, o);
+            q.S = __shfl_xor_sync(0xffffffffu, acc.S, o);
+            q.T = __shfl_xor_sync(0xffffffffu, acc.T, o);
+            q.idx = __shfl_xor_sync(0xffffffffu, acc.idx, o);
+            acc = merge(acc, q);
+        }
+        if (lane == 0) {
+            *reinterpret_cast<float4*>(&p.partials[(long long)row * p.splits + split]) =
+                make_float4(acc.M, acc.S, acc.T, __int_as_float(acc.idx));
+            const int old = p.single_level ? ticket_add(&p.seq_ticket[seq], 1) : ticket_add(&p.row_ticket[row], 1);
+            s_last = old == (p.single_level ? p.rows_per_seq * p.splits : p.splits) - 1;
+        }
     }
-    consumer_sync();   // orders the ticket's acquire before the other threads' reads of the partials
-    if (!(s_last & 1)) return;
-    const bool poisoned = (s_last & 2) != 0;
+    __syncthreads();   // orders the ticket's acquire before the other threads' reads of the partials
+    if (!s_last) return;
 
     if (p.single_level) {
         // ---- last CTA of the sequence: finish every row, then the masked maximum and the decision ----
@@ -545,7 +437,7 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
                 }
             }
         }
-        consumer_sync();
+        __syncthreads();
         if (warp == 0 && p.masked) {
             // ---- confidence-based parallel decoding (Section 2.1 of the paper; threshold 0.9 in its experiments):
             // every masked row above the threshold is decoded; if none is, the masked row of highest confidence
@@ -596,7 +488,7 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
                 if (p.ent_sum_out) p.ent_sum_out[seq] = Hsum;
                 if (p.max_conf_out) p.max_conf_out[seq] = Cmax;
                 p.max_entropy_out[seq] = E;
-                p.decision_out[seq] = poisoned ? -1 : (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
+                p.decision_out[seq] = (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
                 p.seq_ticket[seq] = 0;   // ready for the next call
             }
         } else if (warp == 0) {
@@ -616,7 +508,7 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
                 if (p.ent_sum_out) p.ent_sum_out[seq] = Hsum;
                 if (p.max_conf_out) p.max_conf_out[seq] = Cmax;
                 p.max_entropy_out[seq] = E;
-                p.decision_out[seq] = poisoned ? -1 : (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
+                p.decision_out[seq] = (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
                 p.seq_ticket[seq] = 0;   // ready for the next call
             }
         }
@@ -629,12 +521,10 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
     int seq_last = 0;
     if (lane == 0) {
         p.row_ticket[row] = 0;
-        const int mine = 1 + (poisoned ? kPoison : 0);
-        const int old = ticket_add(&p.seq_ticket[seq], mine);
-        seq_last = ((old & (kPoison - 1)) == p.rows_per_seq - 1 ? 1 : 0) | (old + mine >= kPoison ? 2 : 0);
+        seq_last = ticket_add(&p.seq_ticket[seq], 1) == p.rows_per_seq - 1;
     }
     seq_last = __shfl_sync(0xffffffffu, seq_last, 0);
-    if (!(seq_last & 1)) return;
+    if (!seq_last) return;
     float E = -INFINITY;
     for (int r = lane; r < p.rows_per_seq; r += 32) {
         const int rr = seq * p.rows_per_seq + r;
@@ -644,7 +534,7 @@ __global__ void __launch_bounds__(kGateThreads + (kStaged ? 32 : 0), kCtasPerSm)
     for (int o = 16; o > 0; o >>= 1) E = fmaxf(E, __shfl_xor_sync(0xffffffffu, E, o));
     if (lane == 0) {
         p.max_entropy_out[seq] = E;
-        p.decision_out[seq] = (seq_last & 2) ? -1 : (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
+        p.decision_out[seq] = (E > p.tau) ? EC_RECOMPUTE : EC_SKIP;
         p.seq_ticket[seq] = 0;
     }
 }
@@ -680,24 +570,18 @@ void plan_chunks(int n_rows, int vocab, int* splits, int* chunk, int max_splits 
     *splits = (int)((vocab + per - 1) / per);
 }
 
-template <typename T, bool kStaged>
+template <typename T>
 cudaError_t launch_t(const GateParams& p, cudaStream_t stream) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.splits, p.n_rows, 1);
-    cfg.blockDim = dim3(kGateThreads + (kStaged ? 32 : 0), 1, 1);    // the consumer warps (and the producer warp)
-    cfg.dynamicSmemBytes = kStaged ? kStages * kStageBytes : 0;
-    if (kStaged) {
-        static PerDeviceOnce once;
-        const cudaError_t e = ensure_dynamic_smem(once, gate_kernel<T, kStaged>, kStages * kStageBytes);
-        if (e != cudaSuccess) return e;
-    }
+    cfg.blockDim = dim3(kGateThreads, 1, 1);
     cfg.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch latency may overlap the previous kernel's tail
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gate_kernel<T, kStaged>, p);
+    return cudaLaunchKernelEx(&cfg, gate_kernel<T>, p);
 }
 
 }  // namespace
@@ -744,12 +628,7 @@ cudaError_t launch_gate(const GateArgs& a, cudaStream_t stream) {
     if (p.splits > kMaxSplits) return cudaErrorInvalidValue;   // vocab > 96 * 8192: rejected by the API layer before this
     p.single_level = (a.rows_per_seq <= kSingleLevelMaxRows && p.splits <= 32) ? 1 : 0;
     if (one_cta_finish && !p.single_level) return cudaErrorInvalidValue;   // rows_per_seq > 64 or vocab > 32 * 8192 * ...: rejected by the API layer
-    // small inputs through the bulk-copy ring, large ones (more than a few chunks per CTA slot) with per-thread loads
-    const size_t bytes = (size_t)a.n_rows * a.vocab * (a.dtype == EC_BF16 ? 2 : 4);
-    const bool staged = bytes < ((size_t)24 << 20);
-    if (a.dtype == EC_BF16)
-        return staged ? launch_t<__nv_bfloat16, true>(p, stream) : launch_t<__nv_bfloat16, false>(p, stream);
-    return staged ? launch_t<float, true>(p, stream) : launch_t<float, false>(p, stream);
+    return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16>(p, stream) : launch_t<float>(p, stream);
 }
 
 }  // namespace ec
