@@ -24,9 +24,14 @@
 //            proxy fence) only before the first tile that holds a refreshed position;
 //   warp 0   TMA producer: one 4-D box per operand tile ([2 halves][64 keys][64 columns],
 //            128-byte swizzle), NS stages, full/empty mbarriers;
-//   warps 2+ load Q into swizzled shared memory, then run the softmax: thread = query
-//            row = TMEM lane, running max and sum, exp2 with the scale folded in, lazy
-//            rescale of O;
+//   warps 2+ load Q into swizzled shared memory, then run the softmax: a query row (= TMEM lane)
+//            has two threads, in warps that own the same lanes, each of which takes 32 of a
+//            tile's 64 keys.  A reference in place of the running maximum: probabilities may
+//            exceed it by 2^60 (fp32 and bf16 have room for that, and it is never above the
+//            true maximum) before the two agree on a larger one and rescale O.  The chain of a
+//            tile (scores, softmax, second product) is what bounds the kernel, not memory, as
+//            long as there are fewer than about three CTAs for two SMs: 1.3 us with one thread
+//            per row and a running maximum;
 //   merge    the un-normalised rows (O, m, l) go from TMEM to a staging area grouped by
 //            owner (row r belongs to CTA r mod C of the cluster) and from there with one
 //            bulk shared-to-shared copy per owner into the owner's receive buffer,
@@ -52,6 +57,8 @@
 namespace ec {
 namespace {
 
+using namespace tc;
+
 constexpr int BM = 128, BN = 64, HD = 128;
 constexpr uint32_t KV_SUB = BN * 128;      // [64 keys x 64 bf16], 128-byte swizzle: 8 KB
 constexpr uint32_t KV_TILE = 2 * KV_SUB;   // [64 keys x 128 bf16]
@@ -60,6 +67,7 @@ constexpr int kMaxStages = 6;
 constexpr int kRec = HD + 4;               // floats per exchanged row: O[128], m, l, pad (16-byte multiple)
 constexpr int kMaxRows = 2 * BM;
 constexpr int kMaxCluster = 8;
+constexpr float kRaise = 60.f;             // a score may exceed its row's reference by this power of two
 
 // barrier slots (8 bytes each)
 enum {
@@ -75,100 +83,13 @@ enum {
     B_COUNT = B_RECV + 1
 };
 
-// ---- PTX wrappers -----------------------------------------------------------------
-// mbarriers (bounded waits), shared-memory addresses and the async-proxy fence are the shared wrappers
-using tc::s2u;
-using tc::mbar_init;
-using tc::mbar_arrive;
-using tc::mbar_expect_tx;
-using tc::mbar_try;
-using tc::mbar_wait;
-using tc::fence_async_smem;
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
+// 32 columns of this thread's TMEM lane as floats
+__device__ __forceinline__ void ld32f(uint32_t taddr, float* v) {
     uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
+    ld32(taddr, r);
+    wait_ld();
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const float* v) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-        ::"r"(taddr),
-          "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-          "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-          "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-          "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15])),
-          "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])), "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])),
-          "r"(__float_as_uint(v[20])), "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-          "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])), "r"(__float_as_uint(v[27])),
-          "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])), "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-        : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar) : "memory");
-}
-// bulk copy from this CTA's shared memory into a peer's, completing (bytes) on the peer's mbarrier
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t src_local, uint32_t bytes, uint32_t bar_cluster) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst_cluster), "r"(src_local), "r"(bytes), "r"(bar_cluster) : "memory");
-}
-__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_t cta_rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(cta_rank));
-    return r;
-}
-
-// shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// instruction descriptor: D fp32, A/B bf16, M = 128, N = n; b_mn = 1 when B is MN-major
-__host__ __device__ constexpr uint32_t instr_desc(int n, int b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(BM >> 4) << 24);
-}
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 struct SkipParams {
@@ -183,7 +104,7 @@ struct SkipParams {
     int n_active, ctx_len, n_q_heads, n_kv_heads, group, rows_total;
     int n_splits, tiles_per_split, n_stages, rows_per_cta;
     // shared-memory carve (bytes from the 1024-aligned base)
-    uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_bar;
+    uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_xch, off_bar;
     float scale_log2;
 };
 
@@ -197,10 +118,10 @@ struct SkipShared {
 };
 
 template <int NT>
-__global__ void __launch_bounds__(64 + NT * 128, NT == 1 ? 2 : 1)
+__global__ void __launch_bounds__(64 + NT * 256, NT == 1 ? 2 : 1)
 attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const SkipParams p) {
-    constexpr int kThreads = 64 + NT * 128;
-    constexpr int kSoftThreads = NT * 128;
+    constexpr int kThreads = 64 + NT * 256;
+    constexpr int kSoftThreads = NT * 256;   // per row tile: (keys 0..31 / 32..63 of a key tile) x 128 rows
     constexpr uint32_t TM_COLS = NT * 256;   // per row tile: S0 [0,64), S1 [64,128), O [128,256)
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
@@ -226,8 +147,8 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // softmax warps that own no query row copy the fresh rows; when every warp owns rows, all of them share it
     int n_idle = 0, my_idle = -1;
 #pragma unroll
-    for (int w = 2; w < 2 + NT * 4; ++w) {
-        const int rows_w = min(BM, p.rows_total - ((w - 2) >> 2) * BM);
+    for (int w = 2; w < 2 + NT * 8; ++w) {
+        const int rows_w = min(BM, p.rows_total - ((w - 2) >> 3) * BM);
         if (!((w & 3) * 32 < rows_w)) {
             if (w == warp) my_idle = n_idle;
             ++n_idle;
@@ -243,7 +164,7 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             uint32_t count = 1;
             if (i >= B_PFULL && i < B_PFULL + 2) {
                 const int rows_t = min(BM, p.rows_total - (i - B_PFULL) * BM);
-                count = rows_t > 0 ? 32u * ((rows_t + 31) / 32) : 1u;
+                count = rows_t > 0 ? 64u * ((rows_t + 31) / 32) : 1u;
             } else if (i == B_QFULL) {
                 count = kSoftThreads;
             } else if (i == B_REFRESHED) {
@@ -262,16 +183,17 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s2u(&sh->tmem)), "r"(TM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        tc_fence_before();
+        fence_before();
     }
     __syncthreads();
-    tc_fence_after();
+    fence_after();
     const uint32_t tmem = sh->tmem;
     pdl_wait();                    // the previous kernel of the stream has completed; global memory may be touched
     pdl_launch_dependents();
 
-    // softmax role: warp w >= 2 owns TMEM lanes 32 * (w % 4) of row tile (w - 2) / 4; thread = query row
-    const int soft_tile = warp >= 2 ? (warp - 2) >> 2 : 0;
+    // softmax role: warp w >= 2 owns TMEM lanes 32 * (w % 4) of row tile (w - 2) / 8 and half ((w - 2) / 4) % 2 of the keys
+    const int soft_tile = warp >= 2 ? (warp - 2) >> 3 : 0;
+    const int half = warp >= 2 ? ((warp - 2) >> 2) & 1 : 0;
     const int soft_row = (warp & 3) * 32 + lane;
     const int soft_rows_t = min(BM, p.rows_total - soft_tile * BM);
     const bool soft_active = warp >= 2 && (warp & 3) * 32 < soft_rows_t;   // warp-uniform
@@ -357,35 +279,35 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                     const uint32_t qh = p.rows_pad[t] * 128u;   // bytes of one 64-column half of the Q tile
 #pragma unroll
                     for (int k = 0; k < HD / 16; ++k) {
-                        tc_mma_ss(d, smem_desc(base + p.off_q[t] + (k >> 2) * qh + (k & 3) * 32, 16, 1024),
+                        mma_ss(d, smem_desc(base + p.off_q[t] + (k >> 2) * qh + (k & 3) * 32, 16, 1024),
                                   smem_desc(kst + (k >> 2) * KV_SUB + (k & 3) * 32, 16, 1024), IDESC_S, k > 0);
                     }
-                    tc_commit(bar(B_SFULL + t * 2 + (j & 1)));
+                    commit(bar(B_SFULL + t * 2 + (j & 1)));
                 }
             };
             mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
             mbar_wait(bar(B_FULL + 0), 0, abort_flag, p.dev_status);
-            tc_fence_after();
+            fence_after();
             issue_s(0);
             for (int j = 0; j < T; ++j) {
                 if (j + 1 < T) {
                     mbar_wait(bar(B_FULL + (j + 1) % NS), ((j + 1) / NS) & 1, abort_flag, p.dev_status);
-                    tc_fence_after();
+                    fence_after();
                     issue_s(j + 1);
                 }
                 const uint32_t vst = base + p.off_stage + (j % NS) * STAGE + KV_TILE;
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
                     mbar_wait(bar(B_PFULL + t), j & 1, abort_flag, p.dev_status);
-                    tc_fence_after();
+                    fence_after();
 #pragma unroll
                     for (int k = 0; k < BN / 16; ++k) {
-                        tc_mma_ss(tmem + t * 256 + 128, smem_desc(base + p.off_p[t] + k * 32, 16, 1024),
+                        mma_ss(tmem + t * 256 + 128, smem_desc(base + p.off_p[t] + k * 32, 16, 1024),
                                   smem_desc(vst + k * 2048, KV_SUB, 1024), IDESC_PV, (j > 0 || k > 0));
                     }
-                    tc_commit(bar(B_PVDONE + t));
+                    commit(bar(B_PVDONE + t));
                 }
-                tc_commit(bar(B_EMPTY + j % NS));
+                commit(bar(B_EMPTY + j % NS));
             }
         }
     } else {
@@ -449,102 +371,114 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             }
         }
 
+        // exchange between the two threads of a row: [half][row], rows that exist
+        float* xch = reinterpret_cast<float*>(gbase + p.off_xch) + soft_tile * 2 * (int)p.rows_pad[0];
+        const int rows_x = (int)p.rows_pad[soft_tile], soft_row_x = min(soft_row, rows_x - 1);
         if (soft_active) {
             const float sl2 = p.scale_log2;
+            const f32x2 sl2_2 = pk(sl2, sl2);
             const int t = soft_tile;
             unsigned char* prow = gbase + p.off_p[t] + (soft_row >> 3) * 1024 + (soft_row & 7) * 128;
             const bool store_p = soft_row < (int)p.rows_pad[t];   // rows past the padded tile have no storage
+            const int pair_bar = 1 + t * 4 + (warp & 3);          // named barrier of the two warps that share these rows
 
             for (int j = 0; j < T; ++j) {
                 mbar_wait(bar(B_SFULL + t * 2 + (j & 1)), (j >> 1) & 1, abort_flag, p.dev_status);
-                tc_fence_after();
-                float sc[BN];
-                tc_ld32(tm_t + (j & 1) * 64, sc);
-                tc_ld32(tm_t + (j & 1) * 64 + 32, sc + 32);
-                tc_wait_ld();
+                fence_after();
+                uint32_t sc[32];
+                ld32(tm_t + (j & 1) * 64 + half * 32, sc);
+                wait_ld();
                 int tile = first_tile + j;
                 if (tile >= T) tile -= T;
-                const int key0 = (t_begin + tile) * BN;
-                if (key0 + BN > p.ctx_len) {
+                const int key0 = (t_begin + tile) * BN + half * 32;
+                if (key0 + 32 > p.ctx_len) {
 #pragma unroll
-                    for (int c = 0; c < BN; ++c)
-                        if (key0 + c >= p.ctx_len) sc[c] = -INFINITY;
+                    for (int c = 0; c < 32; ++c)
+                        if (key0 + c >= p.ctx_len) sc[c] = 0xff800000u;   // -inf
                 }
-                float mx4[4] = {sc[0], sc[1], sc[2], sc[3]};
+                float mx4[4];
 #pragma unroll
-                for (int c = 4; c < BN; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], sc[c]);
-                float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                if (!valid) mx = 0.f;                // padded lanes never ask for a rescale
-                const float m_tile = mx * sl2;
+                for (int c = 0; c < 4; ++c) mx4[c] = __uint_as_float(sc[c]);
+#pragma unroll
+                for (int c = 4; c < 32; c += 2) mx4[(c >> 1) & 3] = max3(mx4[(c >> 1) & 3], __uint_as_float(sc[c]), __uint_as_float(sc[c + 1]));
+                const float mx = valid ? fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2 : -INFINITY;
                 float factor = 1.f;
-                if (m_tile > m_used + 8.f || m_used == -INFINITY) {   // stale maximum allowed up to 2^8
-                    factor = (m_used == -INFINITY) ? 0.f : fast_exp2(m_used - m_tile);
-                    m_used = m_tile;
+                const bool raise = named_barrier_or(pair_bar, 64, mx > m_used + kRaise);
+                if (raise) {   // the first tile, and rarely later: the two threads of a row agree on a larger reference
+                    if (soft_row < rows_x) xch[half * rows_x + soft_row] = mx;
+                    named_barrier(pair_bar, 64);
+                    const float m_new = fmaxf(m_used, fmaxf(mx, xch[(1 - half) * rows_x + soft_row_x]));
+                    factor = m_used == -INFINITY ? 0.f : fast_exp2(m_used - m_new);
+                    m_used = m_new;
                 }
-                const bool need_rescale = (j > 0) && __any_sync(0xffffffffu, factor != 1.f);
-                float rs4[4] = {0.f, 0.f, 0.f, 0.f};
-                const float mneg = -m_used;
+                const f32x2 mneg2 = valid ? pk(-m_used, -m_used) : pk(0.f, 0.f);
+                f32x2 sum2[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};
+                uint32_t pw[16];
 #pragma unroll
-                for (int c = 0; c < BN; ++c) {
-                    sc[c] = fast_exp2(fmaf(sc[c], sl2, mneg));
-                    rs4[c & 3] += sc[c];
+                for (int c = 0; c < 16; ++c) {
+                    const f32x2 d2 = fma2(pk(__uint_as_float(sc[2 * c]), __uint_as_float(sc[2 * c + 1])), sl2_2, mneg2);
+                    float d0, d1;
+                    upk(d2, d0, d1);
+                    const float e0 = fast_exp2(d0), e1 = fast_exp2(d1);
+                    sum2[c & 1] = add2(sum2[c & 1], pk(e0, e1));
+                    pw[c] = pack_bf16x2(e0, e1);
                 }
-                l_run = fmaf(l_run, factor, (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]));
+                float a0, a1, b0, b1;
+                upk(sum2[0], a0, a1);
+                upk(sum2[1], b0, b1);
+                l_run = fmaf(l_run, factor, (a0 + a1) + (b0 + b1));   // this half's share of the row sum
 
                 // P buffer free and O stable once P V of the previous tile has completed
                 if (j > 0) mbar_wait(bar(B_PVDONE + t), (j - 1) & 1, abort_flag, p.dev_status);
                 if (store_p) {
 #pragma unroll
-                    for (int ch = 0; ch < BN / 8; ++ch) {
-                        uint4 v;
-                        v.x = pack2(sc[ch * 8 + 0], sc[ch * 8 + 1]);
-                        v.y = pack2(sc[ch * 8 + 2], sc[ch * 8 + 3]);
-                        v.z = pack2(sc[ch * 8 + 4], sc[ch * 8 + 5]);
-                        v.w = pack2(sc[ch * 8 + 6], sc[ch * 8 + 7]);
-                        *reinterpret_cast<uint4*>(prow + ((ch ^ (soft_row & 7)) << 4)) = v;
-                    }
+                    for (int ch = 0; ch < 4; ++ch)
+                        *reinterpret_cast<uint4*>(prow + (((half * 4 + ch) ^ (soft_row & 7)) << 4)) =
+                            make_uint4(pw[4 * ch], pw[4 * ch + 1], pw[4 * ch + 2], pw[4 * ch + 3]);
                 }
-                if (need_rescale) {
-                    tc_fence_after();
+                if (raise && j > 0) {   // each of the two threads scales its 64 columns
+                    fence_after();
 #pragma unroll
-                    for (int c = 0; c < HD / 32; ++c) {
-                        float o[32];
-                        tc_ld32(tm_t + 128 + c * 32, o);
-                        tc_wait_ld();
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t o[32];
+                        ld32(tm_t + 128 + half * 64 + c * 32, o);
+                        wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] *= factor;
-                        tc_st32(tm_t + 128 + c * 32, o);
+                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
+                        st32(tm_t + 128 + half * 64 + c * 32, o);
                     }
-                    tc_wait_st();
+                    wait_st();
                 }
                 fence_async_smem();
-                tc_fence_before();
+                fence_before();
                 mbar_arrive(bar(B_PFULL + t));
             }
+            if (soft_row < rows_x) xch[half * rows_x + soft_row] = l_run;
+            named_barrier(pair_bar, 64);
+            l_run += xch[(1 - half) * rows_x + soft_row_x];
             // all row tiles have finished their last P V: Q, P and the K/V stages are dead from here on
 #pragma unroll
             for (int tt = 0; tt < NT; ++tt) mbar_wait(bar(B_PVDONE + tt), (T - 1) & 1, abort_flag, p.dev_status);
-            tc_fence_after();
+            fence_after();
 
             const int r = t * BM + soft_row;
             if (C == 1) {
                 // ---- single CTA per (sequence, kv head): normalise and store -------------------
                 const int i = valid ? r / p.group : 0, jh = valid ? r % p.group : 0;
-                __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + jh) * HD;
+                __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + jh) * HD + half * 64;
                 const float inv = 1.f / l_run;
 #pragma unroll
-                for (int c = 0; c < HD / 32; ++c) {
+                for (int c = 0; c < 2; ++c) {
                     float o[32];
-                    tc_ld32(tm_t + 128 + c * 32, o);
-                    tc_wait_ld();
+                    ld32f(tm_t + 128 + half * 64 + c * 32, o);
                     if (valid && !*abort_flag) {   // a CTA whose wait gave up stores nothing
 #pragma unroll
                         for (int v4 = 0; v4 < 4; ++v4) {
                             uint4 w;
-                            w.x = pack2(o[v4 * 8 + 0] * inv, o[v4 * 8 + 1] * inv);
-                            w.y = pack2(o[v4 * 8 + 2] * inv, o[v4 * 8 + 3] * inv);
-                            w.z = pack2(o[v4 * 8 + 4] * inv, o[v4 * 8 + 5] * inv);
-                            w.w = pack2(o[v4 * 8 + 6] * inv, o[v4 * 8 + 7] * inv);
+                            w.x = pack_bf16x2(o[v4 * 8 + 0] * inv, o[v4 * 8 + 1] * inv);
+                            w.y = pack_bf16x2(o[v4 * 8 + 2] * inv, o[v4 * 8 + 3] * inv);
+                            w.z = pack_bf16x2(o[v4 * 8 + 4] * inv, o[v4 * 8 + 5] * inv);
+                            w.w = pack_bf16x2(o[v4 * 8 + 6] * inv, o[v4 * 8 + 7] * inv);
                             *reinterpret_cast<uint4*>(dst + c * 32 + v4 * 8) = w;
                         }
                     }
@@ -554,10 +488,9 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 float* rec = reinterpret_cast<float*>(gbase) +
                              (valid ? ((r % C) * p.rows_per_cta + r / C) : 0) * kRec;   // staging reuses the dead Q/P/stage memory
 #pragma unroll
-                for (int c = 0; c < HD / 32; ++c) {
+                for (int c = half * 2; c < half * 2 + 2; ++c) {
                     float o[32];
-                    tc_ld32(tm_t + 128 + c * 32, o);
-                    tc_wait_ld();
+                    ld32f(tm_t + 128 + c * 32, o);
                     if (valid) {
 #pragma unroll
                         for (int v4 = 0; v4 < 8; ++v4)
@@ -565,7 +498,7 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                                 make_float4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
                     }
                 }
-                if (valid) *reinterpret_cast<float4*>(rec + HD) = make_float4(m_used, l_run, 0.f, 0.f);
+                if (valid && half == 0) *reinterpret_cast<float4*>(rec + HD) = make_float4(m_used, l_run, 0.f, 0.f);
                 fence_async_smem();   // staging (generic proxy) -> bulk copies (async proxy)
             }
         }
@@ -625,8 +558,8 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + jh) * HD;
                 const float inv = 1.f / l;
                 uint2 w2;
-                w2.x = pack2(acc.x * inv, acc.y * inv);
-                w2.y = pack2(acc.z * inv, acc.w * inv);
+                w2.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+                w2.y = pack_bf16x2(acc.z * inv, acc.w * inv);
                 if (!*abort_flag) *reinterpret_cast<uint2*>(dst + lane * 4) = w2;   // nothing from a CTA whose wait gave up
             }
         }
@@ -636,18 +569,15 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         cluster_wait();
     }
 
-    tc_fence_before();
+    fence_before();
     __syncthreads();
     if (warp == 1) {
-        tc_fence_after();
+        fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TM_COLS) : "memory");
     }
 }
 
 // ---- host side ---------------------------------------------------------------------------
-using tc::EncodeTiledFn;
-using tc::encode_fn;
-
 // cache [B*Hkv, L, 128] bf16 seen as 4-D {64 columns, key, half, head}: one box {64, 64, 2, 1} lands as
 // [half][key][64 columns], i.e. the two 128-byte-swizzled halves of a [64 keys x 128] tile back to back; keys
 // beyond L read as zero
@@ -665,7 +595,7 @@ bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len) {
 
 struct SkipPlan {
     int nt, rows_total, n_splits, tiles_per_split, n_stages, rows_per_cta;
-    uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_bar, smem_bytes;
+    uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_xch, off_bar, smem_bytes;
 };
 
 constexpr uint32_t kSmemTwoPerSm = 115712;   // (228 KB per SM - 2 x 1 KB reserved) / 2
@@ -701,7 +631,8 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
     // the exchange areas (staging, then receive buffer) reuse the memory below the list once the main loop is over
     const uint32_t recv = pl.n_splits > 1 ? (uint32_t)(pl.n_splits * pl.rows_per_cta * kRec * 4) : 0u;
     const uint32_t list = ((uint32_t)n_active * 8u + 15u) & ~15u;
-    const uint32_t tail = list + B_COUNT * 8u + 32u + 1024u;   // + barrier block + alignment slack
+    const uint32_t xch = (pl.rows_pad[0] + pl.rows_pad[1]) * 8u;   // two floats per row
+    const uint32_t tail = list + xch + B_COUNT * 8u + 32u + 1024u;   // + barrier block + alignment slack
     int ns = 0;
     if (pl.nt == 1) {   // two CTAs per SM when at least two stages fit in half an SM
         ns = off + tail < kSmemTwoPerSm ? (int)((kSmemTwoPerSm - off - tail) / STAGE) : 0;
@@ -717,6 +648,8 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
     pl.off_recv = recv;   // right behind the staging area, which starts at 0
     pl.off_list = off;
     off += list;
+    pl.off_xch = off;
+    off += xch;
     pl.off_bar = off;
     off += B_COUNT * 8u + 32u;
     pl.smem_bytes = off + 1024u;
@@ -730,7 +663,7 @@ cudaError_t launch_nt(const SkipPlan& pl, const SkipParams& p, const CUtensorMap
     if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_skip_kernel<NT>, (int)kSmemMax); ea != cudaSuccess) return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(pl.n_splits, bh, 1);
-    cfg.blockDim = dim3(64 + NT * 128, 1, 1);
+    cfg.blockDim = dim3(64 + NT * 256, 1, 1);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute at[2];
@@ -797,6 +730,7 @@ cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const voi
     p.off_stage = pl.off_stage;
     p.off_recv = pl.off_recv;
     p.off_list = pl.off_list;
+    p.off_xch = pl.off_xch;
     p.off_bar = pl.off_bar;
     p.scale_log2 = a.scale * kLog2e;
     return pl.nt == 1 ? launch_nt<1>(pl, p, map_k, map_v, bh, stream) : launch_nt<2>(pl, p, map_k, map_v, bh, stream);
