@@ -12,16 +12,16 @@
 //            one (sequence, kv head) and split its 64-key tiles into C contiguous ranges;
 //   rows     the n_active x (H_q/H_kv) query rows that share the kv head are packed
 //            into one or two 128-row M tiles (NT); the same K/V tile serves both;
-//   warp 1   scans active_idx for positions inside this CTA's key range (the refresh
-//            list), then issues the tcgen05.mma (S = Q K^T, M128 N64 K16 x 8, into one of
-//            two TMEM S buffers; O += P V, M128 N128 K16 x 4, P from shared memory, V
-//            MN-major);
-//   refresh  a CTA refreshes the cache rows of its own key range (no other CTA reads
-//            them).  Its tiles are visited in rotated order, starting behind the last
-//            tile that holds a refreshed position, so the tiles that need no refresh
-//            stream while softmax warps without query rows copy the fresh rows into the
-//            cache; the producer waits for that copy (generic-proxy writes, then a
-//            proxy fence) only before the first tile that holds a refreshed position;
+//   warp 1   issues the tcgen05.mma (S = Q K^T, M128 N64 K16 x 8, into one of two TMEM S
+//            buffers; O += P V, M128 N128 K16 x 4, P from shared memory, V MN-major), whichever
+//            of the two is ready;
+//   refresh  the fresh rows are attended straight from k_new / v_new, as extra key tiles that
+//            the last CTA of a cluster visits after its cache tiles, while every CTA masks the
+//            stale cached keys of the refreshed positions (a bit per key); softmax warps without
+//            query rows build the masks and copy the fresh rows into the cache, ordered against
+//            nothing.  (Waiting for that copy before the first tile that holds a refreshed
+//            position, and for the list of positions before the first tile at all, cost 3 us a
+//            launch);
 //   warp 0   TMA producer: one 4-D box per operand tile ([2 halves][64 keys][64 columns],
 //            128-byte swizzle), NS stages, full/empty mbarriers;
 //   warps 2+ load Q into swizzled shared memory, then run the softmax: a query row (= TMEM lane)
@@ -41,13 +41,14 @@
 // rows, and the rows past the last packed query row read whatever follows in the CTA's
 // own allocation; rows of S, P and O are independent, so those values never reach a
 // real row and are never stored.
-// The kernel is launched with programmatic stream serialisation: everything before
-// griddepcontrol.wait (barrier set-up, TMEM allocation, descriptor prefetch) may overlap
-// the previous kernel of the stream; nothing in global memory is touched before it.
+// The kernel is launched with programmatic stream serialisation: set-up may overlap the
+// previous kernel of the stream, and so may the first cache tiles when the caller has
+// stated that nothing in flight writes the caches; all else is read after griddepcontrol.wait.
 // Every mbarrier wait is bounded: a wait that runs out sets EC_ERR_TIMEOUT in the
 // caller's dev_status word and a CTA-wide abort flag that makes all later waits fall
 // through; the CTA still frees its TMEM and exits.
 #include "ec_common.cuh"
+#include "ec_skip_keys_pair.cuh"
 #include "ec_tc_ptx.cuh"
 
 #include <cuda.h>
@@ -77,9 +78,8 @@ enum {
     B_PFULL = B_SFULL + 4,            // [tile]
     B_PVDONE = B_PFULL + 2,           // [tile]
     B_QFULL = B_PVDONE + 2,           // Q tiles staged
-    B_LIST = B_QFULL + 1,             // refresh list built
-    B_REFRESHED = B_LIST + 1,         // fresh rows of this CTA's key range are in the cache
-    B_RECV = B_REFRESHED + 1,              // all partial rows this CTA owns have arrived
+    B_LIST = B_QFULL + 1,             // key masks built
+    B_RECV = B_LIST + 1,              // all partial rows this CTA owns have arrived
     B_COUNT = B_RECV + 1
 };
 
@@ -103,6 +103,9 @@ struct SkipParams {
     int32_t* dev_status;
     int n_active, ctx_len, n_q_heads, n_kv_heads, group, rows_total;
     int n_splits, tiles_per_split, n_stages, rows_per_cta;
+    int n_extra;      // key tiles of fresh rows attended by the last CTA of every cluster (0: nothing to refresh)
+    int keys_on_m;    // 1: the CTA runs keys_pair::run
+    int early_cache;  // 1: nothing still running on the stream writes the caches (EC_ATTN_CACHE_SETTLED)
     // shared-memory carve (bytes from the 1024-aligned base)
     uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_xch, off_bar;
     float scale_log2;
@@ -112,24 +115,36 @@ struct SkipParams {
 struct SkipShared {
     uint32_t tmem;
     int abort_flag;
-    int n_mine;       // entries of the refresh list
-    int first_tile;   // rotation: the CTA visits its tiles in the order (first_tile + j) mod T
-    int j_refreshed;  // first visit index j whose tile holds a refreshed position (T if none)
 };
 
 template <int NT>
 __global__ void __launch_bounds__(64 + NT * 256, NT == 1 ? 2 : 1)
-attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const SkipParams p) {
+attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                   const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn, const SkipParams p,
+                   const keys_pair::Params kp) {
     constexpr int kThreads = 64 + NT * 256;
     constexpr int kSoftThreads = NT * 256;   // per row tile: (keys 0..31 / 32..63 of a key tile) x 128 rows
     constexpr uint32_t TM_COLS = NT * 256;   // per row tile: S0 [0,64), S1 [64,128), O [128,256)
     extern __shared__ unsigned char smem_raw[];
-    const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
-    unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
+    const uint32_t base = s2u(smem_raw);
+    unsigned char* gbase = smem_raw;
+    if (base & 1023u) {   // never: the runtime puts dynamic shared memory on a 1024-byte boundary
+        if (threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, (int)EC_ERR_CUDA);
+        return;
+    }
+    if constexpr (NT == 1) {
+        if (p.keys_on_m) {   // few rows, a CTA per kv head: the maps hold 128-key boxes
+            if (p.rows_total <= 48) keys_pair::run<48>(map_k, map_v, map_kn, map_vn, kp, smem_raw);
+            else keys_pair::run<64>(map_k, map_v, map_kn, map_vn, kp, smem_raw);
+            return;
+        }
+    }
     const uint32_t bars = base + p.off_bar;
     SkipShared* sh = reinterpret_cast<SkipShared*>(gbase + p.off_bar + B_COUNT * 8);
     volatile int* abort_flag = &sh->abort_flag;
-    int2* list = reinterpret_cast<int2*>(gbase + p.off_list);   // (active row i, position) pairs of this CTA's key range
+    // [key tile of this CTA, cache tiles first][2]: a bit per key; of a cached key whose position is being refreshed (it does
+    // not count: it is attended from the fresh tile instead), of a fresh key that exists
+    uint32_t* bits = reinterpret_cast<uint32_t*>(gbase + p.off_list);
     auto bar = [&](int idx) { return bars + idx * 8; };
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -139,10 +154,12 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     const int n_tiles_total = (p.ctx_len + BN - 1) / BN;
     const int t_begin = split * p.tiles_per_split;
     const int t_end = min(n_tiles_total, t_begin + p.tiles_per_split);
-    const int T = t_end - t_begin;   // >= 1 by construction of the plan
+    const bool refresh = p.k_new != nullptr;
+    const int TC = t_end - t_begin;  // cache tiles: >= 1 by construction of the plan
+    const int XT = (refresh && split == p.n_splits - 1) ? p.n_extra : 0;   // fresh tiles, visited after them
+    const int T = TC + XT;
     const int NS = p.n_stages;
     const int n_own = (p.rows_total - split + C - 1) / C;   // packed rows r = split + q * C merged by this CTA
-    const bool refresh = p.k_new != nullptr;
 
     // softmax warps that own no query row copy the fresh rows; when every warp owns rows, all of them share it
     int n_idle = 0, my_idle = -1;
@@ -167,18 +184,16 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 count = rows_t > 0 ? 64u * ((rows_t + 31) / 32) : 1u;
             } else if (i == B_QFULL) {
                 count = kSoftThreads;
-            } else if (i == B_REFRESHED) {
+            } else if (i == B_LIST) {
                 count = (uint32_t)n_copy_threads;
             }
             mbar_init(bar(i), count);
         }
         sh->abort_flag = 0;
-        sh->n_mine = 0;
-        sh->first_tile = 0;
-        sh->j_refreshed = T;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (C > 1 && n_own > 0) mbar_expect_tx(bar(B_RECV), (uint32_t)(C * n_own * kRec * 4));
     }
+    for (int w = tid; w < 2 * T; w += kThreads) bits[w] = 0u;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s2u(&sh->tmem)), "r"(TM_COLS)
                      : "memory");
@@ -188,8 +203,9 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     __syncthreads();
     fence_after();
     const uint32_t tmem = sh->tmem;
-    pdl_wait();                    // the previous kernel of the stream has completed; global memory may be touched
-    pdl_launch_dependents();
+    if (warp != 0) pdl_wait();     // the previous kernel of the stream has completed; its results may be read
+    if (tid == 32) pdl_launch_dependents();
+    __syncwarp();
 
     // softmax role: warp w >= 2 owns TMEM lanes 32 * (w % 4) of row tile (w - 2) / 8 and half ((w - 2) / 4) % 2 of the keys
     const int soft_tile = warp >= 2 ? (warp - 2) >> 3 : 0;
@@ -205,109 +221,84 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     if (warp == 0) {
         // ================================ TMA producer ======================================
         if (lane == 0) {
-            int first_tile = 0, j_refreshed = T;
-            if (refresh) {
-                mbar_wait(bar(B_LIST), 0, abort_flag, p.dev_status);
-                first_tile = sh->first_tile;
-                j_refreshed = sh->j_refreshed;
-            }
-            for (int j = 0; j < T; ++j) {
-                const int s = j % NS, u = j / NS;
-                int tile = first_tile + j;
-                if (tile >= T) tile -= T;
-                const int key0 = (t_begin + tile) * BN;
-                if (j == j_refreshed) mbar_wait(bar(B_REFRESHED), 0, abort_flag, p.dev_status);
-                if (u > 0) mbar_wait(bar(B_EMPTY + s), (u - 1) & 1, abort_flag, p.dev_status);
+            auto load = [&](int j) {
+                const int s = j % NS;
                 const uint32_t dst = base + p.off_stage + s * STAGE;
                 mbar_expect_tx(bar(B_FULL + s), STAGE);
-                tma_load_4d(dst, &map_k, 0, key0, 0, bh, bar(B_FULL + s));
-                tma_load_4d(dst + KV_TILE, &map_v, 0, key0, 0, bh, bar(B_FULL + s));
-            }
-        }
-    } else if (warp == 1) {
-        // ================= refresh list, then MMA issue (lane 0) =================================
-        if (refresh) {
-            int posv[kMaxRows / 32];
-#pragma unroll
-            for (int k = 0; k < kMaxRows / 32; ++k) {
-                const int i = k * 32 + lane;
-                posv[k] = -1;
-                if (i < p.n_active) posv[k] = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
-            }
-            int n_mine = 0;
-            int hi_tile = -1;   // last local tile that holds a refreshed position
-#pragma unroll
-            for (int k = 0; k < kMaxRows / 32; ++k) {
-                const bool hit = posv[k] >= key_lo && posv[k] < key_hi;
-                const unsigned m = __ballot_sync(0xffffffffu, hit);
-                if (hit) {
-                    list[n_mine + __popc(m & ((1u << lane) - 1u))] = make_int2(k * 32 + lane, posv[k]);
-                    hi_tile = max(hi_tile, (posv[k] - key_lo) / BN);
-                }
-                n_mine += __popc(m);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) hi_tile = max(hi_tile, __shfl_xor_sync(0xffffffffu, hi_tile, o));
-            // rotate so that the last refreshed tile comes last; the first refreshed tile in that order:
-            const int first_tile = n_mine > 0 ? (hi_tile + 1) % T : 0;
-            int j_ref = T;
-#pragma unroll
-            for (int k = 0; k < kMaxRows / 32; ++k) {
-                if (posv[k] >= key_lo && posv[k] < key_hi) {
-                    int j = (posv[k] - key_lo) / BN - first_tile;
-                    if (j < 0) j += T;
-                    j_ref = min(j_ref, j);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) j_ref = min(j_ref, __shfl_xor_sync(0xffffffffu, j_ref, o));
-            __syncwarp();
-            if (lane == 0) {
-                sh->n_mine = n_mine;
-                sh->first_tile = first_tile;
-                sh->j_refreshed = j_ref;
-                mbar_arrive(bar(B_LIST));
-            }
-        }
-        if (lane == 0) {
-            constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
-            auto issue_s = [&](int j) {
-                const uint32_t kst = base + p.off_stage + (j % NS) * STAGE;
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const uint32_t d = tmem + t * 256 + (j & 1) * 64;
-                    const uint32_t qh = p.rows_pad[t] * 128u;   // bytes of one 64-column half of the Q tile
-#pragma unroll
-                    for (int k = 0; k < HD / 16; ++k) {
-                        mma_ss(d, smem_desc(base + p.off_q[t] + (k >> 2) * qh + (k & 3) * 32, 16, 1024),
-                                  smem_desc(kst + (k >> 2) * KV_SUB + (k & 3) * 32, 16, 1024), IDESC_S, k > 0);
-                    }
-                    commit(bar(B_SFULL + t * 2 + (j & 1)));
+                if (j >= TC) {   // active rows [64 x, 64 x + 64) of this kv head, fresh; rows past n_active read as zero
+                    tma_load_5d(dst, &map_kn, 0, (j - TC) * BN, 0, hk, b, bar(B_FULL + s));
+                    tma_load_5d(dst + KV_TILE, &map_vn, 0, (j - TC) * BN, 0, hk, b, bar(B_FULL + s));
+                } else {
+                    tma_load_4d(dst, &map_k, 0, (t_begin + j) * BN, 0, bh, bar(B_FULL + s));
+                    tma_load_4d(dst + KV_TILE, &map_v, 0, (t_begin + j) * BN, 0, bh, bar(B_FULL + s));
                 }
             };
+            int j = 0;
+            if (p.early_cache)
+                for (const int fill = min(NS, TC); j < fill; ++j) load(j);
+            pdl_wait();
+            for (; j < T; ++j) {
+                if (j >= NS) mbar_wait(bar(B_EMPTY + j % NS), (j / NS - 1) & 1, abort_flag, p.dev_status);
+                load(j);
+            }
+        } else {
+            pdl_wait();
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ================================ MMA issue (lane 0) ========================================
+        if (lane == 0) {
+            constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
+            uint64_t desc_q[NT], desc_p[NT];
+            uint32_t qh[NT];   // one 64-column half of the Q tile, in descriptor units
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                desc_q[t] = smem_desc(base + p.off_q[t], 16, 1024);
+                desc_p[t] = smem_desc(base + p.off_p[t], 16, 1024);
+                qh[t] = p.rows_pad[t] * 8u;
+            }
+            // S of a tile needs the tile, P V of a tile and row tile needs its P: whichever is ready is issued.  S may run
+            // one tile ahead of P V (two S buffers).
+            int next_s = 0, next_pv[NT], n_pv = 0;   // n_pv: tiles whose P V has been issued for every row tile
+#pragma unroll
+            for (int t = 0; t < NT; ++t) next_pv[t] = 0;
             mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
-            mbar_wait(bar(B_FULL + 0), 0, abort_flag, p.dev_status);
-            fence_after();
-            issue_s(0);
-            for (int j = 0; j < T; ++j) {
-                if (j + 1 < T) {
-                    mbar_wait(bar(B_FULL + (j + 1) % NS), ((j + 1) / NS) & 1, abort_flag, p.dev_status);
+            SpinGuard guard;
+            while (n_pv < T) {
+                bool progressed = false;
+                if (next_s < T && next_s <= n_pv + 1 && mbar_test(bar(B_FULL + next_s % NS), (next_s / NS) & 1)) {
+                    const uint64_t desc_k = smem_desc(base + p.off_stage + (next_s % NS) * STAGE, 16, 1024);
                     fence_after();
-                    issue_s(j + 1);
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) {
+#pragma unroll
+                        for (int k = 0; k < HD / 16; ++k)
+                            mma_ss(tmem + t * 256 + (next_s & 1) * 64, desc_q[t] + (k >> 2) * qh[t] + (k & 3) * 2,
+                                   desc_k + (k >> 2) * (KV_SUB / 16) + (k & 3) * 2, IDESC_S, k > 0);
+                        commit(bar(B_SFULL + t * 2 + (next_s & 1)));
+                    }
+                    ++next_s;
+                    progressed = true;
                 }
-                const uint32_t vst = base + p.off_stage + (j % NS) * STAGE + KV_TILE;
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
-                    mbar_wait(bar(B_PFULL + t), j & 1, abort_flag, p.dev_status);
+                    const int j = next_pv[t];
+                    if (j >= next_s || !mbar_test(bar(B_PFULL + t), j & 1)) continue;
+                    const uint64_t desc_v = smem_desc(base + p.off_stage + (j % NS) * STAGE + KV_TILE, KV_SUB, 1024);
                     fence_after();
 #pragma unroll
-                    for (int k = 0; k < BN / 16; ++k) {
-                        mma_ss(tmem + t * 256 + 128, smem_desc(base + p.off_p[t] + k * 32, 16, 1024),
-                                  smem_desc(vst + k * 2048, KV_SUB, 1024), IDESC_PV, (j > 0 || k > 0));
-                    }
+                    for (int k = 0; k < BN / 16; ++k)
+                        mma_ss(tmem + t * 256 + 128, desc_p[t] + k * 2, desc_v + k * 128, IDESC_PV, (j > 0 || k > 0));
                     commit(bar(B_PVDONE + t));
+                    ++next_pv[t];
+                    progressed = true;
                 }
-                commit(bar(B_EMPTY + j % NS));
+                int done = next_pv[0];
+#pragma unroll
+                for (int t = 1; t < NT; ++t) done = min(done, next_pv[t]);
+                for (; n_pv < done; ++n_pv) commit(bar(B_EMPTY + n_pv % NS));
+                if (progressed) guard.progress();
+                else if (!guard.tick(abort_flag, p.dev_status)) break;
             }
         }
     } else {
@@ -333,41 +324,39 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         fence_async_smem();         // Q tiles (generic proxy) -> visible to the tensor core (async proxy)
         mbar_arrive(bar(B_QFULL));
 
-        int first_tile = 0;
-        if (refresh) {
-            mbar_wait(bar(B_LIST), 0, abort_flag, p.dev_status);
-            first_tile = sh->first_tile;
-            // fresh rows of this CTA's key range -> cache in global memory, eight 16-byte pieces in flight per thread
-            if (n_idle == 0 || my_idle >= 0) {
-                const int wid = n_idle == 0 ? stid : my_idle * 32 + lane;
-                const int wn = n_copy_threads;
-                const int chunks = sh->n_mine * 32;
-                for (int c0 = wid; c0 < chunks; c0 += 8 * wn) {
-                    uint4 v[8];
-                    long long dsto[8];
-                    int isv[8];
+        if (refresh && (n_idle == 0 || my_idle >= 0)) {
+            const int wid = n_idle == 0 ? stid : my_idle * 32 + lane;
+            // key masks: stale cached keys of this CTA's range, and the fresh keys that exist
+            for (int i = wid; i < p.n_active; i += n_copy_threads) {
+                const int pos = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
+                if (pos >= key_lo && pos < key_hi) atomicOr(&bits[(pos - key_lo) >> 5], 1u << ((pos - key_lo) & 31));
+                if (XT && pos >= 0 && pos < p.ctx_len) atomicOr(&bits[2 * TC + (i >> 5)], 1u << (i & 31));
+            }
+            mbar_arrive(bar(B_LIST));   // release: the bits above are visible to whoever waits
+            // this CTA's share of the fresh rows -> cache in global memory, for later steps, four 16-byte pieces in flight
+            // per thread; nothing in this launch depends on it
+            const int pieces = p.n_active * 32;   // [row][K, V][16 pieces]
+            for (int q0 = split * n_copy_threads + wid; q0 < pieces; q0 += 4 * C * n_copy_threads) {
+                uint4 v[4];
+                int pos[4];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int c = c0 + u * wn;
-                        isv[u] = -1;
-                        if (c < chunks) {
-                            const int e = c >> 5, piece = c & 15;
-                            isv[u] = (c >> 4) & 1;
-                            const int2 ip = list[e];
-                            const long long src = (((long long)b * p.n_active + ip.x) * p.n_kv_heads + hk) * HD + piece * 8;
-                            dsto[u] = ((long long)bh * p.ctx_len + ip.y) * HD + piece * 8;
-                            v[u] = __ldg(reinterpret_cast<const uint4*>((isv[u] ? p.v_new : p.k_new) + src));
-                        }
+                for (int u = 0; u < 4; ++u) {
+                    const int c = q0 + u * C * n_copy_threads, i = c >> 5;
+                    pos[u] = -1;
+                    if (c < pieces) {
+                        pos[u] = p.active_idx ? __ldg(p.active_idx + (long long)b * p.n_active + i) : i;
+                        const __nv_bfloat16* src = (c & 16) ? p.v_new : p.k_new;
+                        v[u] = __ldg(reinterpret_cast<const uint4*>(
+                            src + (((long long)b * p.n_active + i) * p.n_kv_heads + hk) * HD + (c & 15) * 8));
                     }
+                }
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (isv[u] >= 0) *reinterpret_cast<uint4*>((isv[u] ? p.v_cache : p.k_cache) + dsto[u]) = v[u];
+                for (int u = 0; u < 4; ++u) {
+                    const int c = q0 + u * C * n_copy_threads;
+                    if (pos[u] < 0 || pos[u] >= p.ctx_len) continue;
+                    __nv_bfloat16* dst = (c & 16) ? p.v_cache : p.k_cache;
+                    *reinterpret_cast<uint4*>(dst + ((long long)bh * p.ctx_len + pos[u]) * HD + (c & 15) * 8) = v[u];
                 }
-                if (chunks > 0) {
-                    __threadfence();
-                    fence_async_global();   // generic-proxy writes above before this CTA's TMA reads of the same rows
-                }
-                mbar_arrive(bar(B_REFRESHED));
             }
         }
 
@@ -388,13 +377,17 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 uint32_t sc[32];
                 ld32(tm_t + (j & 1) * 64 + half * 32, sc);
                 wait_ld();
-                int tile = first_tile + j;
-                if (tile >= T) tile -= T;
-                const int key0 = (t_begin + tile) * BN + half * 32;
-                if (key0 + 32 > p.ctx_len) {
+                uint32_t gone = 0;   // keys that do not count
+                if (refresh) {
+                    if (j == 0) mbar_wait(bar(B_LIST), 0, abort_flag, p.dev_status);
+                    gone = j < TC ? bits[2 * j + half] : ~bits[2 * j + half];
+                }
+                const int left = p.ctx_len - (t_begin + j) * BN - half * 32;
+                if (j < TC && left < 32) gone |= left <= 0 ? ~0u : ~0u << left;   // past the end of the context
+                if (gone) {
 #pragma unroll
                     for (int c = 0; c < 32; ++c)
-                        if (key0 + c >= p.ctx_len) sc[c] = 0xff800000u;   // -inf
+                        if ((gone >> c) & 1u) sc[c] = 0xff800000u;   // -inf
                 }
                 float mx4[4];
 #pragma unroll
@@ -411,7 +404,8 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                     factor = m_used == -INFINITY ? 0.f : fast_exp2(m_used - m_new);
                     m_used = m_new;
                 }
-                const f32x2 mneg2 = valid ? pk(-m_used, -m_used) : pk(0.f, 0.f);
+                const float mneg = valid && m_used != -INFINITY ? -m_used : 0.f;   // (no key has counted yet: every d is -inf)
+                const f32x2 mneg2 = pk(mneg, mneg);
                 f32x2 sum2[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};
                 uint32_t pw[16];
 #pragma unroll
@@ -578,23 +572,39 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
 }
 
 // ---- host side ---------------------------------------------------------------------------
-// cache [B*Hkv, L, 128] bf16 seen as 4-D {64 columns, key, half, head}: one box {64, 64, 2, 1} lands as
-// [half][key][64 columns], i.e. the two 128-byte-swizzled halves of a [64 keys x 128] tile back to back; keys
-// beyond L read as zero
-bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len) {
+// cache [B*Hkv, L, 128] bf16 seen as 4-D {64 columns, key, half, head}: one box {64, box_keys, 2, 1}
+// lands as [half][key][64 columns], i.e. the two 128-byte-swizzled halves of a [box_keys x 128] tile back to back;
+// keys beyond L read as zero
+bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len, int box_keys) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[4] = {64, (cuuint64_t)ctx_len, 2, (cuuint64_t)bh};
     const cuuint64_t strides[3] = {(cuuint64_t)HD * 2, 128, (cuuint64_t)ctx_len * HD * 2};
-    const cuuint32_t box[4] = {64, (cuuint32_t)BN, 2, 1};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_keys, 2, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(cache), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// k_new / v_new [B, n, H_kv, 128] bf16 seen as 5-D {64 columns, active row, half, kv head, sequence}: one box
+// {64, box_rows, 2, 1, 1} lands like a cache tile whose keys are active rows of one kv head; rows past n read as zero
+bool make_fresh_map(CUtensorMap* map, const void* fresh, int batch, int n_active, int n_kv_heads, int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)n_active, 2, (cuuint64_t)n_kv_heads, (cuuint64_t)batch};
+    const cuuint64_t strides[4] = {(cuuint64_t)n_kv_heads * HD * 2, 128, (cuuint64_t)HD * 2,
+                                   (cuuint64_t)n_active * n_kv_heads * HD * 2};
+    const cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 2, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(fresh), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct SkipPlan {
-    int nt, rows_total, n_splits, tiles_per_split, n_stages, rows_per_cta;
+    int nt, rows_total, n_splits, tiles_per_split, n_stages, rows_per_cta, n_extra;
+    bool keys_on_m;   // at most 64 packed rows and a CTA per kv head: see ec_skip_keys_pair.cuh
     uint32_t off_q[2], off_p[2], rows_pad[2], off_stage, off_recv, off_list, off_xch, off_bar, smem_bytes;
 };
 
@@ -616,6 +626,7 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
     pl.tiles_per_split = (key_tiles + c - 1) / c;
     pl.n_splits = (key_tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
     pl.rows_per_cta = (pl.rows_total + pl.n_splits - 1) / pl.n_splits;
+    pl.n_extra = (n_active + BN - 1) / BN;
     uint32_t off = 0;
     for (int t = 0; t < 2; ++t) {
         const int rows_t = t < pl.nt ? (pl.rows_total - t * BM < BM ? pl.rows_total - t * BM : BM) : 0;
@@ -630,9 +641,9 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
     pl.off_stage = off;   // multiple of 1024: every piece above is a multiple of 8 rows x 128 bytes
     // the exchange areas (staging, then receive buffer) reuse the memory below the list once the main loop is over
     const uint32_t recv = pl.n_splits > 1 ? (uint32_t)(pl.n_splits * pl.rows_per_cta * kRec * 4) : 0u;
-    const uint32_t list = ((uint32_t)n_active * 8u + 15u) & ~15u;
+    const uint32_t list = ((uint32_t)(pl.tiles_per_split + pl.n_extra) * 8u + 15u) & ~15u;   // key masks
     const uint32_t xch = (pl.rows_pad[0] + pl.rows_pad[1]) * 8u;   // two floats per row
-    const uint32_t tail = list + xch + B_COUNT * 8u + 32u + 1024u;   // + barrier block + alignment slack
+    const uint32_t tail = list + xch + B_COUNT * 8u + 32u;   // + barrier block
     int ns = 0;
     if (pl.nt == 1) {   // two CTAs per SM when at least two stages fit in half an SM
         ns = off + tail < kSmemTwoPerSm ? (int)((kSmemTwoPerSm - off - tail) / STAGE) : 0;
@@ -642,7 +653,8 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
         ns = off + tail < kSmemMax ? (int)((kSmemMax - off - tail) / STAGE) : 0;
         if (ns > kMaxStages) ns = kMaxStages;
     }
-    if (ns > pl.tiles_per_split && ns > 2) ns = pl.tiles_per_split < 2 ? 2 : pl.tiles_per_split;
+    const int visits = pl.tiles_per_split + pl.n_extra;
+    if (ns > visits && ns > 2) ns = visits < 2 ? 2 : visits;
     pl.n_stages = ns;
     off += (uint32_t)ns * STAGE;
     pl.off_recv = recv;   // right behind the staging area, which starts at 0
@@ -652,12 +664,18 @@ SkipPlan make_skip_plan(const ec_attn_desc& d, int n_active) {
     off += xch;
     pl.off_bar = off;
     off += B_COUNT * 8u + 32u;
-    pl.smem_bytes = off + 1024u;
+    pl.smem_bytes = off;
+    // With at least a CTA per kv head and SM in flight, what counts is the time of a key tile; with fewer heads the keys
+    // are split over a cluster, which needs the merge of this kernel.
+    pl.keys_on_m = pl.nt == 1 && pl.n_splits == 1 && pl.rows_total <= keys_pair::kMaxSlots &&
+                   keys_pair::smem_bytes(pl.rows_total, d.ctx_len) <= kSmemTwoPerSm;
+    if (pl.keys_on_m) pl.smem_bytes = keys_pair::smem_bytes(pl.rows_total, d.ctx_len);
     return pl;
 }
 
 template <int NT>
-cudaError_t launch_nt(const SkipPlan& pl, const SkipParams& p, const CUtensorMap& mk, const CUtensorMap& mv, int bh,
+cudaError_t launch_nt(const SkipPlan& pl, const SkipParams& p, const CUtensorMap& mk, const CUtensorMap& mv,
+                      const CUtensorMap& mkn, const CUtensorMap& mvn, const keys_pair::Params& kp, int bh,
                       cudaStream_t stream) {
     static PerDeviceOnce attr_once;
     if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_skip_kernel<NT>, (int)kSmemMax); ea != cudaSuccess) return ea;
@@ -675,7 +693,7 @@ cudaError_t launch_nt(const SkipPlan& pl, const SkipParams& p, const CUtensorMap
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_skip_kernel<NT>, mk, mv, p);
+    return cudaLaunchKernelEx(&cfg, attend_skip_kernel<NT>, mk, mv, mkn, mvn, p, kp);
 }
 
 }  // namespace
@@ -692,8 +710,9 @@ bool attend_skip_supported(const ec_attn_desc& d, int n_active) {
 
 void attend_skip_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len) {
     const SkipPlan pl = make_skip_plan(d, n_active);
-    snprintf(buf, len, "attend_skip_kernel<%d> grid=(%d,%d) cluster=%d stages=%d smem=%u", pl.nt, pl.n_splits,
-             d.batch * d.n_kv_heads, pl.n_splits, pl.n_stages, pl.smem_bytes);
+    snprintf(buf, len, "attend_skip_kernel<%d> grid=(%d,%d) cluster=%d stages=%d smem=%u%s", pl.nt, pl.n_splits,
+             d.batch * d.n_kv_heads, pl.n_splits, pl.keys_on_m ? 1 : pl.n_stages, pl.smem_bytes,
+             pl.keys_on_m ? " keys_on_m" : "");
 }
 
 cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
@@ -701,9 +720,16 @@ cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const voi
     const SkipPlan pl = make_skip_plan(a.d, a.n_active);
     const int bh = a.d.batch * a.d.n_kv_heads;
     CUtensorMap map_k, map_v;
-    if (!make_cache_map(&map_k, a.k_cache, bh, a.d.ctx_len) || !make_cache_map(&map_v, a.v_cache, bh, a.d.ctx_len))
+    const int box = pl.keys_on_m ? keys_pair::BK : BN;
+    if (!make_cache_map(&map_k, a.k_cache, bh, a.d.ctx_len, box) || !make_cache_map(&map_v, a.v_cache, bh, a.d.ctx_len, box))
+        return cudaErrorInvalidValue;
+    CUtensorMap map_kn = map_k, map_vn = map_v;   // placeholders unless refreshing
+    if (k_new && (!make_fresh_map(&map_kn, k_new, a.d.batch, a.n_active, a.d.n_kv_heads, box) ||
+                  !make_fresh_map(&map_vn, v_new, a.d.batch, a.n_active, a.d.n_kv_heads, box)))
         return cudaErrorInvalidValue;
     SkipParams p{};
+    p.n_extra = pl.n_extra;
+    p.early_cache = (a.d.flags & EC_ATTN_CACHE_SETTLED) ? 1 : 0;
     p.q = static_cast<const __nv_bfloat16*>(a.q);
     p.k_new = static_cast<const __nv_bfloat16*>(k_new);
     p.v_new = static_cast<const __nv_bfloat16*>(v_new);
@@ -733,7 +759,12 @@ cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const voi
     p.off_xch = pl.off_xch;
     p.off_bar = pl.off_bar;
     p.scale_log2 = a.scale * kLog2e;
-    return pl.nt == 1 ? launch_nt<1>(pl, p, map_k, map_v, bh, stream) : launch_nt<2>(pl, p, map_k, map_v, bh, stream);
+    p.keys_on_m = pl.keys_on_m ? 1 : 0;
+    const keys_pair::Params kp{p.q, p.k_new, p.v_new, p.k_cache, p.v_cache, p.active_idx, p.out, p.dev_status, p.n_active,
+                               p.ctx_len, p.n_q_heads, p.n_kv_heads, p.group, (65536 + p.group - 1) / p.group,
+                               p.early_cache, p.scale_log2};
+    return pl.nt == 1 ? launch_nt<1>(pl, p, map_k, map_v, map_kn, map_vn, kp, bh, stream)
+                      : launch_nt<2>(pl, p, map_k, map_v, map_kn, map_vn, kp, bh, stream);
 }
 
 }  // namespace ec

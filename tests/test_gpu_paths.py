@@ -27,3 +27,19 @@ def test_first_keys_of_a_tile_all_refreshed(std, L):
     idx = np.concatenate([np.arange(i, i + 32) for i in range(0, min(L, 700), 256)])[None].astype(np.int32)
     w = syn.Workload(98, "stale", syn.BF16, 1, 8, 8, 128, 0, L, 1, 0, 64)
     _check(w, syn.attn_inputs(w, idx.shape[1], active_idx=idx, std_qk=std, std_v=0.5))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,n", [(5, 32, 32, 130, 1), (5, 32, 32, 300, 48), (20, 16, 8, 257, 20), (19, 8, 8, 128, 49),
+                                          (5, 32, 32, 700, 64), (5, 32, 32, 64, 33)])
+def test_many_heads_with_few_rows(B, Hq, Hkv, L, n):
+    """More kv heads than SMs, one CTA each with the keys on the M axis: 48 and 64 query slots, grouped queries, ragged
+    tiles, a context of a single tile that is half refreshed; with and without fresh rows, flat and peaky scores."""
+    import paper_2603_18489_b200 as ec
+
+    w = syn.Workload(99, "many_heads", syn.BF16, B, Hq, Hkv, 128, 0, L, 1, 0, 64)
+    assert "keys_on_m" in ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 128, syn.BF16), n, True, True)
+    idx = syn.arbitrary_active_idx(B, L, n, seed=19 * L + n)
+    for std in (0.5, 6.0):
+        t = syn.attn_inputs(w, n, active_idx=idx, std_qk=std, std_v=0.5)
+        _check(w, t)
+        _check(w, t, refresh=False)
