@@ -56,7 +56,7 @@ constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
 enum { B_FULL = 0, B_EMPTY = kSlots, B_SFULL = 2 * kSlots, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 2,
-       B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 1, B_COUNT = B_VERDICT + 1 };
+       B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 2, B_COUNT = B_VERDICT + 1 };
 
 // first pass: a row's sum may grow to this before the unit is done again with running maxima
 constexpr float kMaxSum = 1.152921504606846976e18f;   // 2^60
@@ -85,7 +85,8 @@ constexpr int kPartFloats = BM * (HD + 2);   // one row tile of one part
 __global__ void __launch_bounds__(kThreads, 1)
 attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kd,
-                    const __grid_constant__ CUtensorMap map_vd, const DenseParams p) {
+                    const __grid_constant__ CUtensorMap map_vd, const __grid_constant__ CUtensorMap map_o,
+                    const DenseParams p) {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
@@ -106,7 +107,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     const int unit = cut ? p.n_full + (lin - p.n_full) / p.split : lin;
     const int part = cut ? (lin - p.n_full) % p.split : 0;
     const int pair = unit % p.n_pairs, bh = unit / p.n_pairs;
-    const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
+    const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads, hk_kv = hk / p.kv_div;
     const int r_pair = pair * 2 * BM;
     const int n_tiles_q = (p.rows_total - r_pair > BM) ? 2 : 1;   // row tiles of this CTA that hold rows
     const int T_all = (p.ctx_len + BN - 1) / BN;
@@ -116,7 +117,13 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
     if (tid == 0) {
         prefetch_map(&map_k);
+        prefetch_map(&map_q);
         prefetch_map(&map_v);
+        if (p.copy) {
+            prefetch_map(&map_kd);
+            prefetch_map(&map_vd);
+        }
+        prefetch_map(&map_o);
         for (int i = 0; i < B_COUNT; ++i)
             mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 2) ? 256u : (p.copy && i >= B_EMPTY && i < B_EMPTY + kSlots) ? 2u : 1u);
         *abort_flag = 0;
@@ -137,12 +144,11 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     if (warp == 0) {
         // ================================ TMA producer ======================================
         if (lane == 0) {
-            const int hk_kv = hk / p.kv_div;
-            // Q first: [half][row][64 columns] per row tile; rows past n_active read as zero
-            prefetch_map(&map_q);
-            mbar_expect_tx(bar(B_QFULL), (uint32_t)n_tiles_q * TILE);
-            for (int t = 0; t < n_tiles_q; ++t)
-                tma_load_5d(base + OFF_Q + t * TILE, &map_q, 0, r_pair + t * BM, hk, 0, b, bar(B_QFULL));
+            // Q: [half][row][64 columns] per row tile; rows past n_active read as zero
+            auto load_q = [&](int t) {
+                mbar_expect_tx(bar(B_QFULL + t), TILE);
+                tma_load_5d(base + OFF_Q + t * TILE, &map_q, 0, r_pair + t * BM, hk, 0, b, bar(B_QFULL + t));
+            };
             for (int n = 0; n < 4 * T; ++n) {   // ring index: K_j = 2j, V_j = 2j + 1; from 2T on the second pass
                 if (n == 2 * T) {
                     mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
@@ -152,6 +158,8 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (u > 0) mbar_wait(bar(B_EMPTY + slot), (u - 1) & 1, abort_flag, p.dev_status);
                 mbar_expect_tx(bar(B_FULL + slot), TILE);
                 tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, (j0 + j) * BN, 0, hk_kv, b, bar(B_FULL + slot));
+                if (n == 0)   // behind the first K tile: the first scores need one row tile of Q
+                    for (int t = 0; t < n_tiles_q; ++t) load_q(t);
             }
         }
     } else if (warp == 1) {
@@ -168,7 +176,6 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
                 commit(bar(B_SFULL + t));
             };
-            mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
             int slot = 0;          // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...
             uint32_t phase = 0, p_phase = 0;
             auto advance = [&]() {
@@ -183,7 +190,11 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
                 mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
                 fence_after();
-                for (int t = 0; t < n_tiles_q; ++t) issue_s(t, slot);
+                for (int t = 0; t < n_tiles_q; ++t) {
+                    mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
+                    fence_after();
+                    issue_s(t, slot);
+                }
                 commit(bar(B_EMPTY + advance()));   // K_0 is free once both S(0) have run
                 for (int j = 0; j < T; ++j, p_phase ^= 1) {
                     mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
@@ -222,7 +233,6 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const uint32_t tm_s = tmem + lane_addr + TM_S + t * 128;
         const uint32_t tm_o = tmem + lane_addr + TM_O + t * 128;
-        const int r = r_pair + t * BM + row;
         float* xch_mine = xch + (t * 2 + h) * BM + row;        // exchanged with the partner thread of the row
         const float* xch_other = xch + (t * 2 + (1 - h)) * BM + row;
         const int pair_bar = 1 + t * 4 + quarter;              // named barrier of the two warps that share these rows
@@ -373,28 +383,34 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             *xch_mine = l_run;
             named_barrier(pair_bar, 64);
             const float l_row = l_run + *xch_other;   // both halves of a row carry the same reference maximum
-            const bool valid = r < p.rows_total;
-            const int i = valid ? r / p.group : 0, jh = valid ? r % p.group : 0;
-            __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + jh) * HD + h * 64;
             if (!cut) {
-                // whole unit: normalise and store this thread's 64 columns
+                // Whole unit: the normalised row goes to shared memory, over the row tile's Q (its last scores are long
+                // formed), and the tile leaves by TMA (rows past n_active are not written).  Rolled: the code of an
+                // epilogue runs once a CTA and is fetched at about its own length in time; unrolled, with 16-byte stores
+                // to global memory, it took 3.5 us.
                 const float inv = 1.f / l_row;
-#pragma unroll
+                unsigned char* qrow = gbase + OFF_Q + t * TILE + h * SUB + (row >> 3) * 1024 + (row & 7) * 128;
+#pragma unroll 1
                 for (int c = 0; c < 2; ++c) {
                     uint32_t o[32];
                     ld32(tm_o + h * 64 + c * 32, o);
                     wait_ld();
-                    if (valid && !*abort_flag) {   // a CTA whose wait gave up stores nothing
 #pragma unroll
-                        for (int v4 = 0; v4 < 4; ++v4) {
-                            uint4 w;
-                            w.x = pack_bf16x2(__uint_as_float(o[v4 * 8 + 0]) * inv, __uint_as_float(o[v4 * 8 + 1]) * inv);
-                            w.y = pack_bf16x2(__uint_as_float(o[v4 * 8 + 2]) * inv, __uint_as_float(o[v4 * 8 + 3]) * inv);
-                            w.z = pack_bf16x2(__uint_as_float(o[v4 * 8 + 4]) * inv, __uint_as_float(o[v4 * 8 + 5]) * inv);
-                            w.w = pack_bf16x2(__uint_as_float(o[v4 * 8 + 6]) * inv, __uint_as_float(o[v4 * 8 + 7]) * inv);
-                            *reinterpret_cast<uint4*>(dst + c * 32 + v4 * 8) = w;
-                        }
+                    for (int v4 = 0; v4 < 4; ++v4) {
+                        uint4 w;
+                        w.x = pack_bf16x2(__uint_as_float(o[v4 * 8 + 0]) * inv, __uint_as_float(o[v4 * 8 + 1]) * inv);
+                        w.y = pack_bf16x2(__uint_as_float(o[v4 * 8 + 2]) * inv, __uint_as_float(o[v4 * 8 + 3]) * inv);
+                        w.z = pack_bf16x2(__uint_as_float(o[v4 * 8 + 4]) * inv, __uint_as_float(o[v4 * 8 + 5]) * inv);
+                        w.w = pack_bf16x2(__uint_as_float(o[v4 * 8 + 6]) * inv, __uint_as_float(o[v4 * 8 + 7]) * inv);
+                        *reinterpret_cast<uint4*>(qrow + (((c * 4 + v4) ^ (row & 7)) << 4)) = w;
                     }
+                }
+                fence_async_smem();
+                named_barrier(10 + t, 256);
+                if ((ws & 7) == 0 && lane == 0 && !*abort_flag) {   // a CTA whose wait gave up stores nothing
+                    tma_store_5d(&map_o, base + OFF_Q + t * TILE, 0, r_pair + t * BM, hk, 0, b);
+                    bulk_commit();
+                    bulk_wait_read();
                 }
             } else {
                 // part of a cut unit: the un-normalised row (relative to m_used), m and l go to the workspace; the
@@ -402,7 +418,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 // bound by what a single SM can pull out of L2: 11 us per extra part)
                 const int cu = unit - p.n_full;
                 float* mine = p.part + ((size_t)(cu * p.split + part) * 2 + t) * kPartFloats;
-#pragma unroll
+#pragma unroll 1
                 for (int c = 0; c < 2; ++c) {
                     uint32_t o[32];
                     ld32(tm_o + h * 64 + c * 32, o);
@@ -428,7 +444,6 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         // nothing.  The units of a kv head (its query heads' row-tile pairs) take turns by tile.  Nobody reads the cache
         // in this launch.  (A warp that copied its share of the rows through registers took longer than the six key
         // tiles of a unit at L = 768.)
-        const int hk_kv = hk / p.kv_div;
         const int n_share = p.n_pairs * p.kv_div, mine = (hk % p.kv_div) * p.n_pairs + pair;
         int slot = 0;
         uint32_t phase = 0;
@@ -447,7 +462,6 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             mbar_arrive(bar(B_EMPTY + slot));
             if (++slot == kSlots) slot = 0, phase ^= 1;
         }
-        bulk_wait();
     }
 
     __syncthreads();
@@ -634,8 +648,8 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
         if (!a.workspace || a.workspace_bytes < attend_dense_workspace_bytes(a.d, a.n_active)) return cudaErrorInvalidValue;
         p.part = static_cast<float*>(a.workspace);
     }
-    CUtensorMap map_q;
-    {
+    CUtensorMap map_q, map_o;
+    for (int i = 0; i < 2; ++i) {   // q and out have the same layout
         EncodeTiledFn fn = encode_fn();
         if (!fn) return cudaErrorInvalidValue;
         const cuuint64_t dims[5] = {64, (cuuint64_t)a.n_active, (cuuint64_t)a.d.n_q_heads, 2, (cuuint64_t)a.d.batch};
@@ -643,7 +657,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
                                        (cuuint64_t)a.n_active * a.d.n_q_heads * HD * 2};
         const cuuint32_t box[5] = {64, (cuuint32_t)BM, 1, 2, 1};
         const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-        if (fn(&map_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.q), dims, strides, box, estr,
+        if (fn(i ? &map_o : &map_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, i ? a.out : const_cast<void*>(a.q), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -660,7 +674,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (const cudaError_t el = cudaLaunchKernelEx(&cfg, attend_dense_kernel, map_k, map_v, map_q, map_kd, map_vd, p); el != cudaSuccess) return el;
+    if (const cudaError_t el = cudaLaunchKernelEx(&cfg, attend_dense_kernel, map_k, map_v, map_q, map_kd, map_vd, map_o, p); el != cudaSuccess) return el;
     if (pl.split == 1) return cudaSuccess;
     CombineParams c{p.part, p.out, pl.n_pairs, pl.n_full, pl.split, a.n_active, a.d.n_q_heads, a.n_active};
     cfg.gridDim = dim3((pl.units - pl.n_full) * 8, 1, 1);   // (cut unit, row tile, 32-row group)
