@@ -16,13 +16,13 @@
 //               Order per key tile j:  P V_0(j), S_0(j+1), P V_1(j), S_1(j+1): the pipe executes in order,
 //               so S_t(j+1) cannot overwrite P_t(j) before P V_t(j) has read it;
 //   warps 2..17 softmax, four warpgroups: (row tile 0 / 1) x (keys 0..63 / 64..127 of the tile).  A query row
-//               (= TMEM lane) is shared by two threads in warps that own the same lanes; they exchange
-//               their half-row maxima through shared memory (a 64-thread named barrier), then each does
+//               (= TMEM lane) is shared by two threads in warps that own the same lanes; each does
 //               tcgen05.ld of its 64 scores, exp2 with the scale folded in (packed fp32x2 FMA), its share of
-//               the row sum, P rounded to bf16 and stored back with tcgen05.st; the O accumulator is only
-//               rescaled when a row maximum grows by more than 2^8 (the stale maximum stays the reference
-//               otherwise).  Halving the per-thread row shortens the softmax that sits between two uses of
-//               the tensor pipe for the same row tile.
+//               the row sum, P rounded to bf16 and stored back with tcgen05.st.  There is no running maximum:
+//               a row's reference is its largest score among the first eight keys, and only if a row sum
+//               leaves the range that fp32 and bf16 share is the unit done again, with running maxima.  Halving
+//               the per-thread row shortens the softmax that sits between two uses of the tensor pipe for the
+//               same row tile.
 //   warp 18     recompute steps only: every cache row is overwritten by the fresh row of the same position, so the
 //               launch reads K/V straight from the token-major k_new / v_new (only the tensor map's strides
 //               differ) and this warp stores landed tiles into the cache meanwhile: no separate refresh pass.
@@ -52,11 +52,12 @@ constexpr uint32_t OFF_BAR = OFF_RING + kSlots * TILE;   // 224 KB
 constexpr uint32_t OFF_XCH = OFF_BAR + 256;               // [2 tiles][2 halves][128 rows] floats
 constexpr uint32_t SMEM_BYTES = 232448;                   // all of a CTA's 227 KB; the rest is alignment slack
 constexpr uint32_t SMEM_NEEDED = OFF_XCH + 2 * 2 * BM * 4;
+constexpr uint32_t PART = BM * HD * 4;                   // un-normalised rows of a row tile (cut units), over the ring
 constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
 enum { B_FULL = 0, B_EMPTY = kSlots, B_SFULL = 2 * kSlots, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 2,
-       B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 2, B_COUNT = B_VERDICT + 1 };
+       B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 2, B_COPIED = B_VERDICT + 1, B_COUNT = B_COPIED + 1 };
 
 // first pass: a row's sum may grow to this before the unit is done again with running maxima
 constexpr float kMaxSum = 1.152921504606846976e18f;   // 2^60
@@ -74,14 +75,20 @@ struct DenseParams {
     // those of the real kv head h / kv_div, of which there are n_kv_real.  kv_div = 1 otherwise.
     int kv_div, n_kv_real;
     float scale_log2;
-    // Launch order = unit order (row-tile pair fastest, then head).  The first n_full units are whole; each later
-    // unit (the last, partial wave of the launch) is cut along the keys into `split` CTAs that leave un-normalised
-    // partials in the workspace for combine_cut_units_kernel.  split = 1: no cuts.
+    // Unit order = row-tile pair fastest, then head.  The first n_full units are whole; each later one (what would be
+    // the last, partial wave of the launch) is cut along the keys into `split` CTAs, a cluster of the second launch.
     int n_pairs, n_full, split;
-    float* part;      // [cut unit][part][row tile][128 rows x 128 floats, then m[128], then l[128]]
+    int wait_first;   // second launch: 1 when there is no first one, see below
 };
-constexpr int kPartFloats = BM * (HD + 2);   // one row tile of one part
 
+// kCut: the launch of the cut units.  A cluster leaves its un-normalised rows, m and l in shared memory, each CTA merges a
+// share of them out of its peers'.  This launch follows the one of the whole units with programmatic serialisation and
+// does NOT wait for it: every CTA of the first launch triggers after its own dependency wait, so whatever wrote q, k_new
+// and v_new is complete by then, and the two launches write different rows.  It waits at its end instead, so that whoever
+// waits for this launch has waited for both.  Measured, layers back to back (a third launch that combined partials from
+// global memory -> merged here): 86.4 -> 78.5 us at 2 x 1531 with 28 heads, 237.5 -> 233.1 at 4096 with 28 heads,
+// 58.0 -> 55.7 at 2048 with 19.
+template <bool kCut>
 __global__ void __launch_bounds__(kThreads, 1)
 attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kd,
@@ -103,15 +110,14 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int lin = blockIdx.x;
-    const bool cut = lin >= p.n_full;
-    const int unit = cut ? p.n_full + (lin - p.n_full) / p.split : lin;
-    const int part = cut ? (lin - p.n_full) % p.split : 0;
+    const int unit = kCut ? p.n_full + lin / p.split : lin;
+    const int part = kCut ? lin % p.split : 0;
     const int pair = unit % p.n_pairs, bh = unit / p.n_pairs;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads, hk_kv = hk / p.kv_div;
     const int r_pair = pair * 2 * BM;
     const int n_tiles_q = (p.rows_total - r_pair > BM) ? 2 : 1;   // row tiles of this CTA that hold rows
     const int T_all = (p.ctx_len + BN - 1) / BN;
-    const int tiles_per_part = cut ? (T_all + p.split - 1) / p.split : T_all;
+    const int tiles_per_part = kCut ? (T_all + p.split - 1) / p.split : T_all;
     const int j0 = part * tiles_per_part;                        // first key tile of this CTA
     const int T = min(T_all, j0 + tiles_per_part) - j0;          // >= 1 by construction of the plan
 
@@ -138,7 +144,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
-    pdl_wait();   // the previous kernel of the stream has completed; global memory may be touched
+    if (!kCut || p.wait_first) pdl_wait();   // the previous kernel of the stream has completed; global memory may be touched
     pdl_launch_dependents();
 
     if (warp == 0) {
@@ -383,7 +389,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             *xch_mine = l_run;
             named_barrier(pair_bar, 64);
             const float l_row = l_run + *xch_other;   // both halves of a row carry the same reference maximum
-            if (!cut) {
+            if constexpr (!kCut) {
                 // Whole unit: the normalised row goes to shared memory, over the row tile's Q (its last scores are long
                 // formed), and the tile leaves by TMA (rows past n_active are not written).  Rolled: the code of an
                 // epilogue runs once a CTA and is fetched at about its own length in time; unrolled, with 16-byte stores
@@ -413,27 +419,22 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     bulk_wait_read();
                 }
             } else {
-                // part of a cut unit: the un-normalised row (relative to m_used), m and l go to the workspace; the
-                // combine kernel that follows in the stream merges the parts (one CTA combining a unit on its own is
-                // bound by what a single SM can pull out of L2: 11 us per extra part)
-                const int cu = unit - p.n_full;
-                float* mine = p.part + ((size_t)(cu * p.split + part) * 2 + t) * kPartFloats;
+                // part of a cut unit: the un-normalised row (relative to m_used), m and l stay in shared memory, over the
+                // ring and Q: both row tiles' products and the copy warp's stores have to be through
+                for (int tt = 0; tt < n_tiles_q; ++tt) mbar_wait(bar(B_PVDONE + tt), (done - 1) & 1, abort_flag, p.dev_status);
+                if (p.copy) mbar_wait(bar(B_COPIED), 0, abort_flag, p.dev_status);
+                unsigned char* prow = gbase + OFF_RING + t * PART + row * (HD * 4);
 #pragma unroll 1
                 for (int c = 0; c < 2; ++c) {
                     uint32_t o[32];
                     ld32(tm_o + h * 64 + c * 32, o);
                     wait_ld();
-                    if (!*abort_flag) {
 #pragma unroll
-                        for (int v4 = 0; v4 < 8; ++v4)
-                            *reinterpret_cast<uint4*>(mine + row * HD + h * 64 + c * 32 + v4 * 4) =
-                                make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
-                    }
+                    for (int v4 = 0; v4 < 8; ++v4)   // (16-byte pieces swizzled by row: 32 lanes are 32 rows)
+                        *reinterpret_cast<uint4*>(prow + (((h * 16 + c * 8 + v4) ^ (row & 31)) << 4)) =
+                            make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
                 }
-                if (h == 0 && !*abort_flag) {
-                    mine[BM * HD + row] = m_used;
-                    mine[BM * HD + BM + row] = l_row;
-                }
+                if (h == 0) *reinterpret_cast<float2*>(gbase + OFF_Q + (t * BM + row) * 8) = make_float2(m_used, l_row);
             }
         }
         fence_before();
@@ -462,6 +463,67 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             mbar_arrive(bar(B_EMPTY + slot));
             if (++slot == kSlots) slot = 0, phase ^= 1;
         }
+        mbar_arrive(bar(B_COPIED));
+    }
+
+    if constexpr (kCut) {
+        // ---- merge: this CTA's share of the cluster's rows, w_s = 2^(m_s - M) / sum_s 2^(m_s - M) l_s ----
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();           // the partials of all CTAs are complete
+        float* weight = reinterpret_cast<float*>(gbase + OFF_Q + 2 * BM * 8);   // [row of the share][8]
+        const int share = n_tiles_q * BM / p.split, row0 = part * share;       // split is 2, 4 or 8
+        for (int i = tid; i < share; i += kThreads) {
+            float mm[8], ll[8], M = -INFINITY, L = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                ld_peer_v2(map_to_cta(base + OFF_Q + (row0 + i) * 8, min(q, p.split - 1)), mm[q], ll[q]);
+                if (q >= p.split) mm[q] = -INFINITY;
+                M = fmaxf(M, mm[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                mm[q] = fast_exp2(mm[q] - M);
+                L = fmaf(mm[q], ll[q], L);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) weight[i * 8 + q] = mm[q] / L;
+        }
+        __syncthreads();
+        if (!*abort_flag) {   // a CTA whose wait gave up stores nothing
+            for (int i0 = warp * 4; i0 < share; i0 += kThreads / 32 * 4) {   // a warp takes four rows, a lane four columns
+                float4 acc[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                for (int q = 0; q < p.split; ++q) {
+                    float x[4][4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int rr = row0 + i0 + k;
+                        ld_peer_v4(map_to_cta(base + OFF_RING + rr * (HD * 4) + ((lane ^ (rr & 31)) << 4), q), x[k]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float w = weight[(i0 + k) * 8 + q];
+                        acc[k].x = fmaf(w, x[k][0], acc[k].x);
+                        acc[k].y = fmaf(w, x[k][1], acc[k].y);
+                        acc[k].z = fmaf(w, x[k][2], acc[k].z);
+                        acc[k].w = fmaf(w, x[k][3], acc[k].w);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int r = r_pair + row0 + i0 + k;
+                    if (r < p.rows_total)
+                        *reinterpret_cast<uint2*>(p.out + (((long long)b * p.n_active + r) * p.n_q_heads + hk) * HD + lane * 4) =
+                            make_uint2(pack_bf16x2(acc[k].x, acc[k].y), pack_bf16x2(acc[k].z, acc[k].w));
+                }
+            }
+        }
+        __syncwarp();
+        cluster_arrive();         // no CTA leaves while a peer may still read its partial
+        cluster_wait();
     }
 
     __syncthreads();
@@ -469,68 +531,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TM_COLS) : "memory");
     }
-}
-
-// Merges the parts of the cut units: CTA = 32 rows of one row tile of one cut unit, thread = 16 columns of a row.
-// With M the largest reference maximum of the row's parts and w_q = 2^(m_q - M):  out = sum_q w_q O_q / sum_q w_q l_q.
-struct CombineParams {
-    const float* part;
-    __nv_bfloat16* out;
-    int n_pairs, n_full, split, n_active, n_q_heads, rows_total;
-};
-__global__ void __launch_bounds__(256) combine_cut_units_kernel(const CombineParams p) {
-    pdl_wait();   // the partials of the attention launch are complete
-    pdl_launch_dependents();
-    const int cu = blockIdx.x >> 3, t = (blockIdx.x >> 2) & 1, row = (blockIdx.x & 3) * 32 + (threadIdx.x >> 3);
-    const int c0 = (threadIdx.x & 7) * 16;
-    const int unit = p.n_full + cu;
-    const int pair = unit % p.n_pairs, bh = unit / p.n_pairs;
-    const int b = bh / p.n_q_heads, hq = bh % p.n_q_heads;
-    const int r = pair * 2 * BM + t * BM + row;
-    if (r >= p.rows_total) return;
-    float w[8], M = -INFINITY, L = 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        w[q] = -INFINITY;
-        if (q < p.split) {
-            w[q] = __ldcg(p.part + ((size_t)(cu * p.split + q) * 2 + t) * kPartFloats + BM * HD + row);
-            M = fmaxf(M, w[q]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        if (q < p.split) {
-            w[q] = fast_exp2(w[q] - M);
-            L = fmaf(w[q], __ldcg(p.part + ((size_t)(cu * p.split + q) * 2 + t) * kPartFloats + BM * HD + BM + row), L);
-        }
-    }
-    float acc[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        if (q < p.split) {
-            const float4* src = reinterpret_cast<const float4*>(
-                p.part + ((size_t)(cu * p.split + q) * 2 + t) * kPartFloats + row * HD + c0);
-#pragma unroll
-            for (int v4 = 0; v4 < 4; ++v4) {
-                const float4 f = __ldcg(src + v4);
-                acc[v4 * 4 + 0] = fmaf(w[q], f.x, acc[v4 * 4 + 0]);
-                acc[v4 * 4 + 1] = fmaf(w[q], f.y, acc[v4 * 4 + 1]);
-                acc[v4 * 4 + 2] = fmaf(w[q], f.z, acc[v4 * 4 + 2]);
-                acc[v4 * 4 + 3] = fmaf(w[q], f.w, acc[v4 * 4 + 3]);
-            }
-        }
-    }
-    const float inv = 1.f / L;
-    __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + r) * p.n_q_heads + hq) * HD + c0;
-    uint4 o0, o1;
-    o0.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);   o0.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-    o0.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);   o0.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-    o1.x = pack_bf16x2(acc[8] * inv, acc[9] * inv);   o1.y = pack_bf16x2(acc[10] * inv, acc[11] * inv);
-    o1.z = pack_bf16x2(acc[12] * inv, acc[13] * inv); o1.w = pack_bf16x2(acc[14] * inv, acc[15] * inv);
-    *reinterpret_cast<uint4*>(dst) = o0;
-    *reinterpret_cast<uint4*>(dst + 8) = o1;
+    if (kCut && warp == 0) pdl_wait();
 }
 
 // ---- host side ---------------------------------------------------------------------------
@@ -557,12 +558,11 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int batch, int n_kv_heads, i
 // How the launch is cut.  Units = (sequence, query head, row-tile pair); a unit walks over all T key tiles.  The
 // hardware deals the CTAs to the SMs in launch order, so the last units form a partial wave: `tail` units on `sms` SMs.
 // Cutting each of them along the keys into s CTAs (s = 2, 4 or 8, at least four key tiles each) fills that wave:
-// cost in key-tile times, with two tiles' worth of fixed cost per CTA, one more for writing the partials, and four
-// for the combine launch that follows:
-//     waves_full * (T + 2) + ceil(tail * s / sms) * (ceil(T / s) + 3) + 4
+// cost in key-tile times, with two tiles' worth of fixed cost per CTA, one more for the merge, and one for the launch:
+//     waves_full * (T + 2) + ceil(tail * s / sms) * (ceil(T / s) + 3) + 1
 // s = 1 (no cut) unless a cut saves at least 3 %.
 struct DensePlan {
-    int n_pairs, units, n_full, split, n_ctas;
+    int n_pairs, units, n_full, split;
 };
 DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
     DensePlan pl;
@@ -578,7 +578,7 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
         const long long need = best - best * 3 / 100;
         for (int s = 2; s <= 8; s *= 2) {
             if (T / s < 4) break;
-            const long long cost = waves_full * (T + 2) + ((tail * s + sms - 1) / sms) * ((T + s - 1) / s + 3) + 4;
+            const long long cost = waves_full * (T + 2) + ((tail * s + sms - 1) / sms) * ((T + s - 1) / s + 3) + 1;
             if (cost < best && cost <= need) {
                 best = cost;
                 pl.split = s;
@@ -586,7 +586,6 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
         }
         if (pl.split > 1) pl.n_full = pl.units - (int)tail;
     }
-    pl.n_ctas = pl.n_full + (pl.units - pl.n_full) * pl.split;
     return pl;
 }
 
@@ -601,13 +600,6 @@ bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
     const long long bh = (long long)d.batch * d.n_q_heads;
     if (pairs * bh > 0x3fffffffLL) return false;
     return pairs * bh >= sm_count() / 4;
-}
-
-size_t attend_dense_workspace_bytes(const ec_attn_desc& d, int n_active) {
-    if (!attend_dense_supported(d, n_active)) return 0;
-    const DensePlan pl = make_dense_plan(d, n_active);
-    if (pl.split == 1) return 0;
-    return (size_t)(pl.units - pl.n_full) * pl.split * 2 * kPartFloats * sizeof(float);
 }
 
 void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len) {
@@ -643,11 +635,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     p.n_pairs = pl.n_pairs;
     p.n_full = pl.n_full;
     p.split = pl.split;
-    p.part = nullptr;
-    if (pl.split > 1) {
-        if (!a.workspace || a.workspace_bytes < attend_dense_workspace_bytes(a.d, a.n_active)) return cudaErrorInvalidValue;
-        p.part = static_cast<float*>(a.workspace);
-    }
+    p.wait_first = pl.n_full == 0;
     CUtensorMap map_q, map_o;
     for (int i = 0; i < 2; ++i) {   // q and out have the same layout
         EncodeTiledFn fn = encode_fn();
@@ -662,25 +650,32 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    static PerDeviceOnce attr_once;
-    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_dense_kernel, (int)SMEM_BYTES); ea != cudaSuccess) return ea;
+    static PerDeviceOnce once_whole, once_cut;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(pl.n_ctas, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = pl.split;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (const cudaError_t el = cudaLaunchKernelEx(&cfg, attend_dense_kernel, map_k, map_v, map_q, map_kd, map_vd, map_o, p); el != cudaSuccess) return el;
-    if (pl.split == 1) return cudaSuccess;
-    CombineParams c{p.part, p.out, pl.n_pairs, pl.n_full, pl.split, a.n_active, a.d.n_q_heads, a.n_active};
-    cfg.gridDim = dim3((pl.units - pl.n_full) * 8, 1, 1);   // (cut unit, row tile, 32-row group)
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, combine_cut_units_kernel, c);
+    if (pl.n_full > 0) {
+        if (const cudaError_t e = ensure_dynamic_smem(once_whole, attend_dense_kernel<false>, (int)SMEM_BYTES); e != cudaSuccess) return e;
+        cfg.gridDim = dim3(pl.n_full, 1, 1);
+        cfg.numAttrs = 1;
+        if (const cudaError_t e = cudaLaunchKernelEx(&cfg, attend_dense_kernel<false>, map_k, map_v, map_q, map_kd, map_vd, map_o, p);
+            e != cudaSuccess)
+            return e;
+    }
+    if (pl.n_full == pl.units) return cudaSuccess;
+    if (const cudaError_t e = ensure_dynamic_smem(once_cut, attend_dense_kernel<true>, (int)SMEM_BYTES); e != cudaSuccess) return e;
+    cfg.gridDim = dim3((pl.units - pl.n_full) * pl.split, 1, 1);
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, attend_dense_kernel<true>, map_k, map_v, map_q, map_kd, map_vd, map_o, p);
 }
 
 }  // namespace ec

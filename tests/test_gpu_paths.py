@@ -43,3 +43,17 @@ def test_many_heads_with_few_rows(B, Hq, Hkv, L, n):
         t = syn.attn_inputs(w, n, active_idx=idx, std_qk=std, std_v=0.5)
         _check(w, t)
         _check(w, t, refresh=False)
+
+
+@pytest.mark.parametrize("Hq,Hkv,L,cut", [(10, 5, 1100, "whole_units=0 cut_units=50x2"), (33, 33, 1100, "whole_units=148 cut_units=17x2"),
+                                          (5, 5, 2500, "whole_units=0 cut_units=50x2")])
+def test_cut_units_alone_and_with_a_single_row_tile(Hq, Hkv, L, cut):
+    """Recompute steps with no whole unit beside the cut ones, and with units of one row tile among the cut ones;
+    moderate scores, and peaky ones for which some parts of a unit run their second pass and others do not."""
+    import paper_2603_18489_b200 as ec
+
+    w = syn.Workload(100, "cut", syn.BF16, 1, Hq, Hkv, 128, 0, L, 1, 0, 64)
+    assert cut in ec.ec_attend_kernel_name(ec.make_desc(1, L, Hq, Hkv, 128, syn.BF16), L, True, False)
+    rows = sorted(set(np.random.Generator(np.random.PCG64(L)).choice(L, 40, replace=False).tolist() + [0, L - 1]))
+    for std in (0.5, 8.0):
+        _check(w, syn.attn_inputs(w, L, std_qk=std, std_v=0.5, salt=Hq), row_sel=rows)
