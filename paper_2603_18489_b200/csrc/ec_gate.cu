@@ -11,7 +11,7 @@
 //           (max, S, T) with S = sum 2^d, T = sum 2^d * d, d = x*log2(e) - base: one ex2.approx per element
 //           and one packed fp32x2 FMA, add and FMA per pair of elements.  The base follows the maximum lazily: it moves, and S and T
 //           are rescaled (S' = 2^dl S, T' = 2^dl (T + dl S), dl = old base - new base), only when a value
-//           exceeds it by more than 2^64, so the common path has no data-dependent branch.  Logits are
+//           exceeds it by more than 2^64 (looked at once per pair of bf16 vectors), so the common path has one branch.  Logits are
 //           clamped from below at -1e38 (packed bf16 max on the raw words), which keeps d finite:
 //           -inf and finfo.min-style masks get probability 0 without a per-element special case;
 //   argmax: the thread remembers the vector that raised its maximum; after the warp's maximum is
@@ -25,11 +25,12 @@
 //           than 32 splits, use two ticket levels instead (last CTA of a row, then last row of the sequence).
 // The entropy identity used: with p_j = 2^{d_j} / S,  -sum p_j ln p_j = ln S - ln2 * T / S
 // for any common base, so no partial ever needs the true row maximum.
-// What bounds it: at [256, 126464] bf16 (17.9 us, 10 of them at the copy rate) about 5 us of launch, ramp, reduction,
-// tickets and the finishing CTA, and 2.5 us of arithmetic that the stream does not hide (15.4 us without any); at
-// [32, 126464] (7.0 us) the fixed part alone.  Also timed at [256, 126464]: twelve vectors ahead through asynchronous
-// copies 17.9 (fp32 26.6 against 24.2), two batches of four in registers 18.6, 3 to 21 CTAs a row 19.5 to 38; a ring of
-// bulk copies with a producer warp took 19.7, and 7.4 at [32, 126464].
+// What bounds it: from about 100 rows on the chain of a thread's vectors (clamps, maximum, exponentials, sums): 31 a
+// thread at [256, 126464] bf16 take 16.9 us, 21 at 192 rows 13.9; the same bytes as fp32 13.7.  (About 3 us are launch,
+// ramp, reduction, ticket and the finishing CTA, 10 the copy rate.)  At [32, 126464] (7.1 us) it is the fixed part.  Also
+// timed at [256, 126464]: twelve vectors ahead through asynchronous copies 17.9 (fp32 26.6 against 24.2), two batches of
+// four in registers 18.6, 3 to 21 CTAs a row 19.5 to 38, five CTAs per SM of 48 registers 20.4, sums of their own for the
+// second vector of a pair 17.0; a ring of bulk copies with a producer warp 19.7, and 7.4 at [32, 126464].
 // The kernel is launched with programmatic stream serialisation, touches global memory only after
 // griddepcontrol.wait and waits for nothing else.
 #include "ec_common.cuh"
@@ -121,6 +122,7 @@ struct Loader<__nv_bfloat16> {
     static __device__ __forceinline__ unsigned int max_word(const uint4& u) {
         return max_bf16x2(max_bf16x2(u.x, u.y), max_bf16x2(u.z, u.w));
     }
+    static __device__ __forceinline__ unsigned int max_words(unsigned int a, unsigned int b) { return max_bf16x2(a, b); }
     static __device__ __forceinline__ float word_max(unsigned int w) {
         return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
     }
@@ -154,6 +156,9 @@ struct Loader<float> {
     static __device__ __forceinline__ unsigned int max_word(const uint4& u) {
         return __float_as_uint(fmaxf(fmaxf(__uint_as_float(u.x), __uint_as_float(u.y)),
                                      fmaxf(__uint_as_float(u.z), __uint_as_float(u.w))));
+    }
+    static __device__ __forceinline__ unsigned int max_words(unsigned int a, unsigned int b) {
+        return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
     }
     static __device__ __forceinline__ float word_max(unsigned int w) { return __uint_as_float(w); }
     static __device__ __forceinline__ void widen(const uint4& u, float (&x)[4]) {
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
     // running state: maximum, exponent base, and S, T as two packed lanes each
     float m = -INFINITY, base = base_of(-INFINITY);
     f32x2 S2 = pack2(0.f, 0.f), T2 = pack2(0.f, 0.f);
-    int mat = -1;               // the vector that raised the maximum last
+    int mat = -1;               // the vector (the first of the pair) that raised the maximum last
     const f32x2 kL2 = pack2(kLog2e, kLog2e);
     auto rebase_if_needed = [&](float vmax) {
         if (fmaf(vmax, kLog2e, -base) > kRebase) {   // rare
@@ -275,12 +280,7 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
             base = nb;
         }
     };
-    auto consume = [&](uint4 v, int i) {
-        L::clamp(v);
-        const float vmax = L::word_max(L::max_word(v));
-        rebase_if_needed(vmax);
-        mat = vmax > m ? i : mat;   // strictly greater: the first vector of a tie survives
-        m = fmaxf(m, vmax);
+    auto add = [&](const uint4& v) {
         const f32x2 nb2 = pack2(-base, -base);
         f32x2 x2[EPV / 2];
         L::widen2(v, x2);
@@ -294,17 +294,47 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
             T2 = fma2(e2, d2, T2);
         }
     };
+    auto raise = [&](float vmax, int i) {
+        rebase_if_needed(vmax);
+        mat = vmax > m ? i : mat;   // strictly greater: the first vectors of a tie survive
+        m = fmaxf(m, vmax);
+    };
+    // bf16: two vectors behind one look at the maximum, which is a branch that the exponentials of one vector and the
+    // clamps and maxima of the next cannot cross ([256, 126464] 17.6 -> 16.9 us); fp32 waits for memory and for the
+    // second of two vectors the longer (22.6 -> 23.2)
+    constexpr bool kPairs = EPV == 8;
+    auto consume2 = [&](uint4 v, uint4 w, int i) {   // vectors i and i + 1
+        L::clamp(v);
+        L::clamp(w);
+        raise(L::word_max(L::max_words(L::max_word(v), L::max_word(w))), i);
+        add(v);
+        add(w);
+    };
+    auto consume = [&](uint4 v, int i) {             // (pairs: the last vector of an odd number)
+        L::clamp(v);
+        raise(L::word_max(L::max_word(v)), i);
+        add(v);
+    };
     int i0 = 0;
     for (; i0 + kInFlight <= n_mine; i0 += kInFlight) {
 #pragma unroll
-        for (int r = 0; r < kInFlight; ++r) {
-            consume(raw[r], i0 + r);
+        for (int r = 0; r < kInFlight; r += 2) {
+            if (kPairs) consume2(raw[r], raw[r + 1], i0 + r);
+            else consume(raw[r], i0 + r);
             fetch(i0 + r + kInFlight, raw[r]);
+            if (!kPairs) consume(raw[r + 1], i0 + r + 1);
+            fetch(i0 + r + 1 + kInFlight, raw[r + 1]);
         }
     }
 #pragma unroll
-    for (int r = 0; r < kInFlight; ++r)
-        if (i0 + r < n_mine) consume(raw[r], i0 + r);
+    for (int r = 0; r < kInFlight; r += 2) {
+        if (kPairs && i0 + r + 1 < n_mine) {
+            consume2(raw[r], raw[r + 1], i0 + r);
+        } else {
+            if (i0 + r < n_mine) consume(raw[r], i0 + r);
+            if (!kPairs && i0 + r + 1 < n_mine) consume(raw[r + 1], i0 + r + 1);
+        }
+    }
     int tail_col = -1;
     {   // the ragged end of the chunk: fewer than EPV columns, one element per thread
         const int col = c0 + n_vec * EPV + tid;
@@ -324,21 +354,29 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
     }
 
     // ---- warp maximum; the threads that attained it find its first column in the vector that raised it --------
-    // (every thread asks again for that vector: an L2 hit, in flight during the reduction)
-    uint4 again = make_uint4(0u, 0u, 0u, 0u);
-    if (mat >= 0) again = __ldg(reinterpret_cast<const uint4*>(mine + (long long)mat * kVStride));
+    // (every thread asks again for that vector or pair: an L2 hit, in flight during the reduction)
+    constexpr int kAgain = kPairs ? 2 : 1;
+    uint4 again[kAgain];
+    if (mat >= 0) {
+#pragma unroll
+        for (int k = 0; k < kAgain; ++k)
+            again[k] = __ldg(reinterpret_cast<const uint4*>(mine + (long long)min(mat + k, n_mine - 1) * kVStride));
+    }
     const float M = tc::redux_max(m);
     int idx = 0x7fffffff;
     if (m == M) {
         if (tail_col >= 0) {
             idx = tail_col;
         } else if (mat >= 0) {
-            float x[EPV];
-            L::clamp(again);
-            L::widen(again, x);
 #pragma unroll
-            for (int e = EPV - 1; e >= 0; --e)   // descending: the smallest column survives
-                if (x[e] == M) idx = c0 + mat * kVStride + tid * EPV + e;
+            for (int k = kAgain - 1; k >= 0; --k) {   // descending: the smallest column survives
+                float x[EPV];
+                L::clamp(again[k]);
+                L::widen(again[k], x);
+#pragma unroll
+                for (int e = EPV - 1; e >= 0; --e)
+                    if (x[e] == M) idx = c0 + min(mat + k, n_mine - 1) * kVStride + tid * EPV + e;
+            }
         }
     }
     // ---- sums against the warp's base, first column of the maximum --------------------------------------

@@ -57,3 +57,21 @@ def test_cut_units_alone_and_with_a_single_row_tile(Hq, Hkv, L, cut):
     rows = sorted(set(np.random.Generator(np.random.PCG64(L)).choice(L, 40, replace=False).tolist() + [0, L - 1]))
     for std in (0.5, 8.0):
         _check(w, syn.attn_inputs(w, L, std_qk=std, std_v=0.5, salt=Hq), row_sel=rows)
+
+
+@pytest.mark.parametrize("dtype", [syn.BF16, syn.F32])
+@pytest.mark.parametrize("V", [8, 2048, 2056, 4096, 2048 * 3 + 40, 2048 * 6, 2048 * 7 + 1003])
+def test_first_maximum_among_the_vectors_of_a_thread(dtype, V):
+    """Rows cut into one chunk, one to eight vectors a thread: the maximum planted in every vector of a pair in turn,
+    with copies of it in the next vector of the same thread, in the last columns and beside it."""
+    import oracle
+    from test_gpu_gate import _compare, _run_gpu
+
+    R, V0 = 608, V // 8 * 8
+    x = np.random.Generator(np.random.PCG64(V)).normal(0, 2, (R, V0 + 16)).astype(np.float32)
+    for r in range(R):
+        at = (r * 1031 + r // 8 * 7) % V
+        x[r, [c for c in (at, at + 1, at + 2048, at + 4096, V - 1) if c < V]] = 9.0 + r % 5
+    st = syn.encode(x, dtype)
+    flags = np.ones(R, np.uint8)
+    _compare(_run_gpu(st, dtype, V, flags, 2.0, 32), oracle.entropy_gate(st, dtype, V, flags, 2.0, 32), 2.0)
