@@ -25,12 +25,13 @@
 //           than 32 splits, use two ticket levels instead (last CTA of a row, then last row of the sequence).
 // The entropy identity used: with p_j = 2^{d_j} / S,  -sum p_j ln p_j = ln S - ln2 * T / S
 // for any common base, so no partial ever needs the true row maximum.
-// What bounds it: from about 100 rows on the chain of a thread's vectors (clamps, maximum, exponentials, sums): 31 a
-// thread at [256, 126464] bf16 take 16.9 us, 21 at 192 rows 13.9; the same bytes as fp32 13.7.  (About 3 us are launch,
-// ramp, reduction, ticket and the finishing CTA, 10 the copy rate.)  At [32, 126464] (7.1 us) it is the fixed part.  Also
-// timed at [256, 126464]: twelve vectors ahead through asynchronous copies 17.9 (fp32 26.6 against 24.2), two batches of
-// four in registers 18.6, 3 to 21 CTAs a row 19.5 to 38, five CTAs per SM of 48 registers 20.4, sums of their own for the
-// second vector of a pair 17.0; a ring of bulk copies with a producer warp 19.7, and 7.4 at [32, 126464].
+// What bounds it: a call is about 5.5 us (launch, ramp, reduction, ticket, the finishing CTA) and its bytes at 6.1 TB/s for
+// bf16, 7.4 for fp32 (from 288 and 576 rows, 256 rows of one and two chunks): [256, 126464] bf16 17.1 us, [32, 126464] 7.2.
+// The difference is arithmetic that the stream does not hide.  Also timed at [256, 126464]: twelve vectors ahead through
+// asynchronous copies 17.9 (fp32 26.6 against 24.2), two batches of four in registers 18.6, 3 to 21 CTAs a row 19.5 to
+// 38, five CTAs per SM of 48 registers 20.4, sums of their own for the second vector of a pair 17.2, 592 equal shares
+// that cross from row to row no better (224 rows 17.1 against 16.8, 160 rows 13.9 against 13.1); a ring of bulk copies
+// with a producer warp 19.7, and 7.4 at [32, 126464].
 // The kernel is launched with programmatic stream serialisation, touches global memory only after
 // griddepcontrol.wait and waits for nothing else.
 #include "ec_common.cuh"
