@@ -5,7 +5,8 @@
 // Work decomposition
 //   - The query rows that share one kv head -- n_active rows x g = H_q/H_kv query
 //     heads -- are flattened into one row axis r = i*g + j (GQA packing), cut into
-//     64-row tiles; one CTA (4 warps x 16 rows) owns one tile.
+//     64-row tiles; one CTA (4 warps x 16 rows) owns one tile.  Where as many tiles of
+//     48 rows hold them (make_plan), the fourth warp only moves data.
 //   - Keys are cut into 64-key tiles.  When there are few row tiles (skip step:
 //     34 active rows) up to eight CTAs, a cluster, split the keys of a row tile; each leaves
 //     (m, l, O) un-normalised in its shared memory and, after a cluster barrier, merges a share
@@ -17,7 +18,7 @@
 //   - Softmax is online (running max / sum per row, exp2 with the scale folded
 //     in); P is re-packed from the S accumulators into A fragments in registers.
 // What bounds it: latency on partial steps of 64-wide heads (four sequences of 1000 keys, 48 rows, 12 query heads on 4:
-// 9.5 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
+// 9.0 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
 // per clock and SM, measured) on full ones.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
@@ -81,11 +82,12 @@ struct MmaParams {
     __nv_bfloat16* out;
     int n_active, ctx_len, n_q_heads, n_kv_heads, group;  // group = H_q / H_kv
     int rows_total;   // n_active * group
-    int row_tiles, n_splits, tiles_per_split;
+    int row_tiles, tile_rows, n_splits, tiles_per_split;   // tile_rows: BM, or 48 (kSpare)
     float scale_log2;  // scale * log2(e)
 };
 
-template <int D>
+// kSpare: the last warp has no rows
+template <int D, bool kSpare>
 __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(const MmaParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int TILE_BYTES = BN * D * 2;
@@ -103,7 +105,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     const int split = blockIdx.x % p.n_splits, unit = blockIdx.x / p.n_splits;
     const int row_tile = unit % p.row_tiles, bh = unit / p.row_tiles;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
-    const int r0 = row_tile * BM;
+    const int r0 = row_tile * (kSpare ? p.tile_rows : BM);
+    const int r_end = kSpare ? min(p.rows_total, r0 + p.tile_rows) : p.rows_total;   // no row of this CTA is beyond it
 
     const int n_tiles_total = (p.ctx_len + BN - 1) / BN;
     const int t_begin = split * p.tiles_per_split;
@@ -124,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     for (int c = tid; c < BM * CHUNKS; c += kThreads) {
         const int row = c / CHUNKS, ch = c % CHUNKS;
         const int r = r0 + row;
-        const bool ok = r < p.rows_total;
+        const bool ok = r < r_end;
         const int i = ok ? r / p.group : 0, j = ok ? r % p.group : 0;
         const __nv_bfloat16* src =
             p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + ch * 8;
@@ -180,88 +183,90 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
         if (t + ST - 1 < t_end) load_kv(t + ST - 1, (t - t_begin + ST - 1) % ST);
         cp_async_commit();
 
-        if (!q_loaded) {
-            q_loaded = true;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks)
-                ldsm_x4(smem_u32(sQ) + swz<D>(warp * 16 + (lane & 15), ks * 2 + (lane >> 4)), qf[ks]);
-        }
-
-        // ---- S = Q K^T --------------------------------------------------------------
-        float s[BN / 8][4];
-#pragma unroll
-        for (int n = 0; n < BN / 8; ++n) { s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f; }
-        const uint32_t kst = smem_u32(sK) + stage * TILE_BYTES;
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-#pragma unroll
-            for (int nb = 0; nb < BN / 16; ++nb) {
-                uint32_t kf[4];
-                const int key = nb * 16 + (lane & 7) + ((lane >> 4) << 3);
-                ldsm_x4(kst + swz<D>(key, ks * 2 + ((lane >> 3) & 1)), kf);
-                mma_bf16(s[2 * nb], qf[ks], kf[0], kf[1]);
-                mma_bf16(s[2 * nb + 1], qf[ks], kf[2], kf[3]);
-            }
-        }
-        // ---- mask keys beyond the context (ragged last tile) ------------------------
         const int key0 = t * BN;
-        if (key0 + BN > p.ctx_len) {
+        if (!kSpare || r0 + warp * 16 < r_end) {
+            if (!q_loaded) {
+                q_loaded = true;
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks)
+                    ldsm_x4(smem_u32(sQ) + swz<D>(warp * 16 + (lane & 15), ks * 2 + (lane >> 4)), qf[ks]);
+            }
+
+            // ---- S = Q K^T --------------------------------------------------------------
+            float s[BN / 8][4];
+#pragma unroll
+            for (int n = 0; n < BN / 8; ++n) { s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f; }
+            const uint32_t kst = smem_u32(sK) + stage * TILE_BYTES;
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+#pragma unroll
+                for (int nb = 0; nb < BN / 16; ++nb) {
+                    uint32_t kf[4];
+                    const int key = nb * 16 + (lane & 7) + ((lane >> 4) << 3);
+                    ldsm_x4(kst + swz<D>(key, ks * 2 + ((lane >> 3) & 1)), kf);
+                    mma_bf16(s[2 * nb], qf[ks], kf[0], kf[1]);
+                    mma_bf16(s[2 * nb + 1], qf[ks], kf[2], kf[3]);
+                }
+            }
+            // ---- mask keys beyond the context (ragged last tile) ------------------------
+            if (key0 + BN > p.ctx_len) {
+#pragma unroll
+                for (int n = 0; n < BN / 8; ++n) {
+                    const int kcol = key0 + n * 8 + 2 * (lane & 3);
+                    if (kcol >= p.ctx_len) { s[n][0] = -INFINITY; s[n][2] = -INFINITY; }
+                    if (kcol + 1 >= p.ctx_len) { s[n][1] = -INFINITY; s[n][3] = -INFINITY; }
+                }
+            }
+            // ---- online softmax ---------------------------------------------------------
+            float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
             for (int n = 0; n < BN / 8; ++n) {
-                const int kcol = key0 + n * 8 + 2 * (lane & 3);
-                if (kcol >= p.ctx_len) { s[n][0] = -INFINITY; s[n][2] = -INFINITY; }
-                if (kcol + 1 >= p.ctx_len) { s[n][1] = -INFINITY; s[n][3] = -INFINITY; }
+                mx[0] = fmaxf(mx[0], fmaxf(s[n][0], s[n][1]));
+                mx[1] = fmaxf(mx[1], fmaxf(s[n][2], s[n][3]));
             }
-        }
-        // ---- online softmax ---------------------------------------------------------
-        float mx[2] = {-INFINITY, -INFINITY};
+            float corr[2], mneg[2];
 #pragma unroll
-        for (int n = 0; n < BN / 8; ++n) {
-            mx[0] = fmaxf(mx[0], fmaxf(s[n][0], s[n][1]));
-            mx[1] = fmaxf(mx[1], fmaxf(s[n][2], s[n][3]));
-        }
-        float corr[2], mneg[2];
+            for (int h = 0; h < 2; ++h) {
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+                const float m_new = fmaxf(m_run[h], mx[h] * p.scale_log2);
+                corr[h] = (m_run[h] == -INFINITY) ? 0.f : fast_exp2(m_run[h] - m_new);
+                m_run[h] = m_new;
+                mneg[h] = -m_new;
+            }
+            float rs[2] = {0.f, 0.f};
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-            const float m_new = fmaxf(m_run[h], mx[h] * p.scale_log2);
-            corr[h] = (m_run[h] == -INFINITY) ? 0.f : fast_exp2(m_run[h] - m_new);
-            m_run[h] = m_new;
-            mneg[h] = -m_new;
-        }
-        float rs[2] = {0.f, 0.f};
+            for (int n = 0; n < BN / 8; ++n) {
+                s[n][0] = fast_exp2(fmaf(s[n][0], p.scale_log2, mneg[0]));
+                s[n][1] = fast_exp2(fmaf(s[n][1], p.scale_log2, mneg[0]));
+                s[n][2] = fast_exp2(fmaf(s[n][2], p.scale_log2, mneg[1]));
+                s[n][3] = fast_exp2(fmaf(s[n][3], p.scale_log2, mneg[1]));
+                rs[0] += s[n][0] + s[n][1];
+                rs[1] += s[n][2] + s[n][3];
+            }
+            l_run[0] = fmaf(l_run[0], corr[0], rs[0]);
+            l_run[1] = fmaf(l_run[1], corr[1], rs[1]);
 #pragma unroll
-        for (int n = 0; n < BN / 8; ++n) {
-            s[n][0] = fast_exp2(fmaf(s[n][0], p.scale_log2, mneg[0]));
-            s[n][1] = fast_exp2(fmaf(s[n][1], p.scale_log2, mneg[0]));
-            s[n][2] = fast_exp2(fmaf(s[n][2], p.scale_log2, mneg[1]));
-            s[n][3] = fast_exp2(fmaf(s[n][3], p.scale_log2, mneg[1]));
-            rs[0] += s[n][0] + s[n][1];
-            rs[1] += s[n][2] + s[n][3];
-        }
-        l_run[0] = fmaf(l_run[0], corr[0], rs[0]);
-        l_run[1] = fmaf(l_run[1], corr[1], rs[1]);
+            for (int n = 0; n < D / 8; ++n) {
+                o[n][0] *= corr[0]; o[n][1] *= corr[0];
+                o[n][2] *= corr[1]; o[n][3] *= corr[1];
+            }
+            // ---- O += P V ---------------------------------------------------------------
+            const uint32_t vst = smem_u32(sV) + stage * TILE_BYTES;
 #pragma unroll
-        for (int n = 0; n < D / 8; ++n) {
-            o[n][0] *= corr[0]; o[n][1] *= corr[0];
-            o[n][2] *= corr[1]; o[n][3] *= corr[1];
-        }
-        // ---- O += P V ---------------------------------------------------------------
-        const uint32_t vst = smem_u32(sV) + stage * TILE_BYTES;
+            for (int ks = 0; ks < BN / 16; ++ks) {
+                uint32_t pf[4];
+                pf[0] = pack_bf16(s[2 * ks][0], s[2 * ks][1]);
+                pf[1] = pack_bf16(s[2 * ks][2], s[2 * ks][3]);
+                pf[2] = pack_bf16(s[2 * ks + 1][0], s[2 * ks + 1][1]);
+                pf[3] = pack_bf16(s[2 * ks + 1][2], s[2 * ks + 1][3]);
 #pragma unroll
-        for (int ks = 0; ks < BN / 16; ++ks) {
-            uint32_t pf[4];
-            pf[0] = pack_bf16(s[2 * ks][0], s[2 * ks][1]);
-            pf[1] = pack_bf16(s[2 * ks][2], s[2 * ks][3]);
-            pf[2] = pack_bf16(s[2 * ks + 1][0], s[2 * ks + 1][1]);
-            pf[3] = pack_bf16(s[2 * ks + 1][2], s[2 * ks + 1][3]);
-#pragma unroll
-            for (int db = 0; db < D / 16; ++db) {
-                uint32_t vf[4];
-                ldsm_x4_t(vst + swz<D>(ks * 16 + (lane & 15), db * 2 + (lane >> 4)), vf);
-                mma_bf16(o[2 * db], pf, vf[0], vf[1]);
-                mma_bf16(o[2 * db + 1], pf, vf[2], vf[3]);
+                for (int db = 0; db < D / 16; ++db) {
+                    uint32_t vf[4];
+                    ldsm_x4_t(vst + swz<D>(ks * 16 + (lane & 15), db * 2 + (lane >> 4)), vf);
+                    mma_bf16(o[2 * db], pf, vf[0], vf[1]);
+                    mma_bf16(o[2 * db + 1], pf, vf[2], vf[3]);
+                }
             }
         }
         // refreshed keys into the cache, from the landed tile: the row tiles that walk over these keys take turns
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     for (int h = 0; h < 2; ++h) {
         const int row = warp * 16 + (lane >> 2) + 8 * h, r = r0 + row;
         if (p.n_splits == 1) {
-            if (r >= p.rows_total) continue;
+            if (r >= r_end) continue;
             __nv_bfloat16* dst = out_row(r);
             const float inv = 1.f / l_run[h];
 #pragma unroll
@@ -300,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
                 const uint32_t v = pack_bf16(o[n][2 * h] * inv, o[n][2 * h + 1] * inv);
                 *reinterpret_cast<uint32_t*>(dst + n * 8 + 2 * (lane & 3)) = v;
             }
-        } else {
+        } else if (!kSpare || r < r_end) {
 #pragma unroll
             for (int n = 0; n < D / 8; ++n)
                 *reinterpret_cast<float2*>(part + row * PP + n * 8 + 2 * (lane & 3)) = make_float2(o[n][2 * h], o[n][2 * h + 1]);
@@ -312,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     // ---- each CTA of the cluster merges a share of the rows: out = sum_s w_s O_s / sum_s w_s l_s, w_s = 2^(m_s - max m) ----
     tc::cluster_arrive();
     tc::cluster_wait();
-    const int valid = min(BM, p.rows_total - r0), per = (valid + p.n_splits - 1) / p.n_splits;
+    const int valid = min(BM, r_end - r0), per = (valid + p.n_splits - 1) / p.n_splits;
     const int rows_here = min(per, valid - split * per);
     for (int idx = tid; idx < rows_here * (D / 4); idx += kThreads) {
         const int row = split * per + idx / (D / 4), ch = idx % (D / 4);
@@ -345,15 +350,19 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
 }
 
 struct Plan {
-    int row_tiles, n_splits, tiles_per_split, rows_total;
+    int row_tiles, tile_rows, n_splits, tiles_per_split, rows_total;
 };
 // Keys of a row tile split over up to eight CTAs (a cluster; at least one tile each) while the launch stays within the
 // three CTAs an SM holds: a CTA is a serial chain of tiles (about 1 us each when nothing hides their latency).
+// Several row tiles of at most 48 rows (144 rows as 3 x 48 instead of 64 + 64 + 16): the padding of the last tile is not
+// computed, and the tensor core (2048 flop per clock and SM) is shared by all tiles of an SM.  9.5 -> 9.0 us for four
+// sequences of 1000 keys and 48 x 3 rows, 14.8 -> 13.8 for eight of 700.  A single tile gains nothing.
 Plan make_plan(const ec_attn_desc& d, int n_active) {
     Plan pl;
     const int g = d.n_q_heads / d.n_kv_heads;
     pl.rows_total = n_active * g;
     pl.row_tiles = (pl.rows_total + BM - 1) / BM;
+    pl.tile_rows = d.head_dim == 64 && pl.row_tiles > 1 && pl.rows_total <= 48 * pl.row_tiles ? 48 : BM;
     const int key_tiles = (d.ctx_len + BN - 1) / BN;
     const long long base = (long long)pl.row_tiles * d.batch * d.n_kv_heads;
     int splits = (int)(3LL * sm_count() / base);
@@ -365,7 +374,7 @@ Plan make_plan(const ec_attn_desc& d, int n_active) {
     return pl;
 }
 
-template <int D>
+template <int D, bool kSpare>
 cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, const void* v_new, const int32_t* active_idx,
                      cudaStream_t stream) {
     MmaParams p;
@@ -383,6 +392,7 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     p.group = a.d.n_q_heads / a.d.n_kv_heads;
     p.rows_total = pl.rows_total;
     p.row_tiles = pl.row_tiles;
+    p.tile_rows = pl.tile_rows;
     p.n_splits = pl.n_splits;
     p.tiles_per_split = pl.tiles_per_split;
     p.scale_log2 = a.scale * kLog2e;
@@ -399,7 +409,7 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     constexpr int smem = (BM + 2 * stages<D>() * BN) * D * 2 + BM * (int)sizeof(float2);
     static_assert(BM * (D + 8) * 4 <= 4 * BN * D * 2, "the partial of the merge fits over the stages");
     static PerDeviceOnce attr_once;
-    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
+    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D, kSpare>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -414,7 +424,7 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D>, p);
+    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D, kSpare>, p);
 }
 
 }  // namespace
@@ -423,8 +433,9 @@ cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const voi
                                cudaStream_t stream) {
     if (a.n_active == 0) return cudaSuccess;
     const Plan pl = make_plan(a.d, a.n_active);
-    return a.d.head_dim == 64 ? launch_d<64>(a, pl, k_new, v_new, active_idx, stream)
-                              : launch_d<128>(a, pl, k_new, v_new, active_idx, stream);
+    if (a.d.head_dim == 128) return launch_d<128, false>(a, pl, k_new, v_new, active_idx, stream);
+    return pl.tile_rows < BM ? launch_d<64, true>(a, pl, k_new, v_new, active_idx, stream)
+                             : launch_d<64, false>(a, pl, k_new, v_new, active_idx, stream);
 }
 
 }  // namespace ec

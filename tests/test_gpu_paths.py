@@ -75,3 +75,13 @@ def test_first_maximum_among_the_vectors_of_a_thread(dtype, V):
     st = syn.encode(x, dtype)
     flags = np.ones(R, np.uint8)
     _compare(_run_gpu(st, dtype, V, flags, 2.0, 32), oracle.entropy_gate(st, dtype, V, flags, 2.0, 32), 2.0)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,n", [(1, 4, 2, 200, 33), (2, 6, 2, 900, 44), (1, 3, 1, 130, 48), (8, 8, 8, 300, 65), (1, 12, 4, 64, 64)])
+def test_row_tiles_of_48_rows(B, Hq, Hkv, L, n):
+    """64-wide heads, two to four row tiles of at most 48 rows: remainders in the last tile, ragged key tiles, one key
+    tile and several; with and without fresh rows."""
+    w = syn.Workload(101, "d64_tiles", syn.BF16, B, Hq, Hkv, 64, 0, L, 1, 0, 64)
+    t = syn.attn_inputs(w, n, active_idx=syn.arbitrary_active_idx(B, L, n, seed=L + n), std_qk=0.9, std_v=0.5)
+    _check(w, t)
+    _check(w, t, refresh=False)
