@@ -11,15 +11,18 @@
 //     34 active rows) up to eight CTAs, a cluster, split the keys of a row tile; each leaves
 //     (m, l, O) un-normalised in its shared memory and, after a cluster barrier, merges a share
 //     of the rows out of its peers' (partials in global memory and a second launch took 5.4 us more).
-//   - K/V tiles are staged in shared memory with 16-byte cp.async copies, XOR-swizzled so ldmatrix
-//     is bank-conflict free.  A key that is being refreshed is read from k_new / v_new (a table of
+//   - K/V tiles are staged in shared memory, XOR-swizzled so ldmatrix is bank-conflict free: by TMA, a box each, when
+//     no index list sends keys elsewhere and heads are 64 wide (the 128-byte swizzle of a 128-byte row is the same
+//     XOR); else with 16-byte cp.async copies.  A key that is being refreshed is read from k_new / v_new (a table of
 //     the CTA's keys, filled from the index list), so nothing waits for the cache update; the row
 //     tiles of a kv head share the writing of the cache.
 //   - Softmax is online (running max / sum per row, exp2 with the scale folded
 //     in); P is re-packed from the S accumulators into A fragments in registers.
 // What bounds it: latency on partial steps of 64-wide heads (four sequences of 1000 keys, 48 rows, 12 query heads on 4:
-// 9.0 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
-// per clock and SM, measured) on full ones.
+// 8.8 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
+// per clock and SM, measured) and the instructions around it on full ones (two sequences of 1024, 24 heads on 8: 60.2 us
+// when all threads issued the copies, 51.0 with TMA; 36 sequences of 1500, 64 rows, no refresh: 45.3, 38.7).  Every wait
+// is bounded: EC_ERR_TIMEOUT in dev_status, and a CTA whose wait gave up stores no output.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
@@ -84,12 +87,16 @@ struct MmaParams {
     int rows_total;   // n_active * group
     int row_tiles, tile_rows, n_splits, tiles_per_split;   // tile_rows: BM, or 48 (kSpare)
     float scale_log2;  // scale * log2(e)
+    int32_t* dev_status;
 };
 
-// kSpare: the last warp has no rows
-template <int D, bool kSpare>
-__global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(const MmaParams p) {
-    extern __shared__ __align__(128) unsigned char smem[];
+// kSpare: the last warp has no rows.  kTma: K/V tiles come by TMA, one box each in the very layout that swz() describes
+// (no index list, so no key is sent elsewhere; 64-wide heads, whose rows are the 128 bytes of the swizzle).
+template <int D, bool kSpare, bool kTma>
+__global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(const MmaParams p, const __grid_constant__ CUtensorMap map_k,
+                                                                                    const __grid_constant__ CUtensorMap map_v) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + (kTma ? -smem_u32(smem_raw) & 1023u : 0u);
     constexpr int TILE_BYTES = BN * D * 2;
     constexpr int CHUNKS = D / 8;  // 16-byte chunks per row
     constexpr int ST = stages<D>();
@@ -97,7 +104,9 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     unsigned char* sK = smem + BM * D * 2;          // ST stages
     unsigned char* sV = sK + ST * TILE_BYTES;       // ST stages
     float2* s_ml = reinterpret_cast<float2*>(sV + ST * TILE_BYTES);   // (m, l) per row, for the merge
-    int* map = reinterpret_cast<int*>(s_ml + BM);   // [key of this CTA]: active row that refreshes it, or -1
+    uint64_t* full = reinterpret_cast<uint64_t*>(s_ml + BM);         // kTma: a barrier per stage
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(full + ST);
+    int* map = reinterpret_cast<int*>(full + ST + 1);   // [key of this CTA]: active row that refreshes it, or -1
     float* part = reinterpret_cast<float*>(sK);     // the partial of the merge, over the stages: [BM][PP]
     constexpr int PP = D + 8;                       // row pitch: fragment stores of eight rows cover all banks
 
@@ -119,19 +128,66 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     const bool fresh = p.k_new != nullptr, mapped = fresh && p.active_idx != nullptr;
     if (mapped)
         for (int k = tid; k < n_keys; k += kThreads) map[k] = -1;
+    // where this thread's pieces of Q are (two divisions each: before the wait, not behind it), -1: no such row
+    constexpr int QN = BM * CHUNKS / kThreads;
+    long long q_at[QN];
+#pragma unroll
+    for (int k = 0; k < QN; ++k) {
+        const int c = tid + k * kThreads, r = r0 + c / CHUNKS, i = r / p.group, j = r - i * p.group;
+        q_at[k] = r < r_end ? (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + c % CHUNKS * 8 : -1;
+    }
+    if (kTma && tid == 0) {
+        tc::prefetch_map(&map_k);
+        tc::prefetch_map(&map_v);
+        for (int s = 0; s < ST; ++s) tc::mbar_init(smem_u32(full + s), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     __syncthreads();
     tc::pdl_wait();
     tc::pdl_launch_dependents();
 
+    // keys that no table sends elsewhere: the cache's panel of this head, or (identity list) the fresh tensor's rows
+    const bool identity = fresh && !mapped;
+    const long long new0 = ((long long)b * p.n_active * p.n_kv_heads + hk) * D;
+    const int new_stride = p.n_kv_heads * D, key_stride = identity ? new_stride : D;
+    const __nv_bfloat16 *ksrc0 = identity ? p.k_new + new0 : kbase, *vsrc0 = identity ? p.v_new + new0 : vbase;
+    auto load_kv = [&](int tile, int stage) {
+        const int key0 = tile * BN;
+        if constexpr (kTma) {   // (rows past the context read as zero)
+            if (tid == 0) {
+                const uint32_t bar = smem_u32(full + stage), k = smem_u32(sK) + stage * TILE_BYTES, v = smem_u32(sV) + stage * TILE_BYTES;
+                tc::mbar_expect_tx(bar, 2 * TILE_BYTES);
+                tc::tma_load_5d(k, &map_k, 0, key0, 0, hk, b, bar);
+                tc::tma_load_5d(v, &map_v, 0, key0, 0, hk, b, bar);
+            }
+        } else {
+            for (int c = tid; c < BN * CHUNKS; c += kThreads) {
+                const int row = c / CHUNKS, ch = c % CHUNKS;
+                const bool ok = key0 + row < p.ctx_len;
+                const long long off = ok ? (long long)(key0 + row) * key_stride : 0;
+                const __nv_bfloat16 *ks = ksrc0 + off, *vs = vsrc0 + off;
+                if (mapped && ok) {
+                    const int i = map[key0 + row - key_lo];
+                    if (i >= 0) {
+                        ks = p.k_new + new0 + (long long)i * new_stride;
+                        vs = p.v_new + new0 + (long long)i * new_stride;
+                    }
+                }
+                cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz<D>(row, ch), ks + ch * 8, ok);
+                cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz<D>(row, ch), vs + ch * 8, ok);
+            }
+        }
+    };
+    if constexpr (kTma) {
+        for (int s = 0; s < ST - 1; ++s)
+            if (t_begin + s < t_end) load_kv(t_begin + s, s);
+    }
     // ---- stage Q (rows beyond rows_total are zero-filled) --------------------------
-    for (int c = tid; c < BM * CHUNKS; c += kThreads) {
-        const int row = c / CHUNKS, ch = c % CHUNKS;
-        const int r = r0 + row;
-        const bool ok = r < r_end;
-        const int i = ok ? r / p.group : 0, j = ok ? r % p.group : 0;
-        const __nv_bfloat16* src =
-            p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + ch * 8;
-        cp_async16(smem_u32(sQ) + swz<D>(row, ch), src, ok);
+#pragma unroll
+    for (int k = 0; k < QN; ++k) {
+        const int c = tid + k * kThreads;
+        cp_async16(smem_u32(sQ) + swz<D>(c / CHUNKS, c % CHUNKS), p.q + max(q_at[k], 0LL), q_at[k] >= 0);
     }
     if (mapped) {
         for (int i = tid; i < p.n_active; i += kThreads) {
@@ -140,31 +196,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
         }
         __syncthreads();
     }
-    // keys that no table sends elsewhere: the cache's panel of this head, or (identity list) the fresh tensor's rows
-    const bool identity = fresh && !mapped;
-    const long long new0 = ((long long)b * p.n_active * p.n_kv_heads + hk) * D;
-    const int new_stride = p.n_kv_heads * D, key_stride = identity ? new_stride : D;
-    const __nv_bfloat16 *ksrc0 = identity ? p.k_new + new0 : kbase, *vsrc0 = identity ? p.v_new + new0 : vbase;
-    auto load_kv = [&](int tile, int stage) {
-        const int key0 = tile * BN;
-        for (int c = tid; c < BN * CHUNKS; c += kThreads) {
-            const int row = c / CHUNKS, ch = c % CHUNKS;
-            const bool ok = key0 + row < p.ctx_len;
-            const long long off = ok ? (long long)(key0 + row) * key_stride : 0;
-            const __nv_bfloat16 *ks = ksrc0 + off, *vs = vsrc0 + off;
-            if (mapped && ok) {
-                const int i = map[key0 + row - key_lo];
-                if (i >= 0) {
-                    ks = p.k_new + new0 + (long long)i * new_stride;
-                    vs = p.v_new + new0 + (long long)i * new_stride;
-                }
-            }
-            cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz<D>(row, ch), ks + ch * 8, ok);
-            cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz<D>(row, ch), vs + ch * 8, ok);
-        }
-    };
     for (int s = 0; s < ST - 1; ++s) {
-        if (t_begin + s < t_end) load_kv(t_begin + s, s);
+        if (!kTma && t_begin + s < t_end) load_kv(t_begin + s, s);
         cp_async_commit();
     }
 
@@ -178,7 +211,12 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     bool q_loaded = false;
     for (int t = t_begin; t < t_end; ++t) {
         const int stage = (t - t_begin) % ST;
-        cp_async_wait<ST - 2>();
+        if constexpr (kTma) {
+            if (t == t_begin) cp_async_wait<0>();   // Q
+            tc::mbar_wait(smem_u32(full + stage), ((t - t_begin) / ST) & 1, abort_flag, p.dev_status);
+        } else {
+            cp_async_wait<ST - 2>();
+        }
         __syncthreads();   // the tile has landed, and everyone is done with the one before it, whose stage is refilled now
         if (t + ST - 1 < t_end) load_kv(t + ST - 1, (t - t_begin + ST - 1) % ST);
         cp_async_commit();
@@ -283,6 +321,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     cp_async_wait<0>();
     __syncthreads();   // everyone is done with the stages before they become the partial
 
+    const bool gave_up = kTma && *abort_flag;   // a CTA whose wait gave up stores nothing
+
     // ---- epilogue ------------------------------------------------------------------
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -297,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     for (int h = 0; h < 2; ++h) {
         const int row = warp * 16 + (lane >> 2) + 8 * h, r = r0 + row;
         if (p.n_splits == 1) {
-            if (r >= r_end) continue;
+            if (r >= r_end || gave_up) continue;
             __nv_bfloat16* dst = out_row(r);
             const float inv = 1.f / l_run[h];
 #pragma unroll
@@ -318,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
     tc::cluster_arrive();
     tc::cluster_wait();
     const int valid = min(BM, r_end - r0), per = (valid + p.n_splits - 1) / p.n_splits;
-    const int rows_here = min(per, valid - split * per);
+    const int rows_here = gave_up ? 0 : min(per, valid - split * per);
     for (int idx = tid; idx < rows_here * (D / 4); idx += kThreads) {
         const int row = split * per + idx / (D / 4), ch = idx % (D / 4);
         float mm[8], ll[8], x[8][4], M = -INFINITY, L = 0.f;
@@ -374,7 +414,20 @@ Plan make_plan(const ec_attn_desc& d, int n_active) {
     return pl;
 }
 
-template <int D, bool kSpare>
+// tile maps of the cache [B, Hkv, L, 64], or of token-major fresh rows [B, L, Hkv, 64]
+bool make_tile_map(CUtensorMap* map, const void* ptr, const ec_attn_desc& d, bool token_major) {
+    tc::EncodeTiledFn fn = tc::encode_fn();
+    if (!fn) return false;
+    const cuuint64_t row = 128, L = (cuuint64_t)d.ctx_len, H = (cuuint64_t)d.n_kv_heads;
+    const cuuint64_t dims[5] = {64, L, 1, H, (cuuint64_t)d.batch};
+    const cuuint64_t strides[4] = {token_major ? row * H : row, row, token_major ? row : row * L, row * L * H};
+    const cuuint32_t box[5] = {64, (cuuint32_t)BN, 1, 1, 1}, estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int D, bool kSpare, bool kTma>
 cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, const void* v_new, const int32_t* active_idx,
                      cudaStream_t stream) {
     MmaParams p;
@@ -396,6 +449,7 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     p.n_splits = pl.n_splits;
     p.tiles_per_split = pl.tiles_per_split;
     p.scale_log2 = a.scale * kLog2e;
+    p.dev_status = a.dev_status;
     const long long ctas = (long long)a.d.batch * a.d.n_kv_heads * pl.row_tiles * pl.n_splits;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     int map_keys = k_new && active_idx ? pl.tiles_per_split * BN : 0;
@@ -406,10 +460,10 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
         p.k_new = p.v_new = nullptr;
         map_keys = 0;
     }
-    constexpr int smem = (BM + 2 * stages<D>() * BN) * D * 2 + BM * (int)sizeof(float2);
+    constexpr int smem = (BM + 2 * stages<D>() * BN) * D * 2 + BM * (int)sizeof(float2) + 8 * (stages<D>() + 1) + (kTma ? 1024 : 0);
     static_assert(BM * (D + 8) * 4 <= 4 * BN * D * 2, "the partial of the merge fits over the stages");
     static PerDeviceOnce attr_once;
-    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D, kSpare>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
+    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D, kSpare, kTma>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -424,7 +478,11 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D, kSpare>, p);
+    CUtensorMap map_k{}, map_v{};
+    if (kTma && (!make_tile_map(&map_k, p.k_new ? k_new : a.k_cache, a.d, p.k_new) ||
+                 !make_tile_map(&map_v, p.v_new ? v_new : a.v_cache, a.d, p.v_new)))
+        return cudaErrorInvalidValue;
+    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D, kSpare, kTma>, p, map_k, map_v);
 }
 
 }  // namespace
@@ -433,9 +491,13 @@ cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const voi
                                cudaStream_t stream) {
     if (a.n_active == 0) return cudaSuccess;
     const Plan pl = make_plan(a.d, a.n_active);
-    if (a.d.head_dim == 128) return launch_d<128, false>(a, pl, k_new, v_new, active_idx, stream);
-    return pl.tile_rows < BM ? launch_d<64, true>(a, pl, k_new, v_new, active_idx, stream)
-                             : launch_d<64, false>(a, pl, k_new, v_new, active_idx, stream);
+    if (a.d.head_dim == 128) return launch_d<128, false, false>(a, pl, k_new, v_new, active_idx, stream);
+    const bool spare = pl.tile_rows < BM;
+    if (k_new && active_idx)
+        return spare ? launch_d<64, true, false>(a, pl, k_new, v_new, active_idx, stream)
+                     : launch_d<64, false, false>(a, pl, k_new, v_new, active_idx, stream);
+    return spare ? launch_d<64, true, true>(a, pl, k_new, v_new, active_idx, stream)
+                 : launch_d<64, false, true>(a, pl, k_new, v_new, active_idx, stream);
 }
 
 }  // namespace ec

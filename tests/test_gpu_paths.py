@@ -85,3 +85,13 @@ def test_row_tiles_of_48_rows(B, Hq, Hkv, L, n):
     t = syn.attn_inputs(w, n, active_idx=syn.arbitrary_active_idx(B, L, n, seed=L + n), std_qk=0.9, std_v=0.5)
     _check(w, t)
     _check(w, t, refresh=False)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L", [(2, 4, 2, 1), (1, 2, 2, 64), (3, 6, 2, 65), (1, 4, 1, 200), (2, 8, 8, 449)])
+def test_recompute_steps_of_64_wide_heads(B, Hq, Hkv, L):
+    """K/V tiles by TMA out of the token-major fresh rows and out of the cache: one key, whole and ragged tiles, more
+    tiles than stages."""
+    w = syn.Workload(102, "d64_full", syn.BF16, B, Hq, Hkv, 64, 0, L, 1, 0, 64)
+    t = syn.attn_inputs(w, L, std_qk=0.9, std_v=0.5)
+    _check(w, t)
+    _check(w, t, refresh=False)
