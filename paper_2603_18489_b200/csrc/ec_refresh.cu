@@ -35,13 +35,11 @@ __global__ void __launch_bounds__(256) refresh_kernel(uint4* __restrict__ k_cach
     const long long b = bi / n_active;
     tc::pdl_wait();
     tc::pdl_launch_dependents();
+    // the piece and its position are asked for together: behind the position's check it is a second round trip
+    const uint4 v = __ldg((blockIdx.y == 0 ? k_new : v_new) + t);
     const int pos = idx ? __ldg(idx + bi) : i;
     if (pos < 0 || pos >= ctx_len) return;  // never write outside the cache
-    const long long dst = ((b * n_kv_heads + h) * ctx_len + pos) * row_vecs + piece;
-    if (blockIdx.y == 0)
-        k_cache[dst] = __ldg(k_new + t);
-    else
-        v_cache[dst] = __ldg(v_new + t);
+    (blockIdx.y == 0 ? k_cache : v_cache)[((b * n_kv_heads + h) * ctx_len + pos) * row_vecs + piece] = v;
 }
 
 }  // namespace
