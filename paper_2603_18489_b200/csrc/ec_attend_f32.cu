@@ -69,16 +69,25 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
     int* map = reinterpret_cast<int*>(sm + C::map);   // [key of this CTA]: active row that refreshes it, or -1
     if (mapped)
         for (int k = tid; k < key_hi - key_lo; k += kThreads) map[k] = -1;
+    // where this thread's pieces of Q are (two divisions each: before the wait, not behind it), -1: no such row
+    constexpr int QN = BM * D4 / kThreads;
+    long long q_at[QN];
+#pragma unroll
+    for (int k = 0; k < QN; ++k) {
+        const int c = tid + k * kThreads, r = r0 + c / D4, i = r / p.group, j = r - i * p.group;
+        q_at[k] = r < p.rows_total ? (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + c % D4 * 4 : -1;
+    }
+    const float *kc = p.k_cache + (long long)bh * p.ctx_len * D, *vc = p.v_cache + (long long)bh * p.ctx_len * D;
+    const long long new0 = ((long long)b * p.n_active * p.n_kv_heads + hk) * D;
+    const int new_stride = p.n_kv_heads * D;
     __syncthreads();
     pdl_wait();
     pdl_launch_dependents();
 
-    for (int c = tid; c < BM * D4; c += kThreads) {
-        const int row = c / D4, ch = c % D4, r = r0 + row;
-        const bool ok = r < p.rows_total;
-        const int i = ok ? r / p.group : 0, j = ok ? r - i * p.group : 0;
-        const float* src = p.q + (((long long)b * p.n_active + i) * p.n_q_heads + hk * p.group + j) * D + ch * 4;
-        cp_async16(s2u(sm + C::q + row * C::P + ch * 4), src, ok);
+#pragma unroll
+    for (int k = 0; k < QN; ++k) {
+        const int c = tid + k * kThreads;
+        cp_async16(s2u(sm + C::q + c / D4 * C::P + c % D4 * 4), p.q + max(q_at[k], 0LL), q_at[k] >= 0);
     }
     if (mapped) {
         for (int i = tid; i < p.n_active; i += kThreads) {
@@ -87,7 +96,6 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
         }
         __syncthreads();
     }
-    const float *kc = p.k_cache + (long long)bh * p.ctx_len * D, *vc = p.v_cache + (long long)bh * p.ctx_len * D;
     // the fresh row behind a key of this CTA, or -1
     auto fresh_row = [&](int key) { return !fresh ? -1 : mapped ? map[key - key_lo] : key; };
     auto load_kv = [&](int t, int stage) {
@@ -98,7 +106,7 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
             const float *ksrc = kc, *vsrc = vc;
             if (ok) {
                 const int i = fresh_row(key);
-                const long long at = i < 0 ? (long long)key * D : (((long long)b * p.n_active + i) * p.n_kv_heads + hk) * D;
+                const long long at = i < 0 ? (long long)key * D : new0 + (long long)i * new_stride;
                 ksrc = (i < 0 ? kc : p.k_new) + at + ch * 4;
                 vsrc = (i < 0 ? vc : p.v_new) + at + ch * 4;
             }
