@@ -2,11 +2,11 @@
 // partial branch; the full branch when every row is active) in ONE launch, entirely in fp32 on the FMA pipes (the
 // tolerance that goes with fp32 tensors, 1e-5 relative, rules out tf32 tensor cores).
 //
-//   grid    a CTA of 128 threads takes 32 packed query rows (active row x query heads of one kv head) and a range of
+//   grid    a CTA of 128 threads takes 32 (16, 8) packed query rows (active row x query heads of one kv head) and a range of
 //           32-key tiles; up to eight CTAs, a cluster, split the keys of a row tile when there are few row tiles, so
 //           that a partial step of a small model still spreads over the chip.
 //   tile    K and V tiles come by 16-byte asynchronous copies into one of two stages.  Thread (tr, tk) = (tid / 16,
-//           tid % 16) holds rows 4 tr .. 4 tr + 3: it forms their scores against keys tk and tk + 16 (packed fp32x2 over even
+//           tid % 16) holds rows R tr .. R tr + R - 1 (R = 4, 2 or 1): it forms their scores against keys tk and tk + 16 (packed fp32x2 over even
 //           and odd columns: two partial sums), the 16 threads of a row exchange maxima and sums by shuffles, and
 //           probabilities go through shared memory to the same warp, which accumulates D / 16 output columns a thread.
 //   refresh a key that is being refreshed is read from k_new / v_new (a table of the CTA's keys, filled from the index
@@ -14,9 +14,9 @@
 //           whose refreshed rows nobody reads.
 //   merge   every CTA leaves O (un-normalised), m and l of its keys in shared memory; after a cluster barrier each
 //           combines a share of the rows out of its peers' memory.
-// What bounds it: latency at the sizes it is for.  34 rows x 4 heads of 64 over 256 keys: 6.0 us a call (a warp per query
+// What bounds it: latency at the sizes it is for.  34 rows x 4 heads of 64 over 256 keys: 4.9 us a call (a warp per query
 // row that walks over all keys, behind a refresh launch, took 30.7).  At large sizes the FMA pipe: 438 rows x 8 heads of
-// four sequences 82 us (511).
+// four sequences 80 us (511).
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
@@ -25,7 +25,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 128, BM = 32, BN = 32;
+constexpr int kThreads = 128, BN = 32;
 constexpr int kMaxMapKeys = 8192;   // keys of one CTA beyond which the refresh is a launch of its own
 
 struct F32Params {
@@ -37,8 +37,9 @@ struct F32Params {
 };
 
 // shared memory, in floats (D-float rows padded by four: eight rows read as float4 then cover all banks)
-template <int D>
+template <int D, int R>
 struct Carve {
+    static constexpr int BM = 8 * R;
     static constexpr int P = D + 4;
     static constexpr int q = 0, kv = q + BM * P, stage = 2 * BN * P, p = kv + 2 * stage, pp = BN + 4;
     static constexpr int ml = p + BM * pp, map = ml + 2 * BM;
@@ -51,9 +52,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sz) : "memory");
 }
 
-template <int D>
+// R: query rows of a thread, an eighth of the CTA's
+template <int D, int R>
 __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p) {
-    using C = Carve<D>;
+    using C = Carve<D, R>;
+    constexpr int BM = 8 * R;
     constexpr int D4 = D / 4, OC = D / 16;   // float4 pieces of a row; output columns of a thread
     extern __shared__ __align__(16) float sm[];
     const int tid = threadIdx.x, tr = tid >> 4, tk = tid & 15;
@@ -117,9 +120,9 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
     };
     if (t0 < t1) load_kv(t0, 0);
 
-    float m[4], l[4], o[4][OC];
+    float m[R], l[R], o[R][OC];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
         m[r] = -INFINITY;
         l[r] = 0.f;
 #pragma unroll
@@ -135,24 +138,24 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
         }
         __syncthreads();
         const float *ks = sm + C::kv + stage * C::stage, *vs = ks + BN * C::P;
-        // ---- scores of four rows against two keys ----
-        f32x2 acc[4][2];
+        // ---- scores of R rows against two keys ----
+        f32x2 acc[R][2];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = pk(0.f, 0.f);
+        for (int r = 0; r < R; ++r) acc[r][0] = acc[r][1] = pk(0.f, 0.f);
 #pragma unroll 4
         for (int ch = 0; ch < D4; ++ch) {
             const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(ks + tk * C::P + ch * 4);
             const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(ks + (tk + 16) * C::P + ch * 4);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(sm + C::q + (4 * tr + r) * C::P + ch * 4);
+            for (int r = 0; r < R; ++r) {
+                const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(sm + C::q + (R * tr + r) * C::P + ch * 4);
                 acc[r][0] = fma2(qv.y, k0.y, fma2(qv.x, k0.x, acc[r][0]));
                 acc[r][1] = fma2(qv.y, k1.y, fma2(qv.x, k1.x, acc[r][1]));
             }
         }
         const bool in0 = t * BN + tk < p.ctx_len, in1 = t * BN + tk + 16 < p.ctx_len;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < R; ++r) {
             float a0, a1, b0, b1;
             upk(acc[r][0], a0, a1);
             upk(acc[r][1], b0, b1);
@@ -170,23 +173,23 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
             m[r] = m_new;
 #pragma unroll
             for (int c = 0; c < OC; ++c) o[r][c] *= corr;
-            sm[C::p + (4 * tr + r) * C::pp + tk] = p0;
-            sm[C::p + (4 * tr + r) * C::pp + tk + 16] = p1;
+            sm[C::p + (R * tr + r) * C::pp + tk] = p0;
+            sm[C::p + (R * tr + r) * C::pp + tk + 16] = p1;
         }
         __syncwarp();   // the probabilities of a row are written and read by the same warp
         // ---- O += P V: output columns 4 tk .. 4 tk + 3 (and 64 + 4 tk .. for D = 128) ----
 #pragma unroll 2
         for (int k4 = 0; k4 < BN; k4 += 4) {
-            float4 pr[4];
+            float4 pr[R];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) pr[r] = *reinterpret_cast<const float4*>(sm + C::p + (4 * tr + r) * C::pp + k4);
+            for (int r = 0; r < R; ++r) pr[r] = *reinterpret_cast<const float4*>(sm + C::p + (R * tr + r) * C::pp + k4);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
 #pragma unroll
                 for (int c = 0; c < OC; c += 4) {
                     const float4 v = *reinterpret_cast<const float4*>(vs + (k4 + k) * C::P + c * 16 + 4 * tk);
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
+                    for (int r = 0; r < R; ++r) {
                         const float pv = k == 0 ? pr[r].x : k == 1 ? pr[r].y : k == 2 ? pr[r].z : pr[r].w;
                         o[r][c] = fmaf(pv, v.x, o[r][c]);
                         o[r][c + 1] = fmaf(pv, v.y, o[r][c + 1]);
@@ -215,9 +218,9 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
     };
     if (p.n_splits == 1) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (r0 + 4 * tr + r >= p.rows_total) continue;
-            float* dst = out_row(r0 + 4 * tr + r);
+        for (int r = 0; r < R; ++r) {
+            if (r0 + R * tr + r >= p.rows_total) continue;
+            float* dst = out_row(r0 + R * tr + r);
             const float inv = 1.f / l[r];
 #pragma unroll
             for (int c = 0; c < OC; c += 4)
@@ -228,12 +231,12 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
     }
     // ---- partial of this CTA, then each CTA of the cluster merges its share of the rows ----
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
 #pragma unroll
         for (int c = 0; c < OC; c += 4)
-            *reinterpret_cast<float4*>(sm + C::part + (4 * tr + r) * D + c * 16 + 4 * tk) =
+            *reinterpret_cast<float4*>(sm + C::part + (R * tr + r) * D + c * 16 + 4 * tk) =
                 make_float4(o[r][c], o[r][c + 1], o[r][c + 2], o[r][c + 3]);
-        if (tk == 0) *reinterpret_cast<float2*>(sm + C::ml + 2 * (4 * tr + r)) = make_float2(m[r], l[r]);
+        if (tk == 0) *reinterpret_cast<float2*>(sm + C::ml + 2 * (R * tr + r)) = make_float2(m[r], l[r]);
     }
     cluster_arrive();
     cluster_wait();
@@ -270,11 +273,11 @@ __global__ void __launch_bounds__(kThreads) attend_f32_kernel(const F32Params p)
     cluster_wait();
 }
 
-template <int D>
+template <int D, int R>
 cudaError_t launch_d(const F32Params& p, int batch, cudaStream_t stream) {
     static PerDeviceOnce once;
-    const size_t smem = Carve<D>::bytes(p.k_new && p.active_idx ? p.tiles_per_split * BN : 0);
-    if (const cudaError_t e = ensure_dynamic_smem(once, attend_f32_kernel<D>, (int)Carve<D>::bytes(kMaxMapKeys)); e != cudaSuccess)
+    const size_t smem = Carve<D, R>::bytes(p.k_new && p.active_idx ? p.tiles_per_split * BN : 0);
+    if (const cudaError_t e = ensure_dynamic_smem(once, attend_f32_kernel<D, R>, (int)Carve<D, R>::bytes(kMaxMapKeys)); e != cudaSuccess)
         return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)((long long)batch * p.n_kv_heads * p.row_tiles * p.n_splits), 1, 1);
@@ -290,7 +293,7 @@ cudaError_t launch_d(const F32Params& p, int batch, cudaStream_t stream) {
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_f32_kernel<D>, p);
+    return cudaLaunchKernelEx(&cfg, attend_f32_kernel<D, R>, p);
 }
 
 }  // namespace
@@ -312,14 +315,24 @@ cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void
     p.n_kv_heads = a.d.n_kv_heads;
     p.group = a.d.n_q_heads / a.d.n_kv_heads;
     p.rows_total = a.n_active * p.group;
-    p.row_tiles = (p.rows_total + BM - 1) / BM;
     p.scale = a.scale;
     // The keys of a row tile are split over as many CTAs (at most eight, at least a tile each) as keep the launch within
-    // four CTAs per SM, which is what shared memory leaves room for.
+    // four CTAs per SM, which is what shared memory leaves room for.  A row tile has 32 rows, or 16 while such a launch
+    // has two CTAs per SM at most, or 8 while it has one: a CTA's time is its threads' rows times its key tiles, but every
+    // row tile reads the keys again and waits for its SM's other ones.  (34 rows x 256 keys x 4 heads: 4.9 us with 16 rows,
+    // 5.1 with 8, 160 CTAs, 5.8 with 32; 40 rows x 400 keys x 12 heads 8.5 with 16, 11.6 with 8, 10.9 with 32.)
     const int n_tiles = (a.d.ctx_len + BN - 1) / BN;
-    const long long units = (long long)a.d.batch * a.d.n_kv_heads * p.row_tiles;
-    int splits = 1;
-    while (splits < 8 && 2 * splits <= n_tiles && 2 * splits * units <= 4LL * sm_count()) splits *= 2;
+    const long long heads = (long long)a.d.batch * a.d.n_kv_heads;
+    long long units = 0;
+    int R = 1, splits = 1;
+    for (;; R *= 2) {
+        p.row_tiles = (p.rows_total + 8 * R - 1) / (8 * R);
+        units = heads * p.row_tiles;
+        splits = n_tiles < 8 ? n_tiles : 8;
+        if (R == 4 || units * splits <= (long long)R * sm_count()) break;
+    }
+    if (units * splits > 4LL * sm_count()) splits = (int)(4LL * sm_count() / units);
+    if (splits < 1) splits = 1;
     p.tiles_per_split = (n_tiles + splits - 1) / splits;
     p.n_splits = (n_tiles + p.tiles_per_split - 1) / p.tiles_per_split;
     if (units * p.n_splits > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -329,7 +342,9 @@ cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void
             return e;
         p.k_new = p.v_new = nullptr;
     }
-    return a.d.head_dim == 64 ? launch_d<64>(p, a.d.batch, stream) : launch_d<128>(p, a.d.batch, stream);
+    if (a.d.head_dim == 64)
+        return R == 1 ? launch_d<64, 1>(p, a.d.batch, stream) : R == 2 ? launch_d<64, 2>(p, a.d.batch, stream) : launch_d<64, 4>(p, a.d.batch, stream);
+    return R == 1 ? launch_d<128, 1>(p, a.d.batch, stream) : R == 2 ? launch_d<128, 2>(p, a.d.batch, stream) : launch_d<128, 4>(p, a.d.batch, stream);
 }
 
 }  // namespace ec

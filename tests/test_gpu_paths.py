@@ -95,3 +95,13 @@ def test_recompute_steps_of_64_wide_heads(B, Hq, Hkv, L):
     t = syn.attn_inputs(w, L, std_qk=0.9, std_v=0.5)
     _check(w, t)
     _check(w, t, refresh=False)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D,L,n", [(1, 2, 1, 64, 70, 35), (1, 4, 4, 64, 256, 2), (1, 4, 4, 64, 256, 34), (1, 3, 1, 128, 33, 17),
+                                            (1, 8, 8, 128, 300, 40), (2, 6, 2, 64, 161, 48), (6, 8, 8, 64, 300, 40)])
+def test_fp32_row_tiles_of_8_16_and_32_rows(B, Hq, Hkv, D, L, n):
+    """Row tiles of every height, remainders in the last one, keys split over three to eight CTAs and uneven shares."""
+    w = syn.Workload(103, "f32_tiles", syn.F32, B, Hq, Hkv, D, 0, L, 1, 0, 64)
+    t = syn.attn_inputs(w, n, active_idx=syn.arbitrary_active_idx(B, L, n, seed=L + n), std_qk=0.9, std_v=0.5)
+    _check(w, t)
+    _check(w, t, refresh=False)
