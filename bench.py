@@ -55,19 +55,19 @@ K64_WORKLOADS = ("c4_llada_l2048", "c5_llada_l4096", "c5_llada_l4096_b8", "c5_dr
 NCU_TRAFFIC = {
     "attend_skip": [
         {"source": "paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",
-         "sha256": "55eea1c65c1cfe60b79f17c4d0f5c2d222cf29ddff308fb432c5a73e07d8b972",
-         "bytes_per_launch": {"c2_llada_l768": 13400000, "c5_llada_l4096": 68730000}},
+         "sha256": "6fd3dc0f298c46a576d57bd3540f12bcb9168ab693ffffbbac8922c8510713b7",
+         "bytes_per_launch": {"c5_llada_l4096": 68160000}},
         {"source": "paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu",
-         "sha256": "bfec166c49fcaea673858dc2e86bfa2b1bffe4d191e2c41857dac13d2d180d5a",
-         "bytes_per_launch": {"c5_llada_l4096_b8": 552480000}}],
+         "sha256": "65b46cc75830b8e859285087271c6c5b40faae59a005274755dbc82fd63d76b5",
+         "bytes_per_launch": {"c5_llada_l4096_b8": 558740000}}],
     "attend_dense": [
         {"source": "paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",
-         "sha256": "4323d044418277f0fa12a7dee721db22bf5b7291e5e7e0507861c74d0b3dd4fe",
-         "bytes_per_launch": {"c2_llada_l768": 18930000, "c4_llada_l2048": 62770000, "c5_llada_l4096": 176240000}}],
+         "sha256": "7a98a8f43f1813c6b2c2e415eaa10ef757f463c24264f763c784fb25d2ae37a6",
+         "bytes_per_launch": {"c5_llada_l4096": 146620000}}],
     "entropy_gate": [
         {"source": "paper_2603_18489_b200/csrc/ec_gate.cu",
-         "sha256": "519bc6a99b3932ab141af3aa77056dff693970d2254c54c7a023263874293215",
-         "bytes_per_launch": {"c5_llada_l4096": 8140000, "c5_llada_l4096_b8": 65060000}}],
+         "sha256": "026fe97ffd51bbd366852fdac150195f9cf2765f3cd9db49fa97c7109723dbe2",
+         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65710000}}],
 }
 
 
