@@ -81,6 +81,11 @@ struct DenseParams {
     int wait_first;   // second launch: 1 when there is no first one, see below
 };
 
+// First key tile of part i of a unit whose T key tiles are cut into s parts.  Every part holds T / s tiles, rounded down or
+// up, so none is empty while T >= s; the longest is no longer than with parts of ceil(T / s) tiles, the last of which
+// start behind the last tile at T = 33 and s = 8, for instance.
+__host__ __device__ constexpr int part_begin(int T, int s, int i) { return (int)((long long)T * i / s); }
+
 // kCut: the launch of the cut units.  A cluster leaves its un-normalised rows, m and l in shared memory, each CTA merges a
 // share of them out of its peers'.  This launch follows the one of the whole units with programmatic serialisation and
 // does NOT wait for it: every CTA of the first launch triggers after its own dependency wait, so whatever wrote q, k_new
@@ -117,9 +122,8 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     const int r_pair = pair * 2 * BM;
     const int n_tiles_q = (p.rows_total - r_pair > BM) ? 2 : 1;   // row tiles of this CTA that hold rows
     const int T_all = (p.ctx_len + BN - 1) / BN;
-    const int tiles_per_part = kCut ? (T_all + p.split - 1) / p.split : T_all;
-    const int j0 = part * tiles_per_part;                        // first key tile of this CTA
-    const int T = min(T_all, j0 + tiles_per_part) - j0;          // >= 1 by construction of the plan
+    const int j0 = kCut ? part_begin(T_all, p.split, part) : 0;                  // first key tile of this CTA
+    const int T = (kCut ? part_begin(T_all, p.split, part + 1) : T_all) - j0;    // >= 4 in a cut unit, see make_dense_plan
 
     if (tid == 0) {
         prefetch_map(&map_k);
@@ -604,8 +608,15 @@ bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
 
 void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len) {
     const DensePlan pl = make_dense_plan(d, n_active);
-    snprintf(buf, len, "attend_dense_kernel grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d", pl.n_pairs,
-             d.batch * d.n_q_heads, pl.n_full, pl.units - pl.n_full, pl.split);
+    const int T = (d.ctx_len + BN - 1) / BN;
+    int lo = T, hi = 0;   // key tiles of the shortest and the longest part of a cut unit
+    for (int i = 0; i < pl.split; ++i) {
+        const int n = part_begin(T, pl.split, i + 1) - part_begin(T, pl.split, i);
+        lo = n < lo ? n : lo;
+        hi = n > hi ? n : hi;
+    }
+    snprintf(buf, len, "attend_dense_kernel grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d part_tiles=%d..%d", pl.n_pairs,
+             d.batch * d.n_q_heads, pl.n_full, pl.units - pl.n_full, pl.split, lo, hi);
 }
 
 cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {

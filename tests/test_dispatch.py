@@ -89,3 +89,25 @@ def test_other_instantiations_and_fallbacks_are_reachable():
     assert "cut_units=0x1" in name(1, 2048, 32, 32, 128, syn.BF16, 2048, idx=False)
     assert "cut_units=0x1" in name(8, 4096, 32, 32, 128, syn.BF16, 4096, idx=False)
     assert ec.ec_attend_kernel_name(ec.make_desc(1, 64, 4, 4, 64, syn.F32), 65, True, True) == ""   # rejected
+
+
+@pytest.mark.parametrize("Hq,Hkv", [(32, 32), (28, 4), (9, 9)])
+def test_every_part_of_a_cut_unit_holds_key_tiles(Hq, Hkv):
+    """The last wave of a recompute step is cut along the keys: whatever the number of key tiles, its parts are level
+    and none of them is empty (a part without a tile would wait for data that nobody loads)."""
+    import re
+
+    import paper_2603_18489_b200 as ec
+
+    n_cut = 0
+    for B in range(1, 9):
+        for tiles in range(1, 65):
+            for L, n in ((128 * tiles, 128 * tiles), (128 * tiles - 57, 128 * tiles - 57), (128 * tiles, min(300, 128 * tiles))):
+                got = ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 128, syn.BF16), n, True, n != L)
+                if not got.startswith(("attend_dense", "refresh_kernel + attend_dense")):
+                    continue
+                cut, parts, lo, hi = (int(v) for v in re.search(r"cut_units=(\d+)x(\d+) part_tiles=(-?\d+)\.\.(\d+)", got).groups())
+                assert lo == tiles // parts and hi == -(-tiles // parts), got
+                assert lo >= 4 or parts == 1, got
+                n_cut += cut > 0
+    assert n_cut > 50

@@ -59,6 +59,19 @@ def test_cut_units_alone_and_with_a_single_row_tile(Hq, Hkv, L, cut):
         _check(w, syn.attn_inputs(w, L, std_qk=std, std_v=0.5, salt=Hq), row_sel=rows)
 
 
+@pytest.mark.parametrize("H,L,cut", [(9, 4100, "cut_units=5x8 part_tiles=4..5"), (9, 4400, "cut_units=14x8 part_tiles=4..5"),
+                                     (6, 6200, "cut_units=2x8 part_tiles=6..7"), (17, 2200, "cut_units=5x4 part_tiles=4..5")])
+def test_cut_units_of_uneven_parts(H, L, cut):
+    """Key tiles that the number of parts does not divide: the cut units are the last ones, those of the last heads."""
+    import paper_2603_18489_b200 as ec
+
+    w = syn.Workload(104, "uneven", syn.BF16, 1, H, H, 128, 0, L, 1, 0, 64)
+    assert cut in ec.ec_attend_kernel_name(ec.make_desc(1, L, H, H, 128, syn.BF16), L, True, False)
+    rows = sorted(set(np.random.Generator(np.random.PCG64(L)).choice(L, 40, replace=False).tolist() + [0, L - 1]))
+    for std in (0.5, 8.0):
+        _check(w, syn.attn_inputs(w, L, std_qk=std, std_v=0.5, salt=H), row_sel=rows)
+
+
 @pytest.mark.parametrize("dtype", [syn.BF16, syn.F32])
 @pytest.mark.parametrize("V", [8, 2048, 2056, 4096, 2048 * 3 + 40, 2048 * 6, 2048 * 7 + 1003])
 def test_first_maximum_among_the_vectors_of_a_thread(dtype, V):
