@@ -158,11 +158,13 @@ public:
     void add(PyObject* given, const char* name, int64_t n, at::ScalarType type) {
         Item& it = items_[count_++];
         it = Item{given, name, n, type, total_};
-        if (given == Py_None) total_ += (n * (int64_t)c10::elementSize(type) + 15) & ~15ll;
+        if (given != Py_None) return;
+        total_ += (n * (int64_t)c10::elementSize(type) + 15) & ~15ll;
+        any_ = true;
     }
     void skip() { items_[count_++] = Item{nullptr, "", 0, at::kFloat, 0}; }   // not wanted: NULL, None
     void allocate() {
-        if (total_) blob_ = at::empty({total_}, like_.options().dtype(at::kByte));
+        if (any_) blob_ = at::empty({total_}, like_.options().dtype(at::kByte));
         for (int i = 0; i < count_; ++i) {
             Item& it = items_[i];
             if (!it.given) continue;
@@ -209,6 +211,7 @@ private:
     Item items_[8];
     int count_ = 0;
     int64_t total_ = 0;
+    bool any_ = false;   // some output is to be made; total_ may still be 0 (a call without rows)
 };
 
 struct Logits {

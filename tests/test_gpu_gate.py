@@ -171,3 +171,26 @@ def test_gate_on_inputs_large_enough_for_the_per_thread_loads(dtype, R, V, strid
     g = _run_gpu(st["logits"], dtype, V, flags, tau, rps)
     o = oracle.entropy_gate(st["logits"], dtype, V, flags, tau, rps)
     _compare(g, o, tau)
+
+
+def test_a_call_without_rows_returns_empty_outputs():
+    """Zero rows is a no-op of the C entry points: outputs that were not given come back empty, given ones untouched."""
+    import paper_2603_18489_b200 as ec
+
+    e = lambda dt: torch.empty(0, dtype=dt, device="cuda")
+    lg, u8 = torch.empty(0, 1024, device="cuda"), e(torch.uint8)
+    got = {"gate": ec.ec_entropy_gate(lg, 1024, 32, u8, 1.5), "metrics": ec.ec_entropy_gate_metrics(lg, 1024, 32, u8, 1.5),
+           "bare": ec.ec_entropy_gate(lg, 1024, 32, u8, 1.5, want_rows=False),
+           "decode": ec.ec_entropy_gate_decode(lg, 1024, 32, u8, 0.9, 1.5, e(torch.int32))}
+    kinds = dict(argmax=torch.int32, decision=torch.int32, decoded=torch.uint8)
+    for name, out in got.items():
+        for key, t in out.items():
+            if name == "bare" and key in ("argmax", "conf", "entropy"):
+                assert t is None
+            else:
+                assert t.numel() == 0 and t.dim() == 1 and t.is_cuda and t.dtype == kinds.get(key, torch.float32), (name, key)
+    mine = e(torch.float32)
+    assert ec.ec_entropy_gate(lg, 1024, 32, u8, 1.5, max_entropy_out=mine)["max_entropy"] is mine
+    with pytest.raises(ec.EcError):   # five rows are not whole sequences: the library's error, not an empty allocation's
+        ec.ec_entropy_gate(torch.zeros(5, 1024, device="cuda"), 1024, 32, torch.zeros(5, dtype=torch.uint8, device="cuda"),
+                           1.5, want_rows=False)
