@@ -6,8 +6,9 @@
 // registers, so one block-wide scan of the per-thread counts (window rows and members of R packed into a word)
 // yields both lists in ascending order.
 //   tau_R = max(min over K, t - dt) without ever finding the k largest: the k-th largest value exceeds t - dt only if
-//           at least k entries do, and is then one of the dt values t - dt + 1 .. t, found by bisection (a probe is
-//           one block-wide count).  Fewer than k decoded positions: the minimum is "-infinity" and t - dt stands.
+//           at least k entries do, and is then one of the dt values t - dt + 1 .. t (one above t, if k entries are:
+//           the first count tells), found by bisection (a probe is one block-wide count).  Fewer than k decoded
+//           positions: the minimum is "-infinity" and t - dt stands.
 // What bounds it: latency.  All global loads are issued in one round (two in sliding mode, whose window rows have to be
 // checked against the mask), then about eight barriers.  Bisecting over all values that occur, behind dependent loads
 // and with two scans, took 6.5 us a call at L = 4096 and 8.9 in sliding mode at L = 1983 under a serialised launch.
@@ -131,10 +132,21 @@ __global__ void __launch_bounds__(kSelThreads) select_recent_kernel(const Select
             for (int j = 0; j < PER; ++j) c += (h[j] >= (int)v) ? 1 : 0;
             return block_sum(c) >= p.k;
         };
-        // no entry exceeds t, so nothing above since can be the k-th largest when dt = 0
-        long long lo = since, hi = (long long)st.t + 1;   // at_least_k(lo) taken for granted, at_least_k(hi) is false
-        if (lo + 1 < hi && !at_least_k(lo + 1)) hi = lo + 1;
-        else if (lo + 1 < hi) lo = lo + 1;
+        // one count: entries that exceed since, and (upper half word) entries that exceed t, which only a loop that sets t
+        // back without its history leaves behind
+        const long long next = since + 1 < INT32_MIN + 1 ? INT32_MIN + 1 : since + 1 > INT32_MAX ? INT32_MAX : since + 1;
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) c += (h[j] >= (int)next ? 1u : 0u) + (h[j] > st.t ? 0x10000u : 0u);
+        const int counts = block_sum(c);
+        // the threshold is since, or the largest v above it that k entries reach: lo may be it, hi may not
+        long long lo = since, hi = (long long)st.t + 1;
+        if (counts >> 16 >= p.k) {
+            lo = lo > hi ? lo : hi;
+            hi = (long long)INT32_MAX + 1;
+        } else if (lo + 1 < hi) {
+            if ((counts & 0xffff) >= p.k) lo = lo + 1; else hi = lo + 1;
+        }
         while (hi - lo > 1) {
             const long long mid = lo + (hi - lo) / 2;
             if (at_least_k(mid)) lo = mid; else hi = mid;

@@ -76,6 +76,39 @@ def test_many_ties_at_the_threshold():
     _trace(2, 512, 32, 4, n_steps=25, seed=9, n_cap=32 + 480, per_step_max=32)
 
 
+@pytest.mark.parametrize("k,dt", [(1, 0), (3, 0), (3, 1), (3, 5), (6, 2), (7, 4), (12, 9), (40, 30)])
+@pytest.mark.parametrize("sliding", [False, True])
+def test_history_entries_above_the_step_index(k, dt, sliding):
+    """K is the k largest values whatever they are: a loop that sets t back without its history has entries above t
+    (six of them here, two tied, one the largest int32), which decide the threshold when there are k of them or more."""
+    import paper_2603_18489_b200 as ec
+
+    L, block, t, n_cap = 700, 16, 50, 256
+    H = np.full(L, -np.inf)
+    H[:60] = np.arange(1, 61) // 2 + 20                      # 20 .. 50: the steps before t
+    H[[3, 70, 90, 200, 333, 650]] = [t + 1, t + 4, t + 4, t + 30, 2 ** 31 - 1, t + 9]
+    masked = np.ones(L, np.uint8)
+    masked[np.isfinite(H)] = 0
+    window = oracle.sliding_window_rows(masked, block) if sliding else np.arange(400, 400 + block)
+    flags = np.zeros(block, np.uint8)
+    flags[[2, 5]] = 1
+    put = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    hist = put(np.where(np.isfinite(H), H, NEVER).astype(np.int32)[None])
+    state = put(np.array([[t, dt, 1, 0]], np.int32))
+    lst = np.full((1, n_cap), -1, np.int32)
+    lst[0, :block] = window
+    idx, decision = put(lst), torch.zeros(1, dtype=torch.int32, device="cuda")
+    if sliding:
+        ec.ec_select_recent_sliding(hist, state, put(masked[None]), put(flags), block, decision, k, idx)
+        rows, skip, dt2, t2 = oracle.sliding_step_bookkeeping(H, masked.copy(), t, dt, window, flags, 0, k, block)
+    else:
+        ec.ec_select_recent(hist, state, put(flags), put(np.array([400], np.int32)), block, decision, k, idx)
+        R, skip, dt2, t2 = oracle.step_bookkeeping(H, t, dt, window[flags != 0], 0, k)
+        rows = oracle.partial_step_rows(400, block, R)
+    assert state.cpu().numpy()[0].tolist() == [t2, dt2, int(skip), rows.size]
+    assert idx.cpu().numpy()[0, :rows.size].tolist() == rows.tolist()
+
+
 def test_window_outside_the_context_leaves_the_sequence_untouched():
     import paper_2603_18489_b200 as ec
 
