@@ -74,19 +74,15 @@ __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
+// 32 N columns of this thread's TMEM lane as floats
+template <int N>
+__device__ __forceinline__ void tc_ld(uint32_t taddr, float* v) {
+    uint32_t r[32 * N];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+    for (int c = 0; c < N; ++c) tc::ld32(taddr + c * 32, r + c * 32);
+    tc::wait_ld<32 * N>(r);
+#pragma unroll
+    for (int i = 0; i < 32 * N; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const float* v) {
     asm volatile(
@@ -104,7 +100,6 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const float* v) {
           "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])), "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
         : "memory");
 }
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1
@@ -256,9 +251,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
             tc_fence_after();
             float sc[BN];
             const uint32_t s_addr = tmem + lane_addr + (s ? TM_S1 : TM_S0);
-#pragma unroll
-            for (int c = 0; c < BN / 32; ++c) tc_ld32(s_addr + c * 32, sc + c * 32);
-            tc_wait_ld();
+            tc_ld<BN / 32>(s_addr, sc);
 
             const int key0 = (t_begin + j) * BN;
             if (key0 + BN > p.ctx_len) {
@@ -303,8 +296,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 #pragma unroll
                 for (int c = 0; c < HD / 32; ++c) {
                     float o[32];
-                    tc_ld32(tmem + lane_addr + TM_O + c * 32, o);
-                    tc_wait_ld();
+                    tc_ld<1>(tmem + lane_addr + TM_O + c * 32, o);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] *= factor;
                     tc_st32(tmem + lane_addr + TM_O + c * 32, o);
@@ -327,8 +319,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 #pragma unroll
             for (int c = 0; c < HD / 32; ++c) {
                 float o[32];
-                tc_ld32(tmem + lane_addr + TM_O + c * 32, o);
-                tc_wait_ld();
+                tc_ld<1>(tmem + lane_addr + TM_O + c * 32, o);
                 if (valid && !*abort_flag) {   // a CTA whose wait gave up stores nothing
 #pragma unroll
                     for (int v4 = 0; v4 < 4; ++v4) {
@@ -347,8 +338,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 #pragma unroll
             for (int c = 0; c < HD / 32; ++c) {
                 float o[32];
-                tc_ld32(tmem + lane_addr + TM_O + c * 32, o);
-                tc_wait_ld();
+                tc_ld<1>(tmem + lane_addr + TM_O + c * 32, o);
                 if (valid) {
 #pragma unroll
                     for (int v4 = 0; v4 < 8; ++v4)

@@ -262,7 +262,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     if (j == 0) {
                         uint32_t r8[8];
                         ld8(tm_s, r8);
-                        wait_ld();
+                        wait_ld<8>(r8);
                         float mx = __uint_as_float(r8[0]);
 #pragma unroll
                         for (int c = 1; c < 8; ++c)
@@ -273,13 +273,13 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     }
                     uint32_t sr[2][32];
                     ld32(tm_s + h * 64, sr[0]);
-                    wait_ld();
+                    wait_ld<32>(sr[0]);
                     ld32(tm_s + h * 64 + 32, sr[1]);   // on its way while the first 32 scores are worked on
                     const int key0 = (j0 + j) * BN + h * 64;
                     const bool ragged = key0 + 64 > p.ctx_len;
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
-                        if (q == 1) wait_ld();
+                        if (q == 1) wait_ld<32>(sr[1]);
                         if (ragged) {
 #pragma unroll
                             for (int c = 0; c < 32; ++c)
@@ -325,7 +325,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 uint32_t sr[BN / 2];
                 ld32(tm_s + h * 64, sr);
                 ld32(tm_s + h * 64 + 32, sr + 32);
-                wait_ld();
+                wait_ld<64>(sr);
                 const int key0 = (j0 + j) * BN + h * 64;
                 if (key0 + 64 > p.ctx_len) {
 #pragma unroll
@@ -374,7 +374,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     for (int c = 0; c < 2; ++c) {
                         uint32_t o[32];
                         ld32(tm_o + h * 64 + c * 32, o);
-                        wait_ld();
+                        wait_ld<32>(o);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
                         st32(tm_o + h * 64 + c * 32, o);
@@ -404,7 +404,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (int c = 0; c < 2; ++c) {
                     uint32_t o[32];
                     ld32(tm_o + h * 64 + c * 32, o);
-                    wait_ld();
+                    wait_ld<32>(o);
 #pragma unroll
                     for (int v4 = 0; v4 < 4; ++v4) {
                         uint4 w;
@@ -432,7 +432,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (int c = 0; c < 2; ++c) {
                     uint32_t o[32];
                     ld32(tm_o + h * 64 + c * 32, o);
-                    wait_ld();
+                    wait_ld<32>(o);
 #pragma unroll
                     for (int v4 = 0; v4 < 8; ++v4)   // (16-byte pieces swizzled by row: 32 lanes are 32 rows)
                         *reinterpret_cast<uint4*>(prow + (((h * 16 + c * 8 + v4) ^ (row & 31)) << 4)) =

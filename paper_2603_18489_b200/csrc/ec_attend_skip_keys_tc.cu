@@ -107,7 +107,7 @@ __device__ __forceinline__ void ld_row(uint32_t taddr, uint32_t* r) {
 #pragma unroll
         for (int c = 0; c < COLS; c += 16) ld16(taddr + c, r + c);
     }
-    wait_ld();
+    wait_ld<COLS>(r);
 }
 struct KeysParams {
     const __nv_bfloat16* q;
@@ -497,7 +497,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 ld16(s_addr, sr[0]);
 #pragma unroll
                 for (int q = 0; q < NH / 16; ++q) {   // sixteen columns at a time, the next ones on their way
-                    wait_ld16(sr[q & 1]);
+                    wait_ld<16>(sr[q & 1]);
                     if (q + 1 < NH / 16) ld16(s_addr + 16 * (q + 1), sr[(q + 1) & 1]);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -517,7 +517,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
 #pragma unroll
                 for (int q = 0; q < NH / 16; ++q) {
                     ld16(s_addr + 16 * q, sr[0]);
-                    wait_ld16(sr[0]);
+                    wait_ld<16>(sr[0]);
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         const float o = redux_max(past_end ? -INFINITY : __uint_as_float(sr[0][c]));
@@ -541,7 +541,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
 #pragma unroll
                     for (int q = 0; q < NH / 16; ++q) {
                         ld16(o_addr + 16 * q, sr[0]);
-                        wait_ld16(sr[0]);
+                        wait_ld<16>(sr[0]);
 #pragma unroll
                         for (int c = 0; c < 16; ++c)
                             sr[0][c] = __float_as_uint(__uint_as_float(sr[0][c]) * sh->factor[j & 1][c0 + 16 * q + c]);

@@ -87,7 +87,7 @@ enum {
 __device__ __forceinline__ void ld32f(uint32_t taddr, float* v) {
     uint32_t r[32];
     ld32(taddr, r);
-    wait_ld();
+    wait_ld<32>(r);
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -376,7 +376,7 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 fence_after();
                 uint32_t sc[32];
                 ld32(tm_t + (j & 1) * 64 + half * 32, sc);
-                wait_ld();
+                wait_ld<32>(sc);
                 uint32_t gone = 0;   // keys that do not count
                 if (refresh) {
                     if (j == 0) mbar_wait(bar(B_LIST), 0, abort_flag, p.dev_status);
@@ -436,7 +436,7 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                     for (int c = 0; c < 2; ++c) {
                         uint32_t o[32];
                         ld32(tm_t + 128 + half * 64 + c * 32, o);
-                        wait_ld();
+                        wait_ld<32>(o);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
                         st32(tm_t + 128 + half * 64 + c * 32, o);

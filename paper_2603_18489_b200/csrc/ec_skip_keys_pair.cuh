@@ -73,9 +73,7 @@ template <int COLS>
 __device__ __forceinline__ void ld_cols(uint32_t taddr, uint32_t* r) {
 #pragma unroll
     for (int c = 0; c < COLS; c += 8) ld8(taddr + c, r + c);
-    wait_ld();
-#pragma unroll
-    for (int c = 0; c < COLS; ++c) asm volatile("" : "+r"(r[c]));   // nothing that reads them moves in front of the wait
+    wait_ld<COLS>(r);
 }
 
 template <int N>
@@ -303,7 +301,7 @@ __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap&
 #pragma unroll
                     for (int q = 0; q < NH; q += 8) {
                         ld8(o_addr + q, o);
-                        wait_ld();
+                        wait_ld<8>(o);
 #pragma unroll
                         for (int c = 0; c < 8; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * sh->factor[c0 + q + c]);
                         st8(o_addr + q, o);

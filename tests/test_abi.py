@@ -115,3 +115,13 @@ def test_descriptor_flags_are_validated_and_mirror_the_header():
     assert ec.ec_attend_workspace_bytes(bad, 34) == 0 and ec.ec_attend_kernel_name(bad, 34) == ""
     st = ec.lib.ec_attend(ctypes.byref(bad), None, None, None, None, None, None, 34, None, None, 0, None, None)
     assert st == 6                                  # EC_ERR_UNSUPPORTED, before any pointer is looked at
+
+
+def test_tensor_memory_loads_are_waited_for_by_name():
+    """tcgen05.ld completes at tcgen05.wait::ld, but to the compiler its results exist when it is issued: only a wait that
+    names the registers keeps arithmetic on them behind it.  So there is one such wait, it names them, and all use it."""
+    csrc = os.path.join(ROOT, "paper_2603_18489_b200", "csrc")
+    code = {fn: re.sub(r"//[^\n]*", "", open(os.path.join(csrc, fn)).read()) for fn in sorted(os.listdir(csrc))}
+    assert {fn: text.count("tcgen05.wait::ld") for fn, text in code.items() if "tcgen05.wait::ld" in text} == {"ec_tc_ptx.cuh": 1}
+    body = re.search(r"void wait_ld\(uint32_t\* r\) \{(.*?)\n\}", code["ec_tc_ptx.cuh"], re.S).group(1)
+    assert "tcgen05.wait::ld" in body and '"+r"(r[i])' in body
