@@ -22,7 +22,7 @@
 // 8.8 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
 // per clock and SM, measured) and the instructions around it on full ones (two sequences of 1024, 24 heads on 8: 60.2 us
 // when all threads issued the copies, 51.0 with TMA; 36 sequences of 1500, 64 rows, no refresh: 45.3, 38.7).  Every wait
-// is bounded: EC_ERR_TIMEOUT in dev_status, and a CTA whose wait gave up stores no output.
+// is bounded: EC_ERR_TIMEOUT in dev_status, and a CTA whose wait gave up stores no output and no further cache rows.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
@@ -308,7 +308,10 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
             }
         }
         // refreshed keys into the cache, from the landed tile: the row tiles that walk over these keys take turns
-        if (fresh && t % p.row_tiles == row_tile) {
+        // (nothing from a stage whose wait gave up: it holds another tile, or none; unrolled by two, as the whole loop
+        // unrolled cost a partial step without fresh rows 0.16 of 7.5 us a layer)
+        if (fresh && t % p.row_tiles == row_tile && !(kTma && *abort_flag)) {
+#pragma unroll 2
             for (int c = tid; c < BN * CHUNKS; c += kThreads) {
                 const int row = c / CHUNKS, ch = c % CHUNKS, key = key0 + row;
                 if (key >= p.ctx_len || (mapped && map[key - key_lo] < 0)) continue;
