@@ -31,22 +31,20 @@ int sm_count() {
 
 namespace {
 
-// bf16 with head_dim 128 runs on the tcgen05 kernels (the fused skip-step kernel when the packed
-// query rows fit two M tiles, the dense kernel otherwise); everything else bf16 on the mma.sync kernel.
-// EC_ATTEND_IMPL (environment, read once) = "mma" forces the mma.sync kernel, "dense" the one-tile dense
-// tcgen05 kernel with a separate refresh launch, "rows" the skip kernel with query rows on the M axis: for A/B
-// measurements only.
+// bf16 with head_dim 128 runs on the tcgen05 kernels (a fused skip-step kernel when the packed query rows fit, a dense
+// kernel otherwise), bf16 with head_dim 64 on the mma.sync kernel, fp32 on the SIMT kernel.
+// EC_ATTEND_IMPL (environment, read once) = "dense" forces the one-tile dense tcgen05 kernel with a separate refresh
+// launch, "rows" the skip kernel with query rows on the M axis: for A/B measurements only.
 int forced_impl() {
     static const int f = [] {
         const char* e = std::getenv("EC_ATTEND_IMPL");
-        if (e && std::strcmp(e, "mma") == 0) return 1;
         if (e && std::strcmp(e, "dense") == 0) return 2;
         if (e && std::strcmp(e, "rows") == 0) return 3;
         return 0;
     }();
     return f;
 }
-bool use_tc(const ec_attn_desc& d) { return d.dtype == EC_BF16 && d.head_dim == 128 && forced_impl() != 1; }
+bool use_tc(const ec_attn_desc& d) { return d.dtype == EC_BF16 && d.head_dim == 128; }
 bool use_skip_keys(const ec_attn_desc& d, int n_active, bool fresh) {
     return forced_impl() == 0 && attend_skip_keys_supported(d, n_active, fresh);
 }

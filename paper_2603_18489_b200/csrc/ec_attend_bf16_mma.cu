@@ -1,4 +1,4 @@
-// ec_attend, bf16 storage, warp-level tensor-core path (mma.sync m16n8k16, fp32
+// ec_attend, bf16 storage, heads of 64, warp-level tensor-core path (mma.sync m16n8k16, fp32
 // accumulation): refresh and active-row bidirectional attention over the full cache
 // (Appendix A of the paper, partial branch; the full branch when n_active == L) in ONE launch.
 //
@@ -12,7 +12,7 @@
 //     (m, l, O) un-normalised in its shared memory and, after a cluster barrier, merges a share
 //     of the rows out of its peers' (partials in global memory and a second launch took 5.4 us more).
 //   - K/V tiles are staged in shared memory, XOR-swizzled so ldmatrix is bank-conflict free: by TMA, a box each, when
-//     no index list sends keys elsewhere and heads are 64 wide (the 128-byte swizzle of a 128-byte row is the same
+//     no index list sends keys elsewhere (the 128-byte swizzle of a 128-byte row is the same
 //     XOR); else with 16-byte cp.async copies.  A key that is being refreshed is read from k_new / v_new (a table of
 //     the CTA's keys, filled from the index list), so nothing waits for the cache update; the row
 //     tiles of a kv head share the writing of the cache.
@@ -32,10 +32,10 @@ namespace {
 constexpr int BM = 64;   // query rows per CTA
 constexpr int BN = 64;   // keys per tile
 constexpr int kThreads = 128;
+constexpr int D = 64;    // head_dim
 // K/V stages in shared memory.  A tile computes in about half the time its data takes to arrive, so two tiles have to be
-// on their way (9.5 us against 13.4 with one); with 128-wide heads two stages are what fits two CTAs per SM.
-template <int D>
-__host__ __device__ constexpr int stages() { return D == 64 ? 3 : 2; }
+// on their way (9.5 us against 13.4 with one).
+constexpr int ST = 3;
 constexpr int kMaxMapKeys = 8192;   // keys of one CTA beyond which the refresh is a launch of its own
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -70,7 +70,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 // byte offset of 16-byte chunk `chunk` of row `row` in a swizzled [rows, D] bf16 tile
-template <int D>
 __device__ __forceinline__ uint32_t swz(int row, int chunk) {
     return (uint32_t)(row * (D * 2) + ((chunk ^ (row & 7)) << 4));
 }
@@ -91,15 +90,14 @@ struct MmaParams {
 };
 
 // kSpare: the last warp has no rows.  kTma: K/V tiles come by TMA, one box each in the very layout that swz() describes
-// (no index list, so no key is sent elsewhere; 64-wide heads, whose rows are the 128 bytes of the swizzle).
-template <int D, bool kSpare, bool kTma>
-__global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(const MmaParams p, const __grid_constant__ CUtensorMap map_k,
-                                                                                    const __grid_constant__ CUtensorMap map_v) {
+// (no index list, so no key is sent elsewhere; a row is the 128 bytes of the swizzle).
+template <bool kSpare, bool kTma>
+__global__ void __launch_bounds__(kThreads, 3) attend_mma_kernel(const MmaParams p, const __grid_constant__ CUtensorMap map_k,
+                                                                  const __grid_constant__ CUtensorMap map_v) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + (kTma ? -smem_u32(smem_raw) & 1023u : 0u);
     constexpr int TILE_BYTES = BN * D * 2;
     constexpr int CHUNKS = D / 8;  // 16-byte chunks per row
-    constexpr int ST = stages<D>();
     unsigned char* sQ = smem;                       // BM x D
     unsigned char* sK = smem + BM * D * 2;          // ST stages
     unsigned char* sV = sK + ST * TILE_BYTES;       // ST stages
@@ -174,8 +172,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
                         vs = p.v_new + new0 + (long long)i * new_stride;
                     }
                 }
-                cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz<D>(row, ch), ks + ch * 8, ok);
-                cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz<D>(row, ch), vs + ch * 8, ok);
+                cp_async16(smem_u32(sK) + stage * TILE_BYTES + swz(row, ch), ks + ch * 8, ok);
+                cp_async16(smem_u32(sV) + stage * TILE_BYTES + swz(row, ch), vs + ch * 8, ok);
             }
         }
     };
@@ -187,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
 #pragma unroll
     for (int k = 0; k < QN; ++k) {
         const int c = tid + k * kThreads;
-        cp_async16(smem_u32(sQ) + swz<D>(c / CHUNKS, c % CHUNKS), p.q + max(q_at[k], 0LL), q_at[k] >= 0);
+        cp_async16(smem_u32(sQ) + swz(c / CHUNKS, c % CHUNKS), p.q + max(q_at[k], 0LL), q_at[k] >= 0);
     }
     if (mapped) {
         for (int i = tid; i < p.n_active; i += kThreads) {
@@ -227,7 +225,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
                 q_loaded = true;
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks)
-                    ldsm_x4(smem_u32(sQ) + swz<D>(warp * 16 + (lane & 15), ks * 2 + (lane >> 4)), qf[ks]);
+                    ldsm_x4(smem_u32(sQ) + swz(warp * 16 + (lane & 15), ks * 2 + (lane >> 4)), qf[ks]);
             }
 
             // ---- S = Q K^T --------------------------------------------------------------
@@ -241,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
                 for (int nb = 0; nb < BN / 16; ++nb) {
                     uint32_t kf[4];
                     const int key = nb * 16 + (lane & 7) + ((lane >> 4) << 3);
-                    ldsm_x4(kst + swz<D>(key, ks * 2 + ((lane >> 3) & 1)), kf);
+                    ldsm_x4(kst + swz(key, ks * 2 + ((lane >> 3) & 1)), kf);
                     mma_bf16(s[2 * nb], qf[ks], kf[0], kf[1]);
                     mma_bf16(s[2 * nb + 1], qf[ks], kf[2], kf[3]);
                 }
@@ -301,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
 #pragma unroll
                 for (int db = 0; db < D / 16; ++db) {
                     uint32_t vf[4];
-                    ldsm_x4_t(vst + swz<D>(ks * 16 + (lane & 15), db * 2 + (lane >> 4)), vf);
+                    ldsm_x4_t(vst + swz(ks * 16 + (lane & 15), db * 2 + (lane >> 4)), vf);
                     mma_bf16(o[2 * db], pf, vf[0], vf[1]);
                     mma_bf16(o[2 * db + 1], pf, vf[2], vf[3]);
                 }
@@ -316,8 +314,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 ? 3 : 2) attend_mma_kernel(c
                 const int row = c / CHUNKS, ch = c % CHUNKS, key = key0 + row;
                 if (key >= p.ctx_len || (mapped && map[key - key_lo] < 0)) continue;
                 const long long at = ((long long)bh * p.ctx_len + key) * D + ch * 8;
-                *reinterpret_cast<uint4*>(p.k_cache + at) = *reinterpret_cast<const uint4*>(sK + stage * TILE_BYTES + swz<D>(row, ch));
-                *reinterpret_cast<uint4*>(p.v_cache + at) = *reinterpret_cast<const uint4*>(sV + stage * TILE_BYTES + swz<D>(row, ch));
+                *reinterpret_cast<uint4*>(p.k_cache + at) = *reinterpret_cast<const uint4*>(sK + stage * TILE_BYTES + swz(row, ch));
+                *reinterpret_cast<uint4*>(p.v_cache + at) = *reinterpret_cast<const uint4*>(sV + stage * TILE_BYTES + swz(row, ch));
             }
         }
     }
@@ -405,7 +403,7 @@ Plan make_plan(const ec_attn_desc& d, int n_active) {
     const int g = d.n_q_heads / d.n_kv_heads;
     pl.rows_total = n_active * g;
     pl.row_tiles = (pl.rows_total + BM - 1) / BM;
-    pl.tile_rows = d.head_dim == 64 && pl.row_tiles > 1 && pl.rows_total <= 48 * pl.row_tiles ? 48 : BM;
+    pl.tile_rows = pl.row_tiles > 1 && pl.rows_total <= 48 * pl.row_tiles ? 48 : BM;
     const int key_tiles = (d.ctx_len + BN - 1) / BN;
     const long long base = (long long)pl.row_tiles * d.batch * d.n_kv_heads;
     int splits = (int)(3LL * sm_count() / base);
@@ -430,8 +428,8 @@ bool make_tile_map(CUtensorMap* map, const void* ptr, const ec_attn_desc& d, boo
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, bool kSpare, bool kTma>
-cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, const void* v_new, const int32_t* active_idx,
+template <bool kSpare, bool kTma>
+cudaError_t launch_d64(const AttendArgs& a, const Plan& pl, const void* k_new, const void* v_new, const int32_t* active_idx,
                      cudaStream_t stream) {
     MmaParams p;
     p.q = static_cast<const __nv_bfloat16*>(a.q);
@@ -463,10 +461,10 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
         p.k_new = p.v_new = nullptr;
         map_keys = 0;
     }
-    constexpr int smem = (BM + 2 * stages<D>() * BN) * D * 2 + BM * (int)sizeof(float2) + 8 * (stages<D>() + 1) + (kTma ? 1024 : 0);
+    constexpr int smem = (BM + 2 * ST * BN) * D * 2 + BM * (int)sizeof(float2) + 8 * (ST + 1) + (kTma ? 1024 : 0);
     static_assert(BM * (D + 8) * 4 <= 4 * BN * D * 2, "the partial of the merge fits over the stages");
     static PerDeviceOnce attr_once;
-    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<D, kSpare, kTma>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
+    if (const cudaError_t ea = ensure_dynamic_smem(attr_once, attend_mma_kernel<kSpare, kTma>, smem + kMaxMapKeys * 4); ea != cudaSuccess) return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -485,7 +483,7 @@ cudaError_t launch_d(const AttendArgs& a, const Plan& pl, const void* k_new, con
     if (kTma && (!make_tile_map(&map_k, p.k_new ? k_new : a.k_cache, a.d, p.k_new) ||
                  !make_tile_map(&map_v, p.v_new ? v_new : a.v_cache, a.d, p.v_new)))
         return cudaErrorInvalidValue;
-    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<D, kSpare, kTma>, p, map_k, map_v);
+    return cudaLaunchKernelEx(&cfg, attend_mma_kernel<kSpare, kTma>, p, map_k, map_v);
 }
 
 }  // namespace
@@ -494,13 +492,12 @@ cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const voi
                                cudaStream_t stream) {
     if (a.n_active == 0) return cudaSuccess;
     const Plan pl = make_plan(a.d, a.n_active);
-    if (a.d.head_dim == 128) return launch_d<128, false, false>(a, pl, k_new, v_new, active_idx, stream);
     const bool spare = pl.tile_rows < BM;
     if (k_new && active_idx)
-        return spare ? launch_d<64, true, false>(a, pl, k_new, v_new, active_idx, stream)
-                     : launch_d<64, false, false>(a, pl, k_new, v_new, active_idx, stream);
-    return spare ? launch_d<64, true, true>(a, pl, k_new, v_new, active_idx, stream)
-                 : launch_d<64, false, true>(a, pl, k_new, v_new, active_idx, stream);
+        return spare ? launch_d64<true, false>(a, pl, k_new, v_new, active_idx, stream)
+                     : launch_d64<false, false>(a, pl, k_new, v_new, active_idx, stream);
+    return spare ? launch_d64<true, true>(a, pl, k_new, v_new, active_idx, stream)
+                 : launch_d64<false, true>(a, pl, k_new, v_new, active_idx, stream);
 }
 
 }  // namespace ec

@@ -63,17 +63,15 @@ enum { B_FULL = 0, B_EMPTY = kSlots, B_SFULL = 2 * kSlots, B_PFULL = B_SFULL + 2
 constexpr float kMaxSum = 1.152921504606846976e18f;   // 2^60
 
 struct DenseParams {
-    const __nv_bfloat16* q;
     __nv_bfloat16* out;
     // recompute step: the K/V this launch reads are the token-major fresh tensors [B, L, Hkv, 128]; its copy warp
     // stores their tiles into the caches [B, Hkv, L, 128]
     int copy;
     int32_t* dev_status;
-    int n_active, ctx_len, n_q_heads, n_kv_heads, group, rows_total;
-    // Grouped-query shapes run with one unit per QUERY head (the kernel then sees n_kv_heads = n_q_heads = H_q and
-    // group = 1, so its row tiles are 128 active rows of one head and come by TMA); the K/V of unit head h are
-    // those of the real kv head h / kv_div, of which there are n_kv_real.  kv_div = 1 otherwise.
-    int kv_div, n_kv_real;
+    int n_active, ctx_len, n_q_heads, n_kv_heads, rows_total;
+    // Grouped-query shapes run with one unit per QUERY head (the kernel's n_kv_heads is H_q, so its row tiles are 128
+    // active rows of one head and come by TMA); the K/V of unit head h are those of the real kv head h / kv_div.
+    int kv_div;
     float scale_log2;
     // Unit order = row-tile pair fastest, then head.  The first n_full units are whole; each later one (what would be
     // the last, partial wave of the launch) is cut along the keys into `split` CTAs, a cluster of the second launch.
@@ -627,7 +625,6 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
         !make_kv_map(&map_v, a.v_cache, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, a.kv_token_major))
         return cudaErrorInvalidValue;
     DenseParams p;
-    p.q = static_cast<const __nv_bfloat16*>(a.q);
     p.out = static_cast<__nv_bfloat16*>(a.out);
     p.copy = a.kv_token_major && a.refresh_k_dst && a.refresh_v_dst;
     CUtensorMap map_kd = map_k, map_vd = map_v;   // placeholders unless copying
@@ -639,10 +636,8 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     p.ctx_len = a.d.ctx_len;
     p.n_q_heads = a.d.n_q_heads;
     p.n_kv_heads = a.d.n_q_heads;   // the kernel's heads are the query heads, see kv_div
-    p.group = 1;
     p.rows_total = a.n_active;
     p.kv_div = a.d.n_q_heads / a.d.n_kv_heads;
-    p.n_kv_real = a.d.n_kv_heads;
     p.scale_log2 = a.scale * kLog2e;
     const DensePlan pl = make_dense_plan(a.d, a.n_active);
     p.n_pairs = pl.n_pairs;

@@ -49,12 +49,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-__device__ __forceinline__ float fast_log2(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // ---- internal launchers (host), one per translation unit ------------------
 struct GateArgs {
     const void* logits;
@@ -120,7 +114,7 @@ struct AttendArgs {
 // fp32: refresh and attention in one launch (k_new == nullptr: attention alone)
 cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                               cudaStream_t stream);
-// mma.sync path (any head_dim): refresh and attention in one launch (k_new == nullptr: attention alone)
+// mma.sync path (head_dim 64): refresh and attention in one launch (k_new == nullptr: attention alone)
 cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                cudaStream_t stream);
 // fused skip-step path (bf16, head_dim 128, n_active * H_q/H_kv <= 256): refresh + attention + merge in one launch

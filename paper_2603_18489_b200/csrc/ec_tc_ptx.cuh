@@ -227,10 +227,6 @@ __device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst_cluster), "r"(src_local), "r"(bytes), "r"(bar_cluster) : "memory");
 }
-// plain store into a peer CTA's shared memory (address from map_to_cta); made visible by the cluster barrier
-__device__ __forceinline__ void st_peer_f32(uint32_t addr_cluster, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr_cluster), "f"(v) : "memory");
-}
 // loads from a peer CTA's shared memory (address from map_to_cta)
 __device__ __forceinline__ void ld_peer_v4(uint32_t addr_cluster, float* r) {
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(addr_cluster) : "memory");
@@ -238,7 +234,6 @@ __device__ __forceinline__ void ld_peer_v4(uint32_t addr_cluster, float* r) {
 __device__ __forceinline__ void ld_peer_v2(uint32_t addr_cluster, float& a, float& b) {
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(addr_cluster) : "memory");
 }
-__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 // named barrier over n_threads threads that also ORs a predicate across them
 __device__ __forceinline__ bool named_barrier_or(int id, int n_threads, bool pred) {
     uint32_t r;
