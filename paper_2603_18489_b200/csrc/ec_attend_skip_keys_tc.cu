@@ -693,20 +693,6 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
 }
 
 // ---- host side ---------------------------------------------------------------------------
-// cache [B*Hkv, L, 128] bf16 seen as 4-D {64 columns, key, half, head}: one box {64, 128, 2, 1} lands as
-// [half][key][64 columns], the two 128-byte-swizzled halves of a [128 keys x 128] tile; keys beyond L read as zero
-bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[4] = {64, (cuuint64_t)ctx_len, 2, (cuuint64_t)bh};
-    const cuuint64_t strides[3] = {(cuuint64_t)HD * 2, 128, (cuuint64_t)ctx_len * HD * 2};
-    const cuuint32_t box[4] = {64, (cuuint32_t)BK, 2, 1};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(cache), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 struct KeysPlan {
     bool ok;
     int group, rows_chunk, n_sub_r, n_sub;   // heads and active rows per CTA column, row chunks, CTA columns per kv head
@@ -883,22 +869,6 @@ KeysPlan make_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
     return plan;
 }
 
-// k_new / v_new [B, n, H_kv, 128] bf16 seen as 5-D {64 columns, active row, half, kv head, sequence}: one box
-// {64, 128, 2, 1, 1} lands as [half][row][64 columns], i.e. exactly like a cache tile whose keys are the active rows
-// 128 j .. 128 j + 127 of one kv head; rows past n read as zero
-bool make_fresh_map(CUtensorMap* map, const void* fresh, int batch, int n_active, int n_kv_heads) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[5] = {64, (cuuint64_t)n_active, 2, (cuuint64_t)n_kv_heads, (cuuint64_t)batch};
-    const cuuint64_t strides[4] = {(cuuint64_t)n_kv_heads * HD * 2, 128, (cuuint64_t)HD * 2,
-                                   (cuuint64_t)n_active * n_kv_heads * HD * 2};
-    const cuuint32_t box[5] = {64, (cuuint32_t)BK, 2, 1, 1};
-    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(fresh), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // bytes per nanosecond assumed for a streaming read when spacing the first ring fill: 0.7 of the nominal rate of the
 // device (clock x bus width, double data rate; a spacing between 1.0 and 1.3 times the measured copy rate's stage
 // time timed best), cached per device
@@ -972,12 +942,12 @@ cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, cons
     if (!pl.ok) return cudaErrorInvalidConfiguration;
     const int bh = a.d.batch * a.d.n_kv_heads;
     CUtensorMap map_k, map_v;
-    if (!make_cache_map(&map_k, a.k_cache, bh, a.d.ctx_len) || !make_cache_map(&map_v, a.v_cache, bh, a.d.ctx_len))
+    if (!make_cache_map(&map_k, a.k_cache, bh, a.d.ctx_len, BK) || !make_cache_map(&map_v, a.v_cache, bh, a.d.ctx_len, BK))
         return cudaErrorInvalidValue;
     KeysParams p{};
     CUtensorMap map_kn = map_k, map_vn = map_v;   // placeholders unless fresh
-    if (fresh && (!make_fresh_map(&map_kn, k_new, a.d.batch, a.n_active, a.d.n_kv_heads) ||
-                  !make_fresh_map(&map_vn, v_new, a.d.batch, a.n_active, a.d.n_kv_heads)))
+    if (fresh && (!make_fresh_map(&map_kn, k_new, a.d.batch, a.n_active, a.d.n_kv_heads, BK) ||
+                  !make_fresh_map(&map_vn, v_new, a.d.batch, a.n_active, a.d.n_kv_heads, BK)))
         return cudaErrorInvalidValue;
     p.q = static_cast<const __nv_bfloat16*>(a.q);
     p.k_new = static_cast<const __nv_bfloat16*>(k_new);

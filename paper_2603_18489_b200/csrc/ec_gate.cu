@@ -83,23 +83,11 @@ __device__ __forceinline__ int ticket_add(int* addr, int v) {
     return old;
 }
 // packed pairs of fp32 (one 64-bit register): two lanes per FMA / add issue slot
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
+using tc::add2;
+using tc::f32x2;
+using tc::fma2;
+using tc::pk;
+using tc::upk;
 __device__ __forceinline__ unsigned int max_bf16x2(unsigned int a, unsigned int b) {
     unsigned int d;
     asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -138,7 +126,7 @@ struct Loader<__nv_bfloat16> {
     static __device__ __forceinline__ void widen2(const uint4& u, f32x2 (&x)[4]) {
         const unsigned int w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+        for (int i = 0; i < 4; ++i) x[i] = pk(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
     }
     static __device__ __forceinline__ float one(const __nv_bfloat16* p) {
         return fmaxf(__bfloat162float(*p), __uint_as_float(kXMinF32));
@@ -167,8 +155,8 @@ struct Loader<float> {
         x[2] = __uint_as_float(u.z); x[3] = __uint_as_float(u.w);
     }
     static __device__ __forceinline__ void widen2(const uint4& u, f32x2 (&x)[2]) {
-        x[0] = pack2(__uint_as_float(u.x), __uint_as_float(u.y));
-        x[1] = pack2(__uint_as_float(u.z), __uint_as_float(u.w));
+        x[0] = pk(__uint_as_float(u.x), __uint_as_float(u.y));
+        x[1] = pk(__uint_as_float(u.z), __uint_as_float(u.w));
     }
     static __device__ __forceinline__ float one(const float* p) { return fmaxf(*p, __uint_as_float(kXMinF32)); }
 };
@@ -263,34 +251,34 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
 
     // running state: maximum, exponent base, and S, T as two packed lanes each
     float m = -INFINITY, base = base_of(-INFINITY);
-    f32x2 S2 = pack2(0.f, 0.f), T2 = pack2(0.f, 0.f);
+    f32x2 S2 = pk(0.f, 0.f), T2 = pk(0.f, 0.f);
     int mat = -1;               // the vector (the first of the pair) that raised the maximum last
-    const f32x2 kL2 = pack2(kLog2e, kLog2e);
+    const f32x2 kL2 = pk(kLog2e, kLog2e);
     auto rebase_if_needed = [&](float vmax) {
         if (fmaf(vmax, kLog2e, -base) > kRebase) {   // rare
             const float nb = base_of(vmax);
             const float dl = fmaxf(base - nb, kDClamp);
             const float c = fast_exp2(dl);
             float s0, s1, t0, t1;
-            unpack2(S2, s0, s1);
-            unpack2(T2, t0, t1);
+            upk(S2, s0, s1);
+            upk(T2, t0, t1);
             t0 = s0 > 0.f ? c * fmaf(dl, s0, t0) : 0.f;
             t1 = s1 > 0.f ? c * fmaf(dl, s1, t1) : 0.f;
-            S2 = pack2(s0 * c, s1 * c);
-            T2 = pack2(t0, t1);
+            S2 = pk(s0 * c, s1 * c);
+            T2 = pk(t0, t1);
             base = nb;
         }
     };
     auto add = [&](const uint4& v) {
-        const f32x2 nb2 = pack2(-base, -base);
+        const f32x2 nb2 = pk(-base, -base);
         f32x2 x2[EPV / 2];
         L::widen2(v, x2);
 #pragma unroll
         for (int e = 0; e < EPV / 2; ++e) {
             const f32x2 d2 = fma2(x2[e], kL2, nb2);
             float d0, d1;
-            unpack2(d2, d0, d1);
-            const f32x2 e2 = pack2(fast_exp2(d0), fast_exp2(d1));
+            upk(d2, d0, d1);
+            const f32x2 e2 = pk(fast_exp2(d0), fast_exp2(d1));
             S2 = add2(S2, e2);
             T2 = fma2(e2, d2, T2);
         }
@@ -345,12 +333,12 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
             tail_col = x > m ? col : -1;
             m = fmaxf(m, x);
             float s0, s1, t0, t1;
-            unpack2(S2, s0, s1);
-            unpack2(T2, t0, t1);
+            upk(S2, s0, s1);
+            upk(T2, t0, t1);
             const float d = fmaf(x, kLog2e, -base);
             const float e = fast_exp2(d);
-            S2 = pack2(s0 + e, s1);
-            T2 = pack2(fmaf(e, d, t0), t1);
+            S2 = pk(s0 + e, s1);
+            T2 = pk(fmaf(e, d, t0), t1);
         }
     }
 
@@ -384,8 +372,8 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
     float S, Tt;
     {
         float s0, s1, t0, t1;
-        unpack2(S2, s0, s1);
-        unpack2(T2, t0, t1);
+        upk(S2, s0, s1);
+        upk(T2, t0, t1);
         S = s0 + s1;
         Tt = t0 + t1;
     }

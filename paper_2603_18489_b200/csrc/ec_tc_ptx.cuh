@@ -310,5 +310,36 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// ---- host: tensor maps of the skip-step kernels (128-wide heads: rows of 256 bytes) ----
+// cache [B*Hkv, L, 128] bf16 seen as 4-D {64 columns, key, half, head}: one box {64, box_keys, 2, 1}
+// lands as [half][key][64 columns], i.e. the two 128-byte-swizzled halves of a [box_keys x 128] tile back to back;
+// keys beyond L read as zero
+inline bool make_cache_map(CUtensorMap* map, const void* cache, int bh, int ctx_len, int box_keys) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[4] = {64, (cuuint64_t)ctx_len, 2, (cuuint64_t)bh};
+    const cuuint64_t strides[3] = {256, 128, (cuuint64_t)ctx_len * 256};
+    const cuuint32_t box[4] = {64, (cuuint32_t)box_keys, 2, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(cache), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// k_new / v_new [B, n, H_kv, 128] bf16 seen as 5-D {64 columns, active row, half, kv head, sequence}: one box
+// {64, box_rows, 2, 1, 1} lands like a cache tile whose keys are active rows of one kv head; rows past n read as zero
+inline bool make_fresh_map(CUtensorMap* map, const void* fresh, int batch, int n_active, int n_kv_heads, int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)n_active, 2, (cuuint64_t)n_kv_heads, (cuuint64_t)batch};
+    const cuuint64_t strides[4] = {(cuuint64_t)n_kv_heads * 256, 128, 256,
+                                   (cuuint64_t)n_active * n_kv_heads * 256};
+    const cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 2, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(fresh), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tc
 }  // namespace ec
