@@ -27,6 +27,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import subprocess
 import sys
 import threading
@@ -50,22 +51,22 @@ K64_WORKLOADS = ("c4_llada_l2048", "c5_llada_l4096", "c5_llada_l4096_b8", "c5_dr
 
 
 # DRAM traffic per launch (reads + writes: dram__bytes.sum.per_second x gpu__time_duration.sum) from the ncu captures
-# summarised under profiles/.  A figure is reported only while the kernel's source file still has the hash it had when the
+# summarised under profiles/.  A figure is reported only while the kernel's source files still have the hash they had when the
 # counters were taken; after any change to the kernel it reads null until the capture is redone.
 NCU_TRAFFIC = {
     "attend_skip": [
-        {"source": "paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",
+        {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",),
          "sha256": "6fd3dc0f298c46a576d57bd3540f12bcb9168ab693ffffbbac8922c8510713b7",
          "bytes_per_launch": {"c5_llada_l4096": 68160000}},
-        {"source": "paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu",
+        {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu", "paper_2603_18489_b200/csrc/ec_skip_keys_pair.cuh"),
          "sha256": "65b46cc75830b8e859285087271c6c5b40faae59a005274755dbc82fd63d76b5",
          "bytes_per_launch": {"c5_llada_l4096_b8": 558740000}}],
     "attend_dense": [
-        {"source": "paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",
+        {"sources": ("paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",),
          "sha256": "7a98a8f43f1813c6b2c2e415eaa10ef757f463c24264f763c784fb25d2ae37a6",
          "bytes_per_launch": {"c5_llada_l4096": 146620000}}],
     "entropy_gate": [
-        {"source": "paper_2603_18489_b200/csrc/ec_gate.cu",
+        {"sources": ("paper_2603_18489_b200/csrc/ec_gate.cu",),
          "sha256": "026fe97ffd51bbd366852fdac150195f9cf2765f3cd9db49fa97c7109723dbe2",
          "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65710000}}],
 }
@@ -78,7 +79,7 @@ def _ncu_traffic(kernel: str, workload: str):
         if workload not in e["bytes_per_launch"]:
             continue
         try:
-            h = hashlib.sha256(open(os.path.join(ROOT, e["source"]), "rb").read()).hexdigest()
+            h = hashlib.sha256(b"".join(open(os.path.join(ROOT, f), "rb").read() for f in e["sources"])).hexdigest()
         except OSError:
             return None
         return e["bytes_per_launch"][workload] if h == e["sha256"] else None
@@ -399,10 +400,19 @@ def run_reference(args) -> None:
 # --------------------------------------------------------------------------- #
 # main arm
 # --------------------------------------------------------------------------- #
+def _attend_launches(name: str) -> int:
+    """Kernels that one ec_attend launches, from its own description of the call (the fp32 and 64-wide kernels refresh
+    inside their one launch)."""
+    m = re.search(r"whole_units=(\d+) cut_units=(\d+)x", name)
+    n = (int(m[1]) > 0) + (int(m[2]) > 0) if m else 1
+    return n + (name.startswith("refresh_kernel + ") and ("attend_dense" in name or "attend_tc" in name))
+
+
 def _rooflines(wl: "DeviceWorkload", peaks: dict, ms_skip_launch: float, ms_rec_launch: float, ms_gate: float) -> dict:
     """The three roofline objects of a workload from the average launch durations (milliseconds) of its regions.
     Units of one launch: skip = one layer-step of the whole batch (refresh + attention + merge: skip_bytes),
-    recompute = one layer-step (recompute_flops; its refresh copy rides in the same launch), gate = R rows."""
+    recompute = one layer-step (recompute_flops; one launch, or two where the last wave is cut, with the refresh copy
+    inside), gate = R rows."""
     w = wl.w
     skip_b, rec_f, gate_b = wl.skip_bytes(), wl.recompute_flops(), wl.gate_bytes()
     att_gbs = skip_b / (ms_skip_launch * 1e-3) / 1e9
@@ -413,7 +423,7 @@ def _rooflines(wl: "DeviceWorkload", peaks: dict, ms_skip_launch: float, ms_rec_
                      "achieved": att_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": att_gbs / peaks["hbm_gbs"],
                      "traffic": _ncu_traffic("attend_skip", w.name), "algorithmic_bytes": skip_b,
                      "us_per_launch": ms_skip_launch * 1e3, "peak_source": peaks["source"]},
-        "roofline_recompute": {"kernel": "ec_attend recompute step (one launch: attention + cache rewrite)",
+        "roofline_recompute": {"kernel": "ec_attend recompute step (attention + cache rewrite: one launch, two where the last wave is cut)",
                                "bound": "tensor", "achieved": rec_tf, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                                "frac": rec_tf / peaks["bf16_tflops"], "traffic": _ncu_traffic("attend_dense", w.name),
                                "algorithmic_flops": rec_f, "us_per_launch": ms_rec_launch * 1e3,
@@ -562,13 +572,14 @@ def run_cuda(args) -> None:
     us_rec = ms_rec * 1e3 / n_layers / world
     cpu = _oracle_layer_step_us(w, 2)
     cfg = _config(w, n_layers)
+    wl_names = wl.kernel_names()
     line = {
         "metric": "us_per_layer_step_skip", "value": us_skip, "unit": "us", "n_gpus": world, "steps": K,
         "warmup": W, "ms_per_step": ms_skip, "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": "bf16" if w.dtype == syn.BF16 else "f32", "data": "synthetic",
         "config": cfg,
         "timing": "one CUDA graph per step, CUDA events on the launching stream, max over ranks",
-        "kernels": wl.kernel_names(),
+        "kernels": wl_names,
         "recompute": {"us_per_layer_step": us_rec, "ms_per_step": ms_rec,
                       "skip_over_recompute": us_skip / us_rec},
         "kernels_us": {"attend_skip": ms_att_skip * 1e3, "attend_skip_without_refresh": ms_att_only * 1e3,
@@ -577,7 +588,8 @@ def run_cuda(args) -> None:
                        "kv_refresh_skip": ms_refresh * 1e3, "select_recent": ms_select * 1e3},
         "e2e": {"value": ms_e2e * 1e3 / n_layers / world, "unit": "us", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
-        "gpu_launches": K * (n_layers + 1),   # a skip layer-step is one launch (refresh + attention + merge), + the gate
+        # the skip step: a layer is one launch (refresh + attention + merge), + the gate
+        "gpu_launches": K * (n_layers * _attend_launches(wl_names["skip"]) + 1),
         "clocks": clocks,
     }
     line.update(_rooflines(wl, peaks, ms_att_skip, ms_att_rec, ms_gate))
@@ -734,8 +746,12 @@ def _run_trace(args, torch, w, dev) -> None:
         E.append(maxh.cpu().numpy().copy())
     tau = float(np.quantile(np.concatenate(E), 0.85))
 
+    n_launch = {(nb, full): _attend_launches(ec.ec_attend_kernel_name(ec.make_desc(nb, L, Hq, Hkv, D, w.dtype),
+                                                                      L if full else q_s.shape[1], True, not full))
+                for nb in range(1, B + 1) for full in (False, True)}
+
     def attend(group, full: bool, layer: int):
-        """One ec_attend per maximal run of consecutive sequences of the group."""
+        """One ec_attend per maximal run of consecutive sequences of the group; returns the kernels launched."""
         for b0, nb in syn.consecutive_runs(group):
             d = ec.make_desc(nb, L, Hq, Hkv, D, w.dtype)
             sl = slice(b0, b0 + nb)
@@ -745,7 +761,7 @@ def _run_trace(args, torch, w, dev) -> None:
             else:
                 ec.ec_attend(d, q_s[sl], kn_s[sl], vn_s[sl], kc[layer][sl], vc[layer][sl], idx[sl], out=out_s[sl],
                              workspace=ws)
-        return len(syn.consecutive_runs(group))
+        return sum(n_launch[nb, full] for _, nb in syn.consecutive_runs(group))
 
     ev = lambda: torch.cuda.Event(enable_timing=True)
     decisions = np.ones(B, np.int64)   # step 1 is a full pass for every sequence
@@ -852,6 +868,9 @@ def _run_trace_sliding(args, torch, w, dev) -> None:
     ev = lambda: torch.cuda.Event(enable_timing=True)
     skip = np.zeros(B, bool)                    # step 1 is a full pass for every sequence
     t_skip = t_rec = t_book = 0.0
+    n_launch = {(nb, full): _attend_launches(ec.ec_attend_kernel_name(ec.make_desc(nb, L, Hq, Hkv, D, w.dtype),
+                                                                      L if full else q_s.shape[1], True, not full))
+                for nb in range(1, B + 1) for full in (False, True)}
     n_skip = n_rec = launches = over_cap = 0
     per_step = []
     torch.cuda.synchronize()
@@ -865,14 +884,14 @@ def _run_trace_sliding(args, torch, w, dev) -> None:
                 sl = slice(b0, b0 + nb)
                 ec.ec_attend(ec.make_desc(nb, L, Hq, Hkv, D, w.dtype), q_s[sl], kn_s[sl], vn_s[sl], kc[l][sl], vc[l][sl],
                              idx[sl], out=out_s[sl], workspace=ws)
-                launches += 1
+                launches += n_launch[nb, False]
         e1.record()
         for l in range(n_layers):
             for b0, nb in syn.consecutive_runs(rc):
                 sl = slice(b0, b0 + nb)
                 ec.ec_attend(ec.make_desc(nb, L, Hq, Hkv, D, w.dtype), q_r[sl], kn_r[sl], vn_r[sl], kc[l][sl], vc[l][sl],
                              None, out=out_r[sl], workspace=ws)
-                launches += 1
+                launches += n_launch[nb, True]
         e2.record()
         row_mask.fill_(1)
         ec.ec_entropy_gate_decode(logits[s_ % period], V, window, row_mask, 0.9, tau, tokens, decoded_out=decoded,
@@ -881,7 +900,7 @@ def _run_trace_sliding(args, torch, w, dev) -> None:
         state_host.copy_(state, non_blocking=True)
         e3.record()
         torch.cuda.synchronize()                # the host reads skip_flag (and the row count): they shape the next step
-        launches += 3
+        launches += 2                           # gate and selection
         st = state_host.numpy()
         skip = (st[:, 2] != 0) & (st[:, 3] <= n_cap)
         over_cap += int(((st[:, 2] != 0) & (st[:, 3] > n_cap)).sum())

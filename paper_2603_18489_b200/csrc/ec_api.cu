@@ -248,7 +248,7 @@ const char* ec_attend_kernel_name(const ec_attn_desc* desc, int32_t n_active, in
     switch (choose_path(*desc, n_active, fresh, with_index_list != 0)) {
         case PATH_SKIP_KEYS: attend_skip_keys_describe(*desc, n_active, fresh, buf, sizeof buf); return buf;
         case PATH_SKIP_ROWS: attend_skip_describe(*desc, n_active, buf, sizeof buf); return buf;
-        // (the fp32 and mma.sync kernels refresh inside their launch; the name lists both steps)
+        // (the fp32 and mma.sync kernels refresh inside their launch; the name lists the steps, see the header)
         case PATH_F32: return fresh ? "refresh_kernel + attend_f32_kernel" : "attend_f32_kernel";
         case PATH_DENSE_FROM_NEW: attend_dense_describe(*desc, n_active, buf, sizeof buf); return buf;
         case PATH_DENSE: {

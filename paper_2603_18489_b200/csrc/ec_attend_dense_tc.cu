@@ -313,7 +313,9 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 *again = redo ? 1 : 0;
                 mbar_arrive(bar(B_VERDICT));
             }
-            // ---- second pass, only if a score left the first one's range: running maxima ----
+            // ---- second pass, only if a score left the first one's range: running maxima.  The unit is done twice: with
+            //      scores of standard deviation 4 (nats) no unit takes it, with 8 some do and with 12 all (L = 768 19.0,
+            //      22.4, 33.1 us a layer; 4096 255, 290, 505) ----
             if (redo) {
                 m_used = -INFINITY;
                 l_run = 0.f;
@@ -564,7 +566,8 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int batch, int n_kv_heads, i
 // Cutting each of them along the keys into s CTAs (s = 2, 4 or 8, at least four key tiles each) fills that wave:
 // cost in key-tile times, with two tiles' worth of fixed cost per CTA, one more for the merge, and one for the launch:
 //     waves_full * (T + 2) + ceil(tail * s / sms) * (ceil(T / s) + 3) + 1
-// s = 1 (no cut) unless a cut saves at least 3 %.
+// s = 1 (no cut) unless a cut saves at least 3 %.  (Not fitted: a unit alone has a fixed part of 6.6 us, 3.9 key tiles of
+// 1.7 us.  The cuts that the rule chooses are gains at the shapes timed, see attend_dense_kernel.)
 struct DensePlan {
     int n_pairs, units, n_full, split;
 };
@@ -596,7 +599,10 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
 
 }  // namespace
 
-// the two-tile kernel is used when its (row-tile pair, head) units fill the GPU
+// The two-tile kernel is used from SMs / 4 of its (row-tile pair, query head) units on.  The one-tile kernel behind a
+// refresh launch, which takes the steps below, is the slower one above the line: L = 320 with 32 heads (64 units) 31.2 us
+// against 11.2, at the line (40 units) 24.9 against 11.4 at L = 300 with 20 heads, 49.1 against 26.1 at 2048 with 5.  (Below
+// the line the two have not been compared; the figures say that it could lie lower.)
 bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
     if (d.dtype != EC_BF16 || d.head_dim != HD || n_active < 1) return false;
     // one unit per (sequence, query head, row-tile pair): grouped-query shapes are run head by head

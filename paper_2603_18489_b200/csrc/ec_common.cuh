@@ -126,11 +126,11 @@ void attend_skip_keys_describe(const ec_attn_desc& d, int n_active, bool fresh, 
 void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len);
 cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                cudaStream_t stream);
-// skip-step path with the keys on the M axis (bf16, head_dim 128, n_active * H_q/H_kv <= 64)
+// skip-step path with the keys on the M axis (bf16, head_dim 128, n_active <= 256, while the launch stays one wave)
 bool attend_skip_keys_supported(const ec_attn_desc& d, int n_active, bool fresh);   // fresh: k_new / v_new are given
 cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                     cudaStream_t stream);
-// two-row-tile dense path (bf16, head_dim 128): used when its (row-tile pair, kv head) units fill the GPU
+// two-row-tile dense path (bf16, head_dim 128): used from SMs / 4 units of (row-tile pair, query head) on
 bool attend_dense_supported(const ec_attn_desc& d, int n_active);
 cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream);
 size_t attend_tc_workspace_bytes(const ec_attn_desc& d, int n_active);

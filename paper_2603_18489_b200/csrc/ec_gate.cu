@@ -26,8 +26,10 @@
 // The entropy identity used: with p_j = 2^{d_j} / S,  -sum p_j ln p_j = ln S - ln2 * T / S
 // for any common base, so no partial ever needs the true row maximum.
 // What bounds it: a call is about 5.5 us (launch, ramp, reduction, ticket, the finishing CTA) and its bytes at 6.1 TB/s for
-// bf16, 7.4 for fp32 (from 288 and 576 rows, 256 rows of one and two chunks): [256, 126464] bf16 17.1 us, [32, 126464] 7.2.
-// The difference is arithmetic that the stream does not hide.  Also timed at [256, 126464]: twelve vectors ahead through
+// bf16, 7.4 for fp32 (from 288 and 576 rows, 256 rows of one and two chunks): [256, 126464] bf16 17.1 us, [32, 126464] 7.2;
+// the decode mode, whose finishing CTA has the decoded set to form, 18.5 to 19.0.
+// Of the 7.8 us above the 9.9 of its transfer (17.7, before pairs) 2.3 were arithmetic (16.9 without the exponentials, 15.4
+// without any) and 5.5 the fixed part, whose pieces have not been timed apart.  Also timed at [256, 126464]: twelve vectors ahead through
 // asynchronous copies 17.9 (fp32 26.6 against 24.2), two batches of four in registers 18.6, 3 to 21 CTAs a row 19.5 to
 // 38, five CTAs per SM of 48 registers 20.4, sums of their own for the second vector of a pair 17.2, 592 equal shares
 // that cross from row to row no better (224 rows 17.1 against 16.8, 160 rows 13.9 against 13.1); a ring of bulk copies
@@ -289,7 +291,7 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
         m = fmaxf(m, vmax);
     };
     // bf16: two vectors behind one look at the maximum, which is a branch that the exponentials of one vector and the
-    // clamps and maxima of the next cannot cross ([256, 126464] 17.6 -> 16.9 us); fp32 waits for memory and for the
+    // clamps and maxima of the next cannot cross ([256, 126464] 17.7 -> 17.1 us); fp32 waits for memory and for the
     // second of two vectors the longer (22.6 -> 23.2)
     constexpr bool kPairs = EPV == 8;
     auto consume2 = [&](uint4 v, uint4 w, int i) {   // vectors i and i + 1

@@ -11,7 +11,8 @@
 //           positions: the minimum is "-infinity" and t - dt stands.
 // What bounds it: latency.  All global loads are issued in one round (two in sliding mode, whose window rows have to be
 // checked against the mask), then about eight barriers.  Bisecting over all values that occur, behind dependent loads
-// and with two scans, took 6.5 us a call at L = 4096 and 8.9 in sliding mode at L = 1983 under a serialised launch.
+// and with two scans, took 6.5 us a call at L = 4096 and 8.9 in sliding mode at L = 1983 under a serialised launch.  Back to
+// back in a graph a call takes 1.7 us at L = 256, 2.9 (dt = 0) to 3.4 at 4096, 4.1 in sliding mode at 1983.
 // The kernel has no waits; an out-of-range window (block mode) or a window list that does not consist of masked
 // positions (sliding mode) leaves the sequence untouched and reports n_active = -1.
 #include "ec_common.cuh"

@@ -6,8 +6,8 @@
 //
 // Why: with the query rows on M a batch of heads is bound by the softmax.  34 rows live in the TMEM lanes of two of the
 // four warp quarters, so one SM sub-partition does 64 exponentials a lane and key tile of 64 for both CTAs (1.0 us a
-// tile) while the others idle.  Here every lane of every quarter owns a key and half of its scores.  Eight sequences of 4096 with 32 heads and 34 rows: 89 us a layer (6.1 TB/s)
-// against 107, five with 40 rows 68 against 87.
+// tile) while the others idle.  Here every lane of every quarter owns a key and half of its scores.  Eight sequences of
+// 4096 with 32 heads and 34 rows: 85 us a layer (6.5 TB/s) against 107, five with 40 rows 68 against 87.
 //   warp 0     TMA producer: one K slot and one V slot of 128 keys, each refilled as soon as its product has run (two
 //              CTAs per SM keep each other's latency covered);
 //   warp 1     tcgen05.mma issue, whichever product is ready, S one tile ahead (two S^T buffers);
