@@ -12,7 +12,9 @@
 // What bounds it: latency.  All global loads are issued in one round (two in sliding mode, whose window rows have to be
 // checked against the mask), then about eight barriers.  Bisecting over all values that occur, behind dependent loads
 // and with two scans, took 6.5 us a call at L = 4096 and 8.9 in sliding mode at L = 1983 under a serialised launch.  Back to
-// back in a graph a call takes 1.7 us at L = 256, 2.9 (dt = 0) to 3.4 at 4096, 4.1 in sliding mode at 1983.
+// back in a graph a call takes 2.1 us at L = 256, 3.1 (dt = 0) to 3.5 at 4096, 3.8 in sliding mode at 1983; searched in 64
+// bits it is 0.1 longer in sliding mode.  The count of the entries above t is a barrier of its own where dt = 0: 0.15 us at
+// 256, 0.25 at 4096.
 // The kernel has no waits; an out-of-range window (block mode) or a window list that does not consist of masked
 // positions (sliding mode) leaves the sequence untouched and reports n_active = -1.
 #include "ec_common.cuh"
@@ -123,45 +125,43 @@ __global__ void __launch_bounds__(kSelThreads) select_recent_kernel(const Select
         }
     }
     // ---- Eq. 3 ----------------------------------------------------------------------------------------
+    // (all values fit 32 bits: a t - dt below them is no limit, and nothing reaches one above them, see reached below)
     const long long since = (long long)st.t - st.dt_recompute;   // t - dt
-    long long tau = since;
-    if (p.k > 0) {
-        auto at_least_k = [&](long long v) {   // do at least k entries reach v?
-            if (v < (long long)INT32_MIN + 1) v = (long long)INT32_MIN + 1;   // (EC_H_NEVER itself never counts)
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < PER; ++j) c += (h[j] >= (int)v) ? 1 : 0;
-            return block_sum(c) >= p.k;
-        };
-        // one count: entries that exceed since, and (upper half word) entries that exceed t, which only a loop that sets t
-        // back without its history leaves behind
-        const long long next = since + 1 < INT32_MIN + 1 ? INT32_MIN + 1 : since + 1 > INT32_MAX ? INT32_MAX : since + 1;
+    const bool reached = p.k > 0 && since <= INT32_MAX;          // k = 0: minimum over the empty set
+    int tau = reached ? (int)(since > INT32_MIN ? since : (long long)INT32_MIN) : INT32_MAX;
+    if (reached) {
+        // the threshold is the largest value from tau to hi that k entries reach; tau itself needs no entry
+        int hi = st.t;
+        // one count: entries that exceed tau and, in the upper half word, entries that exceed t, which only a loop that sets
+        // t back without its history leaves behind
         uint32_t c = 0;
 #pragma unroll
-        for (int j = 0; j < PER; ++j) c += (h[j] >= (int)next ? 1u : 0u) + (h[j] > st.t ? 0x10000u : 0u);
+        for (int j = 0; j < PER; ++j) c += (h[j] > tau ? 1u : 0u) + (h[j] > st.t ? 0x10000u : 0u);
         const int counts = block_sum(c);
-        // the threshold is since, or the largest v above it that k entries reach: lo may be it, hi may not
-        long long lo = since, hi = (long long)st.t + 1;
         if (counts >> 16 >= p.k) {
-            lo = lo > hi ? lo : hi;
-            hi = (long long)INT32_MAX + 1;
-        } else if (lo + 1 < hi) {
-            if ((counts & 0xffff) >= p.k) lo = lo + 1; else hi = lo + 1;
+            tau = max(tau, st.t + 1);
+            hi = INT32_MAX;
+        } else if (tau < hi) {
+            if ((counts & 0xffff) >= p.k) ++tau; else hi = tau;
         }
-        while (hi - lo > 1) {
-            const long long mid = lo + (hi - lo) / 2;
-            if (at_least_k(mid)) lo = mid; else hi = mid;
+        while (tau < hi) {
+            const uint32_t gap = (uint32_t)hi - (uint32_t)tau;
+            const int mid = (int)((uint32_t)tau + (gap >> 1) + (gap & 1u));
+            uint32_t n = 0;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) n += (h[j] >= mid) ? 1 : 0;   // (EC_H_NEVER is below every mid)
+            if (block_sum(n) >= p.k) tau = mid; else hi = mid - 1;
         }
-        tau = lo;
+        tau = max(tau, INT32_MIN + 1);   // never EC_H_NEVER
     }
     // ---- the window's rows and R (outside the block in block mode; a decoded position is never in a sliding window),
     //      ascending: one exclusive scan of both counts ----
     uint32_t rbits = 0;
-    if (p.k > 0) {   // k = 0: minimum over the empty set, nothing reaches it
+    if (reached) {
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
             const int r = i0 + j - w0;
-            const bool in_r = h[j] != EC_H_NEVER && (long long)h[j] >= tau;
+            const bool in_r = h[j] >= tau;
             if (in_r && (sliding || r < 0 || r >= p.block)) rbits |= 1u << j;
         }
     }
