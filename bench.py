@@ -56,19 +56,19 @@ K64_WORKLOADS = ("c4_llada_l2048", "c5_llada_l4096", "c5_llada_l4096_b8", "c5_dr
 NCU_TRAFFIC = {
     "attend_skip": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",),
-         "sha256": "6fd3dc0f298c46a576d57bd3540f12bcb9168ab693ffffbbac8922c8510713b7",
-         "bytes_per_launch": {"c5_llada_l4096": 68160000}},
+         "sha256": "c474a357d342a69efc637af48faa81c785a7ef0647254f9ebb669f52b3b46119",
+         "bytes_per_launch": {"c5_llada_l4096": 68300000}},
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu", "paper_2603_18489_b200/csrc/ec_skip_keys_pair.cuh"),
-         "sha256": "65b46cc75830b8e859285087271c6c5b40faae59a005274755dbc82fd63d76b5",
-         "bytes_per_launch": {"c5_llada_l4096_b8": 558740000}}],
+         "sha256": "f8a1bbeeec1c27874598b6b6d350adaddad2499b98703d06da43b7bafe7f143d",
+         "bytes_per_launch": {"c5_llada_l4096_b8": 556680000}}],
     "attend_dense": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",),
-         "sha256": "7a98a8f43f1813c6b2c2e415eaa10ef757f463c24264f763c784fb25d2ae37a6",
-         "bytes_per_launch": {"c5_llada_l4096": 146620000}}],
+         "sha256": "267ab6f92d2b70bdd83b3c2b3ac6dffd1eef4b0b90ad4057f60ad4d265abb263",
+         "bytes_per_launch": {"c5_llada_l4096": 151530000}}],
     "entropy_gate": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_gate.cu",),
-         "sha256": "026fe97ffd51bbd366852fdac150195f9cf2765f3cd9db49fa97c7109723dbe2",
-         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65710000}}],
+         "sha256": "18611e4521d092e171a3838cfc98ea318657814618c56e10b7bf546a9215100f",
+         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65320000}}],
 }
 
 
