@@ -113,7 +113,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         return;
     }
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int lin = blockIdx.x;
     const int unit = kCut ? p.n_full + lin / p.split : lin;
     const int part = kCut ? lin % p.split : 0;
@@ -174,64 +174,72 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
     } else if (warp == 1) {
         // ================================ MMA issuer ========================================
-        if (lane == 0) {
-            constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
-            const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024);
-            auto issue_s = [&](int t, int slot_k) {
-                const uint64_t desc_k = smem_desc(base + OFF_RING + slot_k * TILE, 16, 1024);
+        // (the whole warp, see elect_one: with one thread this role took 3400 cycles a key tile and set the pace)
+        const bool elected = elect_one();
+        constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
+        const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024);
+        auto issue_s = [&](int t, int slot_k) {
+            const uint64_t desc_k = smem_desc(base + OFF_RING + slot_k * TILE, 16, 1024);
+            if (elected) {
 #pragma unroll
                 for (int k = 0; k < HD / 16; ++k) {
                     const uint32_t koff = ((k >> 2) * SUB + (k & 3) * 32) / 16;
                     mma_ss(tmem + TM_S + t * 128, desc_q + t * (TILE / 16) + koff, desc_k + koff, IDESC_S, k > 0);
                 }
                 commit(bar(B_SFULL + t));
-            };
-            int slot = 0;          // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...
-            uint32_t phase = 0, p_phase = 0;
-            auto advance = [&]() {
-                const int s = slot;
-                if (++slot == kSlots) slot = 0, phase ^= 1;
-                return s;
-            };
-            for (int pass = 0; pass < 2; ++pass) {
-                if (pass == 1) {
-                    mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
-                    if (!*again) break;
-                }
-                mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+            }
+        };
+        int slot = 0;          // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...
+        uint32_t phase = 0, p_phase = 0;
+        auto advance = [&]() {
+            const int s = slot;
+            if (++slot == kSlots) slot = 0, phase ^= 1;
+            return s;
+        };
+        for (int pass = 0; pass < 2; ++pass) {
+            if (pass == 1) {
+                mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                if (!*again) break;
+            }
+            mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+            fence_after();
+            for (int t = 0; t < n_tiles_q; ++t) {
+                mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
                 fence_after();
-                for (int t = 0; t < n_tiles_q; ++t) {
-                    mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
-                    fence_after();
-                    issue_s(t, slot);
-                }
-                commit(bar(B_EMPTY + advance()));   // K_0 is free once both S(0) have run
-                for (int j = 0; j < T; ++j, p_phase ^= 1) {
+                issue_s(t, slot);
+            }
+            const int k0 = advance();
+            if (elected) commit(bar(B_EMPTY + k0));   // K_0 is free once both S(0) have run
+            for (int j = 0; j < T; ++j, p_phase ^= 1) {
+                mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+                const int vs = advance();            // V_j
+                int ks = 0;
+                const bool more = j + 1 < T;
+                if (more) {
                     mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
-                    const int vs = advance();            // V_j
-                    int ks = 0;
-                    const bool more = j + 1 < T;
-                    if (more) {
-                        mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
-                        ks = advance();                  // K_{j+1}
-                    }
-                    const uint64_t desc_v = smem_desc(base + OFF_RING + vs * TILE, SUB, 1024);
-                    for (int t = 0; t < n_tiles_q; ++t) {
-                        mbar_wait(bar(B_PFULL + t), p_phase, abort_flag, p.dev_status);
-                        fence_after();
-                        // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95
+                    ks = advance();                  // K_{j+1}
+                }
+                const uint64_t desc_v = smem_desc(base + OFF_RING + vs * TILE, SUB, 1024);
+                for (int t = 0; t < n_tiles_q; ++t) {
+                    mbar_wait(bar(B_PFULL + t), p_phase, abort_flag, p.dev_status);
+                    fence_after();
+                    // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95
+                    if (elected) {
 #pragma unroll
                         for (int k = 0; k < BN / 16; ++k)
                             mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
                                    IDESC_PV, (j > 0 || k > 0));
-                        if (more) issue_s(t, ks);
-                        commit(bar(B_PVDONE + t));
                     }
+                    if (more) issue_s(t, ks);
+                    if (elected) commit(bar(B_PVDONE + t));
+                }
+                if (elected) {
                     commit(bar(B_EMPTY + vs));
                     if (more) commit(bar(B_EMPTY + ks));
                 }
             }
         }
+        __syncwarp();
     } else if (warp < 2 + kSoftThreads / 32) {
         // ================================ softmax (warps 2..17) ================================
         // A row of a tile is shared by two threads, one per 64-column half, in warps that own the same TMEM

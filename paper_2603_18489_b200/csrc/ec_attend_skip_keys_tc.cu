@@ -177,7 +177,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     uint32_t* stale = reinterpret_cast<uint32_t*>(gbase + p.off_list);   // [cache tile][4]: a bit per stale key
     auto bar = [&](int idx) { return bars + idx * 8; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int split = blockIdx.x, bh = blockIdx.y / p.n_sub, sub = blockIdx.y % p.n_sub;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
     const int hg = sub / p.n_sub_r * p.group;                                  // first query head of this CTA in its kv head
@@ -312,59 +312,71 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ================================ MMA issue (lane 0) ========================================
-        if (lane == 0) {
-            constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
-            constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
-            constexpr uint32_t QHALF = N * 128;                   // bytes of one 64-column half of the Q tile
-            const uint64_t desc_q = smem_desc(base, 16, 1024), desc_p = smem_desc(base + p.off_p, SUB, 1024);
-            auto products_s = [&](int slot, int buf) {
-                const uint64_t desc_k = smem_desc(base + p.off_stage + slot * TILE, 16, 1024);
-                fence_after();
+        // ================================ MMA issue (the whole warp, see elect_one) ==================
+        const bool elected = elect_one();
+        constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
+        constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
+        constexpr uint32_t QHALF = N * 128;                   // bytes of one 64-column half of the Q tile
+        const uint64_t desc_q = smem_desc(base, 16, 1024), desc_p = smem_desc(base + p.off_p, SUB, 1024);
+        auto products_s = [&](int slot, int buf) {
+            const uint64_t desc_k = smem_desc(base + p.off_stage + slot * TILE, 16, 1024);
+            fence_after();
+            if (elected) {
 #pragma unroll
                 for (int k = 0; k < HD / 16; ++k)
                     mma_ss(tmem + TM_S + buf * NP, desc_k + ((k >> 2) * SUB + (k & 3) * 32) / 16,
                            desc_q + ((k >> 2) * QHALF + (k & 3) * 32) / 16, IDESC_S, k > 0);
-            };
-            auto products_pv = [&](int slot, bool accumulate) {
-                const uint64_t desc_v = smem_desc(base + p.off_stage + slot * TILE, SUB, 1024);
-                fence_after();
+            }
+        };
+        auto products_pv = [&](int slot, bool accumulate) {
+            const uint64_t desc_v = smem_desc(base + p.off_stage + slot * TILE, SUB, 1024);
+            fence_after();
+            if (elected) {
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
                     mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (accumulate || k > 0));
-            };
-            // Both products once on whatever shared memory holds, before there is anything to do: the results are
-            // overwritten (S of tile 1, the first P V), but the code has been fetched when the first tile needs it.
-            products_s(0, 1);
-            products_pv(0, false);
-            // S of tile j needs the tile; P V of tile j needs P^T from the softmax.  Whichever is ready
-            // is issued: P V of a tile does not wait for the next tile to land (its commit frees the stage for the
-            // producer), S may run one tile ahead of P V (two S^T buffers).
-            mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
-            int next_s = 0, next_pv = 0;
-            SpinGuard guard;
-            while (next_pv < T) {
-                bool progressed = false;
-                if (next_s < T && next_s <= next_pv + 1 && mbar_test(bar(B_FULL + (2 * next_s) % NS), ((2 * next_s) / NS) & 1)) {
-                    const int s = (2 * next_s) % NS;
-                    products_s(s, next_s & 1);   // (the tile has landed)
-                    commit(bar(B_SFULL + (next_s & 1)));
-                    commit(bar(B_EMPTY + s));    // the K slot is free once these products have run
-                    ++next_s;
-                    progressed = true;
-                }
-                if (mbar_test(bar(B_PFULL), next_pv & 1) &&
-                    mbar_test(bar(B_FULL + (2 * next_pv + 1) % NS), ((2 * next_pv + 1) / NS) & 1)) {   // P^T is there, V has landed
-                    const int s = (2 * next_pv + 1) % NS;
-                    products_pv(s, next_pv > 0);
-                    commit(bar(B_PVDONE));
-                    commit(bar(B_EMPTY + s));
-                    ++next_pv;
-                    progressed = true;
-                }
-                if (progressed) guard.progress();
-                else if (!guard.tick(abort_flag, p.dev_status)) break;
             }
+        };
+        // Both products once on whatever shared memory holds, before there is anything to do: the results are
+        // overwritten (S of tile 1, the first P V), but the code has been fetched when the first tile needs it.
+        products_s(0, 1);
+        products_pv(0, false);
+        // S of tile j needs the tile; P V of tile j needs P^T from the softmax.  Whichever is ready
+        // is issued: P V of a tile does not wait for the next tile to land (its commit frees the stage for the
+        // producer), S may run one tile ahead of P V (two S^T buffers).
+        mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
+        int next_s = 0, next_pv = 0;
+        int ks = 0, vs = 1;               // ring slots of K of tile next_s and V of tile next_pv, and how often they were filled
+        uint32_t k_turn = 0, v_turn = 0;
+        auto step = [&](int& slot, uint32_t& turn) {
+            slot += 2;
+            if (slot >= NS) slot -= NS, turn ^= 1;
+        };
+        SpinGuard guard;
+        while (next_pv < T) {
+            bool progressed = false;
+            if (next_s < T && next_s <= next_pv + 1 && mbar_test_warp(bar(B_FULL + ks), k_turn)) {
+                products_s(ks, next_s & 1);   // (the tile has landed)
+                if (elected) {
+                    commit(bar(B_SFULL + (next_s & 1)));
+                    commit(bar(B_EMPTY + ks));    // the K slot is free once these products have run
+                }
+                step(ks, k_turn);
+                ++next_s;
+                progressed = true;
+            }
+            if (mbar_test_warp(bar(B_PFULL), next_pv & 1) && mbar_test_warp(bar(B_FULL + vs), v_turn)) {   // P^T is there, V has landed
+                products_pv(vs, next_pv > 0);
+                if (elected) {
+                    commit(bar(B_PVDONE));
+                    commit(bar(B_EMPTY + vs));
+                }
+                step(vs, v_turn);
+                ++next_pv;
+                progressed = true;
+            }
+            if (progressed) guard.progress();
+            else if (__any_sync(0xffffffffu, !guard.tick(abort_flag, p.dev_status))) break;
         }
     } else if (warp >= 2 + 4 * WG) {
         // ===== auxiliary warps: stale-key bits; the fresh rows into the cache (for later steps) =====

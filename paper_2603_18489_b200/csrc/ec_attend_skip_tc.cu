@@ -147,7 +147,7 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     uint32_t* bits = reinterpret_cast<uint32_t*>(gbase + p.off_list);
     auto bar = [&](int idx) { return bars + idx * 8; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int split = blockIdx.x, bh = blockIdx.y;
     const int b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
     const int C = p.n_splits;
@@ -246,60 +246,64 @@ attend_skip_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ================================ MMA issue (lane 0) ========================================
-        if (lane == 0) {
-            constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
-            uint64_t desc_q[NT], desc_p[NT];
-            uint32_t qh[NT];   // one 64-column half of the Q tile, in descriptor units
+        // ================================ MMA issue (the whole warp, see elect_one) =====================
+        const bool elected = elect_one();
+        constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
+        uint64_t desc_q[NT], desc_p[NT];
+        uint32_t qh[NT];   // one 64-column half of the Q tile, in descriptor units
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                desc_q[t] = smem_desc(base + p.off_q[t], 16, 1024);
-                desc_p[t] = smem_desc(base + p.off_p[t], 16, 1024);
-                qh[t] = p.rows_pad[t] * 8u;
-            }
-            // S of a tile needs the tile, P V of a tile and row tile needs its P: whichever is ready is issued.  S may run
-            // one tile ahead of P V (two S buffers).
-            int next_s = 0, next_pv[NT], n_pv = 0;   // n_pv: tiles whose P V has been issued for every row tile
+        for (int t = 0; t < NT; ++t) {
+            desc_q[t] = smem_desc(base + p.off_q[t], 16, 1024);
+            desc_p[t] = smem_desc(base + p.off_p[t], 16, 1024);
+            qh[t] = p.rows_pad[t] * 8u;
+        }
+        // S of a tile needs the tile, P V of a tile and row tile needs its P: whichever is ready is issued.  S may run
+        // one tile ahead of P V (two S buffers).
+        int next_s = 0, next_pv[NT], n_pv = 0;   // n_pv: tiles whose P V has been issued for every row tile
 #pragma unroll
-            for (int t = 0; t < NT; ++t) next_pv[t] = 0;
-            mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
-            SpinGuard guard;
-            while (n_pv < T) {
-                bool progressed = false;
-                if (next_s < T && next_s <= n_pv + 1 && mbar_test(bar(B_FULL + next_s % NS), (next_s / NS) & 1)) {
-                    const uint64_t desc_k = smem_desc(base + p.off_stage + (next_s % NS) * STAGE, 16, 1024);
-                    fence_after();
+        for (int t = 0; t < NT; ++t) next_pv[t] = 0;
+        mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
+        SpinGuard guard;
+        while (n_pv < T) {
+            bool progressed = false;
+            if (next_s < T && next_s <= n_pv + 1 && mbar_test_warp(bar(B_FULL + next_s % NS), (next_s / NS) & 1)) {
+                const uint64_t desc_k = smem_desc(base + p.off_stage + (next_s % NS) * STAGE, 16, 1024);
+                fence_after();
 #pragma unroll
-                    for (int t = 0; t < NT; ++t) {
+                for (int t = 0; t < NT; ++t) {
+                    if (elected) {
 #pragma unroll
                         for (int k = 0; k < HD / 16; ++k)
                             mma_ss(tmem + t * 256 + (next_s & 1) * 64, desc_q[t] + (k >> 2) * qh[t] + (k & 3) * 2,
                                    desc_k + (k >> 2) * (KV_SUB / 16) + (k & 3) * 2, IDESC_S, k > 0);
                         commit(bar(B_SFULL + t * 2 + (next_s & 1)));
                     }
-                    ++next_s;
-                    progressed = true;
                 }
+                ++next_s;
+                progressed = true;
+            }
 #pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const int j = next_pv[t];
-                    if (j >= next_s || !mbar_test(bar(B_PFULL + t), j & 1)) continue;
-                    const uint64_t desc_v = smem_desc(base + p.off_stage + (j % NS) * STAGE + KV_TILE, KV_SUB, 1024);
-                    fence_after();
+            for (int t = 0; t < NT; ++t) {
+                const int j = next_pv[t];
+                if (j >= next_s || !mbar_test_warp(bar(B_PFULL + t), j & 1)) continue;
+                const uint64_t desc_v = smem_desc(base + p.off_stage + (j % NS) * STAGE + KV_TILE, KV_SUB, 1024);
+                fence_after();
+                if (elected) {
 #pragma unroll
                     for (int k = 0; k < BN / 16; ++k)
                         mma_ss(tmem + t * 256 + 128, desc_p[t] + k * 2, desc_v + k * 128, IDESC_PV, (j > 0 || k > 0));
                     commit(bar(B_PVDONE + t));
-                    ++next_pv[t];
-                    progressed = true;
                 }
-                int done = next_pv[0];
-#pragma unroll
-                for (int t = 1; t < NT; ++t) done = min(done, next_pv[t]);
-                for (; n_pv < done; ++n_pv) commit(bar(B_EMPTY + n_pv % NS));
-                if (progressed) guard.progress();
-                else if (!guard.tick(abort_flag, p.dev_status)) break;
+                ++next_pv[t];
+                progressed = true;
             }
+            int done = next_pv[0];
+#pragma unroll
+            for (int t = 1; t < NT; ++t) done = min(done, next_pv[t]);
+            for (; n_pv < done; ++n_pv)
+                if (elected) commit(bar(B_EMPTY + n_pv % NS));
+            if (progressed) guard.progress();
+            else if (__any_sync(0xffffffffu, !guard.tick(abort_flag, p.dev_status))) break;
         }
     } else {
         // ================== Q staging, cache refresh, softmax (warps 2..) ========================

@@ -88,7 +88,7 @@ __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap&
     const uint32_t bars = s2u(sh->bars);
     auto bar = [&](int i) { return bars + 8u * i; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int bh = blockIdx.y, b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
     const int rows_total = p.n_active * p.group;
     const bool refresh = p.k_new != nullptr;
@@ -146,42 +146,45 @@ __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap&
                 else if (!guard.tick(abort_flag, p.dev_status)) break;
             }
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
-            constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
-            constexpr uint32_t QHALF = N * 128;
-            const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024), desc_p = smem_desc(base + OFF_P, SUB, 1024);
-            const uint64_t desc_k = smem_desc(base + OFF_K, 16, 1024), desc_v = smem_desc(base + OFF_V, SUB, 1024);
-            mbar_wait(bar(KB_QFULL), 0, abort_flag, p.dev_status);
-            int next_s = 0, next_pv = 0;
-            SpinGuard guard;
-            while (next_pv < T) {
-                bool progressed = false;
-                if (next_s < T && next_s <= next_pv + 1 && mbar_test(bar(KB_KFULL), next_s & 1)) {
-                    fence_after();
+    } else if (warp == 1) {   // (the whole warp, see elect_one)
+        const bool elected = elect_one();
+        constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
+        constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
+        constexpr uint32_t QHALF = N * 128;
+        const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024), desc_p = smem_desc(base + OFF_P, SUB, 1024);
+        const uint64_t desc_k = smem_desc(base + OFF_K, 16, 1024), desc_v = smem_desc(base + OFF_V, SUB, 1024);
+        mbar_wait(bar(KB_QFULL), 0, abort_flag, p.dev_status);
+        int next_s = 0, next_pv = 0;
+        SpinGuard guard;
+        while (next_pv < T) {
+            bool progressed = false;
+            if (next_s < T && next_s <= next_pv + 1 && mbar_test_warp(bar(KB_KFULL), next_s & 1)) {
+                fence_after();
+                if (elected) {
 #pragma unroll
                     for (int k = 0; k < HD / 16; ++k)
                         mma_ss(tmem + TM_S + (next_s & 1) * 64, desc_k + ((k >> 2) * SUB + (k & 3) * 32) / 16,
                                desc_q + ((k >> 2) * QHALF + (k & 3) * 32) / 16, IDESC_S, k > 0);
                     commit(bar(KB_SFULL + (next_s & 1)));
                     commit(bar(KB_KEMPTY));
-                    ++next_s;
-                    progressed = true;
                 }
-                if (next_pv < next_s && mbar_test(bar(KB_PFULL), next_pv & 1) && mbar_test(bar(KB_VFULL), next_pv & 1)) {
-                    fence_after();
+                ++next_s;
+                progressed = true;
+            }
+            if (next_pv < next_s && mbar_test_warp(bar(KB_PFULL), next_pv & 1) && mbar_test_warp(bar(KB_VFULL), next_pv & 1)) {
+                fence_after();
+                if (elected) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
                         mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (next_pv > 0 || k > 0));
                     commit(bar(KB_PVDONE));
                     commit(bar(KB_VEMPTY));
-                    ++next_pv;
-                    progressed = true;
                 }
-                if (progressed) guard.progress();
-                else if (!guard.tick(abort_flag, p.dev_status)) break;
+                ++next_pv;
+                progressed = true;
             }
+            if (progressed) guard.progress();
+            else if (__any_sync(0xffffffffu, !guard.tick(abort_flag, p.dev_status))) break;
         }
     } else {
         const int stid = tid - 64, wg = stid >> 7, c0 = wg * NH, st_w = stid & 127;

@@ -118,6 +118,24 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 __device__ __forceinline__ void commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+// One lane of the (converged) warp, the same one every time.  A role that one thread plays (issuing products, asking for
+// tiles) is run by its whole warp, and only the instructions that must be issued once stand behind this predicate: then the
+// compiler knows descriptors, addresses and barriers as warp-uniform.  Behind `lane == 0` it does not, and moves every
+// operand over for each instruction: eight tcgen05.mma 416 cycles to issue instead of 163 (they run in 512), a wait on a
+// completed mbarrier 165 instead of 54.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+// a barrier as the whole warp sees it: one answer, so what depends on it stays warp-uniform
+__device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)); }
+// threadIdx.x / 32 as a value that the compiler knows to be warp-uniform
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
     asm volatile(
