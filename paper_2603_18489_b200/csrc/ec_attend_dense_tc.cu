@@ -56,7 +56,10 @@ constexpr uint32_t PART = BM * HD * 4;                   // un-normalised rows o
 constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
-enum { B_FULL = 0, B_EMPTY = kSlots, B_SFULL = 2 * kSlots, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 2,
+// B_FREE: ring entries are released in groups, K_0, then {V_0, K_1}, {V_1, K_2}, ... (a second pass goes on: {V of the last
+// tile, K_0}); group c completes phase c / 2 of barrier c % 2.  Entry n belongs to group (n + 1) / 2.
+// B_PFULL: + 2 * part + tile, see the softmax.
+enum { B_FULL = 0, B_FREE = kSlots, B_SFULL = B_FREE + 2, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 4,
        B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 2, B_COPIED = B_VERDICT + 1, B_COUNT = B_COPIED + 1 };
 
 // first pass: a row's sum may grow to this before the unit is done again with running maxima
@@ -135,7 +138,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         prefetch_map(&map_o);
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 2) ? 256u : (p.copy && i >= B_EMPTY && i < B_EMPTY + kSlots) ? 2u : 1u);
+            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 4) ? 256u : (p.copy && i >= B_FREE && i < B_FREE + 2) ? 2u : 1u);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -164,8 +167,8 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
                     if (!*again) break;
                 }
-                const int slot = n % kSlots, u = n / kSlots, j = (n >> 1) % T;
-                if (u > 0) mbar_wait(bar(B_EMPTY + slot), (u - 1) & 1, abort_flag, p.dev_status);
+                const int slot = n % kSlots, j = (n >> 1) % T, c = (n - kSlots + 1) >> 1;   // c: group of the slot's last entry
+                if (n >= kSlots) mbar_wait(bar(B_FREE + (c & 1)), (c >> 1) & 1, abort_flag, p.dev_status);
                 mbar_expect_tx(bar(B_FULL + slot), TILE);
                 tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, (j0 + j) * BN, 0, hk_kv, b, bar(B_FULL + slot));
                 if (n == 0)   // behind the first K tile: the first scores need one row tile of Q
@@ -178,65 +181,84 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const bool elected = elect_one();
         constexpr uint32_t IDESC_S = instr_desc(BN, 0), IDESC_PV = instr_desc(HD, 1);
         const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024);
-        auto issue_s = [&](int t, int slot_k) {
-            const uint64_t desc_k = smem_desc(base + OFF_RING + slot_k * TILE, 16, 1024);
+        auto products_s = [&](int t, uint64_t desc_k, int k0, int k1) {
             if (elected) {
 #pragma unroll
-                for (int k = 0; k < HD / 16; ++k) {
+                for (int k = k0; k < k1; ++k) {
                     const uint32_t koff = ((k >> 2) * SUB + (k & 3) * 32) / 16;
                     mma_ss(tmem + TM_S + t * 128, desc_q + t * (TILE / 16) + koff, desc_k + koff, IDESC_S, k > 0);
                 }
-                commit(bar(B_SFULL + t));
             }
         };
-        int slot = 0;          // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...
+        int slot = 0, group = 0;   // ring slot and phase of the next tile in the order K_0 V_0 K_1 V_1 ...; the next group to release
         uint32_t phase = 0, p_phase = 0;
-        auto advance = [&]() {
+        auto full = [&](int ahead) {   // has the ring entry `ahead` behind the next one landed?
+            const bool wrapped = slot + ahead >= kSlots;
+            return mbar_test(bar(B_FULL + slot + ahead - (wrapped ? kSlots : 0)), phase ^ (wrapped ? 1u : 0u));
+        };
+        auto take = [&](bool landed) {
+            if (!landed) mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
             const int s = slot;
             if (++slot == kSlots) slot = 0, phase ^= 1;
             return s;
         };
+        auto release = [&]() {
+            if (elected) commit(bar(B_FREE + (group & 1)));
+            ++group;
+        };
+        constexpr int kPeek = HD / 16 - 2;
         for (int pass = 0; pass < 2; ++pass) {
             if (pass == 1) {
                 mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
                 if (!*again) break;
             }
-            mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
-            fence_after();
-            for (int t = 0; t < n_tiles_q; ++t) {
-                mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
-                fence_after();
-                issue_s(t, slot);
-            }
-            const int k0 = advance();
-            if (elected) commit(bar(B_EMPTY + k0));   // K_0 is free once both S(0) have run
-            for (int j = 0; j < T; ++j, p_phase ^= 1) {
-                mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
-                const int vs = advance();            // V_j
-                int ks = 0;
-                const bool more = j + 1 < T;
-                if (more) {
-                    mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
-                    ks = advance();                  // K_{j+1}
-                }
-                const uint64_t desc_v = smem_desc(base + OFF_RING + vs * TILE, SUB, 1024);
+            {
+                const uint64_t desc_k = smem_desc(base + OFF_RING + take(false) * TILE, 16, 1024);
                 for (int t = 0; t < n_tiles_q; ++t) {
-                    mbar_wait(bar(B_PFULL + t), p_phase, abort_flag, p.dev_status);
+                    mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
                     fence_after();
-                    // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95
-                    if (elected) {
+                    products_s(t, desc_k, 0, HD / 16);
+                    if (elected) commit(bar(B_SFULL + t));
+                }
+                release();
+            }
+            // The pipe holds about three instructions behind the one that runs; an issuer that comes back from a barrier
+            // later than that leaves it idle.  So the barriers of the next products are looked at while the last two
+            // products of a group are still to be issued, and only what was not ready then is waited for.
+            bool kv_ready = false, p_ready = false;
+            for (int j = 0; j < T; ++j, p_phase ^= 1) {
+                const bool more = j + 1 < T, more2 = j + 2 < T;
+                const uint64_t desc_v = smem_desc(base + OFF_RING + take(kv_ready) * TILE, SUB, 1024);
+                const uint64_t desc_k = smem_desc(base + OFF_RING + (more ? take(kv_ready) : 0) * TILE, 16, 1024);
+                for (int t = 0; t < n_tiles_q; ++t) {
 #pragma unroll
-                        for (int k = 0; k < BN / 16; ++k)
-                            mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
-                                   IDESC_PV, (j > 0 || k > 0));
+                    for (int q = 0; q < 2; ++q) {
+                        if (q == 1 || !p_ready) mbar_wait(bar(B_PFULL + q * 2 + t), p_phase, abort_flag, p.dev_status);
+                        fence_after();
+                        // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95; part 0 are the first
+                        // 48 keys of each half, part 1 the others
+                        if (elected) {
+#pragma unroll
+                            for (int i = 0; i < (q ? 2 : 6); ++i) {
+                                const int k = q ? i * 4 + 3 : (i / 3) * 4 + i % 3;
+                                mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
+                                       IDESC_PV, (j > 0 || k > 0));
+                            }
+                        }
                     }
-                    if (more) issue_s(t, ks);
-                    if (elected) commit(bar(B_PVDONE + t));
+                    p_ready = false;
+                    if (more) {
+                        products_s(t, desc_k, 0, kPeek);
+                        const bool next_tile = t + 1 == n_tiles_q;
+                        const bool p_seen = mbar_test(bar(B_PFULL + (next_tile ? 0 : t + 1)), p_phase ^ (next_tile ? 1u : 0u));
+                        if (t == 0) kv_ready = __all_sync(0xffffffffu, full(0) && (!more2 || full(1)));
+                        p_ready = __all_sync(0xffffffffu, p_seen);
+                        products_s(t, desc_k, kPeek, HD / 16);
+                        if (elected) commit(bar(B_SFULL + t));
+                    }
+                    if (elected && (pass == 1 || !more)) commit(bar(B_PVDONE + t));
                 }
-                if (elected) {
-                    commit(bar(B_EMPTY + vs));
-                    if (more) commit(bar(B_EMPTY + ks));
-                }
+                if (more) release();   // (the last V tile goes with the K_0 of a second pass)
             }
         }
         __syncwarp();
@@ -279,6 +301,10 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         mneg2 = pk(-m_used, -m_used);
                         named_barrier(pair_bar, 64);   // both threads of the row have read what P is about to overwrite
                     }
+                    // P goes out in two parts, 48 columns and 16, so that three quarters of P V run while the rest is worked out:
+                    // the chain of a row tile, scores - softmax - P V - scores, is what the other row tile has to cover.
+                    // us a pass of 32 layers of 768 / 14 of 2 x 1531 (28 heads) / 2 of 8 x 4096 (at 1.5 GHz under the power
+                    // cap): one part 557 / 1095 / 3995, halves 528 / 1045 / 3785, three quarters 523 / 1035 / 3675.
                     uint32_t sr[2][32];
                     ld32(tm_s + h * 64, sr[0]);
                     wait_ld<32>(sr[0]);
@@ -302,20 +328,29 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                             const float e0 = fast_exp2(d0), e1 = fast_exp2(d1);
                             sum2[c & 1] = add2(sum2[c & 1], pk(e0, e1));
                             pw[c] = pack_bf16x2(e0, e1);
+                            if (q == 1 && c == 7) {
+                                st8(tm_s + h * 64 + 16, pw);
+                                wait_st();
+                                fence_before();
+                                mbar_arrive(bar(B_PFULL + t));
+                            }
                         }
-                        // P (bf16 pairs) over the first half of this thread's own scores
-                        st16(tm_s + h * 64 + q * 16, pw);
+                        // (bf16 pairs over the first half of this thread's own scores)
+                        if (q == 0) {
+                            st16(tm_s + h * 64, pw);
+                        } else {
+                            st8(tm_s + h * 64 + 24, pw + 8);
+                            wait_st();
+                            fence_before();
+                            mbar_arrive(bar(B_PFULL + 2 + t));
+                        }
                     }
-                    wait_st();
-                    fence_before();
-                    mbar_arrive(bar(B_PFULL + t));
                 }
                 float a0, a1, b0, b1;
                 upk(sum2[0], a0, a1);
                 upk(sum2[1], b0, b1);
                 l_run = (a0 + a1) + (b0 + b1);   // this half's share of the row sum
             }
-            int done = T;   // tiles of both passes behind us
             const bool redo = named_barrier_or(9, n_tiles_q * 256, !(l_run <= kMaxSum));
             if (ws == 0 && lane == 0) {
                 *again = redo ? 1 : 0;
@@ -327,8 +362,9 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             if (redo) {
                 m_used = -INFINITY;
                 l_run = 0.f;
-                done = 2 * T;
             }
+            // B_PVDONE: one phase at the end of the first pass, one per key tile of the second
+            const uint32_t last = redo ? T & 1 : 0;
             for (int j = 0; redo && j < T; ++j) {
                 mbar_wait(bar(B_SFULL + t), (T + j) & 1, abort_flag, p.dev_status);
                 fence_after();
@@ -378,7 +414,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (need_rescale) {
                     // O holds tiles < j: P V of tile j - 1 must have completed before the accumulator is scaled;
                     // each of the two threads of a row scales its 64 columns
-                    mbar_wait(bar(B_PVDONE + t), (T + j - 1) & 1, abort_flag, p.dev_status);
+                    mbar_wait(bar(B_PVDONE + t), j & 1, abort_flag, p.dev_status);
                     fence_after();
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
@@ -395,10 +431,11 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 wait_st();
                 fence_before();
                 mbar_arrive(bar(B_PFULL + t));
+                mbar_arrive(bar(B_PFULL + 2 + t));
             }
 
             // ---- epilogue ------------------------------------------------------------------------
-            mbar_wait(bar(B_PVDONE + t), (done - 1) & 1, abort_flag, p.dev_status);
+            mbar_wait(bar(B_PVDONE + t), last, abort_flag, p.dev_status);
             fence_after();
             *xch_mine = l_run;
             named_barrier(pair_bar, 64);
@@ -435,7 +472,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             } else {
                 // part of a cut unit: the un-normalised row (relative to m_used), m and l stay in shared memory, over the
                 // ring and Q: both row tiles' products and the copy warp's stores have to be through
-                for (int tt = 0; tt < n_tiles_q; ++tt) mbar_wait(bar(B_PVDONE + tt), (done - 1) & 1, abort_flag, p.dev_status);
+                for (int tt = 0; tt < n_tiles_q; ++tt) mbar_wait(bar(B_PVDONE + tt), last, abort_flag, p.dev_status);
                 if (p.copy) mbar_wait(bar(B_COPIED), 0, abort_flag, p.dev_status);
                 unsigned char* prow = gbase + OFF_RING + t * PART + row * (HD * 4);
 #pragma unroll 1
@@ -474,7 +511,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 bulk_commit();
                 bulk_wait_read();   // the slot has been read
             }
-            mbar_arrive(bar(B_EMPTY + slot));
+            if (!(n & 1)) mbar_arrive(bar(B_FREE + ((n >> 1) & 1)));   // K tiles end a group
             if (++slot == kSlots) slot = 0, phase ^= 1;
         }
         mbar_arrive(bar(B_COPIED));
