@@ -11,8 +11,9 @@
 // so a softmax thread owns one KEY (TMEM lane) and its scores against the query slots: all 128 lanes work, one
 // exponential per (key, query), no padding rows, a pipeline step covers 128 keys.  A thread keeps its key lane's share of
 // every row sum in registers; they are added up over the lanes once, at the end.  (Two auxiliary warps that read P^T back
-// from shared memory took 1.2 us a tile and set the pace: 15.9 us a launch at L = 1983 with 96 rows, now 13.7.)  With
-// N = 96 (the paper's default budget k = 64 gives 96 active rows) two softmax warpgroups share the columns of a key.
+// from shared memory took 1.2 us a tile and set the pace: 15.9 us a launch at L = 1983 with 96 rows, then 13.7.)  Two softmax
+// warpgroups share the columns of a key: with one, for N = 48 and 64, a thread's serial path is twice as long (L = 768, 34
+// rows: 8.6 us a layer, now 7.9; 4096: 16.0, now 15.6).
 //   softmax  the references m[q] (log2 units) are shared by all keys of the CTA and live in shared memory.  The first
 //            is the score of one valid key; p = 2^(s*scale*log2e - m[q]) needs no reduction as long as no score exceeds
 //            its reference by more than 2^60 (bf16 and fp32 have room for that, and a reference is never above the true
@@ -42,12 +43,11 @@
 //            of the peers (128-byte pieces: a warp whose lanes read different rows takes 2.1 us for what this does in 0.6),
 //            combine, normalise and store; a second cluster barrier keeps every CTA's shared memory alive until its
 //            peers have read it.
-// What bounds it: HBM at long contexts (L = 4096, one sequence, 34 rows: 68.8 MB in 16.2 us), the serial path below that:
-// a launch of one tile per CTA takes 7.1 us: dependency wait 0.8, Q 0.5, scores 1.2, softmax 1.2, P V 0.6, the merge 1.9
-// with its barriers, the exit 0.7.  Code that runs once is fetched about as slowly as it runs, so this path is kept
-// short: index arithmetic before the wait, rolled loops in the merge.  One CTA per SM: with 128 registers a thread, which
-// two would need, the softmax spills and the launches of L = 768 to 4096 take 0.7 to 2 us more.
-// warp 0: TMA producer; warp 1: tcgen05.mma issue; next 4 (or 8) warps: Q, softmax; the auxiliary warps: stale-key bits,
+// What bounds it: HBM at long contexts (L = 4096, one sequence, 34 rows: 68.8 MB in 15.6 us), the serial path below that.
+// Code that runs once is fetched about as slowly as it runs, so this path is kept short: index arithmetic before the
+// wait, rolled loops in the merge.  (Q by TMA queues behind the K/V tiles of the first fill in the TMA unit: 0.6 us more at
+// L = 768, 1.6 at 4096.  Parts sent to the owners instead of read by them, one cluster barrier less: 0.7 us more.)
+// warp 0: TMA producer; warp 1: tcgen05.mma issue; warps 2 to 9: Q, softmax; the auxiliary warps: stale-key bits,
 // cache update.  Launched with programmatic stream serialisation; what the previous kernel wrote is read only
 // after griddepcontrol.wait.  Every mbarrier wait is bounded (EC_ERR_TIMEOUT in dev_status, CTA-wide abort flag: an
 // aborted CTA stores no output); the CTA always frees its TMEM and exits.
@@ -66,7 +66,8 @@ using namespace tc;
 
 constexpr int BK = 128, HD = 128;
 constexpr int kAuxThreads = 64;            // auxiliary warps: stale-key bits and cache update
-__host__ __device__ constexpr int block_threads(int n) { return 64 + (n > 64 ? 256 : 128) + kAuxThreads; }
+constexpr int kSoft = 256;                 // two softmax warpgroups: each takes half of the query slots of every key
+constexpr int kThreads = 64 + kSoft + kAuxThreads;
 constexpr uint32_t SUB = 128 * 128;        // [128 rows x 64 bf16], 128-byte swizzle: 16 KB
 constexpr uint32_t TILE = 2 * SUB;         // [128 x 128] bf16
 constexpr uint32_t STAGE = 2 * TILE;       // K tile + V tile: 64 KB
@@ -95,18 +96,18 @@ __device__ __forceinline__ void touch(V v) {
     else asm volatile("" ::"r"((uint32_t)v) : "memory");
 }
 
-// COLS consecutive 32-bit columns of this thread's TMEM lane -> registers.  ALIGNED32: the first column is
-// a multiple of 32 (one 32-column access, then the rest); otherwise 16-column accesses at multiples of 16.
-template <int COLS, bool ALIGNED32>
-__device__ __forceinline__ void ld_row(uint32_t taddr, uint32_t* r) {
-    static_assert(COLS == 48 || COLS == 64, "columns per thread");
-    if (ALIGNED32) {
-        ld32(taddr, r);
-        if (COLS == 48) ld16(taddr + 32, r + 32); else ld32(taddr + 32, r + 32);
-    } else {
+// COLS consecutive 32-bit columns of this thread's TMEM lane -> registers
+template <int COLS>
+__device__ __forceinline__ void ld_row_part(uint32_t taddr, uint32_t* r) {
+    static_assert(COLS % 8 == 0, "columns per thread");
 #pragma unroll
-        for (int c = 0; c < COLS; c += 16) ld16(taddr + c, r + c);
-    }
+    for (int c = 0; c < COLS; c += COLS % 16 ? 8 : 16)   // (accesses start at multiples of their width)
+        if constexpr (COLS % 16) ld8(taddr + c, r + c);
+        else ld16(taddr + c, r + c);
+}
+template <int COLS>
+__device__ __forceinline__ void ld_row(uint32_t taddr, uint32_t* r) {
+    ld_row_part<COLS>(taddr, r);
     wait_ld<COLS>(r);
 }
 struct KeysParams {
@@ -155,15 +156,12 @@ struct alignas(16) KeysShared {
 };
 
 template <int N>
-__global__ void __launch_bounds__(block_threads(N), 1)
+__global__ void __launch_bounds__(kThreads, 1)
 attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                         const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
                         const KeysParams p) {
     static_assert(N == 48 || N == 64 || N == 96, "query-row slots per CTA");
-    constexpr int WG = N > 64 ? 2 : 1;          // softmax warpgroups: each takes NH of a key's N scores
-    constexpr int NH = N / WG;
-    constexpr int kSoft = 128 * WG;
-    constexpr int kThreads = block_threads(N);
+    constexpr int NH = N / 2;                   // query slots of a softmax thread
     // tensor-memory columns: S^T x 2 and O^T at multiples of NP (the slots rounded up to 64 or 128)
     constexpr uint32_t NP = N <= 64 ? 64 : 128;
     constexpr uint32_t TM_S = 0, TM_O = 2 * NP;
@@ -252,7 +250,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     // here, before the wait below, because what follows it is the serial path of a short launch.
     constexpr int kPieces = N * (HD / 8) / kSoft;
     int q_off[kPieces];
-    if (warp >= 2 && warp < 2 + 4 * WG) {
+    if (warp >= 2 && warp < 2 + kSoft / 32) {
         const int stid = tid - 64;
 #pragma unroll
         for (int u = 0; u < kPieces; ++u) {
@@ -378,7 +376,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             if (progressed) guard.progress();
             else if (__any_sync(0xffffffffu, !guard.tick(abort_flag, p.dev_status))) break;
         }
-    } else if (warp >= 2 + 4 * WG) {
+    } else if (warp >= 2 + kSoft / 32) {
         // ===== auxiliary warps: stale-key bits; the fresh rows into the cache (for later steps) =====
         const int atid = tid - (64 + kSoft);
         if (refresh) {
@@ -425,6 +423,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         const int c0 = wg * NH;
         const int st_w = stid & 127;
         constexpr uint32_t QHALF = N * 128;
+        constexpr int W = NH % 16 ? 8 : 16;          // columns that are loaded together
         // Q rows of this kv head -> swizzled K-major tile of N rows (rows past rows_total are zero): all of a thread's
         // loads are issued before the first is stored
         {
@@ -489,7 +488,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 // will do: a reference is never above the true maximum, and probabilities may exceed it by 2^kRaise).
                 if (quarter == 0) {
                     uint32_t sr[NH];
-                    ld_row<NH, WG == 1>(s_addr, sr);
+                    ld_row<NH>(s_addr, sr);
                     const uint32_t valid = __ballot_sync(0xffffffffu, !past_end);
                     if (lane == __ffs(valid) - 1) {
 #pragma unroll
@@ -505,35 +504,34 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             uint32_t pw[NH / 2];
             while (true) {
                 float dmx0 = -INFINITY, dmx1 = -INFINITY;
-                uint32_t sr[2][16];
-                ld16(s_addr, sr[0]);
+                uint32_t sr[2][W];
+                ld_row_part<W>(s_addr, sr[0]);
 #pragma unroll
-                for (int q = 0; q < NH / 16; ++q) {   // sixteen columns at a time, the next ones on their way
-                    wait_ld<16>(sr[q & 1]);
-                    if (q + 1 < NH / 16) ld16(s_addr + 16 * (q + 1), sr[(q + 1) & 1]);
+                for (int q = 0; q < NH / W; ++q) {   // W columns at a time, the next ones on their way
+                    wait_ld<W>(sr[q & 1]);
+                    if (q + 1 < NH / W) ld_row_part<W>(s_addr + W * (q + 1), sr[(q + 1) & 1]);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float2 mm = *reinterpret_cast<const float2*>(&sh->m[c0 + 16 * q + 2 * i]);
+                    for (int i = 0; i < W / 2; ++i) {
+                        const float2 mm = *reinterpret_cast<const float2*>(&sh->m[c0 + W * q + 2 * i]);
                         f32x2 d2 = fma2(pk(__uint_as_float(sr[q & 1][2 * i]), __uint_as_float(sr[q & 1][2 * i + 1])), sl2_2,
                                         pk(-mm.x, -mm.y));
                         if (past_end) d2 = pk(-INFINITY, -INFINITY);   // probability 0 for every query
                         float d0, d1;
                         upk(d2, d0, d1);
                         if (i & 1) dmx1 = max3(dmx1, d0, d1); else dmx0 = max3(dmx0, d0, d1);
-                        pw[8 * q + i] = pack_bf16x2(fast_exp2(d0), fast_exp2(d1));
+                        pw[W / 2 * q + i] = pack_bf16x2(fast_exp2(d0), fast_exp2(d1));
                     }
                 }
                 if (!named_barrier_or(bar_or, 128, fmaxf(dmx0, dmx1) > kRaise)) break;
                 // ---- rare path: raise the references to the column maxima of this tile, rescale O^T and the row sums by
                 //      the same factors, and once more ----
 #pragma unroll
-                for (int q = 0; q < NH / 16; ++q) {
-                    ld16(s_addr + 16 * q, sr[0]);
-                    wait_ld<16>(sr[0]);
+                for (int q = 0; q < NH / W; ++q) {
+                    ld_row<W>(s_addr + W * q, sr[0]);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
+                    for (int c = 0; c < W; ++c) {
                         const float o = redux_max(past_end ? -INFINITY : __uint_as_float(sr[0][c]));
-                        if (lane == (16 * q + c) % 32) sh->col[quarter][c0 + 16 * q + c] = o;
+                        if (lane == (W * q + c) % 32) sh->col[quarter][c0 + W * q + c] = o;
                     }
                 }
                 named_barrier(bar_sync, 128);
@@ -551,13 +549,13 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                     fence_after();
                     const uint32_t o_addr = tmem + lane_addr + TM_O + c0;
 #pragma unroll
-                    for (int q = 0; q < NH / 16; ++q) {
-                        ld16(o_addr + 16 * q, sr[0]);
-                        wait_ld<16>(sr[0]);
+                    for (int q = 0; q < NH / W; ++q) {
+                        ld_row<W>(o_addr + W * q, sr[0]);
 #pragma unroll
-                        for (int c = 0; c < 16; ++c)
-                            sr[0][c] = __float_as_uint(__uint_as_float(sr[0][c]) * sh->factor[j & 1][c0 + 16 * q + c]);
-                        st16(o_addr + 16 * q, sr[0]);
+                        for (int c = 0; c < W; ++c)
+                            sr[0][c] = __float_as_uint(__uint_as_float(sr[0][c]) * sh->factor[j & 1][c0 + W * q + c]);
+                        if constexpr (W == 8) st8(o_addr + W * q, sr[0]);
+                        else st16(o_addr + W * q, sr[0]);
                     }
                     wait_st();
 #pragma unroll
@@ -582,13 +580,14 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             for (int i = 0; i < NH / 2; ++i)   // (while the second product runs)
                 lsum[i] = add2(lsum[i], pk(__uint_as_float(pw[i] << 16), __uint_as_float(pw[i] & 0xffff0000u)));
         }
-        {   // row sums over the warp's 32 keys: each step halves the columns a lane holds, the last adds neighbours
+        {   // row sums over the warp's 32 keys: the first steps halve the columns a lane holds, the last ones add neighbours
+            constexpr int kHalve = NH % 16 ? 3 : 4;
             float v[NH];
 #pragma unroll
             for (int i = 0; i < NH / 2; ++i) upk(lsum[i], v[2 * i], v[2 * i + 1]);
             int first = c0;
 #pragma unroll
-            for (int step = 1; step <= 4; ++step) {
+            for (int step = 1; step <= kHalve; ++step) {
                 const int n = NH >> step, o = 32 >> step;
                 const bool up = (lane & o) != 0;
 #pragma unroll
@@ -599,9 +598,10 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 first += up ? n : 0;
             }
 #pragma unroll
-            for (int i = 0; i < NH / 16; ++i) {
-                v[i] += __shfl_xor_sync(0xffffffffu, v[i], 1);
-                if (!(lane & 1)) sh->col[quarter][first + i] = v[i];
+            for (int i = 0; i < NH >> kHalve; ++i) {
+#pragma unroll
+                for (int o = 16 >> kHalve; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+                if (!(lane & ((32 >> kHalve) - 1))) sh->col[quarter][first + i] = v[i];
             }
         }
         named_barrier(bar_sync, 128);
@@ -613,7 +613,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         mbar_wait(bar(B_PVDONE), (T - 1) & 1, abort_flag, p.dev_status);   // Q, P^T and the K/V stages are dead from here on
         fence_after();
         uint32_t o[NH];
-        ld_row<NH, WG == 1>(tmem + lane_addr + TM_O + c0, o);
+        ld_row<NH>(tmem + lane_addr + TM_O + c0, o);
         fence_before();
         named_arrive(7, kSoft + 32);   // tensor memory has been read: the MMA warp may free it
         if (C == 1) {
@@ -751,7 +751,7 @@ int resident_clusters_of(int c, uint32_t smem) {
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c, 1, 1);
-    cfg.blockDim = dim3(block_threads(N), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -912,7 +912,7 @@ cudaError_t launch_n(const KeysPlan& pl, const KeysParams& p, const CUtensorMap&
         return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(pl.n_splits, bh, 1);
-    cfg.blockDim = dim3(block_threads(N), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute at[2];
