@@ -77,7 +77,7 @@ constexpr int kMaxActive = 256;            // active rows of a sequence (refresh
 constexpr int kMaxTiles = 1024;            // key tiles of one CTA
 
 enum { B_FULL = 0, B_EMPTY = kMaxStages, B_SFULL = 2 * kMaxStages, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 1,
-       B_QFULL = B_PVDONE + 1, B_LIST = B_QFULL + 1, B_COUNT = B_LIST + 1 };
+       B_QFULL = B_PVDONE + 1, B_LIST = B_QFULL + 1, B_DRY = B_LIST + 1, B_COUNT = B_DRY + 1 };
 
 constexpr uint32_t kBarBytes = (B_COUNT * 8u + 15u) & ~15u;   // the barrier block, padded so that what follows is 16-byte aligned
 
@@ -159,13 +159,17 @@ template <int N>
 __global__ void __launch_bounds__(kThreads, 1)
 attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                         const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
-                        const KeysParams p) {
+                        const KeysParams params) {
     static_assert(N == 48 || N == 64 || N == 96, "query-row slots per CTA");
     constexpr int NH = N / 2;                   // query slots of a softmax thread
     // tensor-memory columns: S^T x 2 and O^T at multiples of NP (the slots rounded up to 64 or 128)
     constexpr uint32_t NP = N <= 64 ? 64 : 128;
     constexpr uint32_t TM_S = 0, TM_O = 2 * NP;
     constexpr uint32_t TM_COLS = (3 * NP <= 256) ? 256 : 512;
+    KeysParams p = params;
+    keep_in_registers(p.k_new, p.active_idx, p.out, p.dev_status, p.scale_log2, p.n_active, p.ctx_len, p.n_q_heads, p.n_kv_heads,
+                      p.group, p.group_inv, p.quads_inv, p.n_splits, p.tiles_per_split, p.n_stages, p.shift, p.n_extra, p.dl,
+                      p.off_p, p.off_stage, p.off_list, p.off_bar);
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
@@ -335,14 +339,9 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                     mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (accumulate || k > 0));
             }
         };
-        // Both products once on whatever shared memory holds, before there is anything to do: the results are
-        // overwritten (S of tile 1, the first P V), but the code has been fetched when the first tile needs it.
-        products_s(0, 1);
-        products_pv(0, false);
         // S of tile j needs the tile; P V of tile j needs P^T from the softmax.  Whichever is ready
         // is issued: P V of a tile does not wait for the next tile to land (its commit frees the stage for the
         // producer), S may run one tile ahead of P V (two S^T buffers).
-        mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
         int next_s = 0, next_pv = 0;
         int ks = 0, vs = 1;               // ring slots of K of tile next_s and V of tile next_pv, and how often they were filled
         uint32_t k_turn = 0, v_turn = 0;
@@ -351,26 +350,40 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             if (slot >= NS) slot -= NS, turn ^= 1;
         };
         SpinGuard guard;
+        // The first round is a dry one: both products on whatever shared memory holds (their results are overwritten: S of
+        // tile 1, the first P V), so that the code of the loop has been fetched when the first tile needs it.
+        bool dry = true;
         while (next_pv < T) {
             bool progressed = false;
-            if (next_s < T && next_s <= next_pv + 1 && mbar_test_warp(bar(B_FULL + ks), k_turn)) {
-                products_s(ks, next_s & 1);   // (the tile has landed)
+            const bool s_ready = next_s < T && next_s <= next_pv + 1 && mbar_test_warp(bar(B_FULL + ks), k_turn);   // the tile has landed
+            if (s_ready || dry) {
+                products_s(ks, dry ? 1 : next_s & 1);
                 if (elected) {
-                    commit(bar(B_SFULL + (next_s & 1)));
-                    commit(bar(B_EMPTY + ks));    // the K slot is free once these products have run
+                    commit(bar(dry ? B_DRY : B_SFULL + (next_s & 1)));
+                    commit(bar(dry ? B_DRY : B_EMPTY + ks));    // the K slot is free once these products have run
                 }
-                step(ks, k_turn);
-                ++next_s;
-                progressed = true;
+                if (!dry) {
+                    step(ks, k_turn);
+                    ++next_s;
+                    progressed = true;
+                }
             }
-            if (mbar_test_warp(bar(B_PFULL), next_pv & 1) && mbar_test_warp(bar(B_FULL + vs), v_turn)) {   // P^T is there, V has landed
+            const bool p_ready = mbar_test_warp(bar(B_PFULL), next_pv & 1) && mbar_test_warp(bar(B_FULL + vs), v_turn);   // P^T is there, V has landed
+            if (p_ready || dry) {
                 products_pv(vs, next_pv > 0);
                 if (elected) {
-                    commit(bar(B_PVDONE));
-                    commit(bar(B_EMPTY + vs));
+                    commit(bar(dry ? B_DRY : B_PVDONE));
+                    commit(bar(dry ? B_DRY : B_EMPTY + vs));
                 }
-                step(vs, v_turn);
-                ++next_pv;
+                if (!dry) {
+                    step(vs, v_turn);
+                    ++next_pv;
+                    progressed = true;
+                }
+            }
+            if (dry) {
+                mbar_wait(bar(B_QFULL), 0, abort_flag, p.dev_status);
+                dry = false;
                 progressed = true;
             }
             if (progressed) guard.progress();

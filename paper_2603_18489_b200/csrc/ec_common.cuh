@@ -43,6 +43,28 @@ cudaError_t ensure_dynamic_smem(PerDeviceOnce& once, Kernel kernel, int bytes) {
     return e;
 }
 
+// Kernel parameters are read from the constant bank wherever the code names them, and the SMs' copies of that bank are
+// dropped while a kernel runs, when the GPU makes the next launch of the stream ready (about 3 us after the one before this has
+// completed).  A read behind that costs a few hundred cycles on a path that is otherwise all registers and shared memory
+// (attend_skip_keys_kernel, L = 768: the first exponentials ended 1100 cycles earlier without such reads).  So a kernel of a few
+// microseconds reads what it needs once, at its start.
+template <typename T>
+__device__ __forceinline__ void keep_in_register(T& v) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long u = (unsigned long long)v;
+        asm volatile("" : "+l"(u));
+        v = (T)u;
+    } else if constexpr (sizeof(T) == 4 && T(0.5f) != T(0)) {
+        asm volatile("" : "+f"(v));
+    } else {
+        asm volatile("" : "+r"(v));
+    }
+}
+template <typename... T>
+__device__ __forceinline__ void keep_in_registers(T&... v) {
+    (keep_in_register(v), ...);
+}
+
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
