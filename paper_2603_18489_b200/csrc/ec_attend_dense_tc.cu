@@ -532,7 +532,8 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         cluster_arrive();
         cluster_wait();           // the partials of all CTAs are complete
         float* weight = reinterpret_cast<float*>(gbase + OFF_Q + 2 * BM * 8);   // [row of the share][8]
-        const int share = n_tiles_q * BM / p.split, row0 = part * share;       // split is 2, 4 or 8
+        const int rows = n_tiles_q * BM, per = ((rows + p.split - 1) / p.split + 3) & ~3, row0 = part * per;   // whole groups of four
+        const int share = min(per, rows - row0);
         for (int i = tid; i < share; i += kThreads) {
             float mm[8], ll[8], M = -INFINITY, L = 0.f;
 #pragma unroll
@@ -617,11 +618,12 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int batch, int n_kv_heads, i
 
 // How the launch is cut.  Units = (sequence, query head, row-tile pair); a unit walks over all T key tiles.  The
 // hardware deals the CTAs to the SMs in launch order, so the last units form a partial wave: `tail` units on `sms` SMs.
-// Cutting each of them along the keys into s CTAs (s = 2, 4 or 8, at least four key tiles each) fills that wave:
-// cost in key-tile times, with two tiles' worth of fixed cost per CTA, one more for the merge, and one for the launch:
-//     waves_full * (T + 2) + ceil(tail * s / sms) * (ceil(T / s) + 3) + 1
-// s = 1 (no cut) unless a cut saves at least 3 %.  (Not fitted: a unit alone has a fixed part of 6.6 us, 3.9 key tiles of
-// 1.7 us.  The cuts that the rule chooses are gains at the shapes timed, see attend_dense_kernel.)
+// Cutting each of them along the keys into s CTAs, a cluster, fills that wave.  As many parts as fit at once and leave four
+// tiles each, if that takes five tiles off the wave: a launch of its own with its start and merge costs about as much.
+// us a layer by number of parts (the rule's in brackets): 4 units of 16 tiles (19 heads of 2048) 1: 57.9, 2: 52.4, (4): 49.5,
+// 8: 48.2; 12 of 21 (28 heads of 2600) 1: 105.6, 2: 100.8, 4: 97.4, (5): 96.7, 8: 95.4; 12 of 10 (32 heads of 1280) 1: 41.5,
+// (2): 39.9, 5: 39.4; 12 of 9 (1152) (1): 36.0, 2: 37.5; 40 of 12 (2 x 1531, 28 heads) 1: 71.8, 2: 69.4, (3): 69.0, 4 (two
+// rounds): 82.7; 20 of 12 (28 heads of 1500) 1: 46.7, 2: 44.2, (3): 43.6; 68 of 32 (32 heads of 4096) 1: 217, (2): 205, 3: 222.
 struct DensePlan {
     int n_pairs, units, n_full, split;
 };
@@ -632,20 +634,13 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
     pl.n_full = pl.units;
     pl.split = 1;
     const int sms = sm_count();
-    const long long T = (d.ctx_len + BN - 1) / BN;
-    const long long waves_full = pl.units / sms, tail = pl.units % sms;
-    if (tail > 0) {
-        long long best = (waves_full + 1) * (T + 2);
-        const long long need = best - best * 3 / 100;
-        for (int s = 2; s <= 8; s *= 2) {
-            if (T / s < 4) break;
-            const long long cost = waves_full * (T + 2) + ((tail * s + sms - 1) / sms) * ((T + s - 1) / s + 3) + 1;
-            if (cost < best && cost <= need) {
-                best = cost;
-                pl.split = s;
-            }
-        }
-        if (pl.split > 1) pl.n_full = pl.units - (int)tail;
+    const int T = (d.ctx_len + BN - 1) / BN, tail = pl.units % sms;
+    for (int s = 8; s >= 2 && tail > 0; --s) {
+        const int at_once = 8 * (sms / 8 / s);   // clusters of s, inside the eight GPCs
+        if (T / s < 4 || T - (T + s - 1) / s < 5 || tail > at_once) continue;
+        pl.split = s;
+        pl.n_full = pl.units - tail;
+        break;
     }
     return pl;
 }
