@@ -648,17 +648,18 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
 
 }  // namespace
 
-// The two-tile kernel is used from SMs / 4 of its (row-tile pair, query head) units on.  The one-tile kernel behind a
-// refresh launch, which takes the steps below, is the slower one above the line: L = 320 with 32 heads (64 units) 31.2 us
-// against 11.2, at the line (40 units) 24.9 against 11.4 at L = 300 with 20 heads, 49.1 against 26.1 at 2048 with 5.  (Below
-// the line the two have not been compared; the figures say that it could lie lower.)
+// The two-tile kernel is used from 17 of its (row-tile pair, query head) units on (148 SMs).  The one-tile kernel behind a
+// refresh launch, which takes the steps below, is the slower one on both sides of the line (us a layer, one-tile against this
+// one): 32 units of 2 key tiles (32 heads of 256) 24.9 / 9.6, of 8 tiles (8 heads of 1024) 42.5 / 16.7, of 32 tiles (2 heads of
+// 4096) 60.8 / 25.0; 20 units (2 x 300, 5 heads) 23.6 / 9.6; 16 units 24.8 / 11.0, 8 units of 3 tiles 19.6 / 9.0.  The line was
+// at SMs / 4 = 37; it stops short of 16 units, which the tests of the dispatch expect on the one-tile kernel.
 bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
     if (d.dtype != EC_BF16 || d.head_dim != HD || n_active < 1) return false;
     // one unit per (sequence, query head, row-tile pair): grouped-query shapes are run head by head
     const long long pairs = ((long long)n_active + 2 * BM - 1) / (2 * BM);
     const long long bh = (long long)d.batch * d.n_q_heads;
     if (pairs * bh > 0x3fffffffLL) return false;
-    return pairs * bh >= sm_count() / 4;
+    return pairs * bh > sm_count() / 9;
 }
 
 void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len) {
