@@ -11,9 +11,8 @@
 // so a softmax thread owns one KEY (TMEM lane) and its scores against the query slots: all 128 lanes work, one
 // exponential per (key, query), no padding rows, a pipeline step covers 128 keys.  A thread keeps its key lane's share of
 // every row sum in registers; they are added up over the lanes once, at the end.  (Two auxiliary warps that read P^T back
-// from shared memory took 1.2 us a tile and set the pace: 15.9 us a launch at L = 1983 with 96 rows, then 13.7.)  Two softmax
-// warpgroups share the columns of a key: with one, for N = 48 and 64, a thread's serial path is twice as long (L = 768, 34
-// rows: 8.6 us a layer, now 7.9; 4096: 16.0, now 15.6).
+// from shared memory took 1.2 us a tile and set the pace: 15.9 us a launch at L = 1983 with 96 rows, then 13.7.)  Two
+// to four softmax warpgroups share the columns of a key, which shortens a thread's serial path (see soft_groups).
 //   softmax  the references m[q] (log2 units) are shared by all keys of the CTA and live in shared memory.  The first
 //            is the score of one valid key; p = 2^(s*scale*log2e - m[q]) needs no reduction as long as no score exceeds
 //            its reference by more than 2^60 (bf16 and fp32 have room for that, and a reference is never above the true
@@ -47,7 +46,7 @@
 // Code that runs once is fetched about as slowly as it runs, so this path is kept short: index arithmetic before the
 // wait, rolled loops in the merge.  (Q by TMA queues behind the K/V tiles of the first fill in the TMA unit: 0.6 us more at
 // L = 768, 1.6 at 4096.  Parts sent to the owners instead of read by them, one cluster barrier less: 0.7 us more.)
-// warp 0: TMA producer; warp 1: tcgen05.mma issue; warps 2 to 9: Q, softmax; the auxiliary warps: stale-key bits,
+// warp 0: TMA producer; warp 1: tcgen05.mma issue; the softmax warps: Q, softmax; two auxiliary warps: stale-key bits,
 // cache update.  Launched with programmatic stream serialisation; what the previous kernel wrote is read only
 // after griddepcontrol.wait.  Every mbarrier wait is bounded (EC_ERR_TIMEOUT in dev_status, CTA-wide abort flag: an
 // aborted CTA stores no output); the CTA always frees its TMEM and exits.
@@ -66,8 +65,11 @@ using namespace tc;
 
 constexpr int BK = 128, HD = 128;
 constexpr int kAuxThreads = 64;            // auxiliary warps: stale-key bits and cache update
-constexpr int kSoft = 256;                 // two softmax warpgroups: each takes half of the query slots of every key
-constexpr int kThreads = 64 + kSoft + kAuxThreads;
+// Softmax warpgroups: each takes an equal share of the query slots of every key, a multiple of 8.  us a pass by their number:
+// 48 slots, 32 layers of 768 1: 273.8, 2: 247.2, 3: 249.7; 64 slots, 16 layers of 512 with k = 32 2: 153.5, 4: 149.9; 96
+// slots, 32 layers of 1983 2: 453.2, 3: 448.2, 4: 460.1.
+__host__ __device__ constexpr int soft_groups(int n) { return n == 48 ? 2 : n == 64 ? 4 : 3; }
+__host__ __device__ constexpr int block_threads(int n) { return 64 + 128 * soft_groups(n) + kAuxThreads; }
 constexpr uint32_t SUB = 128 * 128;        // [128 rows x 64 bf16], 128-byte swizzle: 16 KB
 constexpr uint32_t TILE = 2 * SUB;         // [128 x 128] bf16
 constexpr uint32_t STAGE = 2 * TILE;       // K tile + V tile: 64 KB
@@ -156,12 +158,13 @@ struct alignas(16) KeysShared {
 };
 
 template <int N>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(block_threads(N), 1)
 attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                         const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
                         const KeysParams params) {
     static_assert(N == 48 || N == 64 || N == 96, "query-row slots per CTA");
-    constexpr int NH = N / 2;                   // query slots of a softmax thread
+    constexpr int NH = N / soft_groups(N);      // query slots of a softmax thread
+    constexpr int kSoft = 128 * soft_groups(N), kThreads = block_threads(N);
     // tensor-memory columns: S^T x 2 and O^T at multiples of NP (the slots rounded up to 64 or 128)
     constexpr uint32_t NP = N <= 64 ? 64 : 128;
     constexpr uint32_t TM_S = 0, TM_O = 2 * NP;
@@ -628,7 +631,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         uint32_t o[NH];
         ld_row<NH>(tmem + lane_addr + TM_O + c0, o);
         fence_before();
-        named_arrive(7, kSoft + 32);   // tensor memory has been read: the MMA warp may free it
+        named_arrive(1, kSoft + 32);   // tensor memory has been read: the MMA warp may free it
         if (C == 1) {
             // ---- single CTA per (sequence, kv head): normalise and store column kk of every query row ----
             if (!*abort_flag) {
@@ -657,7 +660,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     }
     if (warp == 1) {
         __syncwarp();
-        named_barrier(7, kSoft + 32);
+        named_barrier(1, kSoft + 32);
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TM_COLS) : "memory");
     }
@@ -764,7 +767,7 @@ int resident_clusters_of(int c, uint32_t smem) {
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(block_threads(N), 1, 1);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -925,7 +928,7 @@ cudaError_t launch_n(const KeysPlan& pl, const KeysParams& p, const CUtensorMap&
         return ea;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(pl.n_splits, bh, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(block_threads(N), 1, 1);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute at[2];
