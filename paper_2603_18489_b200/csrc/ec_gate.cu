@@ -4,8 +4,8 @@
 // (Algorithm 1: E > tau -> recompute, else skip).
 //
 // R*V*sizeof(elem) bytes are read exactly once; the arithmetic is about seven instructions per element.
-//   grid  = (splits, R): CTA (s, r) owns the columns [s*chunk, (s+1)*chunk) of row r; the split count is
-//           chosen so that the whole grid is about one resident wave (4 CTAs of 256 threads per SM);
+//   grid  : a CTA owns one chunk of columns of one row; rows have s or s + 1 chunks, so that the CTAs are one resident wave
+//           without a place left over (4 CTAs of 256 threads per SM), see plan_chunks;
 //   loop  : a thread takes the 16-byte vectors (bf16x8 / f32x4) t, t + 256, ... of the chunk in ascending
 //           order through four rolling registers and keeps a running
 //           (max, S, T) with S = sum 2^d, T = sum 2^d * d, d = x*log2(e) - base: one ex2.approx per element
@@ -46,7 +46,8 @@ namespace {
 
 constexpr int kGateThreads = 256;
 constexpr int kCtasPerSm = 4;
-constexpr int kVec = 8;  // columns per thread in one slab of kGateThreads * kVec columns (chunk granularity)
+constexpr int kVec = 8;      // columns per thread in one slab of kGateThreads * kVec columns
+constexpr int kPiece = 256;  // chunks of unequal rows are multiples of this many columns
 constexpr int kMaxSplits = 96;
 constexpr float kDClamp = -150.0f;  // 2^-150 flushes to 0 (ftz)
 constexpr int kInFlight = 4;         // 16-byte vectors a thread keeps in flight
@@ -166,8 +167,11 @@ struct Loader<float> {
 struct GateParams {
     const void* logits;
     long long row_stride;
-    int n_rows, vocab, rows_per_seq, splits;
-    int chunk;          // columns per CTA, a multiple of kGateThreads * kVec
+    int n_rows, vocab, rows_per_seq;
+    // the first n_few rows are cut into `splits` chunks of chunk[0] columns, the others into one more, of chunk[1]
+    int n_few, splits, chunk[2];
+    unsigned int inverse[2];   // ceil(2^32 / splits), ceil(2^32 / (splits + 1)): quotients of a block index (below 2^23) by mulhi
+    int pitch;          // partials of a row
     int single_level;   // 1: the last CTA of a sequence finishes all its rows; 0: per-row then per-sequence tickets
     const uint8_t* flags;
     float tau;
@@ -178,7 +182,7 @@ struct GateParams {
     int* decision_out;
     int* row_ticket;  // [n_rows], zero on entry, zero on exit
     int* seq_ticket;  // [n_seq],  zero on entry, zero on exit
-    Partial* partials;  // [n_rows, splits]
+    Partial* partials;  // [n_rows, pitch]
     // decode mode (masked != nullptr, single_level only): the decoded set comes from the confidences
     uint8_t* masked;       // in/out [n_rows]: rows still masked; cleared for the rows decoded here
     float conf_thr;
@@ -189,12 +193,18 @@ struct GateParams {
     float* max_conf_out;   // [n_seq]
 };
 
+template <bool kUneven>
+__device__ __forceinline__ int splits_of(const GateParams& p, int row) { return p.splits + (kUneven && row >= p.n_few ? 1 : 0); }
+__device__ __forceinline__ const Partial* partials_of(const GateParams& p, int row) { return p.partials + (long long)row * p.pitch; }
+
 // warp-collective: merge the split partials of one row, write the row's outputs, return its entropy (all lanes)
+template <bool kUneven>
 __device__ __forceinline__ float finish_row(const GateParams& p, int row, int lane) {
     Partial acc;
     acc.M = -INFINITY; acc.S = 0.f; acc.T = 0.f; acc.idx = 0x7fffffff;
-    for (int s = lane; s < p.splits; s += 32) {
-        const float4 f = __ldcg(reinterpret_cast<const float4*>(&p.partials[(long long)row * p.splits + s]));
+    const int n = splits_of<kUneven>(p, row);
+    for (int s = lane; s < n; s += 32) {
+        const float4 f = __ldcg(reinterpret_cast<const float4*>(partials_of(p, row) + s));
         Partial q;
         q.M = f.x; q.S = f.y; q.T = f.z; q.idx = __float_as_int(f.w);
         acc = merge(acc, q);
@@ -218,7 +228,9 @@ __device__ __forceinline__ float finish_row(const GateParams& p, int row, int la
     return H;
 }
 
-template <typename T>
+// kUneven: rows of splits or splits + 1 chunks on a grid of one dimension; otherwise (splits, rows).  (One kernel for both cost
+// the even launches 1 to 4 %.)
+template <typename T, bool kUneven>
 __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const GateParams p) {
     constexpr int kWarps = kGateThreads / 32;
     __shared__ float4 s_part[kWarps];
@@ -229,11 +241,22 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
 
     using L = Loader<T>;
     constexpr int EPV = L::EPV;
-    const int row = blockIdx.y, split = blockIdx.x, tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the rows with fewer and larger chunks come first: the SMs are dealt the large chunks, then the small ones
+    int row = blockIdx.y, split = blockIdx.x, n_splits = p.splits, chunk = p.chunk[0];
+    if (kUneven && p.pitch > p.splits) {   // (always; without the second condition the instance spills and is 1 to 2 % slower)
+        const int few = p.n_few * p.splits;
+        const bool more = split >= few;
+        const int at = more ? split - few : split;
+        row = (int)__umulhi((unsigned)at, more ? p.inverse[1] : p.inverse[0]);
+        if (n_splits == 1 && !more) row = at;
+        if (more) ++n_splits, chunk = p.chunk[1];
+        split = at - row * n_splits;
+        if (more) row += p.n_few;
+    }
     const T* rowp = reinterpret_cast<const T*>(p.logits) + (long long)row * p.row_stride;
-    const int c0 = split * p.chunk;
-    const int c_end = min(p.vocab, c0 + p.chunk);
+    const int c0 = split * chunk;
+    const int c_end = min(p.vocab, c0 + chunk);
 
     // Thread t owns the whole vectors t, t + 256, ... of the chunk.  They pass through a rolling set of kInFlight registers:
     // as soon as a vector has been consumed its register is given to the load kInFlight vectors ahead.  The ragged end
@@ -410,10 +433,12 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
             acc = merge(acc, q);
         }
         if (lane == 0) {
-            *reinterpret_cast<float4*>(&p.partials[(long long)row * p.splits + split]) =
+            *reinterpret_cast<float4*>(p.partials + (long long)row * p.pitch + split) =
                 make_float4(acc.M, acc.S, acc.T, __int_as_float(acc.idx));
             const int old = p.single_level ? ticket_add(&p.seq_ticket[seq], 1) : ticket_add(&p.row_ticket[row], 1);
-            s_last = old == (p.single_level ? p.rows_per_seq * p.splits : p.splits) - 1;
+            int all = p.rows_per_seq * p.splits;   // partials of the sequence
+            if (kUneven) all = p.rows_per_seq * (p.splits + 1) - min(max(p.n_few - seq * p.rows_per_seq, 0), p.rows_per_seq);
+            s_last = old == (p.single_level ? all : n_splits) - 1;
         }
     }
     __syncthreads();   // orders the ticket's acquire before the other threads' reads of the partials
@@ -427,11 +452,12 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
             const bool ok = r < p.rows_per_seq;
             const int rr = seq * p.rows_per_seq + (ok ? r : 0);
             float4 f[4];
+            const int n_part = splits_of<kUneven>(p, rr);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int sp = j + 8 * k;
                 f[k] = make_float4(-INFINITY, 0.f, 0.f, __int_as_float(0x7fffffff));
-                if (ok && sp < p.splits) f[k] = __ldcg(reinterpret_cast<const float4*>(&p.partials[(long long)rr * p.splits + sp]));
+                if (ok && sp < n_part) f[k] = __ldcg(reinterpret_cast<const float4*>(partials_of(p, rr) + sp));
             }
             Partial acc;
             acc.M = f[0].x; acc.S = f[0].y; acc.T = f[0].z; acc.idx = __float_as_int(f[0].w);
@@ -546,7 +572,7 @@ __global__ void __launch_bounds__(kGateThreads, kCtasPerSm) gate_kernel(const Ga
 
     // ---- last CTA of the row finishes the row; the last row of the sequence finishes the sequence ----
     if (warp != 0) return;
-    finish_row(p, row, lane);
+    finish_row<kUneven>(p, row, lane);
     int seq_last = 0;
     if (lane == 0) {
         p.row_ticket[row] = 0;
@@ -583,26 +609,40 @@ GateWs carve(int n_rows) {
     return w;
 }
 
-// split count and columns per CTA: about one resident wave (4 CTAs of 256 threads per SM), every CTA a whole number
-// of 2048-column slabs, at most kMaxSplits partials per row
-void plan_chunks(int n_rows, int vocab, int* splits, int* chunk, int max_splits = kMaxSplits) {
+// How the rows are cut: one resident wave of 4 CTAs of 256 threads per SM, all its places taken.  Rows get `splits` chunks
+// or one more, so that the CTAs are as many as the places: with equal splits, 512 CTAs of 256 rows on 592 places, 68 SMs had
+// four CTAs, 80 three, and the former worked 3.4 us longer (bf16 [256, 126464] 20.5 -> 18.4 us with new logits each pass, 160
+// rows 13.2 -> 11.9, 32 rows 6.25 -> 6.04; fp32 [32, 126464] 6.86 -> 6.38).  fp32 waits for memory rather than for its
+// arithmetic, and from about 100 rows on large equal chunks are the better ones (128 rows 13.75 against 13.99).  Equal chunks,
+// where the rule or the limit of splits asks for them, are whole 2048-column slabs.
+void plan_chunks(GateParams& p, int max_splits, bool bf16) {
     const int slab = kGateThreads * kVec;
     const long long slots = (long long)kCtasPerSm * sm_count();
-    long long want = slots / n_rows;
+    long long want = slots / p.n_rows;
+    p.n_few = p.n_rows;
+    if (want >= (bf16 ? 1 : 6) && want + 1 <= max_splits && p.vocab / (want + 1) >= slab) {
+        p.splits = (int)want;
+        p.pitch = p.splits + 1;
+        p.n_few = p.n_rows - (int)(slots - want * p.n_rows);
+        for (int k = 0; k < 2; ++k) {
+            const int n = p.splits + k;
+            p.inverse[k] = (unsigned int)((0x100000000LL + n - 1) / n);
+            p.chunk[k] = ((p.vocab + n - 1) / n + kPiece - 1) / kPiece * kPiece;
+        }
+        return;
+    }
     if (want < 1) want = 1;
     if (want > max_splits) want = max_splits;
-    long long per = (vocab + want - 1) / want;
-    const long long per_min = (vocab + kMaxSplits - 1) / kMaxSplits;
-    if (per < per_min) per = per_min;
-    per = (per + slab - 1) / slab * slab;
-    *chunk = (int)per;
-    *splits = (int)((vocab + per - 1) / per);
+    const int per = (int)((p.vocab + want - 1) / want);
+    p.chunk[0] = p.chunk[1] = (per + slab - 1) / slab * slab;
+    p.splits = p.pitch = (p.vocab + p.chunk[0] - 1) / p.chunk[0];
+    p.inverse[0] = p.inverse[1] = 0;
 }
 
-template <typename T>
+template <typename T, bool kUneven>
 cudaError_t launch_t(const GateParams& p, cudaStream_t stream) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(p.splits, p.n_rows, 1);
+    cfg.gridDim = kUneven ? dim3(p.n_few * p.splits + (p.n_rows - p.n_few) * p.pitch, 1, 1) : dim3(p.splits, p.n_rows, 1);
     cfg.blockDim = dim3(kGateThreads, 1, 1);
     cfg.stream = stream;
     cudaLaunchAttribute at[1];
@@ -610,7 +650,7 @@ cudaError_t launch_t(const GateParams& p, cudaStream_t stream) {
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gate_kernel<T>, p);
+    return cudaLaunchKernelEx(&cfg, gate_kernel<T, kUneven>, p);
 }
 
 }  // namespace
@@ -631,8 +671,6 @@ cudaError_t launch_gate(const GateArgs& a, cudaStream_t stream) {
     p.n_rows = a.n_rows;
     p.vocab = a.vocab;
     p.rows_per_seq = a.rows_per_seq;
-    p.splits = 0;
-    p.chunk = 0;
     p.single_level = 0;
     p.flags = a.flags;
     p.tau = a.tau;
@@ -653,11 +691,11 @@ cudaError_t launch_gate(const GateArgs& a, cudaStream_t stream) {
     // decode mode and the extra metrics need all rows of a sequence in one CTA's hands at the end: the single-level
     // finish (at most 32 splits)
     const bool one_cta_finish = a.masked || a.entropy_sum_out || a.max_conf_out;
-    plan_chunks(a.n_rows, a.vocab, &p.splits, &p.chunk, one_cta_finish ? 32 : kMaxSplits);
-    if (p.splits > kMaxSplits) return cudaErrorInvalidValue;   // vocab > 96 * 8192: rejected by the API layer before this
-    p.single_level = (a.rows_per_seq <= kSingleLevelMaxRows && p.splits <= 32) ? 1 : 0;
+    plan_chunks(p, one_cta_finish ? 32 : kMaxSplits, a.dtype == EC_BF16);
+    p.single_level = (a.rows_per_seq <= kSingleLevelMaxRows && p.pitch <= 32) ? 1 : 0;
     if (one_cta_finish && !p.single_level) return cudaErrorInvalidValue;   // rows_per_seq > 64 or vocab > 32 * 8192 * ...: rejected by the API layer
-    return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16>(p, stream) : launch_t<float>(p, stream);
+    if (p.pitch > p.splits) return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16, true>(p, stream) : launch_t<float, true>(p, stream);
+    return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16, false>(p, stream) : launch_t<float, false>(p, stream);
 }
 
 }  // namespace ec
