@@ -100,8 +100,7 @@ template <bool kCut>
 __global__ void __launch_bounds__(kThreads, 1)
 attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kd,
-                    const __grid_constant__ CUtensorMap map_vd, const __grid_constant__ CUtensorMap map_o,
-                    const DenseParams p) {
+                    const __grid_constant__ CUtensorMap map_vd, const DenseParams p) {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
@@ -136,7 +135,6 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             prefetch_map(&map_kd);
             prefetch_map(&map_vd);
         }
-        prefetch_map(&map_o);
         for (int i = 0; i < B_COUNT; ++i)
             mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 4) ? 256u : (p.copy && i >= B_FREE && i < B_FREE + 2) ? 2u : 1u);
         *abort_flag = 0;
@@ -450,10 +448,10 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             const float l_row = l_run + *xch_other;   // both halves of a row carry the same reference maximum
             if constexpr (!kCut) {
                 // Whole unit: the normalised row goes to shared memory, over the row tile's Q (its last scores are long
-                // formed), and leaves by TMA, a box of 32 rows and half the columns per warp, so that no warp waits for
-                // another (rows past n_active are not written; 510.4 -> 507.7 us a pass of 32 layers of 768).  Rolled: the code of an
-                // epilogue runs once a CTA and is fetched at about its own length in time; unrolled, with 16-byte stores
-                // to global memory, it took 3.5 us.
+                // formed), and from there, a warp its own 32 rows and 64 columns, to global memory in pieces of 128 bytes.
+                // (us a pass of 32 layers of 768: by TMA, a box for each row tile 510.4, for each warp 507.5; like this, with
+                // no copy to wait for, 503.4.  Straight from the registers, a thread 128 bytes of its row: 3.5 us a unit.)
+                // Rolled: the code of an epilogue runs once a unit and is fetched at about its own length in time.
                 const float inv = 1.f / l_row;
                 unsigned char* qrow = gbase + OFF_Q + t * TILE + h * SUB + (row >> 3) * 1024 + (row & 7) * 128;
 #pragma unroll 1
@@ -471,12 +469,19 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         *reinterpret_cast<uint4*>(qrow + (((c * 4 + v4) ^ (row & 7)) << 4)) = w;
                     }
                 }
-                fence_async_smem();
                 __syncwarp();
-                if (lane == 0 && !*abort_flag) {   // a CTA whose wait gave up stores nothing
-                    tma_store_5d(&map_o, base + OFF_Q + t * TILE + h * SUB + quarter * 4096, 0, r_pair + t * BM + quarter * 32, hk, h, b);
-                    bulk_commit();
-                    bulk_wait_read();
+                if (!*abort_flag) {   // a CTA whose wait gave up stores nothing
+                    const unsigned char* mine = gbase + OFF_Q + t * TILE + h * SUB + quarter * 4096;
+                    const int g = lane >> 3, ch = lane & 7;   // four rows at a time, eight lanes a row
+                    const int r0 = r_pair + t * BM + quarter * 32 + g;
+                    __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + r0) * p.n_q_heads + hk) * HD + h * 64 + ch * 8;
+                    const long long step = 4LL * p.n_q_heads * HD;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int rr = k * 4 + g;
+                        const uint4 w = *reinterpret_cast<const uint4*>(mine + (rr >> 3) * 1024 + (rr & 7) * 128 + ((ch ^ (rr & 7)) << 4));
+                        if (r0 + k * 4 < p.rows_total) *reinterpret_cast<uint4*>(dst + k * step) = w;
+                    }
                 }
             } else {
                 // part of a cut unit: the un-normalised row (relative to m_used), m and l stay in shared memory, over the
@@ -700,16 +705,16 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     p.n_full = pl.n_full;
     p.split = pl.split;
     p.wait_first = pl.n_full == 0;
-    CUtensorMap map_q, map_o;
-    for (int i = 0; i < 2; ++i) {   // q and out have the same layout
+    CUtensorMap map_q;
+    {
         EncodeTiledFn fn = encode_fn();
         if (!fn) return cudaErrorInvalidValue;
         const cuuint64_t dims[5] = {64, (cuuint64_t)a.n_active, (cuuint64_t)a.d.n_q_heads, 2, (cuuint64_t)a.d.batch};
         const cuuint64_t strides[4] = {(cuuint64_t)a.d.n_q_heads * HD * 2, (cuuint64_t)HD * 2, 128,
                                        (cuuint64_t)a.n_active * a.d.n_q_heads * HD * 2};
-        const cuuint32_t box[5] = {64, (cuuint32_t)(i ? 32 : BM), 1, (cuuint32_t)(i ? 1 : 2), 1};
+        const cuuint32_t box[5] = {64, (cuuint32_t)BM, 1, 2, 1};
         const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-        if (fn(i ? &map_o : &map_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, i ? a.out : const_cast<void*>(a.q), dims, strides, box, estr,
+        if (fn(&map_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.q), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -731,7 +736,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
         if (const cudaError_t e = ensure_dynamic_smem(once_whole, attend_dense_kernel<false>, (int)SMEM_BYTES); e != cudaSuccess) return e;
         cfg.gridDim = dim3(pl.n_full, 1, 1);
         cfg.numAttrs = 1;
-        if (const cudaError_t e = cudaLaunchKernelEx(&cfg, attend_dense_kernel<false>, map_k, map_v, map_q, map_kd, map_vd, map_o, p);
+        if (const cudaError_t e = cudaLaunchKernelEx(&cfg, attend_dense_kernel<false>, map_k, map_v, map_q, map_kd, map_vd, p);
             e != cudaSuccess)
             return e;
     }
@@ -739,7 +744,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     if (const cudaError_t e = ensure_dynamic_smem(once_cut, attend_dense_kernel<true>, (int)SMEM_BYTES); e != cudaSuccess) return e;
     cfg.gridDim = dim3((pl.units - pl.n_full) * pl.split, 1, 1);
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_dense_kernel<true>, map_k, map_v, map_q, map_kd, map_vd, map_o, p);
+    return cudaLaunchKernelEx(&cfg, attend_dense_kernel<true>, map_k, map_v, map_q, map_kd, map_vd, p);
 }
 
 }  // namespace ec
