@@ -624,10 +624,10 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int batch, int n_kv_heads, i
 // How the launch is cut.  Units = (sequence, query head, row-tile pair); a unit walks over all T key tiles.  The
 // hardware deals the CTAs to the SMs in launch order, so the last units form a partial wave: `tail` units on `sms` SMs.
 // Cutting each of them along the keys into s CTAs, a cluster, fills that wave.  As many parts as fit at once and leave four
-// tiles each, if that takes five tiles off the wave: a launch of its own with its start and merge costs about as much.
+// tiles each, if that takes four tiles off the wave: a launch of its own with its start and merge costs about as much.
 // us a layer by number of parts (the rule's in brackets): 4 units of 16 tiles (19 heads of 2048) 1: 57.9, 2: 52.4, (4): 49.5,
 // 8: 48.2; 12 of 21 (28 heads of 2600) 1: 105.6, 2: 100.8, 4: 97.4, (5): 96.7, 8: 95.4; 12 of 10 (32 heads of 1280) 1: 41.5,
-// (2): 39.9, 5: 39.4; 12 of 9 (1152) (1): 36.0, 2: 37.5; 40 of 12 (2 x 1531, 28 heads) 1: 71.8, 2: 69.4, (3): 69.0, 4 (two
+// (2): 39.9, 5: 39.4; 12 of 9 (1152) 1: 36.0, (2): 37.5; 40 of 12 (2 x 1531, 28 heads) 1: 71.8, 2: 69.4, (3): 69.0, 4 (two
 // rounds): 82.7; 20 of 12 (28 heads of 1500) 1: 46.7, 2: 44.2, (3): 43.6; 68 of 32 (32 heads of 4096) 1: 217, (2): 205, 3: 222.
 struct DensePlan {
     int n_pairs, units, n_full, split;
@@ -642,7 +642,7 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
     const int T = (d.ctx_len + BN - 1) / BN, tail = pl.units % sms;
     for (int s = 8; s >= 2 && tail > 0; --s) {
         const int at_once = 8 * (sms / 8 / s);   // clusters of s, inside the eight GPCs
-        if (T / s < 4 || T - (T + s - 1) / s < 5 || tail > at_once) continue;
+        if (T / s < 4 || T - (T + s - 1) / s < 4 || tail > at_once) continue;
         pl.split = s;
         pl.n_full = pl.units - tail;
         break;
