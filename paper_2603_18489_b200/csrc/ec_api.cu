@@ -32,7 +32,7 @@ int sm_count() {
 namespace {
 
 // bf16 with head_dim 128 runs on the tcgen05 kernels (a fused skip-step kernel when the packed query rows fit, a dense
-// kernel otherwise), bf16 with head_dim 64 on the mma.sync kernel, fp32 on the SIMT kernel.
+// kernel otherwise), bf16 with head_dim 64 on the dense tcgen05 kernel or the mma.sync one, fp32 on the SIMT kernel.
 // EC_ATTEND_IMPL (environment, read once) = "dense" forces the one-tile dense tcgen05 kernel with a separate refresh
 // launch, "rows" the skip kernel with query rows on the M axis: for A/B measurements only.
 int forced_impl() {
@@ -69,7 +69,7 @@ AttendPath choose_path(const ec_attn_desc& d, int n_active, bool fresh_kv, bool 
     if (use_skip_keys(d, n_active, fresh_kv)) return PATH_SKIP_KEYS;
     if (use_skip(d, n_active)) return PATH_SKIP_ROWS;
     if (d.dtype != EC_BF16) return PATH_F32;
-    if (use_tc(d) && forced_impl() != 2 && attend_dense_supported(d, n_active))
+    if (forced_impl() != 2 && attend_dense_supported(d, n_active, fresh_kv))
         return fresh_kv && !index_list ? PATH_DENSE_FROM_NEW : PATH_DENSE;
     return use_tc(d) ? PATH_TC_ONE_TILE : PATH_MMA;
 }

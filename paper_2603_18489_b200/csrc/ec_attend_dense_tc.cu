@@ -1,6 +1,7 @@
-// ec_attend, recompute step and other dense cases (bf16, head_dim 128, more than 256 packed query rows per
-// kv head): bidirectional attention of every active row over the whole cache on the Blackwell tensor cores
-// (Appendix A of the paper, full branch; Algorithm 1 FullPrefill / FullRecompute).
+// ec_attend, recompute step and other dense cases (bf16; head_dim 128 with more than 256 packed query rows per
+// kv head, head_dim 64 where that is faster than mma.sync, see prefers_mma): bidirectional attention of every active row over
+// the whole cache on the Blackwell tensor cores (Appendix A of the paper, full branch; Algorithm 1 FullPrefill /
+// FullRecompute).  What follows describes 128-wide heads; with 64 columns every tile is half as large, and O_t has 64 columns.
 //
 // The step is bound by the tensor pipe and, next to it, by the exponentials of the softmax.  One CTA owns
 // TWO 128-row tiles of the packed (active row x query heads of one kv head) axis and walks over all
@@ -40,19 +41,24 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 128, HD = 128;
+constexpr int BM = 128, BN = 128;
 constexpr int kSoftThreads = 512;          // four softmax warpgroups: (row tile) x (64-column half)
 constexpr int kThreads = 64 + kSoftThreads + 32;   // + one warp that copies fresh K/V into the cache (recompute steps)
 constexpr uint32_t SUB = 128 * 128;        // [128 rows x 64 bf16], 128-byte swizzle: 16 KB
-constexpr uint32_t TILE = 2 * SUB;         // [128 x 128] bf16
 constexpr int kSlots = 5;
-constexpr uint32_t OFF_Q = 0;              // two tiles
-constexpr uint32_t OFF_RING = 2 * TILE;
-constexpr uint32_t OFF_BAR = OFF_RING + kSlots * TILE;   // 224 KB
-constexpr uint32_t OFF_XCH = OFF_BAR + 256;               // [2 tiles][2 halves][128 rows] floats
-constexpr uint32_t SMEM_BYTES = 232448;                   // all of a CTA's 227 KB; the rest is alignment slack
-constexpr uint32_t SMEM_NEEDED = OFF_XCH + 2 * 2 * BM * 4;
-constexpr uint32_t PART = BM * HD * 4;                   // un-normalised rows of a row tile (cut units), over the ring
+// shared memory for heads of HD = 64 or 128 columns
+template <int HD>
+struct Geo {
+    static constexpr uint32_t TILE = HD / 64 * SUB;             // [128 x HD] bf16
+    static constexpr uint32_t OFF_Q = 0;                        // two tiles
+    static constexpr uint32_t OFF_RING = 2 * TILE;
+    static constexpr uint32_t OFF_BAR = OFF_RING + kSlots * TILE;   // 224 KB or 112 KB
+    static constexpr uint32_t OFF_XCH = OFF_BAR + 256;          // [2 tiles][2 halves][128 rows] floats
+    static constexpr uint32_t NEEDED = OFF_XCH + 2 * 2 * BM * 4;
+    static constexpr uint32_t BYTES = HD == 128 ? 232448 : NEEDED + 1024;   // all of a CTA's 227 KB; the rest is alignment slack
+    static constexpr uint32_t PART = BM * HD * 4;               // un-normalised rows of a row tile (cut units), over the ring
+    // (two CTAs never share an SM: they would have 1216 threads of 96 registers)
+};
 constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
@@ -96,11 +102,14 @@ __host__ __device__ constexpr int part_begin(int T, int s, int i) { return i * (
 // waits for this launch has waited for both.  Measured, layers back to back (a third launch that combined partials from
 // global memory -> merged here): 86.4 -> 78.5 us at 2 x 1531 with 28 heads, 237.5 -> 233.1 at 4096 with 28 heads,
 // 58.0 -> 55.7 at 2048 with 19.
-template <bool kCut>
+template <bool kCut, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kd,
                     const __grid_constant__ CUtensorMap map_vd, const DenseParams p) {
+    constexpr uint32_t TILE = Geo<HD>::TILE, OFF_Q = Geo<HD>::OFF_Q, OFF_RING = Geo<HD>::OFF_RING, OFF_BAR = Geo<HD>::OFF_BAR,
+                       OFF_XCH = Geo<HD>::OFF_XCH, PART = Geo<HD>::PART;
+    constexpr int CW = HD / 2, CH = CW / 8;   // output columns of a softmax thread, their 16-byte pieces as bf16
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (s2u(smem_raw) + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - s2u(smem_raw));
@@ -110,7 +119,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     volatile int* again = reinterpret_cast<volatile int*>(gbase + OFF_BAR + B_COUNT * 8 + 8);   // verdict of the first pass
     float* xch = reinterpret_cast<float*>(gbase + OFF_XCH);
     auto bar = [&](int idx) { return bars + idx * 8; };
-    if (base - s2u(smem_raw) + SMEM_NEEDED > SMEM_BYTES) {   // never with the 1024-byte alignment the runtime gives
+    if (base - s2u(smem_raw) + Geo<HD>::NEEDED > Geo<HD>::BYTES) {   // never with the 1024-byte alignment the runtime gives
         if (threadIdx.x == 0 && p.dev_status) atomicExch(p.dev_status, (int)EC_ERR_CUDA);
         return;
     }
@@ -247,7 +256,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll
                             for (int i = 0; i < (q ? 2 : 6); ++i) {
                                 const int k = q ? i * 4 + 3 : (i / 3) * 4 + i % 3;
-                                mma_ts(tmem + TM_O + t * 128, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
+                                mma_ts(tmem + TM_O + t * HD, tmem + TM_S + t * 128 + (k >> 2) * 64 + (k & 3) * 8, desc_v + k * 128,
                                        IDESC_PV, (j > 0 || k > 0));
                             }
                         }
@@ -278,7 +287,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         const int row = quarter * 32 + lane;        // row of the tile == TMEM lane
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const uint32_t tm_s = tmem + lane_addr + TM_S + t * 128;
-        const uint32_t tm_o = tmem + lane_addr + TM_O + t * 128;
+        const uint32_t tm_o = tmem + lane_addr + TM_O + t * HD;
         float* xch_mine = xch + (t * 2 + h) * BM + row;        // exchanged with the partner thread of the row
         const float* xch_other = xch + (t * 2 + (1 - h)) * BM + row;
         const int pair_bar = 1 + t * 4 + quarter;              // named barrier of the two warps that share these rows
@@ -419,17 +428,17 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
                 if (need_rescale) {
                     // O holds tiles < j: P V of tile j - 1 must have completed before the accumulator is scaled;
-                    // each of the two threads of a row scales its 64 columns
+                    // each of the two threads of a row scales its half of the columns
                     mbar_wait(bar(B_PVDONE + t), j & 1, abort_flag, p.dev_status);
                     fence_after();
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
+                    for (int c = 0; c < CW / 32; ++c) {
                         uint32_t o[32];
-                        ld32(tm_o + h * 64 + c * 32, o);
+                        ld32(tm_o + h * CW + c * 32, o);
                         wait_ld<32>(o);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
-                        st32(tm_o + h * 64 + c * 32, o);
+                        st32(tm_o + h * CW + c * 32, o);
                     }
                 }
                 // P (bf16 pairs) over the first half of this thread's own scores
@@ -448,16 +457,20 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             const float l_row = l_run + *xch_other;   // both halves of a row carry the same reference maximum
             if constexpr (!kCut) {
                 // Whole unit: the normalised row goes to shared memory, over the row tile's Q (its last scores are long
-                // formed), and from there, a warp its own 32 rows and 64 columns, to global memory in pieces of 128 bytes.
+                // formed), and from there, a warp its own 32 rows and half of the columns, to global memory in pieces of 128 or 64
+                // bytes.
                 // (us a pass of 32 layers of 768: by TMA, a box for each row tile 510.4, for each warp 507.5; like this, with
                 // no copy to wait for, 503.4.  Straight from the registers, a thread 128 bytes of its row: 3.5 us a unit.)
                 // Rolled: the code of an epilogue runs once a unit and is fetched at about its own length in time.
                 const float inv = 1.f / l_row;
-                unsigned char* qrow = gbase + OFF_Q + t * TILE + h * SUB + (row >> 3) * 1024 + (row & 7) * 128;
+                unsigned char* qtile = gbase + OFF_Q + t * TILE;
+                auto piece = [&](int rw, int g) {   // piece g of the HD / 8 of a row: 128-byte swizzle, so that 32 lanes spread
+                    return reinterpret_cast<uint4*>(qtile + (g >> 3) * SUB + (rw >> 3) * 1024 + (rw & 7) * 128 + (((g & 7) ^ (rw & 7)) << 4));
+                };
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
+                for (int c = 0; c < CW / 32; ++c) {
                     uint32_t o[32];
-                    ld32(tm_o + h * 64 + c * 32, o);
+                    ld32(tm_o + h * CW + c * 32, o);
                     wait_ld<32>(o);
 #pragma unroll
                     for (int v4 = 0; v4 < 4; ++v4) {
@@ -466,21 +479,20 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                         w.y = pack_bf16x2(__uint_as_float(o[v4 * 8 + 2]) * inv, __uint_as_float(o[v4 * 8 + 3]) * inv);
                         w.z = pack_bf16x2(__uint_as_float(o[v4 * 8 + 4]) * inv, __uint_as_float(o[v4 * 8 + 5]) * inv);
                         w.w = pack_bf16x2(__uint_as_float(o[v4 * 8 + 6]) * inv, __uint_as_float(o[v4 * 8 + 7]) * inv);
-                        *reinterpret_cast<uint4*>(qrow + (((c * 4 + v4) ^ (row & 7)) << 4)) = w;
+                        *piece(row, h * CH + c * 4 + v4) = w;
                     }
                 }
                 __syncwarp();
                 if (!*abort_flag) {   // a CTA whose wait gave up stores nothing
-                    const unsigned char* mine = gbase + OFF_Q + t * TILE + h * SUB + quarter * 4096;
-                    const int g = lane >> 3, ch = lane & 7;   // four rows at a time, eight lanes a row
+                    constexpr int RW = 32 / CH;                 // rows at a time, CH lanes a row
+                    const int g = lane / CH, ch = lane % CH;
                     const int r0 = r_pair + t * BM + quarter * 32 + g;
-                    __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + r0) * p.n_q_heads + hk) * HD + h * 64 + ch * 8;
-                    const long long step = 4LL * p.n_q_heads * HD;
+                    __nv_bfloat16* dst = p.out + (((long long)b * p.n_active + r0) * p.n_q_heads + hk) * HD + h * CW + ch * 8;
+                    const long long step = (long long)RW * p.n_q_heads * HD;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int rr = k * 4 + g;
-                        const uint4 w = *reinterpret_cast<const uint4*>(mine + (rr >> 3) * 1024 + (rr & 7) * 128 + ((ch ^ (rr & 7)) << 4));
-                        if (r0 + k * 4 < p.rows_total) *reinterpret_cast<uint4*>(dst + k * step) = w;
+                    for (int k = 0; k < CH; ++k) {
+                        const uint4 w = *piece(quarter * 32 + k * RW + g, h * CH + ch);
+                        if (r0 + k * RW < p.rows_total) *reinterpret_cast<uint4*>(dst + k * step) = w;
                     }
                 }
             } else {
@@ -490,13 +502,13 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 if (p.copy) mbar_wait(bar(B_COPIED), 0, abort_flag, p.dev_status);
                 unsigned char* prow = gbase + OFF_RING + t * PART + row * (HD * 4);
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
+                for (int c = 0; c < CW / 32; ++c) {
                     uint32_t o[32];
-                    ld32(tm_o + h * 64 + c * 32, o);
+                    ld32(tm_o + h * CW + c * 32, o);
                     wait_ld<32>(o);
 #pragma unroll
                     for (int v4 = 0; v4 < 8; ++v4)   // (16-byte pieces swizzled by row: 32 lanes are 32 rows)
-                        *reinterpret_cast<uint4*>(prow + (((h * 16 + c * 8 + v4) ^ (row & 31)) << 4)) =
+                        *reinterpret_cast<uint4*>(prow + (((h * (HD / 8) + c * 8 + v4) ^ (row & (HD / 4 - 1))) << 4)) =
                             make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
                 }
                 if (h == 0) *reinterpret_cast<float2*>(gbase + OFF_Q + (t * BM + row) * 8) = make_float2(m_used, l_row);
@@ -557,7 +569,9 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         __syncthreads();
         if (!*abort_flag) {   // a CTA whose wait gave up stores nothing
-            for (int i0 = warp * 4; i0 < share; i0 += kThreads / 32 * 4) {   // a warp takes four rows, a lane four columns
+            constexpr int LR = HD / 4, RW = 32 / LR;   // lanes of a row, rows side by side in a warp: a lane takes four columns of four rows
+            const int sub = lane / LR, l4 = lane % LR;
+            for (int i0 = warp * 4 * RW + sub; i0 < share; i0 += kThreads / 32 * 4 * RW) {
                 float4 acc[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -566,12 +580,12 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     float x[4][4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int rr = row0 + i0 + k;
-                        ld_peer_v4(map_to_cta(base + OFF_RING + rr * (HD * 4) + ((lane ^ (rr & 31)) << 4), q), x[k]);
+                        const int rr = row0 + i0 + k * RW;
+                        ld_peer_v4(map_to_cta(base + OFF_RING + rr * (HD * 4) + ((l4 ^ (rr & (LR - 1))) << 4), q), x[k]);
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const float w = weight[(i0 + k) * 8 + q];
+                        const float w = weight[(i0 + k * RW) * 8 + q];
                         acc[k].x = fmaf(w, x[k][0], acc[k].x);
                         acc[k].y = fmaf(w, x[k][1], acc[k].y);
                         acc[k].z = fmaf(w, x[k][2], acc[k].z);
@@ -580,9 +594,9 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int r = r_pair + row0 + i0 + k;
-                    if (r < p.rows_total)
-                        *reinterpret_cast<uint2*>(p.out + (((long long)b * p.n_active + r) * p.n_q_heads + hk) * HD + lane * 4) =
+                    const int r = r_pair + row0 + i0 + k * RW;
+                    if (i0 + k * RW < share && r < p.rows_total)
+                        *reinterpret_cast<uint2*>(p.out + (((long long)b * p.n_active + r) * p.n_q_heads + hk) * HD + l4 * 4) =
                             make_uint2(pack_bf16x2(acc[k].x, acc[k].y), pack_bf16x2(acc[k].z, acc[k].w));
                 }
             }
@@ -606,15 +620,15 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 // K or V seen as 5-D {64 columns, key, half, kv head, sequence}: one box {64, 128, 2, 1, 1} lands as
 // [half][key][64 columns], the two 128-byte-swizzled halves of a [128 keys x 128] tile; keys beyond L read as zero.
 // Cache layout [B, Hkv, L, 128] or token-major [B, L, Hkv, 128] (the fresh K/V of a recompute step): only the
-// strides differ.
-bool make_kv_map(CUtensorMap* map, const void* ptr, int batch, int n_kv_heads, int ctx_len, bool token_major) {
+// strides differ.  (64-wide heads: one half.)
+bool make_kv_map(CUtensorMap* map, const void* ptr, int hd, int batch, int n_kv_heads, int ctx_len, bool token_major) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t row = (cuuint64_t)HD * 2;
-    const cuuint64_t dims[5] = {64, (cuuint64_t)ctx_len, 2, (cuuint64_t)n_kv_heads, (cuuint64_t)batch};
+    const cuuint64_t row = (cuuint64_t)hd * 2;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)ctx_len, (cuuint64_t)hd / 64, (cuuint64_t)n_kv_heads, (cuuint64_t)batch};
     const cuuint64_t strides[4] = {token_major ? row * n_kv_heads : row, 128, token_major ? row : row * ctx_len,
                                    row * ctx_len * n_kv_heads};
-    const cuuint32_t box[5] = {64, (cuuint32_t)BN, 2, 1, 1};
+    const cuuint32_t box[5] = {64, (cuuint32_t)BN, (cuuint32_t)hd / 64, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -658,12 +672,29 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
 // one): 32 units of 2 key tiles (32 heads of 256) 24.9 / 9.6, of 8 tiles (8 heads of 1024) 42.5 / 16.7, of 32 tiles (2 heads of
 // 4096) 60.8 / 25.0; 20 units (2 x 300, 5 heads) 23.6 / 9.6; 16 units 24.8 / 11.0, 8 units of 3 tiles 19.6 / 9.0.  The line was
 // at SMs / 4 = 37; it stops short of 16 units, which the tests of the dispatch expect on the one-tile kernel.
-bool attend_dense_supported(const ec_attn_desc& d, int n_active) {
-    if (d.dtype != EC_BF16 || d.head_dim != HD || n_active < 1) return false;
+// 64-wide heads: recompute steps and partial ones of more than 128 rows from 17 units on, others where the estimates below say so.  The mma.sync kernel packs
+// the rows of a kv head's query heads and refreshes in its launch; this one has 128 rows of a query head a tile and a refresh
+// launch in front.  us a layer, mma.sync against this kernel: recompute steps 2 x 1024 with 24 heads on 8 51.5 / 31.4, 4 x
+// 1000 94.1 / 47.5, 1 x 300 with 9 9.4 / 8.1, 1 x 129 with 17 6.9 / 6.6, 1 x 1024 with 6 14.9 / 15.1; index lists 4 x 1000 with 24
+// heads on 8, 96 rows 23.9 / 13.6, 48 rows 16.2 / 13.3, 2 x 1000 with 20 on 4, 200 rows 20.5 / 16.7, 32 x 1000 with 8, 34 rows 37.7 / 27.2, 16 x 2000 with 32, 34 rows 123 /
+// 77.6; left to mma.sync: 64 x 500 with 12 on 4, 40 rows 33.8 / 46.4, 8 x 1000 with 24 on 8, 34 rows 21.7 / 24.4, 4 x 1000 with
+// 12 on 4, 48 rows 8.8 / 12.4, 1 x 1000 with 24, 96 rows 9.3 / 12.8.
+bool prefers_mma(const ec_attn_desc& d, int n_active, bool fresh, long long units) {
+    const int packed = n_active * (d.n_q_heads / d.n_kv_heads), tiles = (packed + 63) / 64;
+    const double rows = (double)tiles * (tiles > 1 && packed <= 48 * tiles ? 48 : 64) * d.batch * d.n_kv_heads;
+    const double mma_us = 5.5 + rows * d.ctx_len / (fresh ? 0.55e6 : 0.8e6);
+    const int T = (d.ctx_len + BN - 1) / BN, sms = sm_count();
+    const double waves = (double)((units + sms - 1) / sms);
+    const double dense_us = waves * (T + 3.3) + (fresh ? 2. : 0.);
+    return mma_us <= dense_us;
+}
+bool attend_dense_supported(const ec_attn_desc& d, int n_active, bool fresh) {
+    if (d.dtype != EC_BF16 || n_active < 1) return false;
     // one unit per (sequence, query head, row-tile pair): grouped-query shapes are run head by head
     const long long pairs = ((long long)n_active + 2 * BM - 1) / (2 * BM);
     const long long bh = (long long)d.batch * d.n_q_heads;
     if (pairs * bh > 0x3fffffffLL) return false;
+    if (d.head_dim == 64 && n_active < d.ctx_len && n_active <= BM && prefers_mma(d, n_active, fresh, pairs * bh)) return false;
     return pairs * bh > sm_count() / 9;
 }
 
@@ -676,21 +707,23 @@ void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_
         lo = n < lo ? n : lo;
         hi = n > hi ? n : hi;
     }
-    snprintf(buf, len, "attend_dense_kernel grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d part_tiles=%d..%d", pl.n_pairs,
+    snprintf(buf, len, "attend_dense_kernel%s grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d part_tiles=%d..%d",
+             d.head_dim == 64 ? "<64>" : "", pl.n_pairs,
              d.batch * d.n_q_heads, pl.n_full, pl.units - pl.n_full, pl.split, lo, hi);
 }
 
-cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
+template <int HD>
+cudaError_t launch_dense(const AttendArgs& a, cudaStream_t stream) {
     CUtensorMap map_k, map_v;
-    if (!make_kv_map(&map_k, a.k_cache, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, a.kv_token_major) ||
-        !make_kv_map(&map_v, a.v_cache, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, a.kv_token_major))
+    if (!make_kv_map(&map_k, a.k_cache, HD, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, a.kv_token_major) ||
+        !make_kv_map(&map_v, a.v_cache, HD, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, a.kv_token_major))
         return cudaErrorInvalidValue;
     DenseParams p;
     p.out = static_cast<__nv_bfloat16*>(a.out);
     p.copy = a.kv_token_major && a.refresh_k_dst && a.refresh_v_dst;
     CUtensorMap map_kd = map_k, map_vd = map_v;   // placeholders unless copying
-    if (p.copy && (!make_kv_map(&map_kd, a.refresh_k_dst, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false) ||
-                   !make_kv_map(&map_vd, a.refresh_v_dst, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false)))
+    if (p.copy && (!make_kv_map(&map_kd, a.refresh_k_dst, HD, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false) ||
+                   !make_kv_map(&map_vd, a.refresh_v_dst, HD, a.d.batch, a.d.n_kv_heads, a.d.ctx_len, false)))
         return cudaErrorInvalidValue;
     p.dev_status = a.dev_status;
     p.n_active = a.n_active;
@@ -709,10 +742,10 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     {
         EncodeTiledFn fn = encode_fn();
         if (!fn) return cudaErrorInvalidValue;
-        const cuuint64_t dims[5] = {64, (cuuint64_t)a.n_active, (cuuint64_t)a.d.n_q_heads, 2, (cuuint64_t)a.d.batch};
+        const cuuint64_t dims[5] = {64, (cuuint64_t)a.n_active, (cuuint64_t)a.d.n_q_heads, HD / 64, (cuuint64_t)a.d.batch};
         const cuuint64_t strides[4] = {(cuuint64_t)a.d.n_q_heads * HD * 2, (cuuint64_t)HD * 2, 128,
                                        (cuuint64_t)a.n_active * a.d.n_q_heads * HD * 2};
-        const cuuint32_t box[5] = {64, (cuuint32_t)BM, 1, 2, 1};
+        const cuuint32_t box[5] = {64, (cuuint32_t)BM, 1, HD / 64, 1};
         const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
         if (fn(&map_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.q), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -722,7 +755,7 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     static PerDeviceOnce once_whole, once_cut;
     cudaLaunchConfig_t cfg{};
     cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.dynamicSmemBytes = Geo<HD>::BYTES;
     cfg.stream = stream;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -733,18 +766,22 @@ cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     if (pl.n_full > 0) {
-        if (const cudaError_t e = ensure_dynamic_smem(once_whole, attend_dense_kernel<false>, (int)SMEM_BYTES); e != cudaSuccess) return e;
+        if (const cudaError_t e = ensure_dynamic_smem(once_whole, attend_dense_kernel<false, HD>, (int)Geo<HD>::BYTES); e != cudaSuccess) return e;
         cfg.gridDim = dim3(pl.n_full, 1, 1);
         cfg.numAttrs = 1;
-        if (const cudaError_t e = cudaLaunchKernelEx(&cfg, attend_dense_kernel<false>, map_k, map_v, map_q, map_kd, map_vd, p);
+        if (const cudaError_t e = cudaLaunchKernelEx(&cfg, attend_dense_kernel<false, HD>, map_k, map_v, map_q, map_kd, map_vd, p);
             e != cudaSuccess)
             return e;
     }
     if (pl.n_full == pl.units) return cudaSuccess;
-    if (const cudaError_t e = ensure_dynamic_smem(once_cut, attend_dense_kernel<true>, (int)SMEM_BYTES); e != cudaSuccess) return e;
+    if (const cudaError_t e = ensure_dynamic_smem(once_cut, attend_dense_kernel<true, HD>, (int)Geo<HD>::BYTES); e != cudaSuccess) return e;
     cfg.gridDim = dim3((pl.units - pl.n_full) * pl.split, 1, 1);
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, attend_dense_kernel<true>, map_k, map_v, map_q, map_kd, map_vd, p);
+    return cudaLaunchKernelEx(&cfg, attend_dense_kernel<true, HD>, map_k, map_v, map_q, map_kd, map_vd, p);
+}
+
+cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream) {
+    return a.d.head_dim == 128 ? launch_dense<128>(a, stream) : launch_dense<64>(a, stream);
 }
 
 }  // namespace ec

@@ -152,8 +152,9 @@ cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const voi
 bool attend_skip_keys_supported(const ec_attn_desc& d, int n_active, bool fresh);   // fresh: k_new / v_new are given
 cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                     cudaStream_t stream);
-// two-row-tile dense path (bf16, head_dim 128): used from SMs / 4 units of (row-tile pair, query head) on
-bool attend_dense_supported(const ec_attn_desc& d, int n_active);
+// two-row-tile dense path (bf16): used from 17 units of (row-tile pair, query head) on, with head_dim 64 on partial steps only
+// where it beats the mma.sync path (fresh: k_new / v_new are given)
+bool attend_dense_supported(const ec_attn_desc& d, int n_active, bool fresh);
 cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream);
 size_t attend_tc_workspace_bytes(const ec_attn_desc& d, int n_active);
 cudaError_t launch_attend_bf16_tc(const AttendArgs& a, cudaStream_t stream);   // tcgen05 path (head_dim 128)

@@ -33,3 +33,35 @@ def test_recompute_steps_with_few_units_and_any_number_of_parts(Hq, Hkv, L, n, c
     rng = np.random.Generator(np.random.PCG64(L + Hq))
     rows = sorted(set(rng.choice(n, min(n, 16), replace=False).tolist() + [0, n - 1]))
     _check(w, t, row_sel=rows)
+
+
+@pytest.mark.parametrize("std_qk", [None, 4.0])
+@pytest.mark.parametrize("B,Hq,Hkv,L,n,cut", [
+    (1, 17, 17, 129, 129, "whole_units=17"),     # one key of a second tile, one row of a second row tile
+    (2, 12, 4, 300, 300, "whole_units=48"),      # grouped query heads, a ragged third tile
+    (1, 7, 7, 1500, 1500, "cut_units=42x3"),
+    (1, 2, 2, 2560, 2560, "cut_units=20x5"),
+    (2, 40, 8, 260, 259, "whole_units=160"),     # an index list, two rounds of units
+    (4, 24, 8, 500, 96, "whole_units=96"),       # a partial step
+])
+def test_heads_of_64_on_the_dense_kernel(B, Hq, Hkv, L, n, cut, std_qk):
+    import paper_2603_18489_b200 as ec
+
+    w = syn.Workload(98, f"d64_h{Hq}_l{L}", syn.BF16, B, Hq, Hkv, 64, L - 64, 64, 32, 2, 1024)
+    full = n == L
+    got = ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 64, syn.BF16), n, True, not full)
+    assert "attend_dense_kernel<64>" in got and cut in got, got
+    idx = None if full else syn.arbitrary_active_idx(B, L, n, seed=7)
+    t = syn.attn_inputs(w, n, active_idx=idx, std_qk=std_qk, salt=6)
+    rng = np.random.Generator(np.random.PCG64(L + Hq))
+    rows = sorted(set(rng.choice(n, min(n, 16), replace=False).tolist() + [0, n - 1]))
+    _check(w, t, row_sel=rows)
+
+
+def test_small_and_packed_steps_of_64_wide_heads_stay_on_mma_sync():
+    import paper_2603_18489_b200 as ec
+
+    for B, L, Hq, Hkv, n, idx in [(1, 449, 8, 8, 449, False), (4, 1000, 12, 4, 48, True), (64, 500, 12, 4, 40, True),
+                                  (8, 1000, 24, 8, 34, True), (1, 1000, 24, 24, 96, True)]:
+        got = ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 64, syn.BF16), n, True, idx)
+        assert got == "refresh_kernel + attend_mma_kernel", (B, L, Hq, Hkv, n, got)
