@@ -63,9 +63,11 @@ constexpr uint32_t TM_COLS = 512;
 constexpr uint32_t TM_S = 0, TM_O = 256;   // + 128 * tile
 
 // B_FREE: ring entries are released in groups, K_0, then {V_0, K_1}, {V_1, K_2}, ... (a second pass goes on: {V of the last
-// tile, K_0}); group c completes phase c / 2 of barrier c % 2.  Entry n belongs to group (n + 1) / 2.
+// tile, K_0}); group c completes phase c / 3 of barrier c % 3, by the products' commit and the copy warp.  Three barriers: the
+// copy warp, which needs no product, walks through the first five entries, groups 0 to 2, at once; its arrival for group
+// c + 3, entry 2 c + 6, waits for group c + 1, and so for the commit of group c.
 // B_PFULL: + 2 * part + tile, see the softmax.
-enum { B_FULL = 0, B_FREE = kSlots, B_SFULL = B_FREE + 2, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 4,
+enum { B_FULL = 0, B_FREE = kSlots, B_SFULL = B_FREE + 3, B_PFULL = B_SFULL + 2, B_PVDONE = B_PFULL + 4,
        B_QFULL = B_PVDONE + 2, B_VERDICT = B_QFULL + 2, B_COPIED = B_VERDICT + 1, B_COUNT = B_COPIED + 1 };
 
 // first pass: a row's sum may grow to this before the unit is done again with running maxima
@@ -145,7 +147,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             prefetch_map(&map_vd);
         }
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 4) ? 256u : (p.copy && i >= B_FREE && i < B_FREE + 2) ? 2u : 1u);
+            mbar_init(bar(i), (i >= B_PFULL && i < B_PFULL + 4) ? 256u : (p.copy && i >= B_FREE && i < B_FREE + 3) ? 2u : 1u);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -172,15 +174,16 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
         };
         load_q(0);   // the first scores need one row tile of Q and the first K tile
-        int slot = 0, key = j0 * BN;
+        int slot = 0, key = j0 * BN, group = 0;   // group: of the entry that had the slot before
+        uint32_t turn = 0;
         for (int n = 0; n < 4 * T; ++n) {   // ring entry: K_j = 2j, V_j = 2j + 1; from 2T on the second pass
             if (n == 2 * T) {
                 mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
                 if (!*again) break;
                 key = j0 * BN;
             }
-            const int c = (n - kSlots + 1) >> 1;   // group of the slot's last entry
-            if (n >= kSlots) mbar_wait(bar(B_FREE + (c & 1)), (c >> 1) & 1, abort_flag, p.dev_status);
+            if (n > kSlots && !(n & 1) && ++group == 3) group = 0, turn ^= 1;   // (five slots: entry n - 5 starts a group where n is even)
+            if (n >= kSlots) mbar_wait(bar(B_FREE + group), turn, abort_flag, p.dev_status);
             if (elected) {
                 mbar_expect_tx(bar(B_FULL + slot), TILE);
                 tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, key, 0, hk_kv, b, bar(B_FULL + slot));
@@ -218,8 +221,8 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             return s;
         };
         auto release = [&]() {
-            if (elected) commit(bar(B_FREE + (group & 1)));
-            ++group;
+            if (elected) commit(bar(B_FREE + group));
+            if (++group == 3) group = 0;
         };
         constexpr int kPeek = HD / 16 - 2;
         for (int pass = 0; pass < 2; ++pass) {
@@ -537,7 +540,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 bulk_commit();
                 bulk_wait_read();   // the slot has been read
             }
-            if (!(n & 1)) mbar_arrive(bar(B_FREE + ((n >> 1) & 1)));   // K tiles end a group
+            if (!(n & 1)) mbar_arrive(bar(B_FREE + (n >> 1) % 3));   // K tiles end a group
             if (++slot == kSlots) slot = 0, phase ^= 1;
         }
         mbar_arrive(bar(B_COPIED));
