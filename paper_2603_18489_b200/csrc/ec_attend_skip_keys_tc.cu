@@ -219,7 +219,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     if (tid == 0) {
         for (int i = 0; i < B_COUNT; ++i) {
             uint32_t count = 1;
-            if (i == B_PFULL || i == B_QFULL) count = kSoft;
+            if (i == B_PFULL || i == B_QFULL) count = kSoft / 32;
             if (i == B_LIST) count = kAuxThreads;
             mbar_init(bar(i), count);
         }
@@ -457,7 +457,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 *reinterpret_cast<uint4*>(gbase + off) = v[u];
             }
             fence_async_smem();     // Q (generic proxy) -> visible to the tensor core (async proxy)
-            mbar_arrive(bar(B_QFULL));
+            mbar_arrive_warp(bar(B_QFULL));
         }
 
         const int quarter = warp & 3;
@@ -591,7 +591,7 @@ attend_skip_keys_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             }
             fence_async_smem();
             fence_before();
-            mbar_arrive(bar(B_PFULL));
+            mbar_arrive_warp(bar(B_PFULL));
 #pragma unroll
             for (int i = 0; i < NH / 2; ++i)   // (while the second product runs)
                 lsum[i] = add2(lsum[i], pk(__uint_as_float(pw[i] << 16), __uint_as_float(pw[i] & 0xffff0000u)));

@@ -134,6 +134,14 @@ __device__ __forceinline__ bool elect_one() {
 }
 // a barrier as the whole warp sees it: one answer, so what depends on it stays warp-uniform
 __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)); }
+// One arrival for the whole warp, behind what all its lanes have done before (each has fenced what the barrier is to publish).
+// Arrivals of 32 lanes at one barrier are taken one after the other: attend_skip_keys_kernel, whose softmax warps are alone on
+// the chain of a tile, is 0.15 to 0.25 us a launch shorter with one (us a pass: llada 768 246.4 -> 241.5, dream 768 204.6 ->
+// 198.8, 1983 with k = 64 447 -> 439.5, 4096 500.6 -> 494.8); the dense kernel (506 / 506) and the pair body (379 / 379) hide them.
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
 // threadIdx.x / 32 as a value that the compiler knows to be warp-uniform
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 // D[tmem] (+)= A[smem] * B[smem]
