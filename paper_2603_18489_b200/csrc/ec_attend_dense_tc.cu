@@ -11,7 +11,7 @@
 //               two Q tiles of the unit, one box each.  (Grouped-query shapes are launched with one unit per
 //               QUERY head, so a row tile is always 128 active rows of one head; the query heads of a kv head
 //               stream the same K/V, which L2 serves.)
-//   warp 1      tcgen05.mma issuer (one thread): S_t = Q_t K^T (both operands K-major in shared memory) into
+//   warp 1      tcgen05.mma issuer (the whole warp, one lane elected): S_t = Q_t K^T (both operands K-major in shared memory) into
 //               the TMEM columns of row tile t, and O_t += P_t V with P_t read from TENSOR MEMORY (it
 //               overwrites the first 64 columns of S_t as packed bf16) and V MN-major from shared memory.
 //               Order per key tile j:  P V_0(j), S_0(j+1), P V_1(j), S_1(j+1): the pipe executes in order,
