@@ -56,19 +56,19 @@ K64_WORKLOADS = ("c4_llada_l2048", "c5_llada_l4096", "c5_llada_l4096_b8", "c5_dr
 NCU_TRAFFIC = {
     "attend_skip": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",),
-         "sha256": "c474a357d342a69efc637af48faa81c785a7ef0647254f9ebb669f52b3b46119",
-         "bytes_per_launch": {"c5_llada_l4096": 68300000}},
+         "sha256": "c8f3be6703ae4e5eda5268ba7accce752972fede0dde7fbb54dbd349b9a77406",
+         "bytes_per_launch": {"c5_llada_l4096": 68770000}},
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu", "paper_2603_18489_b200/csrc/ec_skip_keys_pair.cuh"),
-         "sha256": "f8a1bbeeec1c27874598b6b6d350adaddad2499b98703d06da43b7bafe7f143d",
-         "bytes_per_launch": {"c5_llada_l4096_b8": 556680000}}],
+         "sha256": "ba6748597d440eb2e9986a220077697c6a28e35f238d4fe82a32fc36a356233e",
+         "bytes_per_launch": {"c5_llada_l4096_b8": 557030000}}],
     "attend_dense": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",),
-         "sha256": "267ab6f92d2b70bdd83b3c2b3ac6dffd1eef4b0b90ad4057f60ad4d265abb263",
-         "bytes_per_launch": {"c5_llada_l4096": 151530000}}],
+         "sha256": "f0ec912f389b20564c6f873dd21a1fa3844a972a0c04c76c89b1b96af0ab27cd",
+         "bytes_per_launch": {"c5_llada_l4096": 148540000}}],
     "entropy_gate": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_gate.cu",),
-         "sha256": "18611e4521d092e171a3838cfc98ea318657814618c56e10b7bf546a9215100f",
-         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65320000}}],
+         "sha256": "660af8feb5cbc456545018c79a08fa0ef91987e62268a69798aa2e8e4a489fe5",
+         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65400000}}],
 }
 
 
