@@ -178,12 +178,12 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         uint32_t turn = 0;
         for (int n = 0; n < 4 * T; ++n) {   // ring entry: K_j = 2j, V_j = 2j + 1; from 2T on the second pass
             if (n == 2 * T) {
-                mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                mbar_wait_warp(bar(B_VERDICT), 0, abort_flag, p.dev_status);
                 if (!*again) break;
                 key = j0 * BN;
             }
             if (n > kSlots && !(n & 1) && ++group == 3) group = 0, turn ^= 1;   // (five slots: entry n - 5 starts a group where n is even)
-            if (n >= kSlots) mbar_wait(bar(B_FREE + group), turn, abort_flag, p.dev_status);
+            if (n >= kSlots) mbar_wait_warp(bar(B_FREE + group), turn, abort_flag, p.dev_status);
             if (elected) {
                 mbar_expect_tx(bar(B_FULL + slot), TILE);
                 tma_load_5d(base + OFF_RING + slot * TILE, (n & 1) ? &map_v : &map_k, 0, key, 0, hk_kv, b, bar(B_FULL + slot));
@@ -215,7 +215,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             return mbar_test(bar(B_FULL + slot + ahead - (wrapped ? kSlots : 0)), phase ^ (wrapped ? 1u : 0u));
         };
         auto take = [&](bool landed) {
-            if (!landed) mbar_wait(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
+            if (!landed) mbar_wait_warp(bar(B_FULL + slot), phase, abort_flag, p.dev_status);
             const int s = slot;
             if (++slot == kSlots) slot = 0, phase ^= 1;
             return s;
@@ -227,13 +227,13 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         constexpr int kPeek = HD / 16 - 2;
         for (int pass = 0; pass < 2; ++pass) {
             if (pass == 1) {
-                mbar_wait(bar(B_VERDICT), 0, abort_flag, p.dev_status);
+                mbar_wait_warp(bar(B_VERDICT), 0, abort_flag, p.dev_status);
                 if (!*again) break;
             }
             {
                 const uint64_t desc_k = smem_desc(base + OFF_RING + take(false) * TILE, 16, 1024);
                 for (int t = 0; t < n_tiles_q; ++t) {
-                    mbar_wait(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
+                    mbar_wait_warp(bar(B_QFULL + t), 0, abort_flag, p.dev_status);
                     fence_after();
                     products_s(t, desc_k, 0, HD / 16);
                     if (elected) commit(bar(B_SFULL + t));
@@ -251,7 +251,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                 for (int t = 0; t < n_tiles_q; ++t) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
-                        if (q == 1 || !p_ready) mbar_wait(bar(B_PFULL + q * 2 + t), p_phase, abort_flag, p.dev_status);
+                        if (q == 1 || !p_ready) mbar_wait_warp(bar(B_PFULL + q * 2 + t), p_phase, abort_flag, p.dev_status);
                         fence_after();
                         // P of keys 0..63 lies over S columns 0..31, of keys 64..127 over S columns 64..95; part 0 are the first
                         // 48 keys of each half, part 1 the others

@@ -132,6 +132,13 @@ __device__ __forceinline__ bool elect_one() {
         : "=r"(p));
     return p != 0;
 }
+// A wait in a role that a whole warp plays (see elect_one).  Every lane polls for itself; a lane that came out later than the
+// elected one could, after two more phases of the barrier, look for a parity that has come round again, and only give up at the
+// limit.  So the lanes leave a wait together.
+__device__ __forceinline__ void mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* dev_status) {
+    mbar_wait(bar, parity, abort_flag, dev_status);
+    __syncwarp();
+}
 // a barrier as the whole warp sees it: one answer, so what depends on it stays warp-uniform
 __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)); }
 // One arrival for the whole warp, behind what all its lanes have done before (each has fenced what the barrier is to publish).
