@@ -134,7 +134,8 @@ ec_status ec_attend(const ec_attn_desc *desc, const void *q, const void *k_new, 
  * "refresh_kernel + attend_f32_kernel" (64-wide heads in bf16, fp32) are ONE launch that refreshes and attends, unless
  * a CTA's share of the keys exceeds 8192; with the other kernels "refresh_kernel + " is a launch of its own.
  * "attend_dense_kernel ... whole_units=w cut_units=cxs part_tiles=a..b" is one launch of w CTAs and, when c > 0, a
- * second one of c clusters of s CTAs, each with a to b of the key tiles ("grid" counts uncut units).
+ * second one of c clusters of s CTAs, each with a to b of the key tiles ("grid" counts uncut units); " at_once=n" behind it is
+ * how many such clusters the device keeps resident.
  * with_fresh_kv: k_new/v_new would be given; with_index_list: active_idx would be non-NULL.  Touches no device memory and launches nothing.  Returns "" on arguments ec_attend would reject.  The
  * string lives in a thread-local buffer that the next call on the same thread overwrites. */
 const char *ec_attend_kernel_name(const ec_attn_desc *desc, int32_t n_active, int32_t with_fresh_kv,

@@ -34,6 +34,7 @@
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"
 
+#include <atomic>
 #include <cstdio>
 
 namespace ec {
@@ -649,6 +650,39 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int hd, int batch, int n_kv_
 struct DensePlan {
     int n_pairs, units, n_full, split;
 };
+// How many clusters of s CTAs of the cut launch the current device keeps resident at once.  A cluster stays inside a GPC, and
+// these need neither be alike nor hold a multiple of s SMs: 148 SMs taken as eight GPCs of 18 gave 48 clusters of three, of which
+// 45 ran and the others made a second round (8 heads of 1500, 48 units: 34.2 us a layer in three parts, 21.8 in two).
+// Asked once per device; without a device to ask, that assumption.
+template <int HD>
+int resident_clusters(int s) {
+    static std::atomic<int> cached[kMaxDevices][9] = {};   // + 1
+    static PerDeviceOnce attr_once;
+    int dev = 0, n = 0;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess;
+    const bool slot = known && dev >= 0 && dev < kMaxDevices;
+    if (slot)
+        if (const int v = cached[dev][s].load(std::memory_order_relaxed)) return v - 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(s, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = Geo<HD>::BYTES;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = s;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (!known || ensure_dynamic_smem(attr_once, attend_dense_kernel<true, HD>, (int)Geo<HD>::BYTES) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, attend_dense_kernel<true, HD>, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 8 * (sm_count() / 8 / s);
+    }
+    if (slot) cached[dev][s].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
 DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
     DensePlan pl;
     pl.n_pairs = (n_active + 2 * BM - 1) / (2 * BM);
@@ -658,8 +692,8 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
     const int sms = sm_count();
     const int T = (d.ctx_len + BN - 1) / BN, tail = pl.units % sms;
     for (int s = 8; s >= 2 && tail > 0; --s) {
-        const int at_once = 8 * (sms / 8 / s);   // clusters of s, inside the eight GPCs
-        if (T / s < 4 || T - (T + s - 1) / s < 4 || tail > at_once) continue;
+        if (T / s < 4 || T - (T + s - 1) / s < 4) continue;
+        if (tail > (d.head_dim == 128 ? resident_clusters<128>(s) : resident_clusters<64>(s))) continue;
         pl.split = s;
         pl.n_full = pl.units - tail;
         break;
@@ -710,9 +744,11 @@ void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_
         lo = n < lo ? n : lo;
         hi = n > hi ? n : hi;
     }
-    snprintf(buf, len, "attend_dense_kernel%s grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d part_tiles=%d..%d",
-             d.head_dim == 64 ? "<64>" : "", pl.n_pairs,
-             d.batch * d.n_q_heads, pl.n_full, pl.units - pl.n_full, pl.split, lo, hi);
+    const int n = snprintf(buf, len, "attend_dense_kernel%s grid=(%d,%d) cluster=1 whole_units=%d cut_units=%dx%d part_tiles=%d..%d",
+                           d.head_dim == 64 ? "<64>" : "", pl.n_pairs, d.batch * d.n_q_heads, pl.n_full, pl.units - pl.n_full,
+                           pl.split, lo, hi);
+    if (pl.split > 1 && n > 0 && (size_t)n < len)
+        snprintf(buf + n, len - n, " at_once=%d", d.head_dim == 128 ? resident_clusters<128>(pl.split) : resident_clusters<64>(pl.split));
 }
 
 template <int HD>

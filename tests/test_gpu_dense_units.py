@@ -108,3 +108,23 @@ def test_passes_without_synchronisation_repeat_their_outputs(B, Hq, Hkv, L, D, l
         torch.cuda.synchronize()
         for s, f in zip(st, first):
             assert torch.equal(s[-1], f)
+
+
+def test_cut_units_run_at_once():
+    """The clusters of a cut last wave are no more than the device keeps resident, or the last of them make a second round: 48
+    units of 12 to 16 tiles, which three parts each would fit by the number of SMs alone, and every count of units around."""
+    import re
+
+    import paper_2603_18489_b200 as ec
+
+    seen = set()
+    for D, n in ((128, 300), (64, 200)):
+        for L in range(1024, 4097, 256):
+            for units in range(17, 148):
+                heads = units // 2 if D == 128 else units
+                got = ec.ec_attend_kernel_name(ec.make_desc(1, L, heads, heads, D, syn.BF16), n, True, True)
+                m = re.search(r"cut_units=(\d+)x(\d+) part_tiles=\d+\.\.\d+( at_once=(\d+))?$", got)
+                if m and int(m[1]):
+                    assert m[3] and int(m[1]) <= int(m[4]), got
+                    seen.add(int(m[2]))
+    assert seen >= {2, 3, 4, 5, 6}
