@@ -41,6 +41,8 @@
 
 #include <float.h>
 
+#include <algorithm>
+
 namespace ec {
 namespace {
 
@@ -52,6 +54,7 @@ constexpr int kMaxSplits = 96;
 constexpr float kDClamp = -150.0f;  // 2^-150 flushes to 0 (ftz)
 constexpr int kInFlight = 4;         // 16-byte vectors a thread keeps in flight
 constexpr int kSingleLevelMaxRows = 64;
+constexpr int kFinishSplits = 32;    // chunks of a row that the last CTA of a sequence finishes: eight threads a row, four each
 constexpr float kRebase = 64.f;     // the base moves when a value exceeds it by more than 2^kRebase
 constexpr unsigned int kXMinBf16x2 = 0xFE96FE96u;   // two bf16 of about -1e38: lower clamp of the logits
 constexpr unsigned int kXMinF32 = 0xFE960000u;      // the same value as fp32 bits
@@ -610,26 +613,40 @@ GateWs carve(int n_rows) {
 }
 
 // How the rows are cut: one resident wave of 4 CTAs of 256 threads per SM, all its places taken.  Rows get `splits` chunks
-// or one more, so that the CTAs are as many as the places: with equal splits, 512 CTAs of 256 rows on 592 places, 68 SMs had
-// four CTAs, 80 three, and the former worked 3.4 us longer (bf16 [256, 126464] 20.5 -> 18.4 us with new logits each pass, 160
-// rows 13.2 -> 11.9, 32 rows 6.25 -> 6.04; fp32 [32, 126464] 6.86 -> 6.38).  fp32 waits for memory rather than for its
-// arithmetic, and from about 100 rows on large equal chunks are the better ones (128 rows 13.75 against 13.99).  Equal chunks,
-// where the rule or the limit of splits asks for them, are whole 2048-column slabs.
+// or one more, so that the CTAs are as many as the places: with equal splits, 400 CTAs of 200 rows on 592 places, 104 SMs had
+// three CTAs, 44 two.  (Chunks are whole pieces of 256 columns, so where they are short the last ones of a row may be empty: 8
+// rows of 153700 have 56 of 592 CTAs without work.)  us a call, equal -> as here, on logits that no call before has read, bf16
+// [32, 126464] 6.91 -> 6.66, 128 rows 11.26 -> 10.29, 200 17.45 -> 14.38, 256 16.88 -> 16.80, 300 27.4 -> 19.3, fp32 32 rows
+// 7.56 -> 7.36.  Equal chunks, whole 2048-column slabs, are the better ones where
+//   - a row would have more than the 32 chunks that one CTA finishes, and no more of equal ones: 16 rows of 126464 as 37 or 38
+//     chunks 6.53, as 31 5.29 (10 rows of 152064, 59 or 60 and 38 chunks: fp32 6.92 against 7.28 of equal ones);
+//   - they are no longer than the longest chunk here (rounding them to slabs costs less than 5 %), and rows with one chunk more
+//     are too few to spare every SM one of the long ones: 148 rows of 32000 2 % longer here, 592 of 4104 3 %; with whole rows as
+//     the long chunks the line lies at two fifths, or one half below 48 K columns: 400 rows (192 cut) of 126464 28.5 -> 24.2, of
+//     32000 11.8 -> 12.2, 425 and 450 rows (167, 142 cut) 0 to 3 % longer;
+//   - fp32, which waits for memory rather than for its arithmetic, has large chunks: above 8192 columns [56, 126464], [64,
+//     151936] and [80, 100352] took 1.6 to 2.2 % longer here, below [32, 50304] 8, [32, 126464] 5, [56, 64000] 5 % less.
 void plan_chunks(GateParams& p, int max_splits, bool bf16) {
     const int slab = kGateThreads * kVec;
     const long long slots = (long long)kCtasPerSm * sm_count();
     long long want = slots / p.n_rows;
     p.n_few = p.n_rows;
-    if (want >= (bf16 ? 1 : 6) && want + 1 <= max_splits && p.vocab / (want + 1) >= slab) {
-        p.splits = (int)want;
-        p.pitch = p.splits + 1;
-        p.n_few = p.n_rows - (int)(slots - want * p.n_rows);
-        for (int k = 0; k < 2; ++k) {
-            const int n = p.splits + k;
-            p.inverse[k] = (unsigned int)((0x100000000LL + n - 1) / n);
-            p.chunk[k] = ((p.vocab + n - 1) / n + kPiece - 1) / kPiece * kPiece;
+    if (want >= (bf16 ? 1 : 6) && want + 1 <= max_splits && p.vocab / (want + 1) >= slab && (bf16 || p.vocab / want <= 8192)) {
+        const int longest = (int)((p.vocab + want - 1) / want), more = (int)(slots - want * p.n_rows);
+        const int even = std::min((longest + slab - 1) / slab * slab, p.vocab);
+        const bool finish = want + 1 <= kFinishSplits || (p.vocab + even - 1) / even > kFinishSplits;
+        const bool spares = want > 1 ? 8LL * more >= p.n_rows : (p.vocab < 49152 ? 4LL : 5LL) * more >= 2LL * p.n_rows;
+        if (finish && (spares || longest * 20LL <= even * 19LL)) {
+            p.splits = (int)want;
+            p.pitch = p.splits + 1;
+            p.n_few = p.n_rows - more;
+            for (int k = 0; k < 2; ++k) {
+                const int n = p.splits + k;
+                p.inverse[k] = (unsigned int)((0x100000000LL + n - 1) / n);
+                p.chunk[k] = ((p.vocab + n - 1) / n + kPiece - 1) / kPiece * kPiece;
+            }
+            return;
         }
-        return;
     }
     if (want < 1) want = 1;
     if (want > max_splits) want = max_splits;
@@ -691,8 +708,8 @@ cudaError_t launch_gate(const GateArgs& a, cudaStream_t stream) {
     // decode mode and the extra metrics need all rows of a sequence in one CTA's hands at the end: the single-level
     // finish (at most 32 splits)
     const bool one_cta_finish = a.masked || a.entropy_sum_out || a.max_conf_out;
-    plan_chunks(p, one_cta_finish ? 32 : kMaxSplits, a.dtype == EC_BF16);
-    p.single_level = (a.rows_per_seq <= kSingleLevelMaxRows && p.pitch <= 32) ? 1 : 0;
+    plan_chunks(p, one_cta_finish ? kFinishSplits : kMaxSplits, a.dtype == EC_BF16);
+    p.single_level = (a.rows_per_seq <= kSingleLevelMaxRows && p.pitch <= kFinishSplits) ? 1 : 0;
     if (one_cta_finish && !p.single_level) return cudaErrorInvalidValue;   // rows_per_seq > 64 or vocab > 32 * 8192 * ...: rejected by the API layer
     if (p.pitch > p.splits) return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16, true>(p, stream) : launch_t<float, true>(p, stream);
     return a.dtype == EC_BF16 ? launch_t<__nv_bfloat16, false>(p, stream) : launch_t<float, false>(p, stream);
