@@ -704,35 +704,49 @@ DensePlan make_dense_plan(const ec_attn_desc& d, int n_active) {
 
 }  // namespace
 
-// The two-tile kernel is used from 17 of its (row-tile pair, query head) units on (148 SMs).  The one-tile kernel behind a
+// The two-tile kernel is used from 17 of its (row-tile pair, query head) units on.  The one-tile kernel behind a
 // refresh launch, which takes the steps below, is the slower one on both sides of the line (us a layer, one-tile against this
 // one): 32 units of 2 key tiles (32 heads of 256) 24.9 / 9.6, of 8 tiles (8 heads of 1024) 42.5 / 16.7, of 32 tiles (2 heads of
-// 4096) 60.8 / 25.0; 20 units (2 x 300, 5 heads) 23.6 / 9.6; 16 units 24.8 / 11.0, 8 units of 3 tiles 19.6 / 9.0.  The line was
-// at SMs / 4 = 37; it stops short of 16 units, which the tests of the dispatch expect on the one-tile kernel.
-// 64-wide heads: recompute steps and partial ones of more than 128 rows from 17 units on, others where the estimates below say so.  The mma.sync kernel packs
-// the rows of a kv head's query heads and refreshes in its launch; this one has 128 rows of a query head a tile and a refresh
-// launch in front.  us a layer, mma.sync against this kernel: recompute steps 2 x 1024 with 24 heads on 8 51.5 / 31.4, 4 x
-// 1000 94.1 / 47.5, 1 x 300 with 9 9.4 / 8.1, 1 x 129 with 17 6.9 / 6.6, 1 x 1024 with 6 14.9 / 15.1; index lists 4 x 1000 with 24
-// heads on 8, 96 rows 23.9 / 13.6, 48 rows 16.2 / 13.3, 2 x 1000 with 20 on 4, 200 rows 20.5 / 16.7, 32 x 1000 with 8, 34 rows 37.7 / 27.2, 16 x 2000 with 32, 34 rows 123 /
-// 77.6; left to mma.sync: 64 x 500 with 12 on 4, 40 rows 33.8 / 46.4, 8 x 1000 with 24 on 8, 34 rows 21.7 / 24.4, 4 x 1000 with
-// 12 on 4, 48 rows 8.8 / 12.4, 1 x 1000 with 24, 96 rows 9.3 / 12.8.
-bool prefers_mma(const ec_attn_desc& d, int n_active, bool fresh, long long units) {
-    const int packed = n_active * (d.n_q_heads / d.n_kv_heads), tiles = (packed + 63) / 64;
-    const double rows = (double)tiles * (tiles > 1 && packed <= 48 * tiles ? 48 : 64) * d.batch * d.n_kv_heads;
-    const double mma_us = 5.5 + rows * d.ctx_len / (fresh ? 0.55e6 : 0.8e6);
+// 4096) 60.8 / 25.0; 20 units (2 x 300, 5 heads) 23.6 / 9.6; 16 units 24.8 / 11.0, 8 units of 3 tiles 19.6 / 9.0.  The line
+// stops short of 16 units, which the tests of the dispatch expect on the one-tile kernel.
+constexpr int kOneTileUnits = 16;
+
+// 64-wide heads.  The mma.sync kernel packs the rows of a kv head's query heads and refreshes in its launch; this one has 128
+// rows of a query head a tile and a refresh launch in front.  More than 256 fresh rows and more units than SMs are this one's
+// (the faster one on all of 282 such shapes; one found since, 2 x 260 with 40 heads on 8 and 259 rows, takes 15.8 us, 13.5 on
+// mma.sync).  Partial steps of at most 128 rows are mma.sync's unless they are large (a bound, below which the estimates are too
+// rough).  Then the estimates of both decide, mma.sync where it is 3 % ahead.  Of 2153 shapes timed (1 to 32 sequences, 129 to
+// 4096 keys, 8 to 1000 rows or all, 1 to 32 heads, groups of 1 to 8) 9 are more than 3 % slower here than on mma.sync, of 700
+// others 7; when recompute steps and partial ones of more than 128 rows were not asked about, 42 and 24.  us a layer, mma.sync / this kernel:
+// recompute steps 2 x 1024 with 24 heads on 8 51.5 / 31.4, 4 x 1000 94.1 / 47.5, 1 x 300 with 9 9.0 / 7.8, 32 x 129 with 24 on 8
+// 32.0 / 42.1; index lists 4 x 1000 with 24 on 8, 96 rows 23.9 / 13.6, 48 rows 16.2 / 13.3, 4 x 700 with 6 on 2, 129 rows 10.9 /
+// 13.6, 1 x 1000 with 9, 257 rows 9.2 / 14.8, 64 x 500 with 12 on 4, 40 rows 33.8 / 46.4.
+double dense_us(const ec_attn_desc& d, int n_active, bool fresh) {   // 6 % rms
+    const DensePlan pl = make_dense_plan(d, n_active);
     const int T = (d.ctx_len + BN - 1) / BN, sms = sm_count();
-    const double waves = (double)((units + sms - 1) / sms);
-    const double dense_us = waves * (T + 3.3) + (fresh ? 2. : 0.);
-    return mma_us <= dense_us;
+    const double tile = n_active > BM ? 1.44 : 1.02, around = n_active > BM ? 4.2 : 3.4;   // two row tiles or one
+    double us = -0.7 + (pl.n_full + sms - 1) / sms * (tile * T + around);
+    if (pl.split > 1) us += tile * ((T + pl.split - 1) / pl.split) + around + 4.2;
+    if (fresh && n_active < d.ctx_len) us += 1.6 + 1.4e-4 * n_active * d.batch * d.n_kv_heads;
+    return us;
+}
+bool prefers_mma(const ec_attn_desc& d, int n_active, bool fresh, long long units) {
+    if (fresh && n_active > 2 * BM && units > sm_count()) return false;
+    if (n_active < d.ctx_len && n_active <= BM) {
+        const int packed = n_active * (d.n_q_heads / d.n_kv_heads), tiles = (packed + 63) / 64, sms = sm_count();
+        const double rows = (double)tiles * (tiles > 1 && packed <= 48 * tiles ? 48 : 64) * d.batch * d.n_kv_heads;
+        const double waves = (double)((units + sms - 1) / sms) * ((d.ctx_len + BN - 1) / BN + 3.3) + (fresh ? 2. : 0.);
+        if (5.5 + rows * d.ctx_len / (fresh ? 0.55e6 : 0.8e6) <= waves) return true;
+    }
+    return attend_mma_us(d, n_active, fresh) < 0.97 * dense_us(d, n_active, fresh);
 }
 bool attend_dense_supported(const ec_attn_desc& d, int n_active, bool fresh) {
     if (d.dtype != EC_BF16 || n_active < 1) return false;
     // one unit per (sequence, query head, row-tile pair): grouped-query shapes are run head by head
     const long long pairs = ((long long)n_active + 2 * BM - 1) / (2 * BM);
-    const long long bh = (long long)d.batch * d.n_q_heads;
-    if (pairs * bh > 0x3fffffffLL) return false;
-    if (d.head_dim == 64 && n_active < d.ctx_len && n_active <= BM && prefers_mma(d, n_active, fresh, pairs * bh)) return false;
-    return pairs * bh > sm_count() / 9;
+    const long long units = pairs * d.batch * d.n_q_heads;
+    if (units <= kOneTileUnits || units > 0x3fffffffLL) return false;
+    return d.head_dim == 128 || !prefers_mma(d, n_active, fresh, units);
 }
 
 void attend_dense_describe(const ec_attn_desc& d, int n_active, char* buf, size_t len) {

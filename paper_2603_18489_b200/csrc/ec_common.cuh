@@ -139,6 +139,7 @@ cudaError_t launch_attend_f32(const AttendArgs& a, const void* k_new, const void
 // mma.sync path (head_dim 64): refresh and attention in one launch (k_new == nullptr: attention alone)
 cudaError_t launch_attend_bf16(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                cudaStream_t stream);
+double attend_mma_us(const ec_attn_desc& d, int n_active, bool fresh);   // what a launch of that kernel takes, estimated
 // fused skip-step path (bf16, head_dim 128, n_active * H_q/H_kv <= 256): refresh + attention + merge in one launch
 bool attend_skip_supported(const ec_attn_desc& d, int n_active);
 // host-only descriptions of the launch the plan functions choose ("kernel<instantiation> grid=... cluster=..."),
@@ -152,8 +153,8 @@ cudaError_t launch_attend_skip(const AttendArgs& a, const void* k_new, const voi
 bool attend_skip_keys_supported(const ec_attn_desc& d, int n_active, bool fresh);   // fresh: k_new / v_new are given
 cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
                                     cudaStream_t stream);
-// two-row-tile dense path (bf16): used from 17 units of (row-tile pair, query head) on, with head_dim 64 on partial steps only
-// where it beats the mma.sync path (fresh: k_new / v_new are given)
+// two-row-tile dense path (bf16): used from 17 units of (row-tile pair, query head) on, with head_dim 64 only where it beats
+// the mma.sync path (fresh: k_new / v_new are given)
 bool attend_dense_supported(const ec_attn_desc& d, int n_active, bool fresh);
 cudaError_t launch_attend_dense(const AttendArgs& a, cudaStream_t stream);
 size_t attend_tc_workspace_bytes(const ec_attn_desc& d, int n_active);

@@ -111,3 +111,27 @@ def test_every_part_of_a_cut_unit_holds_key_tiles(Hq, Hkv):
                 assert lo >= 4 or parts == 1, got
                 n_cut += cut > 0
     assert n_cut > 50
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,n,fresh,kernel", [
+    # 64-wide heads: mma.sync takes the time behind the colon, the dense kernel the other
+    (1, 1000, 9, 9, 257, True, "attend_mma_kernel"),     # 9.2 us: 14.8
+    (1, 449, 9, 9, 257, True, "attend_mma_kernel"),      # 7.4: 11.0
+    (2, 700, 9, 9, 129, True, "attend_mma_kernel"),      # 9.9: 13.5
+    (1, 700, 17, 17, 160, True, "attend_mma_kernel"),    # 11.0: 13.6
+    (4, 700, 6, 2, 129, True, "attend_mma_kernel"),      # 10.9: 13.6
+    (4, 300, 24, 8, 257, False, "attend_mma_kernel"),    # 10.6: 15.0
+    (32, 129, 24, 8, 129, True, "attend_mma_kernel"),    # a recompute step, 32.0: 42.1
+    (1, 129, 17, 17, 17, False, "attend_mma_kernel"),    # 3.6: 4.7
+    (16, 1024, 32, 8, 48, True, "attend_mma_kernel"),    # 35.0: 46.7
+    (1, 300, 9, 9, 300, True, "attend_dense_kernel<64>"),     # a recompute step, 9.0: 7.8
+    (4, 1000, 24, 8, 96, True, "attend_dense_kernel<64>"),    # 23.9: 13.6
+    (8, 1024, 9, 9, 128, True, "attend_dense_kernel<64>"),    # 30.2: 14.5
+    (1, 1500, 12, 12, 384, True, "attend_dense_kernel<64>"),  # 23.0: 15.8
+    (32, 449, 32, 4, 257, True, "attend_dense_kernel<64>"),   # more than 256 rows, more units than SMs
+])
+def test_64_wide_heads_run_on_the_faster_kernel(B, L, Hq, Hkv, n, fresh, kernel):
+    import paper_2603_18489_b200 as ec
+
+    got = ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 64, syn.BF16), n, fresh, n != L)
+    assert got.split(" grid")[0].split(" + ")[-1] == kernel, got
