@@ -80,6 +80,9 @@ template <int N>
 __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_kn,
                                     const CUtensorMap& map_vn, const Params& p, unsigned char* gbase) {
     constexpr int NH = N / 2;
+    // Who issues: the whole warp (see elect_one) with 48 slots, which is up to 3 % ahead from 768 keys on and with few rows, one
+    // thread with 64, where the whole warp is the slower one (us a layer, 5 x 32 heads of 200 17.23 -> 17.60, of 768 26.4 -> 26.9).
+    constexpr bool kWarpIssues = N == 48;
     constexpr uint32_t OFF_P = off_p(N), OFF_K = off_k(N), OFF_V = off_v(N), OFF_BITS = off_bits(N);
     const uint32_t base = s2u(gbase);
     uint32_t* bits = reinterpret_cast<uint32_t*>(gbase + OFF_BITS);
@@ -88,7 +91,7 @@ __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap&
     const uint32_t bars = s2u(sh->bars);
     auto bar = [&](int i) { return bars + 8u * i; };
 
-    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const int tid = threadIdx.x, warp = kWarpIssues ? warp_index() : tid >> 5, lane = tid & 31;
     const int bh = blockIdx.y, b = bh / p.n_kv_heads, hk = bh % p.n_kv_heads;
     const int rows_total = p.n_active * p.group;
     const bool refresh = p.k_new != nullptr;
@@ -146,45 +149,52 @@ __device__ __forceinline__ void run(const CUtensorMap& map_k, const CUtensorMap&
                 else if (!guard.tick(abort_flag, p.dev_status)) break;
             }
         }
-    } else if (warp == 1) {   // (the whole warp, see elect_one)
-        const bool elected = elect_one();
-        constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
-        constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
-        constexpr uint32_t QHALF = N * 128;
-        const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024), desc_p = smem_desc(base + OFF_P, SUB, 1024);
-        const uint64_t desc_k = smem_desc(base + OFF_K, 16, 1024), desc_v = smem_desc(base + OFF_V, SUB, 1024);
-        mbar_wait(bar(KB_QFULL), 0, abort_flag, p.dev_status);
-        int next_s = 0, next_pv = 0;
-        SpinGuard guard;
-        while (next_pv < T) {
-            bool progressed = false;
-            if (next_s < T && next_s <= next_pv + 1 && mbar_test_warp(bar(KB_KFULL), next_s & 1)) {
-                fence_after();
-                if (elected) {
+    } else if (warp == 1) {
+        if (kWarpIssues || lane == 0) {
+            const bool elected = kWarpIssues ? elect_one() : true;
+            auto ready = [&](int i, int n) { return kWarpIssues ? mbar_test_lane(bar(i), n & 1) : mbar_test(bar(i), n & 1); };
+            constexpr uint32_t IDESC_S = instr_desc2(N, 0, 0);    // A = K tile (K-major), B = Q (K-major)
+            constexpr uint32_t IDESC_PV = instr_desc2(N, 1, 1);   // A = V tile (MN-major: d contiguous), B = P^T (MN-major)
+            constexpr uint32_t QHALF = N * 128;
+            const uint64_t desc_q = smem_desc(base + OFF_Q, 16, 1024), desc_p = smem_desc(base + OFF_P, SUB, 1024);
+            const uint64_t desc_k = smem_desc(base + OFF_K, 16, 1024), desc_v = smem_desc(base + OFF_V, SUB, 1024);
+            mbar_wait(bar(KB_QFULL), 0, abort_flag, p.dev_status);
+            int next_s = 0, next_pv = 0;
+            SpinGuard guard;
+            while (next_pv < T) {
+                bool progressed = false;
+                if (next_s < T && next_s <= next_pv + 1 && ready(KB_KFULL, next_s)) {
+                    fence_after();
+                    if (elected) {
 #pragma unroll
-                    for (int k = 0; k < HD / 16; ++k)
-                        mma_ss(tmem + TM_S + (next_s & 1) * 64, desc_k + ((k >> 2) * SUB + (k & 3) * 32) / 16,
-                               desc_q + ((k >> 2) * QHALF + (k & 3) * 32) / 16, IDESC_S, k > 0);
-                    commit(bar(KB_SFULL + (next_s & 1)));
-                    commit(bar(KB_KEMPTY));
+                        for (int k = 0; k < HD / 16; ++k)
+                            mma_ss(tmem + TM_S + (next_s & 1) * 64, desc_k + ((k >> 2) * SUB + (k & 3) * 32) / 16,
+                                   desc_q + ((k >> 2) * QHALF + (k & 3) * 32) / 16, IDESC_S, k > 0);
+                        commit(bar(KB_SFULL + (next_s & 1)));
+                        commit(bar(KB_KEMPTY));
+                    }
+                    ++next_s;
+                    progressed = true;
                 }
-                ++next_s;
-                progressed = true;
-            }
-            if (next_pv < next_s && mbar_test_warp(bar(KB_PFULL), next_pv & 1) && mbar_test_warp(bar(KB_VFULL), next_pv & 1)) {
-                fence_after();
-                if (elected) {
+                if (next_pv < next_s && ready(KB_PFULL, next_pv) && ready(KB_VFULL, next_pv)) {
+                    fence_after();
+                    if (elected) {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (next_pv > 0 || k > 0));
-                    commit(bar(KB_PVDONE));
-                    commit(bar(KB_VEMPTY));
+                        for (int k = 0; k < BK / 16; ++k)
+                            mma_ss(tmem + TM_O, desc_v + k * 128, desc_p + k * 128, IDESC_PV, (next_pv > 0 || k > 0));
+                        commit(bar(KB_PVDONE));
+                        commit(bar(KB_VEMPTY));
+                    }
+                    ++next_pv;
+                    progressed = true;
                 }
-                ++next_pv;
-                progressed = true;
+                if (progressed) {
+                    guard.progress();
+                } else {
+                    const bool go_on = guard.tick(abort_flag, p.dev_status);
+                    if (kWarpIssues ? __any_sync(0xffffffffu, !go_on) : !go_on) break;
+                }
             }
-            if (progressed) guard.progress();
-            else if (__any_sync(0xffffffffu, !guard.tick(abort_flag, p.dev_status))) break;
         }
     } else {
         const int stid = tid - 64, wg = stid >> 7, c0 = wg * NH, st_w = stid & 127;

@@ -141,6 +141,14 @@ __device__ __forceinline__ void mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 }
 // a barrier as the whole warp sees it: one answer, so what depends on it stays warp-uniform
 __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)); }
+// the same, looked at by one lane (what it has acquired the others have behind the warp barrier): attend_skip_kernel<1> spills
+// 132 / 272 bytes (stores / loads) with it in keys_pair::run, 144 / 296 where all lanes look (us a layer, 5 x 32 heads of 500, 96
+// rows 27.3, 28.4)
+__device__ __forceinline__ bool mbar_test_lane(uint32_t bar, uint32_t parity) {
+    const bool done = __any_sync(0xffffffffu, (threadIdx.x & 31) == 0 && mbar_test(bar, parity));
+    __syncwarp();
+    return done;
+}
 // One arrival for the whole warp, behind what all its lanes have done before (each has fenced what the barrier is to publish).
 // Arrivals of 32 lanes at one barrier are taken one after the other: attend_skip_keys_kernel, whose softmax warps are alone on
 // the chain of a tile, is 0.15 to 0.25 us a launch shorter with one (us a pass: llada 768 246.4 -> 241.5, dream 768 204.6 ->
