@@ -1,10 +1,13 @@
 """GPU parity of the gate where rows are cut into s or s + 1 chunks, against the fp64 oracle (tolerances of test_gpu_gate)."""
+import numpy as np
 import pytest
 import torch
 
 import ec_synth as syn
 import oracle
-from test_gpu_gate import _compare, _run_gpu
+from _util import to_dev
+from test_gpu_gate import ENT_TOL, _compare, _run_gpu
+from test_gpu_gate_decode import _check as _check_decode, _logits
 
 pytestmark = pytest.mark.gpu
 
@@ -33,6 +36,31 @@ def test_rows_cut_into_unequal_numbers_of_chunks(dtype, R, rps, V, stride):
     o = oracle.entropy_gate(d["logits"], dtype, V, flags, 2.0, rps)
     for _ in range(2):   # (the tickets are zero again)
         _compare(_run_gpu(d["logits"], dtype, V, flags, 2.0, rps), o, 2.0)
+
+
+@pytest.mark.parametrize("dtype,R,rps,V,stride", [
+    (syn.BF16, 256, 32, 9001, 9008),    # 2 or 3 chunks, the change in the middle of the sixth sequence
+    (syn.F32, 42, 7, 40001, 40008),     # 14 or 15, in the sixth
+    (syn.BF16, 350, 35, 4100, 4104),    # 1 or 2, in the fourth
+    (syn.F32, 20, 4, 126464, 126464),   # 29 or 30, in the second
+])
+def test_decoding_and_metrics_where_a_sequence_has_rows_of_both_kinds(dtype, R, rps, V, stride):
+    """One CTA finishes a sequence; it counts the partials of rows with s and with s + 1 chunks."""
+    import paper_2603_18489_b200 as ec
+
+    lg = _logits(R, V, dtype, 62, n_spiked=R // 3, stride=stride)
+    masked = (np.random.Generator(np.random.PCG64(R)).random(R) < 0.7).astype(np.uint8)
+    for _ in range(2):
+        _check_decode(lg, dtype, V, masked, 0.9, 1.5, rps)
+    flags = syn.decoded_flags(R, max(1, rps // 2), rps, cfg_id=63)
+    o = oracle.entropy_gate(lg, dtype, V, flags, 1.5, rps)
+    m = oracle.gate_metrics(o["entropy"], o["conf"], flags, rps)
+    g = ec.ec_entropy_gate_metrics(to_dev(lg), V, rps, to_dev(flags), 1.5)
+    g = {k: v.cpu().numpy() for k, v in g.items()}
+    _compare(g, o, 1.5)
+    n_dec = flags.reshape(-1, rps).sum(axis=1)
+    assert np.all(np.abs(g["entropy_sum"].astype(np.float64) - m["entropy_sum"]) <= ENT_TOL * n_dec)
+    assert np.all(np.abs(g["max_conf"].astype(np.float64) - m["max_conf"]) <= 1e-5 * m["max_conf"])
 
 
 def _chunks_of_a_call(R, rps, V, dtype):

@@ -92,8 +92,8 @@ def test_first_maximum_among_the_vectors_of_a_thread(dtype, V):
 
 @pytest.mark.parametrize("B,Hq,Hkv,L,n", [(1, 4, 2, 200, 33), (2, 6, 2, 900, 44), (1, 3, 1, 130, 48), (8, 8, 8, 300, 65), (1, 12, 4, 64, 64)])
 def test_row_tiles_of_48_rows(B, Hq, Hkv, L, n):
-    """64-wide heads, two to four row tiles of at most 48 rows: remainders in the last tile, ragged key tiles, one key
-    tile and several; with and without fresh rows."""
+    """64-wide heads, two to four row tiles of at most 48 rows on mma.sync: remainders in the last tile, ragged key tiles, one
+    key tile and several; with and without fresh rows.  (8 x 300 with 65 rows runs on the dense kernel.)"""
     w = syn.Workload(101, "d64_tiles", syn.BF16, B, Hq, Hkv, 64, 0, L, 1, 0, 64)
     t = syn.attn_inputs(w, n, active_idx=syn.arbitrary_active_idx(B, L, n, seed=L + n), std_qk=0.9, std_v=0.5)
     _check(w, t)
@@ -102,12 +102,33 @@ def test_row_tiles_of_48_rows(B, Hq, Hkv, L, n):
 
 @pytest.mark.parametrize("B,Hq,Hkv,L", [(2, 4, 2, 1), (1, 2, 2, 64), (3, 6, 2, 65), (1, 4, 1, 200), (2, 8, 8, 449)])
 def test_recompute_steps_of_64_wide_heads(B, Hq, Hkv, L):
-    """K/V tiles by TMA out of the token-major fresh rows and out of the cache: one key, whole and ragged tiles, more
-    tiles than stages."""
+    """K/V tiles by TMA out of the token-major fresh rows and out of the cache: one key, whole and ragged tiles.  (3 x 65 and
+    2 x 449 run on the dense kernel, the others on mma.sync.)"""
     w = syn.Workload(102, "d64_full", syn.BF16, B, Hq, Hkv, 64, 0, L, 1, 0, 64)
     t = syn.attn_inputs(w, L, std_qk=0.9, std_v=0.5)
     _check(w, t)
     _check(w, t, refresh=False)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,n", [(64, 12, 4, 500, 40),    # one CTA walks all eight key tiles
+                                          (32, 12, 4, 500, 30),    # the same with row tiles of 48 rows
+                                          (16, 12, 4, 700, 48),    # three of 48, two CTAs of six and five tiles
+                                          (1, 1, 1, 2048, 2048),   # a recompute step: eight CTAs of four tiles
+                                          (1, 2, 2, 2000, 2000)])  # six CTAs, the last with two tiles, one of them ragged
+def test_mma_sync_kernel_refills_its_stages(B, Hq, Hkv, L, n):
+    """64-wide heads on mma.sync, four and more key tiles a CTA on three stages: an index list with fresh rows, the cache by
+    TMA without them, the fresh rows by TMA on a recompute step."""
+    import paper_2603_18489_b200 as ec
+
+    for fresh in (True, False):
+        got = ec.ec_attend_kernel_name(ec.make_desc(B, L, Hq, Hkv, 64, syn.BF16), n, fresh, n != L)
+        assert got.endswith("attend_mma_kernel"), got
+    w = syn.Workload(105, "d64_ring", syn.BF16, B, Hq, Hkv, 64, 0, L, 1, 0, 64)
+    idx = None if n == L else syn.arbitrary_active_idx(B, L, n, seed=L + n)
+    rows = None if n < L else sorted(set(np.random.Generator(np.random.PCG64(L)).choice(n, 40, replace=False).tolist() + [0, n - 1]))
+    t = syn.attn_inputs(w, n, active_idx=idx, std_qk=0.9, std_v=0.5)
+    _check(w, t, row_sel=rows)
+    _check(w, t, row_sel=rows, refresh=False)
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,D,L,n", [(1, 2, 1, 64, 70, 35), (1, 4, 4, 64, 256, 2), (1, 4, 4, 64, 256, 34), (1, 3, 1, 128, 33, 17),
