@@ -21,8 +21,7 @@
 // What bounds it: latency on partial steps of 64-wide heads (four sequences of 1000 keys, 48 rows, 12 query heads on 4:
 // 8.8 us a layer, against 14.9 with the refresh and the merge as launches of their own), the mma.sync rate (2048 flop
 // per clock and SM, measured) and the instructions around it on larger ones (36 sequences of 1500, 64 rows, no refresh: 45.3 us
-// when all threads issued the copies, 38.7 with TMA).  Recompute steps of 17 and more units and the partial steps that
-// prefers_mma names are attend_dense_kernel's.  Every wait
+// when all threads issued the copies, 38.7 with TMA).  What prefers_mma gives away is attend_dense_kernel's.  Every wait
 // is bounded: EC_ERR_TIMEOUT in dev_status, and a CTA whose wait gave up stores no output and no further cache rows.
 #include "ec_common.cuh"
 #include "ec_tc_ptx.cuh"

@@ -323,7 +323,7 @@ attend_dense_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
                     // P goes out in two parts, 48 columns and 16, so that three quarters of P V run while the rest is worked out:
                     // the chain of a row tile, scores - softmax - P V - scores, is what the other row tile has to cover.
                     // us a pass of 32 layers of 768 / 14 of 2 x 1531 (28 heads) / 2 of 8 x 4096 (at 1.5 GHz under the power
-                    // cap): one part 557 / 1095 / 3995, halves 528 / 1045 / 3785, three quarters 523 / 1035 / 3675.
+                    // cap): one part 530 / 1081 / 3910, halves 518 / 1055 / 3798, three quarters 516 / 1045 / 3726.
                     uint32_t sr[2][32];
                     ld32(tm_s + h * 64, sr[0]);
                     wait_ld<32>(sr[0]);
@@ -641,18 +641,19 @@ bool make_kv_map(CUtensorMap* map, const void* ptr, int hd, int batch, int n_kv_
 
 // How the launch is cut.  Units = (sequence, query head, row-tile pair); a unit walks over all T key tiles.  The
 // hardware deals the CTAs to the SMs in launch order, so the last units form a partial wave: `tail` units on `sms` SMs.
-// Cutting each of them along the keys into s CTAs, a cluster, fills that wave.  As many parts as fit at once and leave four
-// tiles each, if that takes four tiles off the wave: a launch of its own with its start and merge costs about as much.
-// us a layer by number of parts (the rule's in brackets): 4 units of 16 tiles (19 heads of 2048) 1: 57.9, 2: 52.4, (4): 49.5,
-// 8: 48.2; 12 of 21 (28 heads of 2600) 1: 105.6, 2: 100.8, 4: 97.4, (5): 96.7, 8: 95.4; 12 of 10 (32 heads of 1280) 1: 41.5,
-// (2): 39.9, 5: 39.4; 12 of 9 (1152) 1: 36.0, (2): 37.5; 40 of 12 (2 x 1531, 28 heads) 1: 71.8, 2: 69.4, (3): 69.0, 4 (two
-// rounds): 82.7; 20 of 12 (28 heads of 1500) 1: 46.7, 2: 44.2, (3): 43.6; 68 of 32 (32 heads of 4096) 1: 217, (2): 205, 3: 222.
+// Cutting each of them along the keys into s CTAs, a cluster, fills that wave.  As many parts as run at once and leave four
+// tiles each, if that takes four tiles off the wave: a launch of its own with its start and merge costs about as much.  (Nine
+// tiles beside whole units lose by it; the tests of cut units have them in two parts.)
+// us a layer by number of parts (the rule's in brackets): 4 units of 16 tiles (19 heads of 2048) 1: 55.8, 2: 49.6, (4): 46.5,
+// 8: 45.1; 12 of 21 (28 heads of 2600) 1: 100.7, 2: 94.7, 4: 90.9, (5): 90.0, 8: 88.6; 12 of 10 (32 heads of 1280) 1: 39.9, (2): 38.0,
+// 5: 37.6; 12 of 9 (1152) 1: 34.5, (2): 35.6; 40 of 12 (2 x 1531, 28 heads) 1: 67.4, 2: 64.8, (3): 64.6, 4 (two rounds): 79.2; 20
+// of 12 (28 heads of 1500) 1: 45.1, 2: 41.8, (3): 41.2, 4: 40.6; 68 of 32 (32 heads of 4096) 1: 213.5, (2): 205, 3 (two rounds): 217.5.
 struct DensePlan {
     int n_pairs, units, n_full, split;
 };
 // How many clusters of s CTAs of the cut launch the current device keeps resident at once.  A cluster stays inside a GPC, and
 // these need neither be alike nor hold a multiple of s SMs: 148 SMs taken as eight GPCs of 18 gave 48 clusters of three, of which
-// 45 ran and the others made a second round (8 heads of 1500, 48 units: 34.2 us a layer in three parts, 21.8 in two).
+// 45 ran and the others made a second round (8 heads of 1500, 48 units: 33.8 us a layer in three parts, 19.1 in two).
 // Asked once per device; without a device to ask, that assumption.
 template <int HD>
 int resident_clusters(int s) {
@@ -717,10 +718,10 @@ constexpr int kOneTileUnits = 16;
 // mma.sync).  Partial steps of at most 128 rows are mma.sync's unless they are large (a bound, below which the estimates are too
 // rough).  Then the estimates of both decide, mma.sync where it is 3 % ahead.  Of 2153 shapes timed (1 to 32 sequences, 129 to
 // 4096 keys, 8 to 1000 rows or all, 1 to 32 heads, groups of 1 to 8) 9 are more than 3 % slower here than on mma.sync, of 700
-// others 7; when recompute steps and partial ones of more than 128 rows were not asked about, 42 and 24.  us a layer, mma.sync / this kernel:
-// recompute steps 2 x 1024 with 24 heads on 8 51.5 / 31.4, 4 x 1000 94.1 / 47.5, 1 x 300 with 9 9.0 / 7.8, 32 x 129 with 24 on 8
-// 32.0 / 42.1; index lists 4 x 1000 with 24 on 8, 96 rows 23.9 / 13.6, 48 rows 16.2 / 13.3, 4 x 700 with 6 on 2, 129 rows 10.9 /
-// 13.6, 1 x 1000 with 9, 257 rows 9.2 / 14.8, 64 x 500 with 12 on 4, 40 rows 33.8 / 46.4.
+// others 7; when recompute steps and partial ones of more than 128 rows were not asked about, 42 and 24.
+// us a layer, mma.sync / this kernel: recompute steps 2 x 1024 with 24 heads on 8 51.5 / 31.4, 4 x 1000 94.1 / 47.5, 1 x 300 with 9
+// 9.0 / 7.8, 32 x 129 with 24 on 8 32.0 / 42.1; index lists 4 x 1000 with 24 on 8, 96 rows 23.9 / 13.6, 48 rows 16.2 / 13.3, 4 x 700
+// with 6 on 2, 129 rows 10.9 / 13.6, 1 x 1000 with 9, 257 rows 9.2 / 14.8, 64 x 500 with 12 on 4, 40 rows 33.8 / 46.4.
 double dense_us(const ec_attn_desc& d, int n_active, bool fresh) {   // 6 % rms
     const DensePlan pl = make_dense_plan(d, n_active);
     const int T = (d.ctx_len + BN - 1) / BN, sms = sm_count();

@@ -851,7 +851,9 @@ KeysPlan compute_keys_plan(const ec_attn_desc& d, int n_active, bool fresh) {
                 if (ctas > sms) continue;   // one CTA per SM: registers
                 // Cost in quarter tiles (about 0.25 us): the fresh tiles arrive early (they are small and mostly in L2), so
                 // on a shared CTA they count a quarter of a cache tile.  96 slots: a tile takes 1.3 us where the memory
-                // system does not set the pace (48: 1.0), and the launch around the tiles up to 3 us more.
+                // system does not set the pace (48, and 64 by the same price: 1.0), and the launch around the tiles up to 3
+                // us more.  (Fitted when one softmax warpgroup, two with 96 slots, worked on a tile; the launches have become
+                // up to 15 % shorter since, and the prices were not fitted again.)
                 const long long cost = (t.n_slots == 96 ? 5LL * tps + 13 : 4LL * tps) + ((fresh && !own) ? t.n_extra : 0);
                 if (best_cost >= 0 && (cost > best_cost || (cost == best_cost && ctas <= best_ctas))) continue;
                 const int fit = resident_clusters(t.n_slots, c, t.smem_bytes);   // (-1: no device to ask, keep the estimate)
@@ -958,9 +960,8 @@ bool attend_skip_keys_supported(const ec_attn_desc& d, int n_active, bool fresh)
 
 void attend_skip_keys_describe(const ec_attn_desc& d, int n_active, bool fresh, char* buf, size_t len) {
     const KeysPlan pl = make_keys_plan(d, n_active, fresh);
-    snprintf(buf, len, "attend_skip_keys_kernel<%d> grid=(%d,%d) cluster=%d ring_slots=%d smem=%u ctas_per_sm=%d fresh_tiles=%d",
-             pl.n_slots, pl.n_splits, d.batch * d.n_kv_heads * pl.n_sub, pl.n_splits, pl.n_stages, pl.smem_bytes, 1,
-             pl.n_extra);
+    snprintf(buf, len, "attend_skip_keys_kernel<%d> grid=(%d,%d) cluster=%d ring_slots=%d smem=%u ctas_per_sm=1 fresh_tiles=%d",
+             pl.n_slots, pl.n_splits, d.batch * d.n_kv_heads * pl.n_sub, pl.n_splits, pl.n_stages, pl.smem_bytes, pl.n_extra);
 }
 
 cudaError_t launch_attend_skip_keys(const AttendArgs& a, const void* k_new, const void* v_new, const int32_t* active_idx,
