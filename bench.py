@@ -56,19 +56,19 @@ K64_WORKLOADS = ("c4_llada_l2048", "c5_llada_l4096", "c5_llada_l4096_b8", "c5_dr
 NCU_TRAFFIC = {
     "attend_skip": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_keys_tc.cu",),
-         "sha256": "c8f3be6703ae4e5eda5268ba7accce752972fede0dde7fbb54dbd349b9a77406",
-         "bytes_per_launch": {"c5_llada_l4096": 68770000}},
+         "sha256": "5a7dcc92491833645fa51fb0c39931ce520cd9abeeec83e12e01bf59791d29b2",
+         "bytes_per_launch": {"c5_llada_l4096": 68000000}},
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_skip_tc.cu", "paper_2603_18489_b200/csrc/ec_skip_keys_pair.cuh"),
-         "sha256": "ba6748597d440eb2e9986a220077697c6a28e35f238d4fe82a32fc36a356233e",
-         "bytes_per_launch": {"c5_llada_l4096_b8": 557030000}}],
+         "sha256": "9cfdcbeffa857a85d0e0e8234fb8aab7bfe00f7a79e81b8ccb9acffd55a003a6",
+         "bytes_per_launch": {"c5_llada_l4096_b8": 556700000}}],
     "attend_dense": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_attend_dense_tc.cu",),
-         "sha256": "f0ec912f389b20564c6f873dd21a1fa3844a972a0c04c76c89b1b96af0ab27cd",
-         "bytes_per_launch": {"c5_llada_l4096": 148540000}}],
+         "sha256": "734f8adbf7a22d464817271f5d71509462e1b3c8c54d94a2ad69aa470e1daaa4",
+         "bytes_per_launch": {"c5_llada_l4096": 147680000}}],
     "entropy_gate": [
         {"sources": ("paper_2603_18489_b200/csrc/ec_gate.cu",),
-         "sha256": "660af8feb5cbc456545018c79a08fa0ef91987e62268a69798aa2e8e4a489fe5",
-         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65400000}}],
+         "sha256": "fd98ebf1c1140d3108ad75bacf6aa61ffa990ec1098a220d5d9009e4c68b3ab5",
+         "bytes_per_launch": {"c5_llada_l4096": 8150000, "c5_llada_l4096_b8": 65000000}}],
 }
 
 
